@@ -1,10 +1,12 @@
-"""Thin ctypes binding of libap_b200.so: argument marshalling only.
+"""Thin binding of libap_b200.so: argument marshalling only.
 
 Every function has the name of the C entry point it calls (see include/ap.h)
 and takes torch tensors that live on the CUDA device (PyTorch is used for
 device memory and streams only).  All arithmetic happens inside the library's
-kernels.  If the shared library has not been built the import of this module
-fails: there is no fallback path.
+kernels.  The entry points that run once per batch (averaging, selection,
+forward, backward) are marshalled by a native module, _ap_call.so, the others
+by ctypes.  If either shared object has not been built the import of this
+module fails: there is no fallback path.
 """
 from __future__ import annotations
 
@@ -153,6 +155,19 @@ def _check(status: int, where: str) -> None:
         raise ApError(status, where)
 
 
+try:
+    from . import _ap_call as _call
+except ImportError as e:
+    raise ImportError("_ap_call.so is missing or does not match this torch: build it with "
+                      "`python -m paper_2012_02030_b200.build` (there is no fallback implementation)") from e
+_call.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in EXPORTS}, _check)
+
+
+def _tiles_address(tiles):
+    """Address of a tile list's descriptor (None: no list)."""
+    return None if tiles is None else ctypes.addressof(tiles.c)
+
+
 def _dev(t: torch.Tensor, name: str) -> torch.Tensor:
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError("%s must be a contiguous CUDA tensor" % name)
@@ -223,53 +238,23 @@ class Tiles:
 
 
 def ap_accumulate_attention(acc, Q, K, bias=None, causal=False, scale=0.0, stream=None) -> None:
-    _dev(acc, "acc"), _dev(Q, "Q"), _dev(K, "K")
-    B, H, Lq, d = Q.shape
-    Lk = K.shape[2]
-    if K.shape != (B, H, Lk, d) or acc.shape != (H, Lq, Lk) or acc.dtype != torch.float32 or K.dtype != Q.dtype:
-        raise ValueError("shape/dtype mismatch")
-    if bias is not None and (_dev(bias, "bias").shape != (H, Lq, Lk) or bias.dtype != torch.float32):
-        raise ValueError("bias must be float32 [H,Lq,Lk]")
-    _check(lib.ap_accumulate_attention(_ptr(acc), _ptr(Q), _ptr(K), _ptr(bias), B, H, Lq, Lk, d,
-                                       _dtype_code(Q), int(bool(causal)), float(scale), _stream(stream)),
-           "ap_accumulate_attention")
+    _call.accumulate(acc, Q, K, bias, causal, scale, stream)
 
 
 def ap_accumulate_attention_entmax15(acc, Q, K, bias=None, causal=False, scale=0.0, stream=None) -> None:
-    _dev(acc, "acc"), _dev(Q, "Q"), _dev(K, "K")
-    B, H, Lq, d = Q.shape
-    Lk = K.shape[2]
-    if K.shape != (B, H, Lk, d) or acc.shape != (H, Lq, Lk) or acc.dtype != torch.float32 or K.dtype != Q.dtype:
-        raise ValueError("shape/dtype mismatch")
-    if bias is not None and (_dev(bias, "bias").shape != (H, Lq, Lk) or bias.dtype != torch.float32):
-        raise ValueError("bias must be float32 [H,Lq,Lk]")
-    _check(lib.ap_accumulate_attention_entmax15(_ptr(acc), _ptr(Q), _ptr(K), _ptr(bias), B, H, Lq, Lk, d,
-                                                _dtype_code(Q), int(bool(causal)), float(scale), _stream(stream)),
-           "ap_accumulate_attention_entmax15")
-
-
-def _build_mask(fn, name, acc, keep_frac, causal, keep_diag, mask, tiles, nnz_per_head, workspace, stream) -> None:
-    _dev(acc, "acc")
-    H, Lq, Lk = acc.shape
-    if acc.dtype != torch.float32:
-        raise ValueError("acc must be float32")
-    if workspace is None:
-        workspace = torch.empty(ap_build_mask_workspace_bytes(H, Lq, Lk), dtype=torch.uint8, device=acc.device)
-    _check(fn(_ptr(acc), H, Lq, Lk, float(keep_frac), int(bool(causal)), int(bool(keep_diag)),
-              _ptr(mask), ctypes.byref(tiles.c) if tiles is not None else None,
-              _ptr(nnz_per_head), _ptr(workspace), workspace.numel(), _stream(stream)), name)
+    _call.accumulate_entmax15(acc, Q, K, bias, causal, scale, stream)
 
 
 def ap_build_mask(acc, keep_frac, causal=False, keep_diag=True, mask=None, tiles: Tiles | None = None,
                   nnz_per_head=None, workspace=None, stream=None) -> None:
-    _build_mask(lib.ap_build_mask, "ap_build_mask", acc, keep_frac, causal, keep_diag, mask, tiles, nnz_per_head,
-                workspace, stream)
+    _call.build_mask(0, acc, keep_frac, causal, keep_diag, 0, mask, _tiles_address(tiles), nnz_per_head, workspace,
+                     stream)
 
 
 def ap_build_mask_layer(acc, keep_frac, causal=False, keep_diag=True, mask=None, tiles: Tiles | None = None,
                         nnz_per_head=None, workspace=None, stream=None) -> None:
-    _build_mask(lib.ap_build_mask_layer, "ap_build_mask_layer", acc, keep_frac, causal, keep_diag, mask, tiles,
-                nnz_per_head, workspace, stream)
+    _call.build_mask(1, acc, keep_frac, causal, keep_diag, 0, mask, _tiles_address(tiles), nnz_per_head, workspace,
+                     stream)
 
 
 AP_MASK_PER_LAYER, AP_MASK_KEEP_TIES = 1, 2
@@ -277,16 +262,8 @@ AP_MASK_PER_LAYER, AP_MASK_KEEP_TIES = 1, 2
 
 def ap_build_mask_ex(acc, keep_frac, causal=False, keep_diag=True, flags=0, mask=None, tiles: Tiles | None = None,
                      nnz_per_head=None, workspace=None, stream=None) -> None:
-    _dev(acc, "acc")
-    H, Lq, Lk = acc.shape
-    if acc.dtype != torch.float32:
-        raise ValueError("acc must be float32")
-    if workspace is None:
-        workspace = torch.empty(ap_build_mask_workspace_bytes(H, Lq, Lk), dtype=torch.uint8, device=acc.device)
-    _check(lib.ap_build_mask_ex(_ptr(acc), H, Lq, Lk, float(keep_frac), int(bool(causal)), int(bool(keep_diag)),
-                                int(flags), _ptr(mask), ctypes.byref(tiles.c) if tiles is not None else None,
-                                _ptr(nnz_per_head), _ptr(workspace), workspace.numel(), _stream(stream)),
-           "ap_build_mask_ex")
+    _call.build_mask(2, acc, keep_frac, causal, keep_diag, int(flags), mask, _tiles_address(tiles), nnz_per_head,
+                     workspace, stream)
 
 
 def ap_pool_scores(acc, block: int, causal=False, pooled=None, stream=None):
@@ -352,31 +329,11 @@ def ap_dense_tiles(tiles: Tiles, causal=False, stream=None) -> None:
 
 
 def ap_sparse_attention_fwd(Q, K, V, tiles: Tiles, O=None, scale=0.0, stream=None):
-    _dev(Q, "Q"), _dev(K, "K"), _dev(V, "V")
-    B, H, Lq, d = Q.shape
-    Lk = K.shape[2]
-    if K.shape != (B, H, Lk, d) or V.shape != K.shape or K.dtype != Q.dtype or V.dtype != Q.dtype:
-        raise ValueError("shape/dtype mismatch")
-    if O is None:
-        O = torch.empty_like(Q)
-    _check(lib.ap_sparse_attention_fwd(_ptr(Q), _ptr(K), _ptr(V), ctypes.byref(tiles.c), _ptr(_dev(O, "O")),
-                                       B, H, Lq, Lk, d, _dtype_code(Q), float(scale), _stream(stream)),
-           "ap_sparse_attention_fwd")
-    return O
+    return _call.fwd(Q, K, V, _tiles_address(tiles), O, scale, stream)
 
 
 def ap_sparse_attention_entmax15_fwd(Q, K, V, tiles: Tiles, O=None, scale=0.0, stream=None):
-    _dev(Q, "Q"), _dev(K, "K"), _dev(V, "V")
-    B, H, Lq, d = Q.shape
-    Lk = K.shape[2]
-    if K.shape != (B, H, Lk, d) or V.shape != K.shape or K.dtype != Q.dtype or V.dtype != Q.dtype:
-        raise ValueError("shape/dtype mismatch")
-    if O is None:
-        O = torch.empty_like(Q)
-    _check(lib.ap_sparse_attention_entmax15_fwd(_ptr(Q), _ptr(K), _ptr(V), ctypes.byref(tiles.c), _ptr(_dev(O, "O")),
-                                                B, H, Lq, Lk, d, _dtype_code(Q), float(scale), _stream(stream)),
-           "ap_sparse_attention_entmax15_fwd")
-    return O
+    return _call.fwd_entmax15(Q, K, V, _tiles_address(tiles), O, scale, stream)
 
 
 def ap_sparse_attention_bwd_workspace_bytes(B: int, H: int, Lq: int, Lk: int) -> int:
@@ -385,24 +342,7 @@ def ap_sparse_attention_bwd_workspace_bytes(B: int, H: int, Lq: int, Lk: int) ->
 
 def ap_sparse_attention_bwd(Q, K, V, O, dO, tiles: Tiles, dQ=None, dK=None, dV=None, scale=0.0, workspace=None,
                             stream=None):
-    for t, name in ((Q, "Q"), (K, "K"), (V, "V"), (O, "O"), (dO, "dO")):
-        _dev(t, name)
-    B, H, Lq, d = Q.shape
-    Lk = K.shape[2]
-    if (K.shape != (B, H, Lk, d) or V.shape != K.shape or O.shape != Q.shape or dO.shape != Q.shape
-            or any(t.dtype != Q.dtype for t in (K, V, O, dO))):
-        raise ValueError("shape/dtype mismatch")
-    dQ = torch.empty_like(Q) if dQ is None else _dev(dQ, "dQ")
-    dK = torch.empty_like(K) if dK is None else _dev(dK, "dK")
-    dV = torch.empty_like(V) if dV is None else _dev(dV, "dV")
-    if workspace is None:
-        workspace = torch.empty(ap_sparse_attention_bwd_workspace_bytes(B, H, Lq, Lk), dtype=torch.uint8,
-                                device=Q.device)
-    _check(lib.ap_sparse_attention_bwd(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(dO), ctypes.byref(tiles.c),
-                                       _ptr(dQ), _ptr(dK), _ptr(dV), B, H, Lq, Lk, d, _dtype_code(Q), float(scale),
-                                       _ptr(workspace), workspace.numel(), _stream(stream)),
-           "ap_sparse_attention_bwd")
-    return dQ, dK, dV
+    return _call.bwd(Q, K, V, O, dO, _tiles_address(tiles), dQ, dK, dV, scale, workspace, stream)
 
 
 def ap_sparse_attention_fwd_host(hQ, hK, hV, tiles: Tiles, hO, dQ, dK, dV, dO, scale=0.0, stream=None):

@@ -1,4 +1,5 @@
-"""Builds libap_b200.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libap_b200.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _ap_call.so (the
+Python binding's native call path) with the host compiler."""
 from __future__ import annotations
 
 import concurrent.futures
@@ -6,11 +7,14 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libap_b200.so")
+CALL_SRC = os.path.join(CSRC, "ap_call.cpp")
+CALL_LIB = os.path.join(HERE, "_ap_call.so")
 OBJ_DIR = os.path.join(HERE, "build")
 
 NVCC_FLAGS = [
@@ -29,6 +33,21 @@ def _nvcc() -> str:
 
 def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
+
+
+def call_command(target: str):
+    """Host-compiler command of the call path: CPython and torch headers, torch's own ABI."""
+    import torch
+
+    base = os.path.dirname(torch.__file__)
+    libs = os.path.join(base, "lib")
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+            "-I", os.path.join(ROOT, "include"), "-isystem", sysconfig.get_paths()["include"],
+            "-isystem", os.path.join(base, "include"), "-isystem", os.path.join(cuda, "include"),
+            CALL_SRC, "-o", target, "-L", libs, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python",
+            "-Wl,-rpath," + libs]
 
 
 def _stale(target: str, deps) -> bool:
@@ -57,6 +76,11 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         if r.returncode != 0:
             raise RuntimeError("nvcc failed:\n%s\n%s\n%s" % (" ".join(cmd), r.stdout, r.stderr))
         return r.stdout + r.stderr
+
+    if force or _stale(CALL_LIB, [CALL_SRC, os.path.join(ROOT, "include", "ap.h"), os.path.abspath(__file__)]):
+        call_tmp = CALL_LIB + ".%d.tmp" % os.getpid()
+        run(call_command(call_tmp))
+        os.replace(call_tmp, CALL_LIB)
 
     with concurrent.futures.ThreadPoolExecutor(max_workers=min(8, max(1, len(jobs)))) as ex:
         outs = list(ex.map(run, jobs))
