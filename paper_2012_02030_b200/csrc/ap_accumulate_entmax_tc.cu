@@ -76,18 +76,6 @@ struct Barriers {
   int more[kMaxNewton + 2];  // more[s] != 0: some row still moved after sweep s
 };
 
-__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
-                                              unsigned *err) {
-  for (uint32_t i = 0; i < kMaxPolls; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (i > 64) __nanosleep(64);
-  }
-  *abort_flag = 1;
-  atomicOr(err, kDevErrTimeout);
-  return false;
-}
-
 // Sweep s + 1 is the last one when sweep s was a sweep of the iteration after which nothing moved.
 __device__ __forceinline__ bool last_follows(const Barriers *bars, int s) {
   return s >= 1 && (s >= kMaxNewton || *reinterpret_cast<const volatile int *>(&bars->more[s]) == 0);
@@ -142,6 +130,7 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
   tc_fence_after_sync();
   const uint32_t tmem = bars->tmem_base;
   volatile int *abort_flag = &bars->abort_flag;
+  const Waiter wait{abort_flag, err, kMaxPolls};
 
   if (warp == 8) {
     // ------------------------------------------------------------ TMA producer
@@ -157,14 +146,14 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
           const uint32_t ph = (uint32_t)(v / C::kStages) & 1u;
           const int kt = vv / Bc, b = b0 + vv % Bc;
           if (bias_by_tma && vv % Bc == 0) {
-            if (!wait_or_abort(&bars->bias_empty, ((uint32_t)tl & 1u) ^ 1u, abort_flag, err)) { ok = false; break; }
+            if (!wait.one(&bars->bias_empty, ((uint32_t)tl & 1u) ^ 1u)) { ok = false; break; }
             mbar_arrive_expect_tx(&bars->bias_full, kBiasBytes);
 #pragma unroll
             for (int q = 0; q < 4; ++q)
               tma_load_3d(bias_s + q * (kBiasBytes / 4), &map_bias, &bars->bias_full, kt * kTile + 32 * q, qt * kTile, h);
             ++tl;
           }
-          if (!wait_or_abort(&bars->in_empty[st], ph ^ 1u, abort_flag, err)) { ok = false; break; }
+          if (!wait.one(&bars->in_empty[st], ph ^ 1u)) { ok = false; break; }
           unsigned char *q_s = smem + (2 * st) * C::kTileBytes, *k_s = q_s + C::kTileBytes;
           mbar_arrive_expect_tx(&bars->in_full[st], 2 * C::kTileBytes);
 #pragma unroll
@@ -174,7 +163,7 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
           }
         }
         if (!ok || last) break;
-        if (!wait_or_abort(&bars->decided, (uint32_t)sw & 1u, abort_flag, err)) break;
+        if (!wait.one(&bars->decided, (uint32_t)sw & 1u)) break;
         last = last_follows(bars, sw);
       }
       if (*abort_flag) {  // winding down: let the copies in flight land (bounded)
@@ -194,8 +183,8 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
           const int st = v % C::kStages;
           const uint32_t ph = (uint32_t)(v / C::kStages) & 1u;
           const int buf = v & 1;
-          if (!wait_or_abort(&bars->in_full[st], ph, abort_flag, err)) { ok = false; break; }
-          if (!wait_or_abort(&bars->s_empty[buf], ((uint32_t)(v >> 1) & 1u) ^ 1u, abort_flag, err)) { ok = false; break; }
+          if (!wait.one(&bars->in_full[st], ph)) { ok = false; break; }
+          if (!wait.one(&bars->s_empty[buf], ((uint32_t)(v >> 1) & 1u) ^ 1u)) { ok = false; break; }
           tc_fence_after_sync();
           const unsigned char *q_s = smem + (2 * st) * C::kTileBytes, *k_s = q_s + C::kTileBytes;
 #pragma unroll
@@ -209,7 +198,7 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
           mma_commit(&bars->s_full[buf]);
         }
         if (!ok || last) break;
-        if (!wait_or_abort(&bars->decided, (uint32_t)sw & 1u, abort_flag, err)) break;
+        if (!wait.one(&bars->decided, (uint32_t)sw & 1u)) break;
         last = last_follows(bars, sw);
       }
     }
@@ -243,7 +232,7 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         const int j0 = kt * kTile + 64 * wg;  // first column of this thread's slice
         if (b == 0) {  // new key tile: fetch this thread's bias slice once for all samples
           if (bias_by_tma) {
-            ok = wait_or_abort(&bars->bias_full, (uint32_t)tl & 1u, abort_flag, err);
+            ok = wait(&bars->bias_full, (uint32_t)tl & 1u);
             if (!ok) break;
             ++tl;
 #pragma unroll
@@ -278,7 +267,7 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         // statistics of (sample b, this half of the row): fresh at the first key tile of a sweep
         float2 st = kt == 0 ? make_float2(kind == 0 ? -CUDART_INF_F : 0.f, 0.f) : my_stats[b * 128];
         float cnt = (kind != 1 || kt == 0) ? 0.f : my_cnt[b * 128];
-        ok = wait_or_abort(&bars->s_full[buf], (uint32_t)(v >> 1) & 1u, abort_flag, err);
+        ok = wait(&bars->s_full[buf], (uint32_t)(v >> 1) & 1u);
         if (!ok) break;
         tc_fence_after_sync();
         const int n_valid = max(0, min(64, jend - j0));  // columns of this slice inside the row's domain
@@ -383,7 +372,7 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       if (!ok || last) break;
       // ---- end of a sweep: the two halves of every row meet, every (sample, row) takes its step
       mbar_arrive(&bars->sweep_done);
-      ok = wait_or_abort(&bars->sweep_done, (uint32_t)sw & 1u, abort_flag, err);
+      ok = wait(&bars->sweep_done, (uint32_t)sw & 1u);
       if (!ok) break;
       bool moved = false;
       for (int b = 0; b < Bc; ++b) {
@@ -406,7 +395,7 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
       }
       if (moved && row_ok) *reinterpret_cast<volatile int *>(&bars->more[sw]) = 1;
       mbar_arrive(&bars->decided);  // release: the flag and the old statistics' last reads precede it
-      ok = wait_or_abort(&bars->decided, (uint32_t)sw & 1u, abort_flag, err);
+      ok = wait(&bars->decided, (uint32_t)sw & 1u);
       if (!ok) break;
       last = last_follows(bars, sw);
     }

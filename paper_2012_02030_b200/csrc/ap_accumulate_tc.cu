@@ -122,28 +122,6 @@ unsigned *turn_words() {
   return base[dev] + (size_t)(next.fetch_add(1) % kTurnSets) * kTurnWords;
 }
 
-// Bounded wait that also gives up as soon as another thread of the CTA has.
-__device__ __noinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, volatile int *abort_flag, unsigned *err,
-                                           uint32_t max_polls) {
-  for (uint32_t i = 0; i < max_polls; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (i > 1024) __nanosleep(64);
-  }
-  *abort_flag = 1;
-  atomicOr(err, kDevErrTimeout);
-  return false;
-}
-
-// The same wait for a whole (converged) warp: one lane polls - 32 lanes polling one barrier would
-// serialise - and the outcome is shared.
-__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, int lane, volatile int *abort_flag,
-                                          unsigned *err, uint32_t max_polls) {
-  bool ok = true;
-  if (lane == 0 && !mbar_try_wait(bar, parity)) ok = wait_or_abort(bar, parity, abort_flag, err, max_polls);
-  return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-}
-
 // dbg_skip != 0 (test hook): the copies of the first visit are never issued, so the MMA issuer's
 // first wait runs out and the CTA leaves through its error path.
 // kChunked: the instantiation for launches whose samples are cut into chunks (see below); a
@@ -204,6 +182,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   tc_fence_after_sync();
   const uint32_t tmem = bars->tmem_base;
   volatile int *abort_flag = &bars->abort_flag;
+  const Waiter wait{abort_flag, err, max_polls};
 
   if (warp == 8) {
     // ------------------------------------------------------------ TMA producer
@@ -221,14 +200,14 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           // bias tile of the key tile whose visits start here; the buffer is free once all
           // softmax threads have copied the previous tile to registers
           const int tl = v / Bc;
-          if (!wait_or_abort(&bars->bias_empty, ((uint32_t)tl & 1u) ^ 1u, abort_flag, err, max_polls)) break;
+          if (!wait.one(&bars->bias_empty, ((uint32_t)tl & 1u) ^ 1u)) break;
           mbar_arrive_expect_tx(&bars->bias_full, kBiasBytes);
 #pragma unroll
           for (int q = 0; q < 4; ++q)
             tma_load_3d(bias_s + q * (kBiasBytes / 4), &map_bias, &bars->bias_full, kt * kTile + 32 * q, qt * kTile, h);
           bias_loads = tl + 1;
         }
-        if (!wait_or_abort(&bars->in_empty[st], ph ^ 1u, abort_flag, err, max_polls)) break;
+        if (!wait.one(&bars->in_empty[st], ph ^ 1u)) break;
         if (dbg_skip != 0 && v == 0) continue;
         unsigned char *q_s = smem + (2 * st) * C::kTileBytes, *k_s = q_s + C::kTileBytes;
         mbar_arrive_expect_tx(&bars->in_full[st], 2 * C::kTileBytes);
@@ -254,8 +233,8 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         const int st = v % C::kStages;
         const uint32_t ph = (uint32_t)(v / C::kStages) & 1u;
         const int buf = v & 1;
-        if (!wait_or_abort(&bars->in_full[st], ph, abort_flag, err, max_polls)) break;
-        if (!wait_or_abort(&bars->s_empty[buf], ((uint32_t)(v >> 1) & 1u) ^ 1u, abort_flag, err, max_polls)) break;
+        if (!wait.one(&bars->in_full[st], ph)) break;
+        if (!wait.one(&bars->s_empty[buf], ((uint32_t)(v >> 1) & 1u) ^ 1u)) break;
         tc_fence_after_sync();
         const unsigned char *q_s = smem + (2 * st) * C::kTileBytes, *k_s = q_s + C::kTileBytes;
 #pragma unroll
@@ -295,7 +274,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     auto fetch_bias = [&](int kt, int tl) {
       const int j0 = kt * kTile + 64 * wg;
       if (bias_by_tma) {
-        ok = warp_wait(&bars->bias_full, (uint32_t)tl & 1u, lane, abort_flag, err, max_polls);
+        ok = wait(&bars->bias_full, (uint32_t)tl & 1u);
         if (!ok) return;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -331,7 +310,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // (one arrival per warp: 256 threads arriving one by one would take longer than a visit's MMAs).
     auto take_s = [&](int v, uint32_t (&xs)[64]) {
       const int buf = v & 1;
-      ok = warp_wait(&bars->s_full[buf], (uint32_t)(v >> 1) & 1u, lane, abort_flag, err, max_polls);
+      ok = wait(&bars->s_full[buf], (uint32_t)(v >> 1) & 1u);
       if (!ok) return;
       tc_fence_after_sync();
       tmem_ld32(s_addr + 128 * buf, xs);
@@ -398,7 +377,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       tc_fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->sweep1_done);
-      ok = warp_wait(&bars->sweep1_done, 0, lane, abort_flag, err, max_polls);
+      ok = wait(&bars->sweep1_done, 0);
       tc_fence_after_sync();
     }
 

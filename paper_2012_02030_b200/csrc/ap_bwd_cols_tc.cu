@@ -115,7 +115,7 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = sh->tmem_base;
-  const Waiter wait{lane, &sh->abort_flag, err, max_polls};
+  const Waiter wait{&sh->abort_flag, err, max_polls};
   // accumulators of item n: dV at acc, dK at acc + D
   auto acc_of = [&](uint32_t n) { return tmem + kTmemAcc + (C::kAccBufs == 2u ? 128u * (n & 1u) : 0u); };
 

@@ -126,7 +126,7 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = sh->tmem_base;
-  const Waiter wait{lane, &sh->abort_flag, err, max_polls};
+  const Waiter wait{&sh->abort_flag, err, max_polls};
 
   if (warp == 8) {
     // ------------------------------------------------------------ producer

@@ -114,18 +114,6 @@ __device__ __forceinline__ Round decode_round(const RawRound &r) {
   return rd;
 }
 
-__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
-                                              unsigned *err) {
-  for (uint32_t i = 0; i < kMaxPolls; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (i > 64) __nanosleep(64);
-  }
-  *abort_flag = 1;
-  atomicOr(err, kDevErrTimeout);
-  return false;
-}
-
 __device__ __forceinline__ bool last_follows(const Barriers *bars, int s) {
   return s >= 1 && (s >= kMaxNewton || *reinterpret_cast<const volatile int *>(&bars->more[s]) == 0);
 }
@@ -208,6 +196,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
   tc_fence_after_sync();
   const uint32_t tmem = bars->tmem_base;
   volatile int *abort_flag = &bars->abort_flag;
+  const Waiter wait{abort_flag, err, kMaxPolls};
 
   if (T == 0) {
     // nothing kept in these 128 rows: the output is exactly 0
@@ -261,7 +250,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         vv_next = vv_next + 1 == T ? 0 : vv_next + 1;
         next = load_round(round_rows, round_info, t0 + vv_next);
         const int st = v % C::kStages;
-        if (!wait_or_abort(&bars->in_empty[st], ((uint32_t)(v / C::kStages) & 1u) ^ 1u, abort_flag, err)) return false;
+        if (!wait.one(&bars->in_empty[st], ((uint32_t)(v / C::kStages) & 1u) ^ 1u)) return false;
         copy_rows(rd, smem + C::kKOffset + st * C::kTileBytes, &maps.k16, &maps.k128, &bars->in_full[st]);
         ++v;
         return true;
@@ -269,7 +258,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
       auto copy_v = [&](int vv) -> bool {  // V of round vv, the v_loads-th visit of the last sweep
         const int st = v_loads % C::kVStages;
         const Round rd = decode_round(load_round(round_rows, round_info, t0 + vv));
-        if (!wait_or_abort(&bars->v_empty[st], ((uint32_t)(v_loads / C::kVStages) & 1u) ^ 1u, abort_flag, err)) return false;
+        if (!wait.one(&bars->v_empty[st], ((uint32_t)(v_loads / C::kVStages) & 1u) ^ 1u)) return false;
         copy_rows(rd, smem + C::kVOffset + st * C::kTileBytes, &maps.v16, &maps.v128, &bars->v_full[st]);
         ++v_loads;
         return true;
@@ -283,7 +272,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         // (a participant of the barrier: a short sweep could otherwise complete the next phase
         // before this thread has seen this one)
         mbar_arrive(&bars->decided);
-        if (!wait_or_abort(&bars->decided, (uint32_t)sw & 1u, abort_flag, err)) break;
+        if (!wait.one(&bars->decided, (uint32_t)sw & 1u)) break;
         const bool last = last_follows(bars, sw);
         for (int vv = 0; vv < T && ok; ++vv) {
           if (vv >= n_ahead) ok = copy_k();
@@ -306,7 +295,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     if (lane == 0) {
       constexpr uint32_t idesc_pv = idesc_bf16_f32(128, D, false, true, kF16);
       const uint32_t q_addr = smem_u32(smem), k_addr = smem_u32(smem + C::kKOffset), v_addr = smem_u32(smem + C::kVOffset);
-      bool ok = wait_or_abort(&bars->q_full, 0u, abort_flag, err);
+      bool ok = wait.one(&bars->q_full, 0u);
       int v = 0;  // visits whose S has been issued
       auto ng_of = [&](int vv) { return (int)(__ldg(round_info + t0 + vv) & 15u); };
       uint32_t info_next = __ldg(round_info + t0);  // used one visit later: the load stays in flight
@@ -316,10 +305,10 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         const uint32_t idesc_qk = idesc_bf16_f32(128, 16 * (int)(info_next & 15u), false, false, kF16);
         vv_next = vv_next + 1 == T ? 0 : vv_next + 1;
         info_next = __ldg(round_info + t0 + vv_next);
-        if (!wait_or_abort(&bars->in_full[st], (uint32_t)(v / C::kStages) & 1u, abort_flag, err)) return false;
+        if (!wait.one(&bars->in_full[st], (uint32_t)(v / C::kStages) & 1u)) return false;
         // S[buf] was read (and, in the last sweep, its P consumed by a product issued earlier by
         // this thread: products execute in issue order) kSBufs visits ago
-        if (!wait_or_abort(&bars->s_empty[buf], ((uint32_t)(v / kSBufs) & 1u) ^ 1u, abort_flag, err)) return false;
+        if (!wait.one(&bars->s_empty[buf], ((uint32_t)(v / kSBufs) & 1u) ^ 1u)) return false;
         tc_fence_after_sync();
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {
@@ -336,8 +325,8 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
       // threads have arrived; one contraction step of 16 keys per group; then the V stage is free
       auto issue_pv = [&](int u, int j) -> bool {
         const int sb = u % kSBufs, sv = j % C::kVStages, ng_u = ng_of(j);
-        if (!wait_or_abort(&bars->v_full[sv], (uint32_t)(j / C::kVStages) & 1u, abort_flag, err)) return false;
-        if (!wait_or_abort(&bars->s_empty[sb], (uint32_t)(u / kSBufs) & 1u, abort_flag, err)) return false;
+        if (!wait.one(&bars->v_full[sv], (uint32_t)(j / C::kVStages) & 1u)) return false;
+        if (!wait.one(&bars->s_empty[sb], (uint32_t)(u / kSBufs) & 1u)) return false;
         tc_fence_after_sync();
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks)
@@ -355,7 +344,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         for (int vv = 0; vv < n_ahead && ok; ++vv) ok = issue_qk();
         if (!ok) break;
         mbar_arrive(&bars->decided);
-        if (!wait_or_abort(&bars->decided, (uint32_t)sw & 1u, abort_flag, err)) break;
+        if (!wait.one(&bars->decided, (uint32_t)sw & 1u)) break;
         if (!last_follows(bars, sw)) {
           for (int vv = n_ahead; vv < T && ok; ++vv) ok = issue_qk();
         } else {
@@ -405,7 +394,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         const bool full = (info_next & 0x80u) != 0u;  // every entry of the round is kept
         const uint2 bits = bits_next;
         fetch(vv + 1 == T ? 0 : vv + 1, info_next, bits_next);
-        ok = wait_or_abort(&bars->s_full[buf], (uint32_t)(v / kSBufs) & 1u, abort_flag, err);
+        ok = wait(&bars->s_full[buf], (uint32_t)(v / kSBufs) & 1u);
         if (!ok) break;
         tc_fence_after_sync();
         float psum0 = 0.f, psum1 = 0.f;
@@ -477,12 +466,12 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
       cnts[wg * 128 + r] = cnt;
       // ---- end of a sweep: the two halves of every row meet
       mbar_arrive(&bars->sweep_done);
-      ok = wait_or_abort(&bars->sweep_done, (uint32_t)sw & 1u, abort_flag, err);
+      ok = wait(&bars->sweep_done, (uint32_t)sw & 1u);
       if (!ok) break;
       const float2 s0 = stats[r], s1 = stats[128 + r];
       if (last) {
         // epilogue: O / (sum of the rounded weights); this thread writes half of the row's d columns
-        ok = wait_or_abort(&bars->o_done, 0u, abort_flag, err);
+        ok = wait(&bars->o_done, 0u);
         if (!ok) break;
         tc_fence_after_sync();
         const float z = s0.x + s1.x;
@@ -527,7 +516,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
       neg_tau = -tau;
       if (moved && row_ok) *reinterpret_cast<volatile int *>(&bars->more[sw]) = 1;
       mbar_arrive(&bars->decided);
-      ok = wait_or_abort(&bars->decided, (uint32_t)sw & 1u, abort_flag, err);
+      ok = wait(&bars->decided, (uint32_t)sw & 1u);
       if (!ok) break;
       last = last_follows(bars, sw);
     }

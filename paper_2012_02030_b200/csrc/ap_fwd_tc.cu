@@ -54,17 +54,16 @@
 #include <math_constants.h>
 
 #include "ap_common.cuh"
-#include "ap_sm100.cuh"
+#include "ap_pipe.cuh"
 
 namespace ap {
 
 namespace {
 
-using namespace sm100;
+using namespace pipe;
 
 constexpr int kThreads = 480;
 constexpr int kSoftmaxWarps = 8;       // two groups of four; barriers the softmax warps arrive on count warps
-constexpr int kSubBytes = 128 * 128;  // one [128 rows][64 bf16] swizzled sub-tile
 constexpr uint32_t kTmemCols = 512;
 constexpr int kMaxStages = 4;
 
@@ -132,58 +131,7 @@ struct Shared {
   uint32_t tmem_base;
   uint32_t n_items;   // set when the CTA's last item has been handed to the epilogue: how many there were
   int abort_flag;
-  uint32_t max_polls; // poll limit of every wait (directly behind abort_flag: wait_or_abort reads both)
 };
-
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// Bounded wait that also gives up as soon as another thread of the CTA has.
-__device__ __noinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, volatile int *abort_flag, unsigned *err,
-                                           uint32_t max_polls) {
-  for (uint32_t i = 0; i < max_polls; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (i > 1024) __nanosleep(64);
-  }
-  *abort_flag = 1;
-  atomicOr(err, kDevErrTimeout);
-  return false;
-}
-
-// The same wait for a whole (converged) warp: one lane polls - 32 lanes polling one barrier would
-// serialise - and the outcome is shared.
-template <int kPollLane = 0>
-__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, int lane, volatile int *abort_flag,
-                                          unsigned *err, uint32_t max_polls) {
-  bool ok = true;
-  if (lane == kPollLane && !mbar_try_wait(bar, parity)) ok = wait_or_abort(bar, parity, abort_flag, err, max_polls);
-  return __shfl_sync(0xffffffffu, ok ? 1 : 0, kPollLane) != 0;
-}
-
-// Two fp32 values rounded to the tensors' 16-bit type and packed (first value in the low half),
-// and back: exactly the values the tensor cores will see.
-template <bool kF16>
-__device__ __forceinline__ uint32_t pack16x2(float lo, float hi) {
-  if constexpr (kF16) {
-    const __half2 h = __floats2half2_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t *>(&h);
-  } else {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t *>(&h);
-  }
-}
-template <bool kF16>
-__device__ __forceinline__ float2 unpack16x2(uint32_t pk) {
-  if constexpr (kF16) {
-    return __half22float2(*reinterpret_cast<const __half2 *>(&pk));
-  } else {
-    return make_float2(__uint_as_float(pk << 16), __uint_as_float(pk & 0xffff0000u));
-  }
-}
 
 // kGath: the launch may follow gathered rounds (a second instantiation, so that the code for them
 // costs lists without a gathered schedule nothing).  kPairs: the units of work are the pairs of query
@@ -225,7 +173,6 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
     for (int i = 0; i < 2; ++i) mbar_init(&sh->o_free[i], 4);  // epilogue warps
     for (int i = 0; i < 4; ++i) mbar_init(&sh->ml_ready[i], kSoftmaxWarps);
     sh->abort_flag = 0;
-    sh->max_polls = max_polls;
     sh->n_items = 0xffffffffu;
     fence_mbar_init();
   }
@@ -245,6 +192,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
   const uint32_t tmem_o = tmem + 256;
   auto o_of_item = [&](uint32_t n) { return tmem_o + (kOBufs == 2u ? 128u * (n & 1u) : 0u); };
   volatile int *abort_flag = &sh->abort_flag;
+  const Waiter wait{abort_flag, err, max_polls};
   const int item_step = (int)gridDim.x;
 
   if (warp == 8) {
@@ -351,8 +299,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
     // g - 4 was issued, i.e. after that round's softmax, so k_empty implies it.
     static_assert(C::kStages == kMaxStages || C::kStages == 2, "ring discipline");
     auto wait_free = [&](uint64_t *bar, uint32_t ph) {
-      if (lane == 0) ok = wait_or_abort(bar, ph ^ 1u, abort_flag, err, max_polls);
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+      ok = wait(bar, ph ^ 1u);
     };
     // A run of slots (key rows following one another) is copied by the lane of its first slot, in
     // pieces of 8, 4, 2 or 1 slots.
@@ -491,7 +438,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
       // Q of this item into its buffer (free once the last S = Q K^T of item n - 2 has completed)
       const int qb = (int)(n & 1u);
       if (lane == 0) {
-        ok = wait_or_abort(&sh->q_empty[qb], ((n >> 1) & 1u) ^ 1u, abort_flag, err, max_polls);
+        ok = wait.one(&sh->q_empty[qb], ((n >> 1) & 1u) ^ 1u);
         if (ok) {
           mbar_arrive_expect_tx(&sh->q_full[qb], C::kTileBytes);
 #pragma unroll
@@ -606,7 +553,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
     }
   } else if (warp == 9) {
     // ------------------------------------------------------------ issuer of S = Q K^T
-    // The whole warp walks the rounds in lockstep (one lane polls the barriers, another, elected
+    // The whole warp walks the rounds in lockstep (all lanes poll the barriers, an elected
     // one issues the tcgen05 instructions; the state is warp-uniform).
     const uint32_t q_addr = smem_u32(q_s), k_addr = smem_u32(k_s);
     bool ok = true;
@@ -614,17 +561,17 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
     for (uint32_t g = 0; ok; ++g) {
       const int st = (int)(g % C::kStages);
       const uint32_t sb = g & 1u;
-      ok = warp_wait<31>(&sh->k_full[st], (g / C::kStages) & 1u, lane, abort_flag, err, max_polls);
+      ok = wait(&sh->k_full[st], (g / C::kStages) & 1u);
       if (!ok) break;
       const uint32_t info = sh->info[g % kMaxStages];
       if (info & kInfoStop) break;
       const int ng = (int)(info & kInfoSlots);
       const bool first = (info & kInfoFirst) != 0u, last = (info & kInfoLast) != 0u;
       const int qb = (int)(n & 1u);
-      if (first) ok = warp_wait<31>(&sh->q_full[qb], (n >> 1) & 1u, lane, abort_flag, err, max_polls);
+      if (first) ok = wait(&sh->q_full[qb], (n >> 1) & 1u);
       // S[sb] still holds P of round g - 2 until that round's O += P V (issued by another warp) has
       // completed
-      if (ok && g >= 2) ok = warp_wait<31>(&sh->pv_done[sb], ((g >> 1) - 1u) & 1u, lane, abort_flag, err, max_polls);
+      if (ok && g >= 2) ok = wait(&sh->pv_done[sb], ((g >> 1) - 1u) & 1u);
       if (!ok) break;
       tc_fence_after_sync();
       if constexpr (kGath) fence_proxy_async_smem();  // rows of a gathered round may come from plain asynchronous copies
@@ -655,18 +602,18 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
     for (uint32_t g = 0; ok; ++g) {
       const int st = (int)(g % C::kStages);
       const uint32_t sb = g & 1u;
-      ok = warp_wait<31>(&sh->b_full[g % kMaxStages], (g / kMaxStages) & 1u, lane, abort_flag, err, max_polls);
+      ok = wait(&sh->b_full[g % kMaxStages], (g / kMaxStages) & 1u);
       if (!ok) break;
       const uint32_t info = sh->info[g % kMaxStages];
       if (info & kInfoStop) break;
       const int ng = (int)(info & kInfoSlots);
       const bool first = (info & kInfoFirst) != 0u, last = (info & kInfoLast) != 0u;
       // (what is ready early first; P, which the softmax has just finished, last)
-      ok = warp_wait<31>(&sh->v_full[st], (g / C::kStages) & 1u, lane, abort_flag, err, max_polls);
+      ok = wait(&sh->v_full[st], (g / C::kStages) & 1u);
       // the first round of an item overwrites O: the epilogue of the previous item must have read it
       if (ok && first && n >= kOBufs)
-        ok = warp_wait<31>(&sh->o_free[kOBufs == 2u ? (n & 1u) : 0u], ((n / kOBufs) - 1u) & 1u, lane, abort_flag, err, max_polls);
-      if (ok) ok = warp_wait<31>(&sh->p_full[sb], (g >> 1) & 1u, lane, abort_flag, err, max_polls);
+        ok = wait(&sh->o_free[kOBufs == 2u ? (n & 1u) : 0u], ((n / kOBufs) - 1u) & 1u);
+      if (ok) ok = wait(&sh->p_full[sb], (g >> 1) & 1u);
       if (!ok) break;
       tc_fence_after_sync();
       if constexpr (kGath) fence_proxy_async_smem();  // rows of a gathered round may come from plain asynchronous copies
@@ -713,7 +660,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
       const int st = (int)(g % kMaxStages);  // info / bitmap slot of the round
       const uint32_t sb = g & 1u;
       const uint32_t tmem_s = tmem + 128u * sb;
-      ok = warp_wait(&sh->b_full[st], (g / kMaxStages) & 1u, lane, abort_flag, err, max_polls);
+      ok = wait(&sh->b_full[st], (g / kMaxStages) & 1u);
       if (!ok) break;
       const uint32_t info = sh->info[st];
       if (info & kInfoStop) break;
@@ -738,7 +685,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
         w0 = brow[grp];
         w1 = brow[grp + 2];
       }
-      ok = warp_wait(&sh->s_full[sb], (g >> 1) & 1u, lane, abort_flag, err, max_polls);
+      ok = wait(&sh->s_full[sb], (g >> 1) & 1u);
       if (!ok) break;
       tc_fence_after_sync();
       // straight-line: both chunks always (a chunk the round does not reach holds stale scores whose
@@ -775,7 +722,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
       // Rescale the group's running output where the reference moved.  O += P V of the previous
       // round may still be running (this round's S was computed ahead of it): wait for it first.
       if (o_started && __any_sync(0xffffffffu, alpha != 1.f)) {
-        ok = warp_wait(&sh->pv_done[(g - 1u) & 1u], ((g - 1u) >> 1) & 1u, lane, abort_flag, err, max_polls);
+        ok = wait(&sh->pv_done[(g - 1u) & 1u], ((g - 1u) >> 1) & 1u);
         if (!ok) break;
         tc_fence_after_sync();
 #pragma unroll 1
@@ -798,8 +745,8 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
         for (int e = 0; e < 16; ++e) {
           const float p0 = ex2_approx(fmaf(__uint_as_float(xs[32 * c + 2 * e]), scale_log2, neg_mc));
           const float p1 = ex2_approx(fmaf(__uint_as_float(xs[32 * c + 2 * e + 1]), scale_log2, neg_mc));
-          pk[e] = pack16x2<kF16>(p0, p1);
-          const float2 pr = unpack16x2<kF16>(pk[e]);
+          pk[e] = pack2<kF16>(p0, p1);
+          const float2 pr = unpack2<kF16>(pk[e]);
           sum0 += pr.x;
           sum1 += pr.y;
         }
@@ -843,7 +790,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     bool ok = true;
     for (uint32_t n = 0; ok; ++n) {
-      ok = warp_wait(&sh->ml_ready[n & 3u], (n >> 2) & 1u, lane, abort_flag, err, max_polls);
+      ok = wait(&sh->ml_ready[n & 3u], (n >> 2) & 1u);
       if (!ok) break;
       if (n >= *reinterpret_cast<volatile uint32_t *>(&sh->n_items)) break;
       const int item_qt = sh->ml_qt[n & 3u], item_bh = sh->ml_bh[n & 3u];
@@ -858,7 +805,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
       const float l_tot = g0.y * a0 + g1.y * a1;
       const float inv = l_tot > 0.f ? 1.f / l_tot : 0.f;
       const float f0 = a0 * inv, f1 = a1 * inv;
-      ok = warp_wait(&sh->o_done[kOBufs == 2u ? (n & 1u) : 0u], (n / kOBufs) & 1u, lane, abort_flag, err, max_polls);
+      ok = wait(&sh->o_done[kOBufs == 2u ? (n & 1u) : 0u], (n / kOBufs) & 1u);
       if (!ok) break;
       tc_fence_after_sync();
 #pragma unroll 1
@@ -883,7 +830,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
               const float x0 = (f0 > 0.f ? __uint_as_float(o0[j]) * f0 : 0.f) + (f1 > 0.f ? __uint_as_float(o1[j]) * f1 : 0.f);
               const float x1 = (f0 > 0.f ? __uint_as_float(o0[j + 1]) * f0 : 0.f) +
                                (f1 > 0.f ? __uint_as_float(o1[j + 1]) * f1 : 0.f);
-              pk[e] = pack16x2<kF16>(x0, x1);
+              pk[e] = pack2<kF16>(x0, x1);
             }
             *reinterpret_cast<uint4 *>(orow + 32 * c + 8 * q) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
           }

@@ -1,5 +1,4 @@
-// What the warp-specialised kernels share: bounded waits that a whole warp takes, the 16-bit packing of
-// the tensors' types, copies of runs of key rows, and the coalesced store of accumulator rows.
+// What the warp-specialised kernels share: the 16-bit packing of the tensors' types, copies of runs of key rows, and the coalesced store of accumulator rows.
 #pragma once
 
 #include "ap_common.cuh"
@@ -42,34 +41,6 @@ __device__ __forceinline__ float2 unpack2(uint32_t pk) {
     return make_float2(__uint_as_float(pk << 16), __uint_as_float(pk & 0xffff0000u));
   }
 }
-
-// Bounded wait that also gives up as soon as another thread of the CTA has.
-static __device__ __noinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, volatile int *abort_flag, unsigned *err,
-                                           uint32_t max_polls) {
-  for (uint32_t i = 0; i < max_polls; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (i > 1024) __nanosleep(64);
-  }
-  *abort_flag = 1;
-  atomicOr(err, kDevErrTimeout);
-  return false;
-}
-
-// What a role needs to wait: its lane, the CTA's abort flag, the device status word, the poll limit.
-struct Waiter {
-  int lane;
-  volatile int *abort_flag;
-  unsigned *err;
-  uint32_t max_polls;
-
-  // The wait for a whole converged warp: one lane polls, the outcome is shared.
-  __device__ __forceinline__ bool operator()(uint64_t *bar, uint32_t parity) const {
-    bool ok = true;
-    if (lane == 0 && !mbar_try_wait(bar, parity)) ok = wait_or_abort(bar, parity, abort_flag, err, max_polls);
-    return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-  }
-};
 
 // Layout of a staged tile of D columns.  kSplit = false: [slab][row][128 B], one box per 64-column slab;
 // kSplit = true (d = 128, whole groups of eight rows): [row / 8][slab][8 rows][128 B], one box for both.

@@ -5,9 +5,7 @@
 // tcgen05.mma takes.  Every wait in here is bounded.
 #pragma once
 
-#include <cuda.h>
-#include <cuda_runtime.h>
-#include <stdint.h>
+#include "ap_common.cuh"
 
 namespace ap {
 namespace sm100 {
@@ -91,6 +89,40 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32
   }
   return false;
 }
+
+// Bounded wait that also gives up as soon as another thread of the CTA has: the slow path of the waits below,
+// kept out of line.
+static __device__ __noinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
+                                                  unsigned *err, uint32_t max_polls) {
+  for (uint32_t i = 0; i < max_polls; ++i) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if (*abort_flag) return false;
+    if (i > 1024) __nanosleep(64);
+  }
+  *abort_flag = 1;
+  atomicOr(err, kDevErrTimeout);
+  return false;
+}
+
+// The waits of a role: the CTA's abort flag, the device status word, the poll limit.
+struct Waiter {
+  volatile int *abort_flag;
+  unsigned *err;
+  uint32_t max_polls;
+
+  // For a whole converged warp; the outcome is the same for every lane.  All lanes poll: a round trip through two
+  // mbarriers between two warps then takes some 280 cycles.  With one polling lane that shares the outcome by a
+  // shuffle it took 600 (the divergence costs more than 31 more pollers), which made every hand-over between the
+  // roles of a kernel that much slower: 5 to 10 % of the attention kernels' time.
+  __device__ __forceinline__ bool operator()(uint64_t *bar, uint32_t parity) const {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, wait_or_abort(bar, parity, abort_flag, err, max_polls)) != 0;
+  }
+  // For a single thread.
+  __device__ __forceinline__ bool one(uint64_t *bar, uint32_t parity) const {
+    return mbar_try_wait(bar, parity) || wait_or_abort(bar, parity, abort_flag, err, max_polls);
+  }
+};
 
 // True in exactly one lane of a fully converged warp.
 __device__ __forceinline__ bool elect_one() {
