@@ -176,6 +176,7 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16_f32(128, 128, false, false, f16 != 0);
+      const uint32_t desc0 = smem_desc_lo(smem_u32(smem), 16);
       int v = 0;
       bool last = false, ok = true;
       for (int sw = 0; ok; ++sw) {
@@ -186,13 +187,12 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
           if (!wait.one(&bars->in_full[st], ph)) { ok = false; break; }
           if (!wait.one(&bars->s_empty[buf], ((uint32_t)(v >> 1) & 1u) ^ 1u)) { ok = false; break; }
           tc_fence_after_sync();
-          const unsigned char *q_s = smem + (2 * st) * C::kTileBytes, *k_s = q_s + C::kTileBytes;
+          const uint32_t q_lo = desc0 + 2 * st * (C::kTileBytes >> 4), k_lo = q_lo + (C::kTileBytes >> 4);
+          constexpr uint32_t kHi = smem_desc_hi_sw128(1024);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) {
-            const int sub = ks / 4, o = (ks % 4) * 32;
-            const uint64_t da = smem_desc_sw128(smem_u32(q_s + sub * kSubBytes + o), 16, 1024);
-            const uint64_t db = smem_desc_sw128(smem_u32(k_s + sub * kSubBytes + o), 16, 1024);
-            mma_ss(tmem + 128 * buf, da, db, idesc, ks > 0);
+            const uint32_t step = (ks / 4) * (kSubBytes >> 4) + (ks % 4) * 2;
+            mma_ss<kHi, kHi>(tmem + 128 * buf, q_lo + step, k_lo + step, idesc, ks > 0);
           }
           mma_commit(&bars->in_empty[st]);
           mma_commit(&bars->s_full[buf]);

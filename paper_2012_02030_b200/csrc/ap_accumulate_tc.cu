@@ -186,10 +186,12 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
   if (warp == 8) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    {
+      if (lane == 0) {
       prefetch_tensormap(&map_q);
       prefetch_tensormap(&map_k);
       if (bias_by_tma) prefetch_tensormap(&map_bias);
+      }
       int v = 0, bias_loads = 0;
       for (; v < n_visits; ++v) {
         const int st = v % C::kStages;
@@ -200,24 +202,30 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           // bias tile of the key tile whose visits start here; the buffer is free once all
           // softmax threads have copied the previous tile to registers
           const int tl = v / Bc;
-          if (!wait.one(&bars->bias_empty, ((uint32_t)tl & 1u) ^ 1u)) break;
+          if (!wait(&bars->bias_empty, ((uint32_t)tl & 1u) ^ 1u)) break;
+          if (lane == 0) {
           mbar_arrive_expect_tx(&bars->bias_full, kBiasBytes);
 #pragma unroll
           for (int q = 0; q < 4; ++q)
             tma_load_3d(bias_s + q * (kBiasBytes / 4), &map_bias, &bars->bias_full, kt * kTile + 32 * q, qt * kTile, h);
+          }
+          __syncwarp();
           bias_loads = tl + 1;
         }
-        if (!wait.one(&bars->in_empty[st], ph ^ 1u)) break;
+        if (!wait(&bars->in_empty[st], ph ^ 1u)) break;
         if (dbg_skip != 0 && v == 0) continue;
         unsigned char *q_s = smem + (2 * st) * C::kTileBytes, *k_s = q_s + C::kTileBytes;
+        if (lane == 0) {
         mbar_arrive_expect_tx(&bars->in_full[st], 2 * C::kTileBytes);
 #pragma unroll
         for (int s = 0; s < C::kSub; ++s) {
           tma_load_3d(q_s + s * kSubBytes, &map_q, &bars->in_full[st], 64 * s, qt * kTile, b * H + h);
           tma_load_3d(k_s + s * kSubBytes, &map_k, &bars->in_full[st], 64 * s, kt * kTile, b * H + h);
         }
+        }
+        __syncwarp();
       }
-      if (*abort_flag) {  // winding down: let the copies in flight land (bounded)
+      if (lane == 0 && *abort_flag) {  // winding down: let the copies in flight land (bounded)
         for (int j = max(0, v - C::kStages); j < v; ++j) {
           if (dbg_skip != 0 && j == 0) continue;
           mbar_wait(&bars->in_full[j % C::kStages], (uint32_t)(j / C::kStages) & 1u, max_polls);
@@ -227,25 +235,28 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     }
   } else if (warp == 9) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_bf16_f32(128, 128, false, false, f16 != 0);
+      const uint32_t desc0 = smem_desc_lo(smem_u32(smem), 16);
       for (int v = 0; v < n_visits; ++v) {
         const int st = v % C::kStages;
         const uint32_t ph = (uint32_t)(v / C::kStages) & 1u;
         const int buf = v & 1;
-        if (!wait.one(&bars->in_full[st], ph)) break;
-        if (!wait.one(&bars->s_empty[buf], ((uint32_t)(v >> 1) & 1u) ^ 1u)) break;
+        if (!wait(&bars->in_full[st], ph)) break;
+        if (!wait(&bars->s_empty[buf], ((uint32_t)(v >> 1) & 1u) ^ 1u)) break;
         tc_fence_after_sync();
-        const unsigned char *q_s = smem + (2 * st) * C::kTileBytes, *k_s = q_s + C::kTileBytes;
+        if (elect_one()) {
+        const uint32_t q_lo = desc0 + 2 * st * (C::kTileBytes >> 4), k_lo = q_lo + (C::kTileBytes >> 4);
+        constexpr uint32_t kHi = smem_desc_hi_sw128(1024);
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {
-          const int sub = ks / 4, off = (ks % 4) * 32;
-          const uint64_t da = smem_desc_sw128(smem_u32(q_s + sub * kSubBytes + off), 16, 1024);
-          const uint64_t db = smem_desc_sw128(smem_u32(k_s + sub * kSubBytes + off), 16, 1024);
-          mma_ss(tmem + 128 * buf, da, db, idesc, ks > 0);
+          const uint32_t step = (ks / 4) * (kSubBytes >> 4) + (ks % 4) * 2;
+          mma_ss<kHi, kHi>(tmem + 128 * buf, q_lo + step, k_lo + step, idesc, ks > 0);
         }
         mma_commit(&bars->in_empty[st]);
         mma_commit(&bars->s_full[buf]);
+        }
+        __syncwarp();
       }
     }
   } else {

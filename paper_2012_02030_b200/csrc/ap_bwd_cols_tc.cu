@@ -253,21 +253,22 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
     // C[128 keys x queries] = A B^T over the visit's span
     auto issue_abt = [&](uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t info) {
       const uint32_t g0 = first_group(info), idesc = idesc_bf16_f32(128, 16 * (int)span(info), false, false, kF16);
+      const uint32_t a_lo = smem_desc_lo(a_addr, 16), b_lo = smem_desc_lo(b_addr + g0 * 2048u, 16), d = d_tmem + 16u * g0;
+      constexpr uint32_t kHi = smem_desc_hi_sw128(1024);
 #pragma unroll
       for (int ks = 0; ks < D / 16; ++ks) {
-        const int sub = ks / 4, off = (ks % 4) * 32;
-        mma_ss(d_tmem + 16u * g0, smem_desc_sw128(a_addr + sub * kSubBytes + off, 16, 1024),
-               smem_desc_sw128(b_addr + sub * kSubBytes + g0 * 2048u + off, 16, 1024), idesc, ks > 0);
+        const uint32_t step = (ks / 4) * (kSubBytes >> 4) + (ks % 4) * 2;
+        mma_ss<kHi, kHi>(d, a_lo + step, b_lo + step, idesc, ks > 0);
       }
     };
     // acc[128 keys x D] (+)= A[keys x queries, TMEM] B[queries x D], steps of empty query groups left out
     auto issue_acc = [&](uint32_t acc, uint32_t a_tmem, uint32_t b_addr, uint32_t info) {
       uint32_t started = (info & kInfoFirst) ? 0u : 1u;
+      const uint32_t b_lo = smem_desc_lo(b_addr, kSubBytes);
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks)
         if ((info >> ks) & 1u) {
-          mma_ts(acc, a_tmem + 32 * (ks >> 1) + 8 * (ks & 1), smem_desc_sw128(b_addr + ks * 2048, kSubBytes, 1024),
-                 idesc_acc, started);
+          mma_ts<smem_desc_hi_sw128(1024)>(acc, a_tmem + 32 * (ks >> 1) + 8 * (ks & 1), b_lo + ks * 128, idesc_acc, started);
           started = 1u;
         }
     };

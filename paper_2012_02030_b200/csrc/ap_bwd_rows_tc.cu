@@ -242,7 +242,8 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
     }
   } else if (warp == 9) {
     // ------------------------------------------------------------ issuer of all products
-    const uint32_t q_addr = smem_u32(q_s), do_addr = smem_u32(do_s), stage_addr = smem_u32(stage_s);
+    const uint32_t q_lo = smem_desc_lo(smem_u32(q_s), 16), do_lo = smem_desc_lo(smem_u32(do_s), 16);
+    const uint32_t stage_lo = smem_desc_lo(smem_u32(stage_s), 16), stage_mn = smem_desc_lo(smem_u32(stage_s), L::kSlabStride);
     constexpr uint32_t idesc_dq = idesc_bf16_f32(128, D, false, true, kF16);
     uint32_t n_front = 0, n_back = 0;  // items started by S / by dQ
     uint32_t info_front = 0u;
@@ -263,13 +264,13 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
       if (!ok) return false;
       tc_fence_after_sync();
       const uint32_t idesc = idesc_bf16_f32(128, 16 * (int)(info_front & kInfoSlots), false, false, kF16);
-      const uint32_t k_addr = stage_addr + st * C::kStageBytes;
+      const uint32_t k_lo = stage_lo + st * (C::kStageBytes >> 4);
       if (elect_one()) {
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {
-          const int sub = ks / 4, off = (ks % 4) * 32;
-          mma_ss(tmem + 128u * sb, smem_desc_sw128(q_addr + sub * kSubBytes + off, 16, 1024),
-                 smem_desc_sw128(k_addr + sub * L::kSlabStride + off, 16, L::kSbo), idesc, ks > 0);
+          const uint32_t a_step = (ks / 4) * (kSubBytes >> 4) + (ks % 4) * 2;
+          const uint32_t b_step = (ks / 4) * (L::kSlabStride >> 4) + (ks % 4) * 2;
+          mma_ss<smem_desc_hi_sw128(1024), smem_desc_hi_sw128(L::kSbo)>(tmem + 128u * sb, q_lo + a_step, k_lo + b_step, idesc, ks > 0);
         }
         mma_commit(&sh->s_full[sb]);
       }
@@ -282,9 +283,9 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
         if (!stats) {
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) {
-            const int sub = ks / 4, off = (ks % 4) * 32;
-            mma_ss(tmem + kTmemDp, smem_desc_sw128(do_addr + sub * kSubBytes + off, 16, 1024),
-                   smem_desc_sw128(k_addr + L::kBytes + sub * L::kSlabStride + off, 16, L::kSbo), idesc, ks > 0);
+            const uint32_t a_step = (ks / 4) * (kSubBytes >> 4) + (ks % 4) * 2;
+            const uint32_t b_step = (L::kBytes >> 4) + (ks / 4) * (L::kSlabStride >> 4) + (ks % 4) * 2;
+            mma_ss<smem_desc_hi_sw128(1024), smem_desc_hi_sw128(L::kSbo)>(tmem + kTmemDp, do_lo + a_step, k_lo + b_step, idesc, ks > 0);
           }
           if (last) mma_commit(&sh->q_empty);
         }
@@ -311,13 +312,12 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
       tc_fence_after_sync();
       if (elect_one()) {
         if (!stats) {
-          const uint32_t k_addr = stage_addr + st * C::kStageBytes, a_addr = tmem + 128u * sb;
+          const uint32_t k_lo = stage_mn + st * (C::kStageBytes >> 4), a_addr = tmem + 128u * sb;
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)
             if (ks < ng)
-              mma_ts(tmem + kTmemDq, a_addr + 32 * (ks >> 1) + 8 * (ks & 1),
-                     smem_desc_sw128(k_addr + ks * L::kSlotStride, L::kSlabStride, L::kSbo), idesc_dq,
-                     ks > 0 || !first);
+              mma_ts<smem_desc_hi_sw128(L::kSbo)>(tmem + kTmemDq, a_addr + 32 * (ks >> 1) + 8 * (ks & 1),
+                                                  k_lo + ks * (L::kSlotStride >> 4), idesc_dq, ks > 0 || !first);
           if (last) mma_commit(&sh->o_done);
         }
         mma_commit(&sh->kv_empty[st]);

@@ -292,10 +292,12 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     // ------------------------------------------------------------ MMA issuer
     // S = Q K^T of the first visits of the next sweep is issued before the decision as well
     // (three S buffers).
-    if (lane == 0) {
+    {
       constexpr uint32_t idesc_pv = idesc_bf16_f32(128, D, false, true, kF16);
-      const uint32_t q_addr = smem_u32(smem), k_addr = smem_u32(smem + C::kKOffset), v_addr = smem_u32(smem + C::kVOffset);
-      bool ok = wait.one(&bars->q_full, 0u);
+      constexpr uint32_t kHi = smem_desc_hi_sw128(1024);
+      const uint32_t q_lo = smem_desc_lo(smem_u32(smem), 16), k_lo = smem_desc_lo(smem_u32(smem + C::kKOffset), 16);
+      const uint32_t v_lo = smem_desc_lo(smem_u32(smem + C::kVOffset), kSubBytes);
+      bool ok = wait(&bars->q_full, 0u);
       int v = 0;  // visits whose S has been issued
       auto ng_of = [&](int vv) { return (int)(__ldg(round_info + t0 + vv) & 15u); };
       uint32_t info_next = __ldg(round_info + t0);  // used one visit later: the load stays in flight
@@ -305,19 +307,21 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         const uint32_t idesc_qk = idesc_bf16_f32(128, 16 * (int)(info_next & 15u), false, false, kF16);
         vv_next = vv_next + 1 == T ? 0 : vv_next + 1;
         info_next = __ldg(round_info + t0 + vv_next);
-        if (!wait.one(&bars->in_full[st], (uint32_t)(v / C::kStages) & 1u)) return false;
+        if (!wait(&bars->in_full[st], (uint32_t)(v / C::kStages) & 1u)) return false;
         // S[buf] was read (and, in the last sweep, its P consumed by a product issued earlier by
         // this thread: products execute in issue order) kSBufs visits ago
-        if (!wait.one(&bars->s_empty[buf], ((uint32_t)(v / kSBufs) & 1u) ^ 1u)) return false;
+        if (!wait(&bars->s_empty[buf], ((uint32_t)(v / kSBufs) & 1u) ^ 1u)) return false;
         tc_fence_after_sync();
+        if (elect_one()) {
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {
-          const int sub = ks / 4, o = (ks % 4) * 32;
-          mma_ss(tmem + 128 * buf, smem_desc_sw128(q_addr + sub * kSubBytes + o, 16, 1024),
-                 smem_desc_sw128(k_addr + st * C::kTileBytes + sub * kSubBytes + o, 16, 1024), idesc_qk, ks > 0);
+          const uint32_t step = (ks / 4) * (kSubBytes >> 4) + (ks % 4) * 2;
+          mma_ss<kHi, kHi>(tmem + 128 * buf, q_lo + step, k_lo + st * (C::kTileBytes >> 4) + step, idesc_qk, ks > 0);
         }
         mma_commit(&bars->in_empty[st]);
         mma_commit(&bars->s_full[buf]);
+        }
+        __syncwarp();
         ++v;
         return true;
       };
@@ -325,16 +329,19 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
       // threads have arrived; one contraction step of 16 keys per group; then the V stage is free
       auto issue_pv = [&](int u, int j) -> bool {
         const int sb = u % kSBufs, sv = j % C::kVStages, ng_u = ng_of(j);
-        if (!wait.one(&bars->v_full[sv], (uint32_t)(j / C::kVStages) & 1u)) return false;
-        if (!wait.one(&bars->s_empty[sb], (uint32_t)(u / kSBufs) & 1u)) return false;
+        if (!wait(&bars->v_full[sv], (uint32_t)(j / C::kVStages) & 1u)) return false;
+        if (!wait(&bars->s_empty[sb], (uint32_t)(u / kSBufs) & 1u)) return false;
         tc_fence_after_sync();
+        if (elect_one()) {
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks)
           if (ks < ng_u)
-            mma_ts(tmem + 128 * kSBufs, tmem + 128 * sb + 32 * (ks >> 1) + 8 * (ks & 1),
-                   smem_desc_sw128(v_addr + sv * C::kTileBytes + ks * 2048, kSubBytes, 1024), idesc_pv,
-                   (j == 0 && ks == 0) ? 0u : 1u);
+            mma_ts<kHi>(tmem + 128 * kSBufs, tmem + 128 * sb + 32 * (ks >> 1) + 8 * (ks & 1),
+                        v_lo + sv * (C::kTileBytes >> 4) + ks * 128, idesc_pv, (j == 0 && ks == 0) ? 0u : 1u);
         mma_commit(&bars->v_empty[sv]);
+        if (j == T - 1) mma_commit(&bars->o_done);
+        }
+        __syncwarp();
         return true;
       };
       const int n_ahead = T < kSBufs ? T : kSBufs;
@@ -343,8 +350,9 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         const int v_head = v;
         for (int vv = 0; vv < n_ahead && ok; ++vv) ok = issue_qk();
         if (!ok) break;
-        mbar_arrive(&bars->decided);
-        if (!wait.one(&bars->decided, (uint32_t)sw & 1u)) break;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->decided);
+        if (!wait(&bars->decided, (uint32_t)sw & 1u)) break;
         if (!last_follows(bars, sw)) {
           for (int vv = n_ahead; vv < T && ok; ++vv) ok = issue_qk();
         } else {
@@ -353,7 +361,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
             if (vv >= n_ahead) ok = issue_qk();
             if (ok && vv > 0) ok = issue_pv(v_head + vv - 1, vv - 1);
           }
-          if (ok && issue_pv(v_head + T - 1, T - 1)) mma_commit(&bars->o_done);
+          if (ok) issue_pv(v_head + T - 1, T - 1);
           break;
         }
       }

@@ -555,7 +555,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
     // ------------------------------------------------------------ issuer of S = Q K^T
     // The whole warp walks the rounds in lockstep (all lanes poll the barriers, an elected
     // one issues the tcgen05 instructions; the state is warp-uniform).
-    const uint32_t q_addr = smem_u32(q_s), k_addr = smem_u32(k_s);
+    const uint32_t q_desc = smem_desc_lo(smem_u32(q_s), 16), k_desc = smem_desc_lo(smem_u32(k_s), 16);
     bool ok = true;
     uint32_t n = 0;  // non-empty items started so far
     for (uint32_t g = 0; ok; ++g) {
@@ -578,13 +578,12 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
       // N = 16 ng, D/16 steps of K = 16 (32 bytes inside the swizzled rows)
       if (elect_one()) {
         const uint32_t idesc_qk = idesc_bf16_f32(128, 16 * ng, false, false, kF16);
-        const uint32_t q_buf = q_addr + qb * C::kTileBytes, k_stage = k_addr + st * C::kTileBytes;
+        const uint32_t q_lo = q_desc + qb * (C::kTileBytes >> 4), k_lo = k_desc + st * (C::kTileBytes >> 4);
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const int sub = ks / 4, off = (ks % 4) * 32;
-          mma_ss(tmem + 128u * sb, smem_desc_sw128(q_buf + sub * kSubBytes + off, 16, 1024),
-                 smem_desc_sw128(k_stage + sub * C::kHalfStride + off, 16, C::kSbo), idesc_qk, ks > 0);
-        }
+        for (int ks = 0; ks < D / 16; ++ks)
+          mma_ss<smem_desc_hi_sw128(1024), smem_desc_hi_sw128(C::kSbo)>(
+              tmem + 128u * sb, q_lo + (ks / 4) * (kSubBytes >> 4) + (ks % 4) * 2,
+              k_lo + (ks / 4) * (C::kHalfStride >> 4) + (ks % 4) * 2, idesc_qk, ks > 0);
         mma_commit(&sh->k_empty[st]);
         if (last) mma_commit(&sh->q_empty[qb]);
         mma_commit(&sh->s_full[sb]);
@@ -595,7 +594,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
   } else if (warp == 10) {
     // ------------------------------------------------------------ issuer of O += P V
     constexpr uint32_t idesc_pv = idesc_bf16_f32(128, D, false, true, kF16);
-    const uint32_t v_addr = smem_u32(v_s);
+    const uint32_t v_desc = smem_desc_lo(smem_u32(v_s), C::kHalfStride);
     bool ok = true;
     uint32_t n = 0;                          // non-empty items started so far
     uint32_t started0 = 0u, started1 = 0u;  // the item's O_0 / O_1 holds a partial result already
@@ -624,15 +623,15 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
       // O_1; a group's first step of an item overwrites its accumulator.
       if (first) started0 = started1 = 0u;
       if (elect_one()) {
-        const uint32_t v_stage = v_addr + st * C::kTileBytes;
+        const uint32_t v_lo = v_desc + st * (C::kTileBytes >> 4);
         const uint32_t p_base = tmem + 128u * sb;
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
           if (ks < ng) {
             const int grp = (ks >> 1) & 1;
             const uint32_t acc = ks == 0 ? started0 : ks == 2 ? started1 : 1u;  // slots 0 / 2 open their group
-            mma_ts(o_of_item(n) + kOGroup * grp, p_base + 32 * (ks >> 1) + 8 * (ks & 1),
-                   smem_desc_sw128(v_stage + ks * C::kSlotStride, C::kHalfStride, C::kSbo), idesc_pv, acc);
+            mma_ts<smem_desc_hi_sw128(C::kSbo)>(o_of_item(n) + kOGroup * grp, p_base + 32 * (ks >> 1) + 8 * (ks & 1),
+                                                v_lo + ks * (C::kSlotStride >> 4), idesc_pv, acc);
           }
         }
         mma_commit(&sh->v_empty[st]);
