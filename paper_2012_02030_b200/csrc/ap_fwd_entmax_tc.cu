@@ -8,13 +8,17 @@
 // of its list row (the schedule of the tile list: up to eight non-empty groups of 16 key columns,
 // taken from one or several key tiles, per round) several times, recomputing S = Q K^T on the tensor
 // cores each time:
-//   sweep 0          row maxima over the kept entries, tau = max - 0.625 (the root lies in [max - 1, max))
-//   sweeps 1 .. n    over the support of the trial threshold (the n entries with x > tau):
-//                    S1 = sum (x - tau), S2 = sum (x - tau)^2 -> tau moves to the smaller root of the
-//                    support's parabola, tau + (S2 - 1) / (S1 + sqrt(S1^2 - n (S2 - 1))), which is the
-//                    answer once the support is right and lies on the other side of it otherwise
-//                    (Newton's step (S2 - 1) / (2 S1) where the parabola has no root); until no row
-//                    of the CTA moves (or kMaxNewton sweeps)
+//   sweep 0          row maxima over the kept entries; and the entries that can lie above tau, i.e. above the running
+//                    maximum - 1 (the root lies in [max - 1, max)), appended to a list per thread in shared memory.  A
+//                    list that fills up is pruned by the threshold of what it holds (more entries only raise the
+//                    root), which for spread-out scores leaves a dozen entries of any number
+//   then             tau from the lists alone: over the support of the trial threshold (the n entries with x > tau,
+//                    first max - 0.625) S1 = sum (x - tau), S2 = sum (x - tau)^2 -> tau moves to the smaller root
+//                    of the support's parabola, tau + (S2 - 1) / (S1 + sqrt(S1^2 - n (S2 - 1))), which is the
+//                    answer once the support is right and lies on the other side of it otherwise (Newton's step
+//                    (S2 - 1) / (2 S1) where the parabola has no root); until no row moves (or kMaxNewton steps)
+//   sweeps 1 .. n    only where a list overflowed (a row with more than kListCap entries of nearly the same, largest
+//                    score): the same steps, each with the sums of a sweep over all rounds
 //   last sweep       P = max(x - tau, 0)^2 rounded to the tensors' type, written over S in TMEM;
 //                    O += P V (A operand from TMEM); the epilogue divides by the sum of the rounded
 //                    weights, so that O is an exact convex combination of V rows.
@@ -23,6 +27,9 @@
 // one box of 128 rows for eight adjacent groups, into a ring of 4 to 6 stages; V rows in the last
 // sweep), warp 9 issues the products.
 // Every mbarrier wait is bounded.
+//
+// What bounds it: the normalising warps' two passes over the scores and the chain of a list row's few rounds.  With
+// a sweep per step of tau (seven to eight sweeps) 16 x 16 heads of 512 tokens (10 % kept, d = 64) took 125 us.
 #include <math_constants.h>
 
 #include "ap_common.cuh"
@@ -35,7 +42,10 @@ namespace {
 using namespace sm100;
 
 constexpr int kThreads = 320;
-constexpr int kNormThreads = 256;
+constexpr int kNormWarps = 8;
+// Candidate lists: entries per thread before a list is pruned, and room for one more step of 16 columns.
+constexpr int kListCap = 32, kListRows = kListCap + 16;
+constexpr int kListPitch = 2 * 128 + 32;  // thread (wg, r) at 144 wg + r: the two halves of a row on different banks
 constexpr int kSubBytes = 128 * 128;
 constexpr uint32_t kTmemCols = 512;  // S x 3 (columns 0..383), O (columns 384..384 + d)
 constexpr int kSBufs = 3;            // S buffers in flight: a visit's hand-offs take longer than its work
@@ -51,7 +61,7 @@ struct Cfg {
   static constexpr int kTileBytes = kSub * kSubBytes;
   // K is copied again in every sweep and a list row is a few rounds long: a ring deep enough to hold
   // a short row whole keeps the copies several visits ahead of the products.  V is needed once.
-  static constexpr int kStages = D == 64 ? 6 : 4;         // K ring
+  static constexpr int kStages = D == 64 ? 4 : 3;         // K ring
   static constexpr int kVStages = D == 64 ? 2 : 1;        // V ring (last sweep)
   static constexpr int kKOffset = kTileBytes;             // after Q
   static constexpr int kVOffset = kKOffset + kStages * kTileBytes;
@@ -61,7 +71,8 @@ struct Cfg {
   static constexpr int kCntBytes = 2 * 128 * 4;           // [wg][row] support size n
   static constexpr int kTauOffset = kCntOffset + kCntBytes;
   static constexpr int kTauBytes = 2 * 128 * 4;           // [wg][row]: each half keeps its own copy
-  static constexpr int kBarOffset = kTauOffset + kTauBytes;
+  static constexpr int kListOffset = kTauOffset + kTauBytes;
+  static constexpr int kBarOffset = kListOffset + kListRows * kListPitch * 4;
   static constexpr int kSmemBytes = kBarOffset + 512 + 1024;
   static_assert(kSmemBytes > 114 * 1024 && kSmemBytes <= 227 * 1024, "one CTA per SM, within the limit");
 };
@@ -76,7 +87,7 @@ struct Barriers {
   uint64_t o_done;
   uint32_t tmem_base;
   int abort_flag;
-  int more[kMaxNewton + 2];
+  int more[kMaxNewton + 2];  // [0]: a list overflowed; [s]: a row moved in sweep s
 };
 
 struct Maps {
@@ -115,7 +126,7 @@ __device__ __forceinline__ Round decode_round(const RawRound &r) {
 }
 
 __device__ __forceinline__ bool last_follows(const Barriers *bars, int s) {
-  return s >= 1 && (s >= kMaxNewton || *reinterpret_cast<const volatile int *>(&bars->more[s]) == 0);
+  return s >= kMaxNewton || *reinterpret_cast<const volatile int *>(&bars->more[s]) == 0;
 }
 
 // v when sel < 0, -inf otherwise (one select instruction on the sign of an integer).
@@ -170,7 +181,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     mbar_init(&bars->q_full, 1);
     for (int s = 0; s < kSBufs; ++s) {
       mbar_init(&bars->s_full[s], 1);
-      mbar_init(&bars->s_empty[s], kNormThreads);
+      mbar_init(&bars->s_empty[s], kNormWarps);
     }
     for (int s = 0; s < C::kStages; ++s) {
       mbar_init(&bars->in_full[s], 1);
@@ -180,8 +191,8 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
       mbar_init(&bars->v_full[s], 1);
       mbar_init(&bars->v_empty[s], 1);
     }
-    mbar_init(&bars->sweep_done, kNormThreads);
-    mbar_init(&bars->decided, kNormThreads + 2);  // + the copy and product threads, which run ahead of it
+    mbar_init(&bars->sweep_done, kNormWarps);
+    mbar_init(&bars->decided, kNormWarps + 2);  // + the copy and product threads, which run ahead of it
     mbar_init(&bars->o_done, 1);
     bars->abort_flag = 0;
     for (int s = 0; s < kMaxNewton + 2; ++s) bars->more[s] = 0;
@@ -265,6 +276,8 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
       };
       const int n_ahead = T < C::kStages ? T : C::kStages;
       for (int vv = 0; vv < T && ok; ++vv) ok = copy_k();  // sweep 0
+      const int v_ahead = T < C::kVStages ? T : C::kVStages;  // (the V ring serves the last sweep only)
+      for (int vv = 0; vv < v_ahead && ok; ++vv) ok = copy_v(vv);
       for (int sw = 0; ok; ++sw) {
         // sweep sw is issued and is not the last: the head of sweep sw + 1, before the decision
         for (int vv = 0; vv < n_ahead && ok; ++vv) ok = copy_k();
@@ -276,7 +289,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         const bool last = last_follows(bars, sw);
         for (int vv = 0; vv < T && ok; ++vv) {
           if (vv >= n_ahead) ok = copy_k();
-          if (ok && last) ok = copy_v(vv);
+          if (ok && last && vv >= v_ahead) ok = copy_v(vv);
         }
         if (last) break;
       }
@@ -376,6 +389,39 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     float2 *my_stats = stats + wg * 128 + r;
     float *my_tau = taus + wg * 128 + r;
     float cnt = 0.f;
+    float *list = reinterpret_cast<float *>(smem + C::kListOffset) + 144 * wg + r;  // entry k at list[k * kListPitch]
+    int n_list = 0;
+    bool overflow = false;
+    // This thread's list without the entries that cannot lie above tau: three Newton steps on the list from `thr`, a
+    // lower bound of its root; they stay below it (the sum is convex in tau).
+    auto prune = [&](float thr) {
+#pragma unroll 1
+      for (int it = 0; it < 3; ++it) {
+        float S1 = 0.f, S2 = 0.f;
+#pragma unroll 4
+        for (int k = 0; k < n_list; ++k) {
+          const float u = __saturatef(list[k * kListPitch] - thr);
+          S1 += u;
+          S2 = fmaf(u, u, S2);
+        }
+        if (S2 > 1.f) thr += 0.999f * (S2 - 1.f) / (2.f * S1);  // (0.999: never above the root by rounding)
+      }
+      int kept = 0;
+      for (int k = 0; k < n_list; ++k) {
+        const float x = list[k * kListPitch];
+        if (x > thr) {
+          list[kept * kListPitch] = x;
+          ++kept;
+        }
+      }
+      n_list = kept;
+      if (n_list > kListCap) {
+        overflow = true;
+        n_list = 0;
+      }
+      return thr;
+    };
+    float list_thr = -CUDART_INF_F;  // entries at or below it cannot lie above tau
 
     // kept-entry bits of this thread's 64 columns of the round (0 for the columns of unused groups),
     // fetched one visit ahead
@@ -431,6 +477,17 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
               m3 = fmax3(m3, t[e + 3], t[e + 7]);
             }
             st.x = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
+            list_thr = fmaxf(list_thr, st.x - 1.f);
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+#pragma unroll
+              for (int e = 16 * half; e < 16 * half + 16; ++e)
+                if (t[e] > list_thr) {
+                  list[n_list * kListPitch] = t[e];
+                  ++n_list;
+                }
+              if (__any_sync(0xffffffffu, n_list > kListCap)) list_thr = prune(list_thr);
+            }
           } else if (kind == 1) {
             float a0 = st.x, a1 = 0.f, a2 = 0.f, a3 = 0.f, q0 = st.y, q1 = 0.f, q2 = 0.f, q3 = 0.f;
 #pragma unroll
@@ -467,13 +524,16 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         }
         // S[buf] is read; in the last sweep it now holds P for the product
         tc_fence_before_sync();
-        mbar_arrive(&bars->s_empty[buf]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->s_empty[buf]);
       }
       if (!ok) break;
       *my_stats = st;
-      cnts[wg * 128 + r] = cnt;
+      cnts[wg * 128 + r] = sw == 0 ? __int_as_float(n_list) : cnt;
+      if (sw == 0 && overflow) *reinterpret_cast<volatile int *>(&bars->more[0]) = 1;
       // ---- end of a sweep: the two halves of every row meet
-      mbar_arrive(&bars->sweep_done);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->sweep_done);
       ok = wait(&bars->sweep_done, (uint32_t)sw & 1u);
       if (!ok) break;
       const float2 s0 = stats[r], s1 = stats[128 + r];
@@ -510,6 +570,39 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         const float m = fmaxf(s0.x, s1.x);
         // No kept entry: every weight is 0 whatever the score
         tau = m == -CUDART_INF_F ? CUDART_INF_F : m - kFirstGap;
+        if (!last_follows(bars, 0)) {
+          *my_tau = tau;
+        } else {
+          // No list overflowed: this warp finds tau of rows 16 warp .. 16 warp + 15, lane l from the list of half l / 16
+          // (both lanes of a row see the same sums: they add the same two numbers).
+          const int lr = 16 * warp + (lane & 15), lh = lane >> 4;
+          const float *ll = reinterpret_cast<const float *>(smem + C::kListOffset) + 144 * lh + lr;
+          const int ln = __float_as_int(cnts[lh * 128 + lr]);
+          const float lm = fmaxf(stats[lr].x, stats[128 + lr].x);
+          float lt = lm == -CUDART_INF_F ? CUDART_INF_F : lm - kFirstGap;
+          bool going = lm != -CUDART_INF_F;
+#pragma unroll 1
+          for (int it = 0; it < kMaxNewton && __any_sync(0xffffffffu, going); ++it) {
+            float S1 = 0.f, S2 = 0.f, n = 0.f;
+#pragma unroll 4
+            for (int k = 0; k < ln; ++k) {
+              const float u = __saturatef(ll[k * kListPitch] - lt);
+              S1 += u;
+              S2 = fmaf(u, u, S2);
+              n += u > 0.f ? 1.f : 0.f;
+            }
+            S1 += __shfl_xor_sync(0xffffffffu, S1, 16);
+            S2 += __shfl_xor_sync(0xffffffffu, S2, 16);
+            n += __shfl_xor_sync(0xffffffffu, n, 16);
+            const float disc = S1 * S1 - n * (S2 - 1.f);
+            const float step = S1 > 0.f ? (S2 - 1.f) / (S1 + (disc >= 0.f ? sqrtf(disc) : S1)) : 0.f;
+            if (going) {
+              lt += step;
+              going = fabsf(step) > 2e-6f * fmaxf(1.f, fabsf(lt));
+            }
+          }
+          taus[lh * 128 + lr] = lt;
+        }
       } else {
         tau = *my_tau;
         const float S1 = s0.x + s1.x, S2 = s0.y + s1.y, n = cnts[r] + cnts[128 + r];
@@ -520,12 +613,13 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         // below the resolution of tau itself a step is rounding noise of the sums
         moved = fabsf(step) > 2e-6f * fmaxf(1.f, fabsf(tau));
       }
-      *my_tau = tau;
-      neg_tau = -tau;
+      if (sw > 0) *my_tau = tau;
       if (moved && row_ok) *reinterpret_cast<volatile int *>(&bars->more[sw]) = 1;
-      mbar_arrive(&bars->decided);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->decided);
       ok = wait(&bars->decided, (uint32_t)sw & 1u);
       if (!ok) break;
+      neg_tau = -*my_tau;
       last = last_follows(bars, sw);
     }
   }
