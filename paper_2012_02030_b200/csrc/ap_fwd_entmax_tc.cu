@@ -44,11 +44,9 @@ using namespace sm100;
 constexpr int kThreads = 320;
 constexpr int kNormWarps = 8;
 // Candidate lists: entries per thread before a list is pruned, and room for one more step of 16 columns.
-constexpr int kListCap = 32, kListRows = kListCap + 16;
+constexpr int kListCap = 24, kListRows = kListCap + 8;
 constexpr int kListPitch = 2 * 128 + 32;  // thread (wg, r) at 144 wg + r: the two halves of a row on different banks
 constexpr int kSubBytes = 128 * 128;
-constexpr uint32_t kTmemCols = 512;  // S x 3 (columns 0..383), O (columns 384..384 + d)
-constexpr int kSBufs = 3;            // S buffers in flight: a visit's hand-offs take longer than its work
 constexpr uint32_t kMaxPolls = 1u << 22;
 constexpr int kMaxNewton = 30;
 // The first trial threshold: this far below the row maximum (the root lies in [max - 1, max); from
@@ -61,8 +59,13 @@ struct Cfg {
   static constexpr int kTileBytes = kSub * kSubBytes;
   // K is copied again in every sweep and a list row is a few rounds long: a ring deep enough to hold
   // a short row whole keeps the copies several visits ahead of the products.  V is needed once.
-  static constexpr int kStages = D == 64 ? 4 : 3;         // K ring
-  static constexpr int kVStages = D == 64 ? 2 : 1;        // V ring (last sweep)
+  // d = 64: two CTAs share an SM and fill each other's waits (a list row is a few rounds long, so most of a CTA's
+  // time is one chain), each with half of TMEM: one S buffer.  d = 128: one CTA, three S buffers in flight.
+  static constexpr int kCtas = D == 64 ? 2 : 1;
+  static constexpr int kSBufs = D == 64 ? 1 : 3;
+  static constexpr uint32_t kTmemCols = D == 64 ? 256 : 512;  // S x kSBufs, then O
+  static constexpr int kStages = D == 64 ? 2 : 3;         // K ring
+  static constexpr int kVStages = 1;                      // V ring (last sweep)
   static constexpr int kKOffset = kTileBytes;             // after Q
   static constexpr int kVOffset = kKOffset + kStages * kTileBytes;
   static constexpr int kStatsOffset = kVOffset + kVStages * kTileBytes;
@@ -74,12 +77,13 @@ struct Cfg {
   static constexpr int kListOffset = kTauOffset + kTauBytes;
   static constexpr int kBarOffset = kListOffset + kListRows * kListPitch * 4;
   static constexpr int kSmemBytes = kBarOffset + 512 + 1024;
-  static_assert(kSmemBytes > 114 * 1024 && kSmemBytes <= 227 * 1024, "one CTA per SM, within the limit");
+  static_assert(kSmemBytes <= 227 * 1024 / kCtas - 1024, "within the limit");
+  static_assert((kCtas + 1) * kSmemBytes > 228 * 1024, "no more CTAs than TMEM has room for");
 };
 
 struct Barriers {
   uint64_t q_full;
-  uint64_t s_full[kSBufs], s_empty[kSBufs];
+  uint64_t s_full[3], s_empty[3];
   uint64_t in_full[6], in_empty[6];  // K ring: rows landed / S = Q K^T of the visit completed
   uint64_t v_full[2], v_empty[2];    // V ring: rows landed / O += P V of the visit completed
   uint64_t sweep_done;  // all statistics of the sweep are in shared memory
@@ -156,12 +160,14 @@ __device__ __forceinline__ float2 unpack2(uint32_t v) {
 }
 
 template <int D, bool kF16>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, Cfg<D>::kCtas)
 fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, const int32_t *__restrict__ round_ptr,
                   const int32_t *__restrict__ round_rows, const uint8_t *__restrict__ round_info,
                   const uint32_t *__restrict__ round_bitmap, int BH, int H, int Lq, int n_qt, float half_scale,
                   unsigned *err) {
   using C = Cfg<D>;
+  constexpr int kSBufs = C::kSBufs;
+  constexpr uint32_t kTmemCols = C::kTmemCols;
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem =
       reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -304,7 +310,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
   } else if (warp == 9) {
     // ------------------------------------------------------------ MMA issuer
     // S = Q K^T of the first visits of the next sweep is issued before the decision as well
-    // (three S buffers).
+    // (as many as there are S buffers).
     {
       constexpr uint32_t idesc_pv = idesc_bf16_f32(128, D, false, true, kF16);
       constexpr uint32_t kHi = smem_desc_hi_sw128(1024);
@@ -371,8 +377,10 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         } else {
           // visit by visit: S of the visit (unless issued above), then O += P V of the one before
           for (int vv = 0; vv < T && ok; ++vv) {
-            if (vv >= n_ahead) ok = issue_qk();
-            if (ok && vv > 0) ok = issue_pv(v_head + vv - 1, vv - 1);
+            // (a single S buffer holds P of the visit before until its product is over)
+            if (kSBufs == 1 && vv > 0) ok = issue_pv(v_head + vv - 1, vv - 1);
+            if (ok && vv >= n_ahead) ok = issue_qk();
+            if (kSBufs > 1 && ok && vv > 0) ok = issue_pv(v_head + vv - 1, vv - 1);
           }
           if (ok) issue_pv(v_head + T - 1, T - 1);
           break;
@@ -396,7 +404,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     // lower bound of its root; they stay below it (the sum is convex in tau).
     auto prune = [&](float thr) {
 #pragma unroll 1
-      for (int it = 0; it < 3; ++it) {
+      for (int it = 0; it < 1; ++it) {
         float S1 = 0.f, S2 = 0.f;
 #pragma unroll 4
         for (int k = 0; k < n_list; ++k) {
@@ -479,9 +487,9 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
             st.x = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
             list_thr = fmaxf(list_thr, st.x - 1.f);
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
+            for (int half = 0; half < 4; ++half) {
 #pragma unroll
-              for (int e = 16 * half; e < 16 * half + 16; ++e)
+              for (int e = 8 * half; e < 8 * half + 8; ++e)
                 if (t[e] > list_thr) {
                   list[n_list * kListPitch] = t[e];
                   ++n_list;
