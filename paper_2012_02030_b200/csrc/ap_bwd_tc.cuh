@@ -6,16 +6,12 @@
 namespace ap {
 namespace bwd {
 
-// Everything the two kernels read that is not a tensor: carved out of the caller's workspace.
+// What the two kernels hand on to one another.
 struct Plan {
-  float *neg_l;       // [B*H][n_qt*128]  -log2 of the row's sum of 2^(c S); -inf: no kept entry
-  float *dsum;        // [B*H][n_qt*128]  D_i = dO_i . O_i
-  int32_t *next;      // [2]              next item to hand out (rows kernel, columns kernel)
-  int32_t *tile_id;   // [H][n_qt][n_kt]  list position of a tile, -1 if it is not stored
-  int32_t *order;     // [H][8*n_kt]      16-key group at each position of the head's key order
-  int32_t *n_visits;  // [H][n_kt]        query tiles a key block of eight groups is visited by
-  uint32_t *visit;    // [H][n_kt][n_qt]  bits 0..23: query tile; bits 24..31: its 16-row groups that keep an entry
-  uint32_t *bits;     // [H][n_kt][n_qt][128 keys][4]  transposed bitmap of a visit: bit q of key row k
+  float *neg_l;     // [B*H][Lq]        -log2 of the row's sum of 2^(c S); -inf: no kept entry
+  float *dsum;      // [B*H][Lq]        D_i = dO_i . O_i
+  uint32_t *table;  // [H][n_qt][n_kt]  bits 0..23: list position of a tile; 24..31: its groups that keep an entry (0: not stored)
+  int32_t *next;    // [2]              next item to hand out (rows kernel, columns kernel)
 };
 
 struct RowsMaps {
@@ -38,9 +34,6 @@ struct Args {
   cudaStream_t s;
 };
 
-size_t plan_bytes(int B, int H, int Lq, int Lk);
-Plan plan_at(void *workspace, int B, int H, int Lq, int Lk);
-cudaError_t launch_plan(const Args &a);
 cudaError_t launch_rows(const RowsMaps &maps, const Args &a);
 cudaError_t launch_cols(const ColsMaps &maps, const Args &a);
 
