@@ -67,7 +67,7 @@ struct Shared {
   alignas(16) uint32_t words[kRing + 1][8 * kTile];  // plain: [query][4]; gathered: [group][query], the word that holds it
   alignas(16) float neg_l[kRing + 1][kTile];
   alignas(16) float dsum[kRing + 1][kTile];
-  uint8_t heavy[kMaxHeavy];               // [h][key tile]: its heavy groups
+  uint32_t order[kMaxHeavy];              // [h][key tile]: bits 0..7 its heavy groups; above: light groups in the tiles below
   uint64_t b_full[kRing + 1];             // words and statistics of a visit there
   uint64_t q_full[kRing], do_full[kRing];
   uint64_t s_full[kRing], dp_full[kRing];
@@ -90,8 +90,8 @@ struct Cfg {
   static constexpr int kKvBufs = D == 64 ? 2 : 1;
   static constexpr uint32_t kAccBufs = D == 64 ? 2 : 1;
   static constexpr int kSlotOffset = kKvBufs * 2 * L::kBytes;             // behind the (K, V) pairs
-  static constexpr int kOutOffset = kSlotOffset + kRing * 2 * L::kBytes;  // 4 KB per finishing warp
-  static constexpr int kSharedOffset = kOutOffset + 4 * 4096;
+  static constexpr int kOutOffset = kSlotOffset + kRing * 2 * L::kBytes;  // 2 KB per finishing warp
+  static constexpr int kSharedOffset = kOutOffset + 4 * 2048;
   static constexpr int kSmemBytes = kSharedOffset + (int)sizeof(Sh) + 1024;
   static_assert(kSmemBytes <= 227 * 1024, "shared memory");
   static_assert(kSmemBytes > 114 * 1024, "one CTA per SM: all of TMEM is taken");
@@ -179,7 +179,24 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
         for (int p = 0; p < 8; ++p) below += 2u * ((c[p >> 1] >> (16 * (p & 1))) & 0xffffu) + 2u < mine ? 1 : 0;
         heavy |= (below >= 4 ? 1u : 0u) << q;
       }
-      sh->heavy[x] = (uint8_t)heavy;
+      sh->order[x] = heavy;
+    }
+    __syncthreads();
+    for (int h = warp; h < H; h += kThreads / 32) {
+      uint32_t below = 0u;
+      for (int kt0 = 0; kt0 < n_kt; kt0 += 32) {
+        uint32_t *mine = sh->order + h * n_kt + kt0 + lane;
+        const bool there = kt0 + lane < n_kt;
+        const uint32_t heavy = there ? *mine : 0xffu, light = 8u - __popc(heavy);
+        uint32_t incl = light;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += y;
+        }
+        if (there) *mine = heavy | (below + incl - light) << 8;
+        below += __shfl_sync(0xffffffffu, incl, 31);
+      }
     }
   }
   tc_fence_before_sync();
@@ -203,11 +220,8 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
     uint32_t g = 0, n = 0;    // visits / items with visits so far
     int k_armed = -1, v_armed = -1;
     uint32_t last1 = 0, last2 = 0;  // last visit of the item before, and of the one before that
-    auto draw = [&]() {
-      int x = 0;
-      if (lane == 0) x = atomicAdd(next, 1);  // (every CTA begins with the item of its own number)
-      return (int)gridDim.x + __shfl_sync(0xffffffffu, x, 0);
-    };
+    // (every CTA begins with the item of its own number; a number is drawn an item ahead of its use)
+    auto draw = [&]() { return lane == 0 ? (int)gridDim.x + atomicAdd(next, 1) : 0; };
     // Items: four neighbouring key blocks of a (b, h) in a row (they share query tiles, which are then read from L2
     // once for all four), the sets of four from the last to the first (the last hold the keys that most query
     // tiles keep, so the long items come first), all (b, h) of a set in a row.
@@ -226,7 +240,8 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
         it.word[q] = qt < n_qt ? ldg_now_u32(row + kt) : 0u;
       }
     };
-    auto look_up = [&](int k) {
+    auto look_up = [&](int drawn) {
+      const int k = __shfl_sync(0xffffffffu, drawn, 0);
       Item it;
       it.bh = 0, it.block = -1, it.group = 0, it.plain = true;
       if (k >= BH * n_kt) return it;
@@ -235,40 +250,21 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
       it.block = n_kt - 1 - 4 * set - x % in_set;
       it.group = 8 * it.block + (lane & 7);
       if (ordered) {
-        // lane q < 8: the group at position 8 block + q of the order; positions count the light groups first
-        const uint8_t *heavy = sh->heavy + (it.bh % H) * n_kt;
-        int n_light = 0;
-        for (int kt0 = 0; kt0 < n_kt; kt0 += 32)
-          n_light += __reduce_add_sync(0xffffffffu, kt0 + lane < n_kt ? 8 - __popc((uint32_t)heavy[kt0 + lane]) : 0);
+        // lane q < 8: the group at position 8 block + q of the order, which counts the light groups first
+        const uint32_t *order = sh->order + (it.bh % H) * n_kt;
+        const int n_light = (int)(order[n_kt - 1] >> 8) + 8 - __popc(order[n_kt - 1] & 0xffu);
         if (n_light < 8 * n_kt) {
-          int found = 0;
-          int before[2] = {0, 0};  // light / heavy groups in the key tiles below kt0
-          for (int kt0 = 0; kt0 < n_kt; kt0 += 32) {
-            const uint32_t hv = kt0 + lane < n_kt ? heavy[kt0 + lane] : 0x100u;
-#pragma unroll
-            for (int kind = 0; kind < 2; ++kind) {
-              const uint32_t mine = hv == 0x100u ? 0u : kind ? hv : ~hv & 0xffu;
-              int incl = __popc(mine);
-#pragma unroll
-              for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-              }
-              const int total = __shfl_sync(0xffffffffu, incl, 31);
-#pragma unroll 1
-              for (int q = 0; q < 8; ++q) {
-                const int pos = 8 * it.block + q - (kind ? n_light : 0) - before[kind];  // among this kind, in these tiles
-                if ((8 * it.block + q >= n_light) != (kind == 1) || pos < 0 || pos >= total) continue;
-                const int src = __popc(__ballot_sync(0xffffffffu, incl <= pos));  // the tile that holds it
-                const int below = __shfl_sync(0xffffffffu, incl - __popc(mine), src);
-                uint32_t set_bits = __shfl_sync(0xffffffffu, mine, src);
-                for (int skip = pos - below; skip > 0; --skip) set_bits &= set_bits - 1u;
-                if (lane == q) found = 8 * (kt0 + src) + __ffs((int)set_bits) - 1;
-              }
-              before[kind] += total;
-            }
+          const bool heavy = it.group >= n_light;
+          const int pos = heavy ? it.group - n_light : it.group;  // among its kind
+          auto below = [&](int kt) { return heavy ? 8 * kt - (int)(order[kt] >> 8) : (int)(order[kt] >> 8); };
+          int lo = 0, hi = n_kt - 1;  // the last key tile with no more than pos of the kind below it holds the group ...
+          while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (below(mid) <= pos) lo = mid; else hi = mid - 1;
           }
-          it.group = found;
+          uint32_t kind = heavy ? order[lo] & 0xffu : ~order[lo] & 0xffu;
+          for (int skip = pos - below(lo); skip > 0; --skip) kind &= kind - 1u;  // ... as its (pos - below)-th
+          it.group = 8 * lo + __ffs((int)kind) - 1;
           const int first = __shfl_sync(0xffffffffu, it.group, 0);
           it.plain = (first & 7) == 0 && __all_sync(0xffffffffu, lane >= 8 || it.group == first + lane);
         }
@@ -542,7 +538,6 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
   } else if (warp < kComputeWarps) {
     // ------------------------------------------------------------ P and dS
     const int chunk0 = warp >> 2;          // queries [32 ch, 32 ch + 32) of every visit, ch = chunk0, chunk0 + 2
-    const int r = (warp & 3) * 32 + lane;  // key row of the block == TMEM lane
     const uint32_t tmem_s = tmem + ((uint32_t)((warp & 3) * 32) << 16), tmem_dp = tmem_s + kTmemDp;
     const float c = scale * kLog2e;
     // Before the transpose lane l holds query 4 (7 - l mod 8) + l / 8 of the chunk, so that a key's word holds the bits of
@@ -655,7 +650,7 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
     // ------------------------------------------------------------ dV and dK of the last item
     const int wr = (warp & 3) * 32;
     const uint32_t lane_addr = (uint32_t)wr << 16;
-    unsigned char *out_s = smem + C::kOutOffset + (warp - kFinish) * 4096;
+    unsigned char *out_s = smem + C::kOutOffset + (warp - kFinish) * 2048;
     bool ok = true;
     for (uint32_t n = 0; ok; ++n) {
       const uint32_t ab = n % C::kAccBufs;
@@ -686,10 +681,10 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
         __syncwarp();
         if (lane == 0) mbar_arrive(which ? &sh->dk_free[ab] : &sh->dv_free[ab]);
 #pragma unroll
-        for (int x = 0; x < D / 64; ++x)
-          store_rows64(out_s, lane, &pk[32 * x], [&](int rr) -> uint16_t * {
+        for (int x = 0; x < D / 32; ++x)
+          store_rows<32>(out_s, lane, &pk[16 * x], [&](int rr) -> uint16_t * {
             const int j = (rr < 16 ? j0 : j1 - 16) + rr;
-            return j < Lk ? out + (size_t)j * D + 64 * x : nullptr;
+            return j < Lk ? out + (size_t)j * D + 32 * x : nullptr;
           });
       }
     }

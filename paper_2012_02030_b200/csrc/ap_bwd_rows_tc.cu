@@ -644,7 +644,7 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
           __syncwarp();
           if (lane == 0) mbar_arrive(&sh->o_free);  // the next item may overwrite dQ
         }
-        store_rows64(out_s, lane, pk,
+        store_rows<64>(out_s, lane, pk,
                      [&](int rr) -> uint16_t * { return rr < n_rows ? rows_out + (size_t)rr * D + 64 * x : nullptr; });
       }
     }
