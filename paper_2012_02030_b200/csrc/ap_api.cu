@@ -210,13 +210,11 @@ ap_status build_mask_impl(const float *acc, int H, int Lq, int Lk, double keep_f
   a.nnz = nnz_per_head;
   a.stage_bitmap = tiles ? reinterpret_cast<uint32_t *>(ws) : nullptr;
   a.stage_count = tiles ? reinterpret_cast<int32_t *>(ws + (size_t)n_tiles * kBitmapWords * sizeof(uint32_t)) : nullptr;
+  a.stage_groups = tiles ? reinterpret_cast<uint32_t *>(a.stage_count) + ((size_t)n_tiles * 4 + 255) / 256 * 64 : nullptr;
   a.scratch = ws + stage;
-  if (launch_build_mask(a, s) != cudaSuccess) return AP_ERR_CUDA;
-  if (tiles) {
-    fill_tiles_shape(tiles, H, Lq, Lk);
-    if (launch_compact_tiles(a.stage_bitmap, a.stage_count, *tiles, s) != cudaSuccess) return AP_ERR_CUDA;
-  }
-  return AP_OK;
+  if (tiles) fill_tiles_shape(tiles, H, Lq, Lk);
+  a.tiles = tiles;
+  return launch_build_mask(a, s) == cudaSuccess ? AP_OK : AP_ERR_CUDA;
 }
 }  // namespace
 

@@ -2,37 +2,44 @@
 //
 // Order of the entries of one head: forced (diagonal) first, then larger fp32
 // value, then lower linear index i*Lk + j.  The k-th entry of that order is
-// found with a most-significant-digit-first radix select over order-preserving
-// 32-bit keys: three digits of 11, 11 and 10 bits, one histogram pass over the
-// accumulator each.  Large heads first try a shortcut that needs one pass: a
-// random sample of the head brackets the threshold between two pivot keys, one
+// found with a most-significant-digit-first radix select over the pair (order-preserving
+// 32-bit key of the value, complement of the index): digits of 11, 11 and 10 bits each.  The
+// first three give the threshold; the last three, the index of the last kept entry equal to it,
+// run only where some of those entries are kept and others are not.
+//
+// Small inputs (up to kDirectEntries in all, a few times less than L2 holds) select straight over the
+// accumulator, one pass over it per digit.  Larger ones take a shortcut that reads it once: a
+// random sample of the selection brackets the threshold between two pivot keys, one
 // pass counts the keys above the upper pivot and collects those between the
-// pivots, and the threshold is selected among the collected keys (the same radix
-// select on their offsets from the lower pivot, grid-wide); it is exact
-// whenever the bracket holds the threshold and the collected keys fit their
-// buffer (checked with the exact counts), else the head takes the three passes.  Entries equal to the threshold key are all kept when the
-// count allows it (the usual case); otherwise they are ranked by linear index
-// with per-row-segment tie counts and a prefix sum, so that exactly k entries
-// are kept.  The emit pass writes the element mask and per-tile bitmaps;
-// ap_tiles.cu compacts them.  Integer work throughout: no floating-point
-// arithmetic decides a bit.
+// pivots, and the select runs over the collected entries; it is exact whenever the bracket holds
+// the threshold and the collected entries fit their buffer (checked with the exact counts), else
+// the selection takes the passes over the accumulator.  All of the select is ONE cooperative kernel
+// (select_kernel): the CTAs of a selection meet at a bounded barrier after each digit.  As a chain of
+// kernels (a histogram per digit, a pick, a tie count, a scan, each launched whether or not it had
+// work) the mask of one layer of 16 heads x 512 tokens took 18 launches and 132 us.
+//
+// The emit pass writes the element mask and per-tile bitmaps; ap_tiles.cu compacts them.  Integer work
+// throughout: no floating-point arithmetic decides a bit.
 //
 // One threshold for the whole layer (Eq. 2 as stated) is the same selection run
 // once over a virtual head of H*Lq rows: row i' = h*Lq + i has the domain of row
 // i, and the linear index i'*Lk + j is the layer-wide tie order.
 #include "ap_common.cuh"
+#include "ap_grid.cuh"
 
 namespace ap {
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 256;  // collect_kernel
 constexpr int kWarps = kThreads / 32;
 constexpr int kBins = 2048;
-constexpr int kPasses = 3;
+constexpr int kPasses = 3;     // digits of a key (and of an index)
 
 __host__ __device__ constexpr int digit_shift(int pass) { return pass == 0 ? 21 : (pass == 1 ? 10 : 0); }
 __host__ __device__ constexpr uint32_t digit_mask(int pass) { return pass == 2 ? 0x3ffu : 0x7ffu; }
+// the bits above a digit
+__host__ __device__ constexpr uint32_t above_digit(int pass) { return pass == 0 ? 0u : pass == 1 ? 0xffe00000u : 0xfffffc00u; }
 
 // Larger float <=> larger key; -0 is mapped onto +0 first.
 __device__ __forceinline__ uint32_t key_of(float f) {
@@ -48,73 +55,34 @@ __device__ __forceinline__ float float_of_key(uint32_t key) {
   return __uint_as_float((key & 0x80000000u) ? (key ^ 0x80000000u) : ~key);
 }
 
-struct SelectState {  // per selection
-  uint32_t prefix;    // digits of the threshold key found so far
-  uint32_t thr;       // threshold key (valid after the last digit)
-  unsigned long long remaining;  // rank still to resolve inside the current prefix
-  unsigned long long ties_kept;  // entries equal to thr that are kept (lowest indices first)
-  uint32_t all_ties_kept;        // every entry equal to thr is kept: no ranking needed
-  uint32_t done;                 // thr, ties_kept, all_ties_kept are final (set by the one-pass shortcut)
+struct alignas(64) SelectState {  // per selection; all zero before the first kernel of a call
+  uint32_t thr;                  // threshold key; 0xffffffff: nothing but the forced entries is kept
+  uint32_t tie_cut;              // entries equal to the threshold are kept up to this linear index
   // the shortcut's bracket and what the collecting pass found
   uint32_t lo, hi;               // pivot keys, lo <= hi; hi == 0xffffffff: no upper pivot
   unsigned long long above_hi;   // keys > hi
   uint32_t n_cand;               // keys in [lo, hi] (may exceed the buffer: then the shortcut fails)
   uint32_t use_shortcut;
-  // when not all entries equal to thr are kept: those with linear index i*Lk + j <= tie_cut are
-  // (valid if have_cut; otherwise the ties are ranked with tie counts and a prefix sum)
-  uint32_t tie_cut, have_cut;
-  // selection among the collected keys
-  uint32_t cand_select;          // the bracket holds the threshold: the passes over the collected keys run
-  uint32_t thr_count;            // entries equal to the threshold key
-  uint32_t tie_n;                // entries gathered in the tie list
-  // the classifying pass and the patch pass have written this selection's mask and tile bitmaps: the
+  // the classifying pass and the select have written this selection's mask and tile bitmaps: the
   // emit pass has nothing left to do for it
   uint32_t emitted;
-  // CTAs of the running kernel that have finished their share of this selection: the last one goes on
-  // with the step that needs all of them (digit pick, tie scan, finish) and puts the count back to zero
-  uint32_t ticket;
+  uint32_t barrier;              // arrivals of the selection's CTAs so far
 };
 
-// Called by all threads of a CTA when its share of selection h is done (its global writes issued):
-// true in exactly the CTA that finishes last, which then sees everything the others wrote.
-__device__ __forceinline__ bool last_cta_of(SelectState *state, int h, uint32_t n_ctas) {
-  __shared__ uint32_t last_s;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const bool last = atomicAdd(&state[h].ticket, 1u) == n_ctas - 1u;
-    if (last) state[h].ticket = 0u;
-    last_s = last ? 1u : 0u;
-  }
-  __syncthreads();
-  if (last_s) __threadfence();
-  return last_s != 0u;
-}
-
-// Selection among the keys the one-pass shortcut collected (see below).
-// The bracket holds the threshold (the (k_rest - above_hi)-th largest collected key) and every key
-// of the bracket was collected.  All fields are final once the collecting pass has ended.
-__device__ __forceinline__ bool bracket_holds(const SelectState &st, uint32_t cand_cap, unsigned long long k_rest) {
-  return st.use_shortcut && st.n_cand <= cand_cap && st.above_hi < k_rest && k_rest - st.above_hi <= st.n_cand;
-}
-// All offsets are at most hi - lo: a leading digit in which that span is zero is zero for every
-// key and needs no pass (the pick leaves the digit at zero).
-__device__ __forceinline__ bool digit_is_zero(const SelectState &st, int pass) {
-  return pass < kPasses - 1 && ((st.hi - st.lo) >> digit_shift(pass)) == 0u;
-}
-
-constexpr int kMaxCutTies = 4096;  // ties with the threshold ranked inside the shortcut (more: tie counts + scan)
+constexpr int kHistBuffers = 3;      // a digit's counts; zeroed again two digits later
+constexpr int kMaxSharedSelections = 128;  // selections with more than one CTA (see select_kernel), at most
 
 struct Scratch {
-  uint32_t *hist;       // [H][kBins]
   SelectState *state;   // [H]
-  uint32_t *tie_count;  // [H][Lq][n_kt] -> exclusive prefix after the scan
-  uint32_t *tie_list;   // [H][kMaxCutTies] linear indices of the collected entries equal to the threshold
+  uint32_t *hist;       // [min(H, kMaxSharedSelections)][kHistBuffers][kBins]
   uint2 *cand;          // [H][cand_cap] (key, linear index) of the entries collected by the shortcut
 };
 
-// The shortcut is tried for heads of at least this many selectable entries.
+// The shortcut is tried for selections of at least this many entries, when all of them together have more
+// than kDirectEntries: passes over an accumulator that L2 holds cost less than drawing the pivots and
+// collecting (16 heads x 512 causal, one selection of 2.1 M entries: see launch_build_mask).
 constexpr long long kShortcutMinEntries = 1ll << 20;
+constexpr long long kDirectEntries = 12ll << 20;
 constexpr int kSamples = 16384;  // draws per head (over the Lq x Lk rectangle; draws outside the domain are dropped)
 __host__ __device__ inline long long cand_capacity(long long n_rest) {
   return n_rest >= kShortcutMinEntries ? n_rest / 16 : 0;
@@ -134,195 +102,40 @@ __device__ __forceinline__ void load4(const float *__restrict__ row, int j0, int
   }
 }
 
-// n_sel selections (one per head, or one for the layer); nnz[H] starts at nnz_init.
-__global__ void init_state_kernel(SelectState *state, uint32_t *hist, int n_sel, unsigned long long k_rest, int H,
-                                  long long nnz_init, int64_t *nnz) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < n_sel * kBins) hist[idx] = 0u;
-  if (nnz && idx < H) nnz[idx] = nnz_init;
-  if (idx < n_sel) {
-    state[idx].prefix = 0u;
-    state[idx].thr = 0xffffffffu;
-    state[idx].remaining = k_rest;
-    state[idx].ties_kept = 0ull;
-    state[idx].all_ties_kept = 0u;
-    state[idx].done = 0u;
-    state[idx].lo = 0u;
-    state[idx].hi = 0xffffffffu;
-    state[idx].above_hi = 0ull;
-    state[idx].n_cand = 0u;
-    state[idx].use_shortcut = 0u;
-    state[idx].tie_cut = 0u;
-    state[idx].have_cut = 0u;
-    state[idx].cand_select = 0u;
-    state[idx].thr_count = 0u;
-    state[idx].tie_n = 0u;
-    state[idx].emitted = 0u;
-    state[idx].ticket = 0u;
-  }
-}
-
-__device__ void pick_digit(SelectState *state, uint32_t *hist, int h, int pass, int from_cand, uint32_t cand_cap,
-                           unsigned long long k_rest);
-
-// Histogram of one digit over the non-forced domain entries whose higher digits
-// equal the prefix found so far; the CTA that finishes last picks the digit.  grid = (row blocks, selections); a warp takes a row at
-// a time and its lanes stride over the row, two float4 loads in flight each.
-// Here and in the kernels below Lq counts the rows of the selection and row i has
-// the domain of row i % period of a head (period == Lq unless heads are stacked).
-// Under the causal constraint row r of a head sees the keys j <= r + (Lk - period):
-// Lk - period memory keys, then its own segment; its own position r + (Lk - period)
-// is the forced entry when the diagonal is kept.
-__global__ void __launch_bounds__(kThreads) digit_histogram_kernel(const float *__restrict__ acc, int Lq, int Lk,
-                                                                   int period, int causal, int diag, int pass,
-                                                                   SelectState *state, uint32_t *hist) {
-  __shared__ uint32_t sh[kBins];
-  const int h = blockIdx.y;
-  if (state[h].done) return;  // resolved by the shortcut
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int b = threadIdx.x; b < kBins; b += kThreads) sh[b] = 0u;
-  __syncthreads();
-  const int shift = digit_shift(pass);
-  const uint32_t dmask = digit_mask(pass);
-  const uint32_t prefix = state[h].prefix;
-  const uint32_t hi_mask = pass == 0 ? 0u : ~((1u << (shift + (pass == 1 ? 11 : 10))) - 1u);
-  const uint32_t want_hi = prefix & hi_mask;
-  const bool vec = (Lk & 3) == 0;
-  const int off = (causal || diag) ? Lk - period : 0;
-  for (int i = blockIdx.x * kWarps + warp; i < Lq; i += gridDim.x * kWarps) {
-    const float *row = acc + ((size_t)h * Lq + i) * Lk;
-    const int own = i % period + off;  // the row's own position among the keys
-    const int jend = causal ? min(Lk, own + 1) : Lk;
-    for (int base = 0; base < jend; base += 256) {  // warp-uniform trip count
-      float v[2][4];
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int j0 = base + 128 * u + 4 * lane;
-        v[u][0] = v[u][1] = v[u][2] = v[u][3] = 0.f;
-        if (j0 < jend) load4(row, j0, jend, vec, v[u]);
-      }
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int j0 = base + 128 * u + 4 * lane;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int j = j0 + c;
-          const uint32_t key = key_of(v[u][c]);
-          const bool take = j < jend && !(diag && j == own) && ((key & hi_mask) == want_hi);
-          const uint32_t bin = (key >> shift) & dmask;
-          // lanes that hit the same bin elect one to add their count
-          const unsigned voters = __ballot_sync(0xffffffffu, take);
-          if (take) {
-            const unsigned peers = __match_any_sync(voters, bin);
-            if (lane == __ffs(peers) - 1) atomicAdd(&sh[bin], (uint32_t)__popc(peers));
-          }
-        }
-      }
-    }
-  }
-  __syncthreads();
-  for (int b = threadIdx.x; b < kBins; b += kThreads) {
-    const uint32_t s = sh[b];
-    if (s) atomicAdd(&hist[h * kBins + b], s);
-  }
-  if (last_cta_of(state, h, gridDim.x)) pick_digit(state, hist, h, pass, 0, 0u, 0ull);
-}
-
-// One CTA per head: picks the digit whose bin contains the wanted rank.  Thread t
-// owns bins [kBins-1-8t, kBins-8-8t] (descending); a block-wide prefix over the
-// threads' sums locates the owner, which then walks its eight bins.
-// from_cand: the histogram came from the collected keys (offsets from the lower pivot); the first
-// such pass opens the selection among them if the bracket holds the threshold.
-// Run by the last CTA (256 threads) of the histogram pass that filled hist.
-__device__ void pick_digit(SelectState *state, uint32_t *hist, int h, int pass, int from_cand, uint32_t cand_cap,
-                           unsigned long long k_rest) {
-  __shared__ uint32_t warp_sums[8];
-  if (!from_cand && state[h].done) return;  // resolved by the shortcut
-  if (from_cand) {
-    const SelectState cur = state[h];
-    if (!(pass == 0 ? bracket_holds(cur, cand_cap, k_rest) : cur.cand_select != 0u)) return;
-    if (digit_is_zero(cur, pass)) {
-      if (pass == 0 && threadIdx.x == 0) {
-        state[h].remaining = k_rest - cur.above_hi;
-        state[h].prefix = 0u;
-        state[h].cand_select = 1u;
-      }
-      return;
-    }
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t cnt[8];
-  uint32_t mine = 0u;
-#pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    const int bin = kBins - 1 - (8 * (int)threadIdx.x + e);
-    cnt[e] = __ldcg(hist + h * kBins + bin);
-    hist[h * kBins + bin] = 0u;
-    mine += cnt[e];
-  }
-  uint32_t incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
-  }
-  if (lane == 31) warp_sums[warp] = incl;
-  SelectState st = state[h];  // read by everyone before the barrier, written by the owner after it
-  if (from_cand && pass == 0) {
-    st.remaining = k_rest - st.above_hi;
-    st.prefix = 0u;
-    st.cand_select = 1u;
-  }
-  __syncthreads();
-  unsigned long long before = incl - mine;  // entries in bins above this thread's
-  for (int w = 0; w < warp; ++w) before += warp_sums[w];
-  // the owner: fewer than `remaining` entries above its bins, at least that many including them;
-  // the last thread also takes the case of an over-long rank (cannot happen for valid k)
-  const bool owner = before < st.remaining && (before + mine >= st.remaining || threadIdx.x == 255);
-  if (owner) {
-    unsigned long long above = before;
-    int e = 0;
-    for (; e < 7; ++e) {
-      if (above + cnt[e] >= st.remaining) break;
-      above += cnt[e];
-    }
-    const int bin = kBins - 1 - (8 * (int)threadIdx.x + e);
-    SelectState out = st;
-    out.remaining = st.remaining - above;
-    out.prefix = st.prefix | ((uint32_t)bin << digit_shift(pass));
-    if (pass == kPasses - 1) {
-      out.thr = out.prefix;
-      out.ties_kept = out.remaining;
-      out.all_ties_kept = out.remaining == cnt[e] ? 1u : 0u;
-      out.thr_count = cnt[e];
-    }
-    state[h] = out;
-  }
-}
+// Here and below `rows` counts the rows of a selection and row i has the domain of row i % period
+// of a head (period == rows unless heads are stacked).  Under the causal constraint row r of a head
+// sees the keys j <= r + (Lk - period): Lk - period memory keys, then its own segment; its own
+// position r + (Lk - period) is the forced entry when the diagonal is kept.
 
 // ---- the one-pass shortcut ------------------------------------------------------------------
 
-// CTA-wide (1024 threads) radix select: the key of rank `rank` (1 = largest) among keys[0..n),
-// 1 <= rank <= n.  Returns the key, how many keys equal it, and the rank inside that group of
-// equals.  hist: 2048 words of shared memory; xch: 4 words.
-struct Picked {
-  uint32_t key, count, rank_in_ties;
-};
-// scan(fn) calls fn(key) once for every key, the keys spread over the CTA's threads in any way.
-template <typename Scan>
-__device__ Picked block_select_over(uint32_t n, uint32_t rank, uint32_t *hist, uint32_t *xch, Scan scan) {
+__device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
+  x += 0x9e3779b97f4a7c15ull;
+  x = (x ^ (x >> 30)) * 0xbf58476d1ce4e5b9ull;
+  x = (x ^ (x >> 27)) * 0x94d049bb133111ebull;
+  return x ^ (x >> 31);
+}
+
+// CTA-wide (1024 threads): the leading 22 bits of the key of rank `rank` (1 = largest) among keys[0..n),
+// 1 <= rank <= n.  hist: kBins words of shared memory; xch: 2 words.
+__device__ uint32_t block_select22(const uint32_t *keys, uint32_t n, uint32_t rank, uint32_t *hist, uint32_t *xch) {
   __shared__ uint32_t warp_sums[32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  uint32_t prefix = 0u, hi_mask = 0u, count = n;
-  for (int pass = 0; pass < kPasses; ++pass) {
+  uint32_t prefix = 0u;
+  for (int pass = 0; pass < 2; ++pass) {
     const int shift = digit_shift(pass);
-    const uint32_t dmask = digit_mask(pass);
     hist[t] = 0u;
     hist[t + 1024] = 0u;
     __syncthreads();
-    scan([&](uint32_t key) {
-      if ((key & hi_mask) == prefix) atomicAdd(&hist[(key >> shift) & dmask], 1u);
-    });
+    for (uint32_t idx0 = t; idx0 < n; idx0 += 8 * 1024) {  // eight loads in flight per thread
+      uint32_t kk[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) kk[u] = idx0 + u * 1024 < n ? keys[idx0 + u * 1024] : 0u;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (idx0 + u * 1024 < n && (kk[u] & above_digit(pass)) == prefix)
+          atomicAdd(&hist[(kk[u] >> shift) & digit_mask(pass)], 1u);
+    }
     __syncthreads();
     // thread t owns bins 2047 - 2t and 2046 - 2t (descending order of keys)
     const uint32_t c0 = hist[kBins - 1 - 2 * t], c1 = hist[kBins - 2 - 2 * t];
@@ -341,56 +154,27 @@ __device__ Picked block_select_over(uint32_t n, uint32_t rank, uint32_t *hist, u
       const bool first = before + c0 >= rank;
       xch[0] = (uint32_t)(kBins - 1 - 2 * t - (first ? 0 : 1));
       xch[1] = rank - before - (first ? 0u : c0);
-      xch[2] = first ? c0 : c1;
     }
     __syncthreads();
     prefix |= xch[0] << shift;
     rank = xch[1];
-    count = xch[2];
-    hi_mask |= dmask << shift;
     __syncthreads();
   }
-  Picked p;
-  p.key = prefix;
-  p.count = count;
-  p.rank_in_ties = rank;
-  return p;
-}
-__device__ Picked block_select(const uint32_t *keys, uint32_t n, uint32_t rank, uint32_t *hist, uint32_t *xch) {
-  return block_select_over(n, rank, hist, xch, [&](auto fn) {
-    for (uint32_t idx0 = threadIdx.x; idx0 < n; idx0 += 8 * 1024) {  // eight loads in flight per thread
-      uint32_t kk[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const uint32_t idx = idx0 + u * 1024;
-        kk[u] = idx < n ? keys[idx] : 0xffffffffu;
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (idx0 + u * 1024 < n) fn(kk[u]);
-    }
-  });
-}
-
-__device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
-  x += 0x9e3779b97f4a7c15ull;
-  x = (x ^ (x >> 30)) * 0xbf58476d1ce4e5b9ull;
-  x = (x ^ (x >> 27)) * 0x94d049bb133111ebull;
-  return x ^ (x >> 31);
+  return prefix;
 }
 
 // Two CTAs per selection (blockIdx.y = 0: upper pivot, 1: lower pivot), each of which samples the
 // selection's entries (the same draws) and sets its end of the bracket [lo, hi] around the
-// expected threshold.
-__global__ void __launch_bounds__(1024) sample_pivots_kernel(const float *__restrict__ acc, int Lq, int Lk, int period,
+// expected threshold (rounded outwards to 22 bits: a third digit would not narrow it noticeably).
+__global__ void __launch_bounds__(1024) sample_pivots_kernel(const float *__restrict__ acc, int rows, int Lk, int period,
                                                              int causal, int diag, unsigned long long k_rest,
                                                              unsigned long long n_rest, SelectState *state) {
   extern __shared__ uint32_t sm_dyn[];
   uint32_t *keys = sm_dyn;               // kSamples
   uint32_t *hist = sm_dyn + kSamples;    // kBins
-  __shared__ uint32_t xch[4];
+  __shared__ uint32_t xch[2];
   __shared__ uint32_t n_valid_s;
-  const int h = blockIdx.x, t = threadIdx.x;
+  const int h = blockIdx.x, t = threadIdx.x, lane = t & 31;
   if (t == 0) n_valid_s = 0u;
   __syncthreads();
   const int off = (causal || diag) ? Lk - period : 0;
@@ -403,15 +187,20 @@ __global__ void __launch_bounds__(1024) sample_pivots_kernel(const float *__rest
     // row and column from the two halves of one 64-bit draw, scaled by multiplication (64-bit
     // divisions, emulated in dozens of instructions each, made up most of this kernel's time)
     const unsigned long long m = mix64(((unsigned long long)h << 32) | (unsigned)s);
-    const int i = (int)(((m >> 32) * (unsigned long long)Lq) >> 32);
+    const int i = (int)(((m >> 32) * (unsigned long long)rows) >> 32);
     const int j = (int)(((m & 0xffffffffull) * (unsigned long long)Lk) >> 32);
     const int own = i % period + off;
     valid[u] = !((causal && j > own) || (diag && j == own));
-    drawn[u] = valid[u] ? acc[((size_t)h * Lq + i) * Lk + j] : 0.f;
+    drawn[u] = valid[u] ? acc[((size_t)h * rows + i) * Lk + j] : 0.f;
   }
 #pragma unroll
-  for (int u = 0; u < kDraws; ++u)
-    if (valid[u]) keys[atomicAdd(&n_valid_s, 1u)] = key_of(drawn[u]);
+  for (int u = 0; u < kDraws; ++u) {  // one reservation per warp
+    const uint32_t vote = __ballot_sync(0xffffffffu, valid[u]);
+    uint32_t at = 0u;
+    if (lane == 0) at = atomicAdd(&n_valid_s, (uint32_t)__popc(vote));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(vote & ((1u << lane) - 1u));
+    if (valid[u]) keys[at] = key_of(drawn[u]);
+  }
   __syncthreads();
   const uint32_t nv = n_valid_s;
   if (nv < 1024u) return;  // too few draws landed in the domain: no shortcut for this head
@@ -422,11 +211,11 @@ __global__ void __launch_bounds__(1024) sample_pivots_kernel(const float *__rest
   const long long r_hi = (long long)floor(r - dev), r_lo = (long long)ceil(r + dev);
   if (blockIdx.y == 0) {
     uint32_t hi = 0xffffffffu;
-    if (r_hi >= 1) hi = block_select(keys, nv, (uint32_t)r_hi, hist, xch).key;
+    if (r_hi >= 1) hi = block_select22(keys, nv, (uint32_t)r_hi, hist, xch) | 0x3ffu;
     if (t == 0) state[h].hi = hi;
   } else {
     uint32_t lo = 0u;
-    if (r_lo <= (long long)nv) lo = block_select(keys, nv, (uint32_t)r_lo, hist, xch).key;
+    if (r_lo <= (long long)nv) lo = block_select22(keys, nv, (uint32_t)r_lo, hist, xch);
     if (t == 0) state[h].lo = lo;
   }
   if (t == 0) state[h].use_shortcut = 1u;  // both CTAs take the same decision
@@ -530,276 +319,210 @@ __global__ void __launch_bounds__(kThreads) collect_kernel(const float *__restri
   if (lane == 0 && above_warp) atomicAdd(&state[h].above_hi, above_warp);
 }
 
-// ---- selection among the collected keys: the radix select on their offsets from the lower pivot ----
+// ---- the select -----------------------------------------------------------------------------
 
+constexpr int kSelThreads = 512;
+constexpr int kSelCtasPerSm = 2;
 
-// grid = (CTAs, selections)
-__global__ void __launch_bounds__(kThreads) cand_histogram_kernel(SelectState *state, const uint2 *__restrict__ cand,
-                                                                  uint32_t cand_cap, unsigned long long k_rest,
-                                                                  int pass, uint32_t *hist) {
-  __shared__ uint32_t sh[kBins];
-  const int h = blockIdx.y;
-  const SelectState st = state[h];
-  if (!(pass == 0 ? bracket_holds(st, cand_cap, k_rest) : st.cand_select != 0u)) return;
-  if (digit_is_zero(st, pass)) {  // no pass needed; the first CTA lets the pick open the selection
-    if (blockIdx.x == 0) pick_digit(state, hist, h, pass, 1, cand_cap, k_rest);
-    return;
-  }
-  const int lane = threadIdx.x & 31;
-  for (int b = threadIdx.x; b < kBins; b += kThreads) sh[b] = 0u;
-  __syncthreads();
-  const int shift = digit_shift(pass);
-  const uint32_t dmask = digit_mask(pass);
-  const uint32_t hi_mask = pass == 0 ? 0u : ~((1u << (shift + (pass == 1 ? 11 : 10))) - 1u);
-  const uint32_t want_hi = (pass == 0 ? 0u : st.prefix) & hi_mask;
-  const uint32_t n = st.n_cand, lo = st.lo;
-  const uint2 *mine = cand + (size_t)h * cand_cap;
-  for (uint32_t base = blockIdx.x * (4 * kThreads); base < n; base += gridDim.x * (4 * kThreads)) {  // warp-uniform
-    uint32_t key[4];
+// fn(value, linear index, whether the lane's entry is one of the selection's) for the selection's entries, spread over
+// `n_warps` warps of which this is the `warp`-th: four 128-column pieces of rows at a time, a lane four consecutive
+// entries of each.  Called by whole warps, fn by all lanes together.
+template <class F>
+__device__ __forceinline__ void scan_domain(const float *__restrict__ base, int rows, int Lk, int period, int causal,
+                                            int diag, uint32_t warp, uint32_t n_warps, int lane, F fn) {
+  const int n_kt = (Lk + kTile - 1) / kTile, off = (causal || diag) ? Lk - period : 0;
+  const uint32_t pieces = (uint32_t)rows * (uint32_t)n_kt;
+  const bool vec = (Lk & 3) == 0;
+  for (uint32_t p0 = 4u * warp; p0 < pieces; p0 += 4u * n_warps) {
+    int i = (int)(p0 / (uint32_t)n_kt), kt = (int)(p0 - (uint32_t)i * (uint32_t)n_kt);
+    float v[4][4];
+    int row[4], col[4], jend[4], own[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {  // four loads in flight
-      const uint32_t idx = base + u * kThreads + threadIdx.x;
-      key[u] = idx < n ? mine[idx].x - lo : 0u;
+    for (int u = 0; u < 4; ++u) {
+      row[u] = i;
+      col[u] = kt * kTile + 4 * lane;
+      own[u] = i % period + off;
+      jend[u] = i >= rows ? 0 : causal ? min(Lk, own[u] + 1) : Lk;
+      v[u][0] = v[u][1] = v[u][2] = v[u][3] = 0.f;
+      if (col[u] < jend[u]) load4(base + (size_t)i * Lk, col[u], jend[u], vec, v[u]);
+      if (++kt == n_kt) {
+        kt = 0;
+        ++i;
+      }
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const uint32_t idx = base + u * kThreads + threadIdx.x;
-      const bool take = idx < n && (key[u] & hi_mask) == want_hi;
-      const uint32_t bin = (key[u] >> shift) & dmask;
-      const unsigned voters = __ballot_sync(0xffffffffu, take);
-      if (take) {
-        const unsigned peers = __match_any_sync(voters, bin);
-        if (lane == __ffs(peers) - 1) atomicAdd(&sh[bin], (uint32_t)__popc(peers));
+      if (!__any_sync(0xffffffffu, col[u] < jend[u])) continue;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int j = col[u] + c;
+        fn(v[u][c], (uint32_t)row[u] * (uint32_t)Lk + (uint32_t)j, j < jend[u] && !(diag && j == own[u]));
       }
     }
   }
-  __syncthreads();
-  for (int b = threadIdx.x; b < kBins; b += kThreads) {
-    const uint32_t s = sh[b];
-    if (s) atomicAdd(&hist[h * kBins + b], s);
-  }
-  if (last_cta_of(state, h, gridDim.x)) pick_digit(state, hist, h, pass, 1, cand_cap, k_rest);
 }
 
-// Ranks `count` <= kMaxCutTies distinct linear indices: returns (in *cut_s, after a barrier) the one
-// with exactly rank - 1 smaller ones.  By all threads of a CTA.
-__device__ void rank_ties(const uint32_t *tie_idx, uint32_t count, uint32_t rank, uint32_t *cut_s) {
-  for (uint32_t e = threadIdx.x; e < count; e += blockDim.x) {
-    const uint32_t me = tie_idx[e];
-    uint32_t smaller = 0u;
-    for (uint32_t f = 0; f < count; ++f) smaller += tie_idx[f] < me ? 1u : 0u;
-    if (smaller == rank - 1u) *cut_s = me;
+// The collected entries of a selection that the classifying pass left out and that are kept after all:
+// above the threshold, or equal to it and within the ties that are kept.  By all threads of the selection's CTAs
+// (warp-uniform trip count); entries that follow one another in the buffer were collected by one warp
+// from one stretch of a tile, so lanes that hit the same bitmap word or tile combine their updates.
+__device__ __forceinline__ void patch(const uint2 *__restrict__ cand, uint32_t n, uint32_t thr, uint32_t tie_cut, int h,
+                                      uint32_t first, uint32_t step, int Lq, int Lk, int n_qt, int n_kt,
+                                      uint8_t *__restrict__ mask, uint32_t *__restrict__ stage_bitmap,
+                                      int32_t *__restrict__ stage_count, uint32_t *__restrict__ stage_groups) {
+  const int lane = threadIdx.x & 31;
+  for (uint32_t base = first - lane; base < n; base += step) {
+    const uint32_t idx = base + lane;
+    uint2 c = make_uint2(0u, 0u);
+    if (idx < n) c = cand[idx];
+    const bool keep = idx < n && (c.x > thr || (c.x == thr && c.y <= tie_cut));
+    const uint32_t i = c.y / (uint32_t)Lk, j = c.y - i * (uint32_t)Lk;
+    if (keep && mask) mask[((size_t)h * Lq + i) * Lk + j] = 1;
+    if (stage_bitmap) {
+      const uint32_t tile = (uint32_t)((h * n_qt + (int)(i >> 7)) * n_kt + (int)(j >> 7));
+      const uint32_t word = tile * (uint32_t)kBitmapWords + 4u * (i & 127u) + ((j & 127u) >> 5);
+      const unsigned voters = __ballot_sync(0xffffffffu, keep);
+      if (keep) {
+        const unsigned same_word = __match_any_sync(voters, word);
+        const uint32_t all_bits = __reduce_or_sync(same_word, 1u << (j & 31u));
+        if (lane == __ffs((int)same_word) - 1) atomicOr(stage_bitmap + word, all_bits);
+        const unsigned same_tile = __match_any_sync(voters, tile);
+        const uint32_t all_groups = __reduce_or_sync(same_tile, 1u << ((j & 127u) >> 4));
+        if (lane == __ffs((int)same_tile) - 1) {
+          atomicAdd(stage_count + tile, __popc(same_tile));
+          if (all_groups & ~stage_groups[tile]) atomicOr(stage_groups + tile, all_groups);
+        }
+      }
+    }
   }
-  __syncthreads();
 }
 
-// Closes the selection among the collected keys.  grid = (CTAs, selections).  First the linear indices
-// of the collected entries equal to the threshold are gathered, when they must be ranked and are few
-// enough; the CTA that finishes last then turns the digits found among the collected keys into the
-// threshold, ranks those ties (the lowest linear indices are kept) and marks the selection as done.
-__global__ void __launch_bounds__(kThreads) cand_finish_kernel(SelectState *state, const uint2 *__restrict__ cand,
-                                                               uint32_t cand_cap, uint32_t *tie_list,
-                                                               int classified) {
-  __shared__ uint32_t tie_idx[kMaxCutTies];
-  __shared__ uint32_t cut_s;
-  const int h = blockIdx.y;
-  const SelectState st = state[h];
-  if (!st.cand_select) return;
-  const bool rank_them = !st.all_ties_kept && st.thr_count <= (uint32_t)kMaxCutTies;
-  if (rank_them) {
-    const uint32_t want = st.prefix + st.lo;
+// Cooperative.  Selection h belongs to per_sel CTAs (one CTA takes several selections in turn where there are more
+// of them than CTAs): finds its threshold and the index of the last kept entry equal to it, and, where the
+// classifying pass has written the mask and the bitmaps, adds the collected entries that are kept.
+//
+// What bounds it: three times (load latency + a few microseconds of shared-memory histogram + a barrier of about
+// 1.5 us); the passes read from L2.  Two CTAs of 512 threads per SM, so that one's loads run under the other's counting.
+__global__ void __launch_bounds__(kSelThreads, kSelCtasPerSm)
+select_kernel(const float *__restrict__ acc, int rows, int Lk, int period, int causal, int diag,
+              unsigned long long k_rest, int n_sel, int per_sel, SelectState *state, uint32_t *hist,
+              const uint2 *__restrict__ cand, uint32_t cand_cap, int keep_ties, int H, long long nnz_init,
+              int64_t *__restrict__ nnz, int classified, int Lq, int n_qt, int n_kt, uint8_t *__restrict__ mask,
+              uint32_t *__restrict__ stage_bitmap, int32_t *__restrict__ stage_count,
+              uint32_t *__restrict__ stage_groups, unsigned *err) {
+  __shared__ uint32_t sh[kBins];
+  __shared__ uint32_t warp_sums[kSelThreads / 32];
+  __shared__ uint32_t pick_bin, pick_count;
+  __shared__ unsigned long long pick_rest;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (nnz)
+    for (int x = blockIdx.x * kSelThreads + threadIdx.x; x < H; x += gridDim.x * kSelThreads) nnz[x] = nnz_init;
+  const int rank = (int)blockIdx.x % per_sel;
+  for (int h = (int)blockIdx.x / per_sel; h < n_sel; h += (int)gridDim.x / per_sel) {
+    SelectState &st = state[h];
+    if (k_rest == 0ull) {  // nothing but the forced entries is kept
+      if (rank == 0 && threadIdx.x == 0) st.thr = 0xffffffffu;
+      continue;
+    }
+    // the bracket holds the threshold and every key of the bracket was collected
+    const bool from_cand = st.use_shortcut && st.n_cand <= cand_cap && st.above_hi < k_rest &&
+                           k_rest - st.above_hi <= st.n_cand;
+    const uint32_t lo = from_cand ? st.lo : 0u, span = from_cand ? st.hi - st.lo : 0xffffffffu;
+    const uint32_t n_cand = st.n_cand;
     const uint2 *mine = cand + (size_t)h * cand_cap;
-    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < st.n_cand; idx += gridDim.x * kThreads) {
-      const uint2 c = mine[idx];
-      if (c.x == want) {
-        const uint32_t pos = atomicAdd(&state[h].tie_n, 1u);
-        if (pos < (uint32_t)kMaxCutTies) tie_list[(size_t)h * kMaxCutTies + pos] = c.y;
+    const float *base = acc + (size_t)h * rows * Lk;
+    unsigned long long rest = from_cand ? k_rest - st.above_hi : k_rest;
+    uint32_t prefix = 0u, thr = 0u, arrived = 0u;
+    uint32_t tie_cut = 0xffffffffu;
+    int turn = 0;  // histogram buffers used so far
+    for (int digit = 0; digit < 2 * kPasses; ++digit) {
+      const int pass = digit % kPasses;
+      const bool of_index = digit >= kPasses;
+      if (digit == kPasses) {
+        thr = prefix + lo;
+        prefix = 0u;
+        if (keep_ties || rest == pick_count) break;  // every entry equal to the threshold is kept
       }
-    }
-  }
-  if (!last_cta_of(state, h, gridDim.x)) return;
-  if (rank_them) {
-    for (uint32_t e = threadIdx.x; e < st.thr_count; e += kThreads)
-      tie_idx[e] = __ldcg(tie_list + (size_t)h * kMaxCutTies + e);
-    __syncthreads();
-    rank_ties(tie_idx, st.thr_count, (uint32_t)st.ties_kept, &cut_s);
-  }
-  if (threadIdx.x == 0) {
-    state[h].tie_cut = rank_them ? cut_s : 0u;
-    state[h].have_cut = rank_them ? 1u : 0u;
-    state[h].thr = st.prefix + st.lo;
-    state[h].prefix = st.prefix + st.lo;
-    state[h].done = 1u;
-    // with the classifying pass before it, the patch pass can finish the mask unless the ties would
-    // have to be ranked by their counts per row segment
-    state[h].emitted = (classified && (st.all_ties_kept || rank_them)) ? 1u : 0u;
-  }
-}
-
-// ---- small selections: everything in one CTA ----------------------------------------------------
-
-constexpr long long kSelectSmallEntries = 1ll << 15;  // rows x Lk of a selection, at most
-
-// One CTA of 1024 threads per selection of at most kSelectSmallEntries entries: sets up the
-// selection's state (and nnz), finds the threshold with the CTA-wide radix select straight over
-// the selection's domain, and where only some of the entries equal to the threshold are kept, the
-// linear index of the last kept one (tie_cut): by ranking the ties when there are at most
-// kMaxCutTies of them, else by bisection on the index (each probe counts the ties up to it).  Such a
-// selection needs no other kernel before the emit pass.
-__global__ void __launch_bounds__(1024) select_small_kernel(const float *__restrict__ acc, int rows, int Lk,
-                                                            int period, int causal, int diag,
-                                                            unsigned long long k_rest, SelectState *state, int H,
-                                                            long long nnz_init, int64_t *nnz) {
-  __shared__ uint32_t hist[kBins];
-  __shared__ uint32_t xch[4];
-  __shared__ uint32_t tie_idx[kMaxCutTies];
-  __shared__ uint32_t tie_n_s, cut_s;
-  const int h = blockIdx.x;
-  if (nnz && h == 0)
-    for (int x = threadIdx.x; x < H; x += 1024) nnz[x] = nnz_init;
-  SelectState st;
-  st.prefix = 0u, st.thr = 0xffffffffu, st.remaining = k_rest, st.ties_kept = 0ull, st.all_ties_kept = 0u;
-  st.done = 1u, st.lo = 0u, st.hi = 0xffffffffu, st.above_hi = 0ull, st.n_cand = 0u, st.use_shortcut = 0u;
-  st.tie_cut = 0u, st.have_cut = 0u, st.cand_select = 0u, st.thr_count = 0u, st.tie_n = 0u, st.ticket = 0u;
-  st.emitted = 0u;
-  if (k_rest == 0ull) {  // nothing but the forced entries is kept
-    if (threadIdx.x == 0) state[h] = st;
-    return;
-  }
-  const float *base = acc + (size_t)h * rows * Lk;
-  const int off = (causal || diag) ? Lk - period : 0;
-  const uint32_t n = (uint32_t)rows * (uint32_t)Lk;
-  const bool vec = (Lk & 3) == 0;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // fn(key, linear index) for every selectable entry of rows [0, row_end): a warp takes a row at a time,
-  // its lanes four consecutive entries each, two loads in flight
-  auto scan_rows = [&](int row_end, auto fn) {
-    for (int i = warp; i < row_end; i += 32) {
-      const float *row = base + (size_t)i * Lk;
-      const int own = i % period + off;  // the row's own position among the keys
-      const int jend = causal ? min(Lk, own + 1) : Lk;
-      for (int j00 = 0; j00 < jend; j00 += 256) {
-        float v[2][4];
+      // offsets from the lower pivot are at most span: a leading digit in which that is zero is zero for all
+      if (from_cand && !of_index && pass < kPasses - 1 && (span >> digit_shift(pass)) == 0u) continue;
+      const int shift = digit_shift(pass);
+      const uint32_t dmask = digit_mask(pass), hi_mask = above_digit(pass);
+      for (int b = threadIdx.x; b < kBins; b += kSelThreads) sh[b] = 0u;
+      __syncthreads();
+      auto count = [&](uint32_t key, uint32_t index, bool there) {  // key: offset from the lower pivot
+        const uint32_t word = of_index ? ~index : key;
+        if (there && (word & hi_mask) == prefix && (!of_index || key == thr - lo)) atomicAdd(&sh[(word >> shift) & dmask], 1u);
+      };
+      if (from_cand) {
+        const uint32_t step = (uint32_t)per_sel * kSelThreads * 4u;
+        for (uint32_t x0 = (uint32_t)rank * (4u * kSelThreads) + threadIdx.x; x0 < n_cand + threadIdx.x; x0 += step) {
+          uint2 c[4];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int j0 = j00 + 128 * u + 4 * lane;
-          v[u][0] = v[u][1] = v[u][2] = v[u][3] = 0.f;
-          if (j0 < jend) load4(row, j0, jend, vec, v[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int j = j00 + 128 * u + 4 * lane + c;
-            if (j < jend && !(diag && j == own)) fn(key_of(v[u][c]), (uint32_t)i * (uint32_t)Lk + (uint32_t)j);
+          for (int u = 0; u < 4; ++u) {  // four loads in flight
+            const uint32_t x = x0 + u * kSelThreads;
+            c[u] = x < n_cand ? mine[x] : make_uint2(0u, 0u);
           }
-      }
-    }
-  };
-  const Picked p = block_select_over(n, (uint32_t)k_rest, hist, xch, [&](auto fn) {
-    scan_rows(rows, [&](uint32_t key, uint32_t) { fn(key); });
-  });
-  st.prefix = st.thr = p.key;
-  st.remaining = st.ties_kept = p.rank_in_ties;
-  st.thr_count = p.count;
-  st.all_ties_kept = p.rank_in_ties == p.count ? 1u : 0u;
-  if (!st.all_ties_kept) {
-    if (p.count <= (uint32_t)kMaxCutTies) {
-      if (threadIdx.x == 0) tie_n_s = 0u;
-      __syncthreads();
-      scan_rows(rows, [&](uint32_t key, uint32_t idx) {
-        if (key == p.key) tie_idx[atomicAdd(&tie_n_s, 1u)] = idx;
-      });
-      __syncthreads();
-      rank_ties(tie_idx, p.count, p.rank_in_ties, &cut_s);
-    } else {
-      // the smallest index L with rank_in_ties ties at indices <= L
-      uint32_t lo = 0u, hi = n - 1u;
-      while (lo < hi) {  // the same for every thread
-        const uint32_t mid = lo + (hi - lo) / 2u;
-        uint32_t mine = 0u;
-        scan_rows((int)(mid / (uint32_t)Lk) + 1, [&](uint32_t key, uint32_t idx) {
-          mine += (key == p.key && idx <= mid) ? 1u : 0u;
-        });
-        if (threadIdx.x == 0) tie_n_s = 0u;
-        __syncthreads();
-        mine = __reduce_add_sync(0xffffffffu, mine);
-        if (lane == 0 && mine) atomicAdd(&tie_n_s, mine);
-        __syncthreads();
-        const uint32_t upto = tie_n_s;
-        __syncthreads();
-        if (upto >= p.rank_in_ties) hi = mid; else lo = mid + 1u;
-      }
-      if (threadIdx.x == 0) cut_s = lo;
-      __syncthreads();
-    }
-    st.tie_cut = cut_s;
-    st.have_cut = 1u;
-  }
-  if (threadIdx.x == 0) state[h] = st;
-}
-
-// Entries equal to the threshold key per (row, 128-column segment); only for heads
-// where the ties must be ranked.  grid = (row blocks, H); a warp takes a row.  The CTA that finishes
-// last turns the head's counts into their exclusive prefix sum, in place.
-__global__ void __launch_bounds__(kThreads) tie_count_kernel(const float *__restrict__ acc, int Lq, int Lk, int period,
-                                                             int n_kt, int causal, int diag, SelectState *state,
-                                                             uint32_t *tie_count) {
-  const int h = blockIdx.y;
-  if (state[h].all_ties_kept || state[h].have_cut) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t thr = state[h].thr;
-  const bool vec = (Lk & 3) == 0;
-  const int off = (causal || diag) ? Lk - period : 0;
-  for (int i = blockIdx.x * kWarps + warp; i < Lq; i += gridDim.x * kWarps) {
-    const float *row = acc + ((size_t)h * Lq + i) * Lk;
-    const int own = i % period + off;  // the row's own position among the keys
-    const int jend = causal ? min(Lk, own + 1) : Lk;
-    for (int kt = 0; kt < n_kt; ++kt) {
-      const int j0 = kt * kTile + 4 * lane;
-      int ties = 0;
-      if (j0 < jend) {
-        float v[4];
-        load4(row, j0, jend, vec, v);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int j = j0 + c;
-          ties += (j < jend && !(diag && j == own) && key_of(v[c]) == thr) ? 1 : 0;
+          for (int u = 0; u < 4; ++u) count(c[u].x - lo, c[u].y, x0 + u * kSelThreads < n_cand);
         }
+      } else {
+        scan_domain(base, rows, Lk, period, causal, diag, (uint32_t)(rank * (kSelThreads / 32) + warp),
+                    (uint32_t)(per_sel * (kSelThreads / 32)), lane,
+                    [&](float f, uint32_t index, bool there) { count(key_of(f), index, there); });
       }
+      __syncthreads();
+      const uint32_t *counts = sh;
+      if (per_sel > 1) {
+        uint32_t *all = hist + ((size_t)h * kHistBuffers + turn % kHistBuffers) * kBins;
+        for (int b = threadIdx.x; b < kBins; b += kSelThreads)
+          if (sh[b]) atomicAdd(all + b, sh[b]);
+        if (turn >= 2) {  // the buffer of two digits ago has been read by all: ready for the next digit but ...
+          uint32_t *old = hist + ((size_t)h * kHistBuffers + (turn - 2) % kHistBuffers) * kBins;
+          for (int b = rank * kSelThreads + threadIdx.x; b < kBins; b += per_sel * kSelThreads) old[b] = 0u;
+        }
+        arrived += (uint32_t)per_sel;
+        if (!cta_barrier(&st.barrier, arrived, err)) return;
+        for (int b = threadIdx.x; b < kBins; b += kSelThreads) sh[b] = __ldcg(all + b);
+        __syncthreads();
+        ++turn;
+      }
+      // thread t owns bins 2047 - 4t .. 2044 - 4t (descending); the owner of the wanted rank picks the digit
+      uint32_t c[4], sum = 0u;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) ties += __shfl_xor_sync(0xffffffffu, ties, o);
-      if (lane == 0) tie_count[((size_t)h * Lq + i) * n_kt + kt] = (uint32_t)ties;
-    }
-  }
-  if (!last_cta_of(state, h, gridDim.x)) return;
-  __shared__ uint32_t warp_sums[kWarps];
-  __shared__ uint32_t carry_s;
-  const int n_per_head = Lq * n_kt;
-  uint32_t *a = tie_count + (size_t)h * n_per_head;
-  if (threadIdx.x == 0) carry_s = 0u;
-  __syncthreads();
-  for (int base = 0; base < n_per_head; base += kThreads) {
-    const int idx = base + threadIdx.x;
-    const uint32_t x = idx < n_per_head ? __ldcg(a + idx) : 0u;
-    uint32_t incl = x;
+      for (int e = 0; e < 4; ++e) {
+        c[e] = counts[kBins - 1 - 4 * (int)threadIdx.x - e];
+        sum += c[e];
+      }
+      uint32_t incl = sum;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      if (lane == 31) warp_sums[warp] = incl;
+      __syncthreads();
+      unsigned long long before = incl - sum;  // entries in bins above this thread's
+      for (int w = 0; w < warp; ++w) before += warp_sums[w];
+      if (before < rest && before + sum >= rest) {  // exactly one thread
+        int e = 0;
+        for (; e < 3 && before + c[e] < rest; ++e) before += c[e];
+        pick_bin = (uint32_t)(kBins - 1 - 4 * (int)threadIdx.x - e);
+        pick_rest = rest - before;
+        pick_count = e == 0 ? c[0] : e == 1 ? c[1] : e == 2 ? c[2] : c[3];
+      }
+      __syncthreads();
+      prefix |= pick_bin << shift;
+      rest = pick_rest;
+      if (digit == 2 * kPasses - 1) tie_cut = ~prefix;
     }
-    if (lane == 31) warp_sums[warp] = incl;
-    __syncthreads();
-    uint32_t before = 0u, total = 0u;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-      if (w < warp) before += warp_sums[w];
-      total += warp_sums[w];
+    if (rank == 0 && threadIdx.x == 0) {
+      st.thr = thr;
+      st.tie_cut = tie_cut;
+      st.emitted = classified && from_cand ? 1u : 0u;
     }
-    const uint32_t carry = carry_s;
-    if (idx < n_per_head) a[idx] = carry + before + incl - x;
-    __syncthreads();
-    if (threadIdx.x == 0) carry_s = carry + total;
+    if (classified && from_cand)
+      patch(mine, n_cand, thr, tie_cut, h, (uint32_t)(rank * kSelThreads + threadIdx.x), (uint32_t)(per_sel * kSelThreads),
+            Lq, Lk, n_qt, n_kt, mask, stage_bitmap, stage_count, stage_groups);
     __syncthreads();
   }
 }
@@ -842,34 +565,35 @@ struct Collector {
 struct EmitSel {
   float thr_f;  // the threshold as a float (NaN when nothing but the forced entries is kept)
   float lo_f;   // classifying pass: thr_f is the bracket's upper pivot, lo_f its lower one
-  unsigned long long ties_kept;
-  bool all_ties, have_cut;
-  uint32_t tie_cut;
+  uint32_t tie_cut;    // entries equal to the threshold are kept up to this index
   uint32_t first_row;  // of this head in the tie order
 };
 
-// The rows of one tile; returns this lane's share of the tile's popcount (lanes 0, 8, 16, 24).
+// The rows of one tile, kCtaWarps warps; returns this lane's share of the tile's popcount (lanes 0, 8, 16, 24) and adds
+// the bitmap words it has written to `any` (same lanes).
 // kInterior: every row and column of the tile exists and lies in the domain and none is forced,
 // so nothing is checked per entry.
 // kClassify: the classifying pass of the one-pass shortcut instead of the emit pass proper.  Entries
-// above the bracket are kept, entries inside it are collected (col) and left out for the patch pass
+// above the bracket are kept, entries inside it are collected (col) and left out for the select
 // to decide, entries above the bracket are counted (above).
-template <bool kInterior, bool kClassify>
-__device__ __forceinline__ int emit_tile_rows(const float *__restrict__ acc, int Lq, int Lk, int n_kt, int h, int qt,
-                                              int kt, int tile, int causal, int diag, const EmitSel &sel,
-                                              const uint32_t *__restrict__ tie_prefix, uint8_t *__restrict__ mask,
-                                              uint32_t *__restrict__ stage_bitmap, Collector &col, uint32_t &above) {
+template <bool kInterior, bool kClassify, int kCtaWarps>
+__device__ __forceinline__ int emit_tile_rows(const float *__restrict__ acc, int Lq, int Lk, int h, int qt, int kt,
+                                              int tile, int causal, int diag, const EmitSel &sel,
+                                              uint8_t *__restrict__ mask, uint32_t *__restrict__ stage_bitmap,
+                                              Collector &col, uint32_t &above, uint32_t &any) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool vec = (Lk & 3) == 0;
   const int j0 = kt * kTile + 4 * lane;
   const float thr_f = sel.thr_f;
+  // the lowest value that needs a closer look: the threshold, or the bracket's lower pivot
+  const float floor_f = kClassify ? sel.lo_f : thr_f;
   const int off = (causal || diag) ? Lk - Lq : 0;  // row i's own position is key i + off
   int count = 0;
-  for (int r0 = warp; r0 < kTile; r0 += 16) {
+  for (int r0 = warp; r0 < kTile; r0 += 4 * kCtaWarps) {
     float v[4][4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {  // rows r0, r0+4, r0+8, r0+12: four loads in flight
-      const int i = qt * kTile + r0 + 4 * u;
+    for (int u = 0; u < 4; ++u) {  // four loads in flight
+      const int i = qt * kTile + r0 + kCtaWarps * u;
       if (kInterior) {
         const float4 t = *reinterpret_cast<const float4 *>(acc + ((size_t)h * Lq + i) * Lk + j0);
         v[u][0] = t.x; v[u][1] = t.y; v[u][2] = t.z; v[u][3] = t.w;
@@ -883,95 +607,67 @@ __device__ __forceinline__ int emit_tile_rows(const float *__restrict__ acc, int
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int r = r0 + 4 * u;
+      const int r = r0 + kCtaWarps * u;
       const int i = qt * kTile + r;
       uint32_t nib = 0u;
-      if (kInterior || i < Lq) {  // warp-uniform
-        uint32_t tie_bits = 0u, gt_bits = 0u;
-        // the lowest value that needs a closer look: the threshold, or the bracket's lower pivot
-        const float floor_f = kClassify ? sel.lo_f : thr_f;
-        uint32_t forced_bits = 0u;
-        if (kInterior) {
-          // (most pieces of a row lie wholly below it: one test instead of eight)
-          if (!(v[u][0] < floor_f && v[u][1] < floor_f && v[u][2] < floor_f && v[u][3] < floor_f)) {
+      bool close = false;  // some lane of the warp has an entry that needs a closer look
+      if (kInterior) {
+        // (most pieces of a row lie wholly below: one test for the warp, and zeros are written)
+        close = __any_sync(0xffffffffu, !(v[u][0] < floor_f && v[u][1] < floor_f && v[u][2] < floor_f && v[u][3] < floor_f));
+      } else {
+        close = i < Lq;
+      }
+      if (close) {  // warp-uniform
+        uint32_t tie_bits = 0u, gt_bits = 0u, forced_bits = 0u;
+        const int jend = kInterior ? j0 + 4 : causal ? min(Lk, i + 1 + off) : Lk;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < 4; ++c) {
+          const int j = j0 + c;
+          if (kInterior || j < jend) {
+            if (!kInterior && diag && j == i + off) {
+              forced_bits |= 1u << c;
+            } else {
               gt_bits |= (v[u][c] > thr_f ? 1u : 0u) << c;
               tie_bits |= ((kClassify ? !(v[u][c] < floor_f) && !(v[u][c] > thr_f) : v[u][c] == thr_f) ? 1u : 0u) << c;
             }
           }
-        } else {
-          const int jend = causal ? min(Lk, i + 1 + off) : Lk;
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int j = j0 + c;
-            if (j < jend) {
-              if (diag && j == i + off) {
-                forced_bits |= 1u << c;
-              } else {
-                gt_bits |= (v[u][c] > thr_f ? 1u : 0u) << c;
-                tie_bits |= ((kClassify ? !(v[u][c] < floor_f) && !(v[u][c] > thr_f) : v[u][c] == thr_f) ? 1u : 0u) << c;
-              }
-            }
-          }
         }
         nib = gt_bits | forced_bits;
-        if (kClassify) {
-          above += (uint32_t)__popc(gt_bits);
-          if (tie_bits) {
+        if (kClassify) above += (uint32_t)__popc(gt_bits);
+        if (tie_bits) {
+          const uint32_t first = (sel.first_row + (uint32_t)i) * (uint32_t)Lk + (uint32_t)j0;
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-              if (tie_bits & (1u << c))
-                col.push(v[u][c], (sel.first_row + (uint32_t)i) * (uint32_t)Lk + (uint32_t)(j0 + c));
-          }
-        } else if (sel.all_ties) {
-          nib |= tie_bits;
-        } else if (sel.have_cut) {
-          if (tie_bits) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-              if ((tie_bits & (1u << c)) &&
-                  (sel.first_row + (uint32_t)i) * (uint32_t)Lk + (uint32_t)(j0 + c) <= sel.tie_cut)
-                nib |= 1u << c;
-          }
-        } else if (__any_sync(0xffffffffu, tie_bits != 0u)) {
-          // rank of each tie in linear-index order = ties before this row segment
-          // + ties in lower lanes + ties in lower columns of this lane
-          int before = __popc(tie_bits);
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            int t = __shfl_up_sync(0xffffffffu, before, o);
-            if (lane >= o) before += t;
-          }
-          before -= __popc(tie_bits);
-          unsigned long long rank = (unsigned long long)tie_prefix[((size_t)h * Lq + i) * n_kt + kt] + before;
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
+          for (int c = 0; c < 4; ++c)
             if (tie_bits & (1u << c)) {
-              if (rank < sel.ties_kept) nib |= 1u << c;
-              ++rank;
+              if (kClassify)
+                col.push(v[u][c], first + c);
+              else if (first + c <= sel.tie_cut)
+                nib |= 1u << c;
             }
-          }
-        }
-        if (mask) {
-          uint8_t *mrow = mask + ((size_t)h * Lq + i) * Lk;
-          if (kInterior || (vec && j0 + 4 <= Lk)) {
-            *reinterpret_cast<uchar4 *>(mrow + j0) =
-                make_uchar4(nib & 1u, (nib >> 1) & 1u, (nib >> 2) & 1u, (nib >> 3) & 1u);
-          } else {
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-              if (j0 + c < Lk) mrow[j0 + c] = (nib >> c) & 1u;
-          }
         }
       }
-      // 8 lanes x 4 bits -> one bitmap word, complete in the first lane of each group of eight
-      uint32_t w = nib << (4 * (lane & 7));
-      w |= __shfl_xor_sync(0xffffffffu, w, 1);
-      w |= __shfl_xor_sync(0xffffffffu, w, 2);
-      w |= __shfl_xor_sync(0xffffffffu, w, 4);
+      if ((kInterior || i < Lq) && mask) {
+        uint8_t *mrow = mask + ((size_t)h * Lq + i) * Lk;
+        if (kInterior || (vec && j0 + 4 <= Lk)) {
+          *reinterpret_cast<uchar4 *>(mrow + j0) =
+              make_uchar4(nib & 1u, (nib >> 1) & 1u, (nib >> 2) & 1u, (nib >> 3) & 1u);
+        } else {
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (j0 + c < Lk) mrow[j0 + c] = (nib >> c) & 1u;
+        }
+      }
+      uint32_t w = 0u;
+      if (close) {
+        // 8 lanes x 4 bits -> one bitmap word, complete in the first lane of each group of eight
+        w = nib << (4 * (lane & 7));
+        w |= __shfl_xor_sync(0xffffffffu, w, 1);
+        w |= __shfl_xor_sync(0xffffffffu, w, 2);
+        w |= __shfl_xor_sync(0xffffffffu, w, 4);
+      }
       if ((lane & 7) == 0) {
         count += __popc(w);
+        any |= w;
         if (stage_bitmap) stage_bitmap[(size_t)tile * kBitmapWords + 4 * r + (lane >> 3)] = w;
       }
     }
@@ -981,146 +677,135 @@ __device__ __forceinline__ int emit_tile_rows(const float *__restrict__ acc, int
   return count;
 }
 
-// One CTA per tile of the (h, qt, kt) grid; warp w takes tile rows w, w+4, ...
-// (four rows loaded ahead) and each lane four consecutive columns.  Writes the
-// element mask, the tile's bitmap and popcount into the staging area.  Values are
+// A CTA per tile of the (h, qt, kt) grid (a CTA takes several in turn where the grid is smaller); warp w takes tile rows
+// w, w + kCtaWarps, ... (four rows loaded ahead) and each lane four consecutive columns.  Writes the
+// element mask, the tile's bitmap, popcount and group summary into the staging area.  Values are
 // compared with the threshold as floats (the same order as their keys).  per_layer:
 // all heads share selection 0, ties are ordered by (h*Lq + i)*Lk + j, and the
 // tiles' popcounts are added up into nnz[h].  keep_ties: every entry equal to the threshold is
-// kept (no ranking), and the popcounts are added up as well (the count is not known beforehand).
+// kept, and the popcounts are added up as well (the count is not known beforehand).
 // kClassify: the shortcut's one pass over the accumulator, which does the collecting pass's work
 // (entries above the upper pivot counted, entries inside the bracket appended to the selection's
 // buffer) and most of the emit pass's at once: everything above the bracket is kept, everything else
-// left out, and patch_kernel adds the collected entries that turn out to be kept.  Only for exact
+// left out, and the select adds the collected entries that turn out to be kept.  Only for exact
 // per-head selections (the kept count is known beforehand, nothing is counted here).
-template <bool kClassify>
-__global__ void __launch_bounds__(128) emit_kernel(const float *__restrict__ acc, int Lq, int Lk, int n_qt, int n_kt,
-                                                   int causal, int diag, int per_layer, int keep_ties,
-                                                   SelectState *state, const uint32_t *__restrict__ tie_prefix,
-                                                   uint8_t *__restrict__ mask, uint32_t *__restrict__ stage_bitmap,
-                                                   int32_t *__restrict__ stage_count, int64_t *__restrict__ nnz,
-                                                   uint2 *__restrict__ cand, uint32_t cand_cap) {
-  const int tile = blockIdx.x;
-  const int kt = tile % n_kt;
-  const int qt = (tile / n_kt) % n_qt;
-  const int h = tile / (n_kt * n_qt);
+template <bool kClassify, int kCtaWarps>
+__global__ void __launch_bounds__(32 * kCtaWarps) emit_kernel(const float *__restrict__ acc, int Lq, int Lk, int n_qt,
+                                                              int n_kt, int n_tiles, int causal, int diag, int per_layer,
+                                                              int keep_ties, SelectState *state,
+                                                              uint8_t *__restrict__ mask,
+                                                              uint32_t *__restrict__ stage_bitmap,
+                                                              int32_t *__restrict__ stage_count,
+                                                              uint32_t *__restrict__ stage_groups,
+                                                              int64_t *__restrict__ nnz, uint2 *__restrict__ cand,
+                                                              uint32_t cand_cap) {
+  __shared__ int warp_count[kCtaWarps];
+  __shared__ uint32_t warp_groups[kCtaWarps];
+  __shared__ uint2 stage_all[kClassify ? kCtaWarps : 1][kClassify ? kWarpStage : 1];
+  __shared__ uint32_t stage_n_all[kCtaWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __shared__ int warp_count[4];
-  __shared__ uint2 stage_all[kClassify ? 4 : 1][kClassify ? kWarpStage : 1];
-  __shared__ uint32_t stage_n_all[4];
-  SelectState &st = state[per_layer ? 0 : h];
-  if (kClassify ? !st.use_shortcut : st.emitted != 0u) return;  // not this pass's selection
-  // own positions of the tile's rows among the keys: columns own_lo .. own_hi
-  const int own_lo = qt * kTile + ((causal || diag) ? Lk - Lq : 0), own_hi = own_lo + kTile - 1;
-  if (causal && kt * kTile > own_hi) {
-    // the whole tile lies above the diagonal: nothing is kept, nothing needs to be read
-    const bool vec = (Lk & 3) == 0;
-    const int j0 = kt * kTile + 4 * lane;
-    for (int r = warp; r < kTile; r += 4) {
-      const int i = qt * kTile + r;
-      if (i < Lq && mask) {
-        uint8_t *mrow = mask + ((size_t)h * Lq + i) * Lk;
-        if (vec && j0 + 4 <= Lk) {
-          *reinterpret_cast<uchar4 *>(mrow + j0) = make_uchar4(0, 0, 0, 0);
-        } else {
-          for (int c = 0; c < 4; ++c)
-            if (j0 + c < Lk) mrow[j0 + c] = 0;
+  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    const int kt = tile % n_kt;
+    const int qt = (tile / n_kt) % n_qt;
+    const int h = tile / (n_kt * n_qt);
+    SelectState &st = state[per_layer ? 0 : h];
+    if (kClassify ? !st.use_shortcut : st.emitted != 0u) continue;  // not this pass's selection
+    // own positions of the tile's rows among the keys: columns own_lo .. own_hi
+    const int own_lo = qt * kTile + ((causal || diag) ? Lk - Lq : 0), own_hi = own_lo + kTile - 1;
+    if (causal && kt * kTile > own_hi) {
+      // the whole tile lies above the diagonal: nothing is kept, nothing needs to be read
+      const bool vec = (Lk & 3) == 0;
+      const int j0 = kt * kTile + 4 * lane;
+      for (int r = warp; r < kTile; r += kCtaWarps) {
+        const int i = qt * kTile + r;
+        if (i < Lq && mask) {
+          uint8_t *mrow = mask + ((size_t)h * Lq + i) * Lk;
+          if (vec && j0 + 4 <= Lk) {
+            *reinterpret_cast<uchar4 *>(mrow + j0) = make_uchar4(0, 0, 0, 0);
+          } else {
+            for (int c = 0; c < 4; ++c)
+              if (j0 + c < Lk) mrow[j0 + c] = 0;
+          }
         }
       }
-      if (stage_bitmap && lane == 0)
-        reinterpret_cast<uint4 *>(stage_bitmap + (size_t)tile * kBitmapWords)[r] = make_uint4(0u, 0u, 0u, 0u);
-    }
-    if (stage_count && threadIdx.x == 0) stage_count[tile] = 0;
-    return;
-  }
-  EmitSel sel;
-  sel.thr_f = float_of_key(kClassify ? st.hi : st.thr);
-  sel.lo_f = float_of_key(st.lo);
-  sel.ties_kept = st.ties_kept;
-  sel.all_ties = st.all_ties_kept != 0u || keep_ties != 0;
-  sel.have_cut = st.have_cut != 0u;
-  sel.tie_cut = st.tie_cut;
-  sel.first_row = per_layer ? (uint32_t)h * (uint32_t)Lq : 0u;
-  Collector col;
-  col.stage = stage_all[kClassify ? warp : 0];
-  col.stage_n = &stage_n_all[warp];
-  col.out = cand + (size_t)(per_layer ? 0 : h) * cand_cap;
-  col.n_cand = &st.n_cand;
-  col.cap = cand_cap;
-  if (lane == 0) stage_n_all[warp] = 0u;
-  __syncwarp();
-  uint32_t above = 0u;
-  const bool below = !causal || kt * kTile + kTile - 1 <= own_lo;  // every column in every row's domain
-  const bool has_diag = diag && own_lo <= kt * kTile + kTile - 1 && own_hi >= kt * kTile;
-  const bool interior = (qt + 1) * kTile <= Lq && (kt + 1) * kTile <= Lk && (Lk & 3) == 0 && below && !has_diag;
-  int count = interior ? emit_tile_rows<true, kClassify>(acc, Lq, Lk, n_kt, h, qt, kt, tile, causal, diag, sel,
-                                                         tie_prefix, mask, stage_bitmap, col, above)
-                       : emit_tile_rows<false, kClassify>(acc, Lq, Lk, n_kt, h, qt, kt, tile, causal, diag, sel,
-                                                          tie_prefix, mask, stage_bitmap, col, above);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
-  if (kClassify) {
-    above = __reduce_add_sync(0xffffffffu, above);
-    if (lane == 0 && above) atomicAdd(&st.above_hi, (unsigned long long)above);
-  }
-  if (lane == 0) warp_count[warp] = count;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int total = warp_count[0] + warp_count[1] + warp_count[2] + warp_count[3];
-    if (stage_count) stage_count[tile] = total;
-    if (!kClassify && (per_layer || keep_ties) && nnz && total)
-      atomicAdd(reinterpret_cast<unsigned long long *>(nnz + h), (unsigned long long)total);
-  }
-}
-
-// The collected entries of a selection that the classifying pass left out and that are kept after all:
-// above the threshold, or equal to it and within the ties that are kept.  grid = (CTAs, selections).
-__global__ void __launch_bounds__(kThreads) patch_kernel(const SelectState *__restrict__ state,
-                                                         const uint2 *__restrict__ cand, uint32_t cand_cap, int Lq,
-                                                         int Lk, int n_qt, int n_kt, uint8_t *__restrict__ mask,
-                                                         uint32_t *__restrict__ stage_bitmap,
-                                                         int32_t *__restrict__ stage_count) {
-  const int h = blockIdx.y;
-  const SelectState st = state[h];
-  if (!st.emitted) return;
-  const uint2 *mine = cand + (size_t)h * cand_cap;
-  const int lane = threadIdx.x & 31;
-  const uint32_t n = st.n_cand;
-  // (warp-uniform trip count; entries that follow one another in the buffer were collected by one warp
-  // from one stretch of a tile, so lanes that hit the same bitmap word or tile combine their updates)
-  for (uint32_t base = blockIdx.x * kThreads; base < n; base += gridDim.x * kThreads) {
-    const uint32_t idx = base + threadIdx.x;
-    uint2 c = make_uint2(0u, 0u);
-    if (idx < n) c = mine[idx];
-    const bool keep = idx < n && (c.x > st.thr || (c.x == st.thr && (st.all_ties_kept != 0u || c.y <= st.tie_cut)));
-    const uint32_t i = c.y / (uint32_t)Lk, j = c.y - i * (uint32_t)Lk;
-    if (keep && mask) mask[((size_t)h * Lq + i) * Lk + j] = 1;
-    if (stage_bitmap) {
-      const uint32_t tile = (uint32_t)((h * n_qt + (int)(i >> 7)) * n_kt + (int)(j >> 7));
-      const uint32_t word = tile * (uint32_t)kBitmapWords + 4u * (i & 127u) + ((j & 127u) >> 5);
-      const unsigned voters = __ballot_sync(0xffffffffu, keep);
-      if (keep) {
-        const unsigned same_word = __match_any_sync(voters, word);
-        const uint32_t all_bits = __reduce_or_sync(same_word, 1u << (j & 31u));
-        if (lane == __ffs((int)same_word) - 1) atomicOr(stage_bitmap + word, all_bits);
-        const unsigned same_tile = __match_any_sync(voters, tile);
-        if (lane == __ffs((int)same_tile) - 1) atomicAdd(stage_count + tile, __popc(same_tile));
+      // (the bitmap of an empty tile is not read)
+      if (stage_count && threadIdx.x == 0) {
+        stage_count[tile] = 0;
+        stage_groups[tile] = 0u;
       }
+      continue;
     }
+    EmitSel sel;
+    sel.thr_f = float_of_key(kClassify ? st.hi : st.thr);
+    sel.lo_f = float_of_key(st.lo);
+    sel.tie_cut = st.tie_cut;
+    sel.first_row = per_layer ? (uint32_t)h * (uint32_t)Lq : 0u;
+    Collector col;
+    col.stage = stage_all[kClassify ? warp : 0];
+    col.stage_n = &stage_n_all[warp];
+    col.out = cand + (size_t)(per_layer ? 0 : h) * cand_cap;
+    col.n_cand = &st.n_cand;
+    col.cap = cand_cap;
+    if (kClassify && lane == 0) stage_n_all[warp] = 0u;
+    __syncwarp();
+    uint32_t above = 0u, any = 0u;
+    const bool below = !causal || kt * kTile + kTile - 1 <= own_lo;  // every column in every row's domain
+    const bool has_diag = diag && own_lo <= kt * kTile + kTile - 1 && own_hi >= kt * kTile;
+    const bool interior = (qt + 1) * kTile <= Lq && (kt + 1) * kTile <= Lk && (Lk & 3) == 0 && below && !has_diag;
+    int count = interior ? emit_tile_rows<true, kClassify, kCtaWarps>(acc, Lq, Lk, h, qt, kt, tile, causal, diag, sel,
+                                                                      mask, stage_bitmap, col, above, any)
+                         : emit_tile_rows<false, kClassify, kCtaWarps>(acc, Lq, Lk, h, qt, kt, tile, causal, diag, sel,
+                                                                       mask, stage_bitmap, col, above, any);
+    if (kClassify) {
+      above = __reduce_add_sync(0xffffffffu, above);
+      if (lane == 0 && above) atomicAdd(&st.above_hi, (unsigned long long)above);
+    }
+    if (!stage_bitmap && !(nnz && !kClassify && (per_layer || keep_ties))) continue;
+    count = __reduce_add_sync(0xffffffffu, count);
+    // groups 2q and 2q + 1 of the tile are the halves of word q, which lane 8q has seen
+    const uint32_t bits = ((any & 0xffffu) ? 1u : 0u) | ((any >> 16) ? 2u : 0u);
+    const uint32_t groups = __reduce_or_sync(0xffffffffu, (lane & 7) == 0 ? bits << (2 * (lane >> 3)) : 0u);
+    if (lane == 0) {
+      warp_count[warp] = count;
+      warp_groups[warp] = groups;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int total = 0;
+      uint32_t all = 0u;
+#pragma unroll
+      for (int w = 0; w < kCtaWarps; ++w) {
+        total += warp_count[w];
+        all |= warp_groups[w];
+      }
+      if (stage_count) {
+        stage_count[tile] = total;
+        stage_groups[tile] = all;
+      }
+      if (!kClassify && (per_layer || keep_ties) && nnz && total)
+        atomicAdd(reinterpret_cast<unsigned long long *>(nnz + h), (unsigned long long)total);
+    }
+    __syncthreads();  // warp_count is read
   }
 }
 
-Scratch carve(void *scratch, int H, int Lq, int Lk) {
+// Where the arrays of the select scratch lie.  The header and the states (and the histograms, where the select shares
+// them between CTAs) are zeroed before the first kernel of a call.
+struct Header {
+  uint32_t compact_barrier;
+  uint32_t pad[15];
+};
+
+Scratch carve(void *scratch, int H, Header **header) {
   char *p = static_cast<char *>(scratch);
   Scratch s;
-  s.hist = reinterpret_cast<uint32_t *>(p);
-  p += align256((size_t)H * kBins * sizeof(uint32_t));
+  *header = reinterpret_cast<Header *>(p);
+  p += sizeof(Header);
   s.state = reinterpret_cast<SelectState *>(p);
-  p += align256((size_t)H * sizeof(SelectState));
-  s.tie_count = reinterpret_cast<uint32_t *>(p);
-  p += align256((size_t)H * Lq * ceil_div(Lk, kTile) * sizeof(uint32_t));
-  s.tie_list = reinterpret_cast<uint32_t *>(p);
-  p += align256((size_t)H * kMaxCutTies * sizeof(uint32_t));
+  p += (size_t)H * sizeof(SelectState);
+  p = reinterpret_cast<char *>(align256(reinterpret_cast<size_t>(p)));
+  s.hist = reinterpret_cast<uint32_t *>(p);
+  p += (size_t)min(H, kMaxSharedSelections) * kHistBuffers * kBins * sizeof(uint32_t);
   s.cand = reinterpret_cast<uint2 *>(p);
   return s;
 }
@@ -1130,111 +815,101 @@ Scratch carve(void *scratch, int H, int Lq, int Lk) {
 size_t select_scratch_bytes(int H, int Lq, int Lk) {
   // the candidate buffer is sized for the larger of the causal and the full domain, and for one
   // selection over all heads (never smaller than H selections of one head each)
-  return align256((size_t)H * kBins * sizeof(uint32_t)) + align256((size_t)H * sizeof(SelectState)) +
-         align256((size_t)H * Lq * ceil_div(Lk, kTile) * sizeof(uint32_t)) +
-         align256((size_t)H * kMaxCutTies * sizeof(uint32_t)) +
+  return align256(sizeof(Header) + (size_t)H * sizeof(SelectState)) + 256 +
+         (size_t)min(H, kMaxSharedSelections) * kHistBuffers * kBins * sizeof(uint32_t) +
          align256((size_t)cand_capacity((long long)H * Lq * Lk) * sizeof(uint2));
 }
 
 cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
-  const int n_qt = ceil_div(a.Lq, kTile), n_kt = ceil_div(a.Lk, kTile);
+  const int n_qt = ceil_div(a.Lq, kTile), n_kt = ceil_div(a.Lk, kTile), n_tiles = a.H * n_qt * n_kt;
   const int diag = (a.keep_diag && (a.Lq == a.Lk || a.causal)) ? 1 : 0;
-  Scratch sc = carve(a.scratch, a.H, a.Lq, a.Lk);
+  const int sms = sm_count();
+  unsigned *err = device_error_word();
+  if (sms <= 0 || !err) return cudaErrorUnknown;
+  Header *header;
+  Scratch sc = carve(a.scratch, a.H, &header);
   // the selections: one per head over Lq rows, or one over the H*Lq rows of the layer
   const int n_sel = a.per_layer ? 1 : a.H;
   const int rows = a.per_layer ? a.H * a.Lq : a.Lq;
   const int period = a.Lq;
-  cudaError_t e;
+  // CTAs per selection: all that fit, as far as there is a row for each of their warps
+  const int max_ctas = kSelCtasPerSm * sms;
+  int per_sel = max_ctas / n_sel;
+  const long long pieces = (long long)rows * n_kt;
+  if ((long long)per_sel * (kSelThreads / 32) > pieces) per_sel = (int)((pieces + kSelThreads / 32 - 1) / (kSelThreads / 32));
+  if (per_sel < 1 || n_sel > kMaxSharedSelections) per_sel = 1;
+  const size_t hist_bytes = per_sel > 1 ? (size_t)n_sel * kHistBuffers * kBins * sizeof(uint32_t) : 0;
+  cudaError_t e = cudaMemsetAsync(header, 0, (reinterpret_cast<char *>(sc.hist) - reinterpret_cast<char *>(header)) + hist_bytes, s);
+  if (e != cudaSuccess) return e;
   // per head nnz = k; per layer, or with all ties kept, the emit pass counts it
   const bool count_nnz = a.per_layer || a.keep_ties;
+  const long long n_valid = domain_size(a.Lq, a.Lk, a.causal);
+  const long long n_rest = (n_valid - (diag ? a.Lq : 0)) * (a.per_layer ? a.H : 1);
+  const long long cap = cand_capacity(n_rest);
+  const bool shortcut = a.k_rest > 0 && cap > 0 && n_valid * a.H > kDirectEntries;
+  // Exact per-head selections: the one pass over the accumulator also writes what is certain of the
+  // mask and the tile bitmaps (the select adds the collected entries that are kept), so
+  // the emit pass at the end has nothing to read for the selections the shortcut resolves.  Other
+  // selections count what they keep in the emit pass, which therefore has to see every entry.
+  const bool classify = shortcut && !a.per_layer && !a.keep_ties;
+  if (shortcut) {
+    const size_t smem = (kSamples + kBins) * sizeof(uint32_t);
+    e = cudaFuncSetAttribute(sample_pivots_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    sample_pivots_kernel<<<dim3(n_sel, 2), 1024, smem, s>>>(a.acc, rows, a.Lk, period, a.causal, diag,
+                                                            (unsigned long long)a.k_rest, (unsigned long long)n_rest,
+                                                            sc.state);
+    if (classify) {
+      emit_kernel<true, 4><<<n_tiles, 128, 0, s>>>(a.acc, a.Lq, a.Lk, n_qt, n_kt, n_tiles, a.causal, diag, 0, 0, sc.state,
+                                                   a.mask, a.stage_bitmap, a.stage_count, a.stage_groups, a.nnz, sc.cand,
+                                                   (uint32_t)cap);
+    } else {
+      // one wave of CTAs (five fit an SM), so that no SM idles while a second, partial wave runs
+      int collect_blocks = ceil_div(rows, kWarps);
+      if (collect_blocks > 148 * 5 / n_sel) collect_blocks = max(148 * 5 / n_sel, 1);
+      collect_kernel<<<dim3(collect_blocks, n_sel), kThreads, 0, s>>>(a.acc, rows, a.Lk, period, a.causal, diag, sc.state,
+                                                                     sc.cand, (uint32_t)cap);
+    }
+    count_launches(2);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   {
-    // very small selections: one kernel instead of the passes below (measured: one CTA per selection
-    // beats the ten launches of the passes up to about 2^15 entries per selection: 0.085 -> 0.065 ms on
-    // B32 H12 L128; at 2^17 and more it loses, the passes spread a selection over many CTAs)
-    if ((long long)rows * a.Lk <= kSelectSmallEntries) {
-      select_small_kernel<<<n_sel, 1024, 0, s>>>(a.acc, rows, a.Lk, period, a.causal, diag,
-                                                 (unsigned long long)a.k_rest, sc.state, a.H,
-                                                 count_nnz ? 0ll : (long long)a.k, a.nnz);
-      count_launches(1);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      emit_kernel<false><<<a.H * n_qt * n_kt, 128, 0, s>>>(a.acc, a.Lq, a.Lk, n_qt, n_kt, a.causal, diag,
-                                                           a.per_layer, a.keep_ties, sc.state, sc.tie_count, a.mask,
-                                                           a.stage_bitmap, a.stage_count, a.nnz, nullptr, 0u);
-      count_launches(1);
-      return cudaGetLastError();
-    }
+    const int grid = per_sel > 1 ? n_sel * per_sel : n_sel < max_ctas ? n_sel : max_ctas;
+    unsigned long long k_rest = (unsigned long long)a.k_rest;
+    long long nnz_init = count_nnz ? 0ll : (long long)a.k;
+    int classified = classify ? 1 : 0, n_sel_arg = n_sel, rows_arg = rows, period_arg = period, per_sel_arg = per_sel;
+    int diag_arg = diag, n_qt_arg = n_qt, n_kt_arg = n_kt, Lk = a.Lk, Lq = a.Lq, H = a.H, causal = a.causal;
+    int keep_ties = a.keep_ties;
+    uint32_t cap_arg = shortcut ? (uint32_t)cap : 0u;
+    const float *acc = a.acc;
+    const uint2 *cand = sc.cand;
+    int64_t *nnz = a.nnz;
+    uint8_t *mask = a.mask;
+    uint32_t *stage_bitmap = a.stage_bitmap, *stage_groups = a.stage_groups;
+    int32_t *stage_count = a.stage_count;
+    void *args[] = {&acc, &rows_arg, &Lk, &period_arg, &causal, &diag_arg, &k_rest, &n_sel_arg, &per_sel_arg, &sc.state,
+                    &sc.hist, &cand, &cap_arg, &keep_ties, &H, &nnz_init, &nnz, &classified, &Lq, &n_qt_arg, &n_kt_arg,
+                    &mask, &stage_bitmap, &stage_count, &stage_groups, &err};
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(select_kernel), dim3(grid), dim3(kSelThreads), args, 0, s);
+    if (e != cudaSuccess) return e;
+    count_launches(1);
   }
-  init_state_kernel<<<ceil_div(max(n_sel * kBins, a.H), 256), 256, 0, s>>>(
-      sc.state, sc.hist, n_sel, (unsigned long long)a.k_rest, a.H, count_nnz ? 0ll : (long long)a.k, a.nnz);
-  count_launches(1);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  // enough CTAs per selection to fill the GPU, at most one warp-row each
-  int row_blocks = ceil_div(rows, kWarps);
-  const int want = ceil_div(148 * 8, n_sel);
-  if (row_blocks > want) row_blocks = want;
-  dim3 grid(row_blocks, n_sel);
-  if (a.k_rest > 0) {
-    // large selections: the one-pass shortcut first (those it resolves skip the three passes below)
-    const long long n_valid = domain_size(a.Lq, a.Lk, a.causal);
-    const long long n_rest = (n_valid - (diag ? a.Lq : 0)) * (a.per_layer ? a.H : 1);
-    const long long cap = cand_capacity(n_rest);
-    if (cap > 0) {
-      const size_t smem = (kSamples + kBins) * sizeof(uint32_t);
-      e = cudaFuncSetAttribute(sample_pivots_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      sample_pivots_kernel<<<dim3(n_sel, 2), 1024, smem, s>>>(a.acc, rows, a.Lk, period, a.causal, diag,
-                                                     (unsigned long long)a.k_rest, (unsigned long long)n_rest, sc.state);
-      // Exact per-head selections: the one pass over the accumulator also writes what is certain of the
-      // mask and the tile bitmaps (the patch pass below adds the collected entries that are kept), so
-      // the emit pass at the end has nothing to read for the selections the shortcut resolves.  Other
-      // selections count what they keep in the emit pass, which therefore has to see every entry.
-      const bool classify = !a.per_layer && !a.keep_ties;
-      if (classify) {
-        emit_kernel<true><<<a.H * n_qt * n_kt, 128, 0, s>>>(a.acc, a.Lq, a.Lk, n_qt, n_kt, a.causal, diag, 0, 0,
-                                                            sc.state, sc.tie_count, a.mask, a.stage_bitmap,
-                                                            a.stage_count, a.nnz, sc.cand, (uint32_t)cap);
-      } else {
-        // one wave of CTAs (five fit an SM), so that no SM idles while a second, partial wave runs
-        int collect_blocks = ceil_div(rows, kWarps);
-        if (collect_blocks > 148 * 5 / n_sel) collect_blocks = max(148 * 5 / n_sel, 1);
-        collect_kernel<<<dim3(collect_blocks, n_sel), kThreads, 0, s>>>(a.acc, rows, a.Lk, period, a.causal, diag,
-                                                                       sc.state, sc.cand, (uint32_t)cap);
-      }
-      // the threshold among the collected keys: the same three digits, on offsets from the lower pivot
-      const dim3 cand_grid(ceil_div(148 * 8, n_sel), n_sel);
-      for (int pass = 0; pass < kPasses; ++pass) {
-        cand_histogram_kernel<<<cand_grid, kThreads, 0, s>>>(sc.state, sc.cand, (uint32_t)cap,
-                                                             (unsigned long long)a.k_rest, pass, sc.hist);
-      }
-      cand_finish_kernel<<<cand_grid, kThreads, 0, s>>>(sc.state, sc.cand, (uint32_t)cap, sc.tie_list,
-                                                        classify ? 1 : 0);
-      count_launches(3 + kPasses);
-      if (classify) {
-        patch_kernel<<<cand_grid, kThreads, 0, s>>>(sc.state, sc.cand, (uint32_t)cap, a.Lq, a.Lk, n_qt, n_kt, a.mask,
-                                                    a.stage_bitmap, a.stage_count);
-        count_launches(1);
-      }
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    for (int pass = 0; pass < kPasses; ++pass) {
-      digit_histogram_kernel<<<grid, kThreads, 0, s>>>(a.acc, rows, a.Lk, period, a.causal, diag, pass, sc.state,
-                                                       sc.hist);
-      count_launches(1);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if (!a.keep_ties) {  // the ties' ranks are needed only where some of them are pruned
-      // both return at once for selections whose ties with the threshold are all kept
-      tie_count_kernel<<<grid, kThreads, 0, s>>>(a.acc, rows, a.Lk, period, n_kt, a.causal, diag, sc.state,
-                                                 sc.tie_count);
-      count_launches(1);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+  // Few tiles: sixteen warps each, so that a tile's rows are all in flight at once.  With the mask written by then (the
+  // usual end of a classified selection) the launch only has to look.
+  if (n_tiles <= 4 * sms) {
+    emit_kernel<false, 16><<<n_tiles, 512, 0, s>>>(a.acc, a.Lq, a.Lk, n_qt, n_kt, n_tiles, a.causal, diag, a.per_layer,
+                                                   a.keep_ties, sc.state, a.mask, a.stage_bitmap, a.stage_count,
+                                                   a.stage_groups, a.nnz, nullptr, 0u);
+  } else {
+    emit_kernel<false, 4><<<n_tiles < 16 * sms ? n_tiles : 16 * sms, 128, 0, s>>>(
+        a.acc, a.Lq, a.Lk, n_qt, n_kt, n_tiles, a.causal, diag, a.per_layer, a.keep_ties, sc.state, a.mask, a.stage_bitmap,
+        a.stage_count, a.stage_groups, a.nnz, nullptr, 0u);
   }
-  emit_kernel<false><<<a.H * n_qt * n_kt, 128, 0, s>>>(a.acc, a.Lq, a.Lk, n_qt, n_kt, a.causal, diag, a.per_layer,
-                                                       a.keep_ties, sc.state, sc.tie_count, a.mask, a.stage_bitmap,
-                                                       a.stage_count, a.nnz, nullptr, 0u);
   count_launches(1);
-  return cudaGetLastError();
+  if ((e = cudaGetLastError()) != cudaSuccess || !a.tiles) return e;
+  // the histograms are free by now: the compaction keeps its CTAs' totals there
+  return launch_compact_staged(a.stage_bitmap, a.stage_count, a.stage_groups, *a.tiles, reinterpret_cast<int2 *>(sc.hist),
+                               (size_t)kHistBuffers * kBins * sizeof(uint32_t) / sizeof(int2), &header->compact_barrier, s);
 }
 
 }  // namespace ap

@@ -98,6 +98,10 @@ cudaError_t launch_stage_from_mask(const uint8_t *mask, int H, int Lq, int Lk, u
 // Staging area -> compacted tile list.
 cudaError_t launch_compact_tiles(const uint32_t *stage_bitmap, const int32_t *stage_count,
                                  const ap_tiles &t, cudaStream_t s);
+// The same from a staging area that holds the tiles' group summaries too (stage_groups[H*n_qt*n_kt]), in one cooperative
+// kernel.  totals: room for n_totals pairs, one per CTA; barrier: a word that is zero.
+cudaError_t launch_compact_staged(const uint32_t *stage_bitmap, const int32_t *stage_count, const uint32_t *stage_groups,
+                                  const ap_tiles &t, int2 *totals, size_t n_totals, uint32_t *barrier, cudaStream_t s);
 cudaError_t launch_dense_tiles(const ap_tiles &t, int causal, cudaStream_t s);
 
 size_t stage_bytes(int H, int Lq, int Lk);
@@ -113,6 +117,8 @@ struct BuildMaskArgs {
   int64_t *nnz;    // may be NULL
   uint32_t *stage_bitmap;  // may be NULL (no tile list wanted)
   int32_t *stage_count;
+  uint32_t *stage_groups;
+  const ap_tiles *tiles;  // may be NULL
   void *scratch;  // select scratch
 };
 size_t select_scratch_bytes(int H, int Lq, int Lk);

@@ -6,6 +6,7 @@
 // assigns list positions to the non-empty ones in that order, and a copy
 // kernel moves their bitmaps to the compacted list.
 #include "ap_common.cuh"
+#include "ap_grid.cuh"
 
 namespace ap {
 
@@ -393,6 +394,227 @@ __global__ void __launch_bounds__(128) fill_rounds_kernel(const int32_t *__restr
   }
 }
 
+// ---- all of the above in one launch ----------------------------------------------------------
+
+constexpr int kCompactCtasPerSm = 8;
+
+// Cooperative: staging area with group summaries -> tile list and rounds.  A CTA counts the tiles and rounds of its share
+// of the list rows; after a barrier it knows what lies before them and writes their offsets; after another, `parts`
+// CTAs per list row (n_rows * parts pieces, taken in turn) copy the row's bitmaps and write its rounds, straight from
+// the staging area.  The five kernels it stands for (still those of ap_mask_to_tiles) took 23 us on 16 heads x 512
+// tokens, most of it launches and the latency of short grids.
+__global__ void __launch_bounds__(128, kCompactCtasPerSm)
+compact_kernel(const uint32_t *__restrict__ stage_bitmap, const int32_t *__restrict__ stage_count,
+               const uint32_t *__restrict__ stage_groups, int n_rows, int n_kt, int cap, int parts, int32_t *row_ptr,
+               int32_t *__restrict__ col_idx, uint8_t *__restrict__ flags, uint32_t *__restrict__ bitmap,
+               uint8_t *__restrict__ groups, int32_t *round_ptr, int32_t *__restrict__ round_rows,
+               uint8_t *__restrict__ round_info, uint32_t *__restrict__ round_bitmap, int2 *totals, uint32_t *barrier,
+               unsigned *err) {
+  constexpr int kSeg = 128;                    // key tiles per pass
+  __shared__ uint32_t slot_src[kSeg * 8 + 8];  // key tile << 4 | group << 1 | tile fully kept
+  __shared__ int32_t seg_kt[kSeg];             // the pass's stored tiles
+  __shared__ int2 warp_sums[4];
+  const int r = threadIdx.x, lane = r & 31, warp = r >> 5, n_ctas = (int)gridDim.x;
+  // ---- counts of this CTA's rows
+  const int per_cta = (n_rows + n_ctas - 1) / n_ctas, row0 = min(n_rows, (int)blockIdx.x * per_cta),
+            row1 = min(n_rows, row0 + per_cta);
+  int2 mine = make_int2(0, 0);  // (tiles, rounds); lane 0 of each warp
+  for (int row = row0 + warp; row < row1; row += 4) {
+    int tiles = 0, slots = 0;
+    for (int kt = lane; kt < n_kt; kt += 32) {
+      const size_t tile = (size_t)row * n_kt + kt;
+      if (stage_count[tile] > 0) {
+        ++tiles;
+        slots += __popc(stage_groups[tile]);
+      }
+    }
+    tiles = __reduce_add_sync(0xffffffffu, tiles);
+    slots = __reduce_add_sync(0xffffffffu, slots);
+    if (lane == 0) {
+      row_ptr[row + 1] = tiles;
+      round_ptr[row + 1] = (slots + 7) / 8;
+      mine.x += tiles;
+      mine.y += (slots + 7) / 8;
+    }
+  }
+  if (lane == 0) warp_sums[warp] = mine;
+  __syncthreads();
+  if (r == 0)
+    totals[blockIdx.x] = make_int2(warp_sums[0].x + warp_sums[1].x + warp_sums[2].x + warp_sums[3].x,
+                                   warp_sums[0].y + warp_sums[1].y + warp_sums[2].y + warp_sums[3].y);
+  if (!cta_barrier(barrier, (uint32_t)n_ctas, err)) return;
+  // ---- offsets: what lies before this CTA's rows, then a running sum over them
+  int2 before = make_int2(0, 0);
+  int all_tiles = 0;
+  for (int c = r; c < n_ctas; c += 128) {
+    const int2 t = __ldcg(totals + c);
+    all_tiles += t.x;
+    if (c < (int)blockIdx.x) {
+      before.x += t.x;
+      before.y += t.y;
+    }
+  }
+  before.x = __reduce_add_sync(0xffffffffu, before.x);
+  before.y = __reduce_add_sync(0xffffffffu, before.y);
+  all_tiles = __reduce_add_sync(0xffffffffu, all_tiles);
+  __shared__ int tiles_s[4];
+  if (lane == 0) {
+    warp_sums[warp] = before;
+    tiles_s[warp] = all_tiles;
+  }
+  __syncthreads();
+  before = make_int2(warp_sums[0].x + warp_sums[1].x + warp_sums[2].x + warp_sums[3].x,
+                     warp_sums[0].y + warp_sums[1].y + warp_sums[2].y + warp_sums[3].y);
+  all_tiles = tiles_s[0] + tiles_s[1] + tiles_s[2] + tiles_s[3];
+  __syncthreads();
+  for (int base = row0; base < row1; base += 128) {
+    const int row = base + r;
+    const int2 own = row < row1 ? make_int2(row_ptr[row + 1], round_ptr[row + 1]) : make_int2(0, 0);
+    int2 incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl.x, o), y = __shfl_up_sync(0xffffffffu, incl.y, o);
+      if (lane >= o) incl.x += x, incl.y += y;
+    }
+    if (lane == 31) warp_sums[warp] = incl;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) incl.x += warp_sums[w].x, incl.y += warp_sums[w].y;
+    if (row < row1) {
+      row_ptr[row + 1] = min(before.x + incl.x, cap);
+      round_ptr[row + 1] = before.y + incl.y;
+    }
+#pragma unroll
+    for (int w = 0; w < 4; ++w) before.x += warp_sums[w].x, before.y += warp_sums[w].y;
+    __syncthreads();
+  }
+  if (blockIdx.x == 0 && r == 0) {
+    row_ptr[0] = 0;
+    round_ptr[0] = 0;
+    if (all_tiles > cap) atomicOr(err, kDevErrCapacity);
+  }
+  if (!cta_barrier(barrier, 2u * (uint32_t)n_ctas, err)) return;
+  if (all_tiles > cap) {
+    // (the error case: the list is cut off, and so are the rounds; one warp counts them again)
+    if (blockIdx.x == 0 && warp == 0) {
+      int at = 0;
+      for (int row = 0; row < n_rows; ++row) {
+        const int keep = __ldcg(row_ptr + row + 1) - __ldcg(row_ptr + row);
+        int seen = 0, slots = 0;
+        for (int kt0 = 0; kt0 < n_kt && seen < keep; kt0 += 32) {
+          const size_t tile = (size_t)row * n_kt + kt0 + lane;
+          const bool there = kt0 + lane < n_kt && stage_count[tile] > 0;
+          const uint32_t vote = __ballot_sync(0xffffffffu, there);
+          const bool in = there && seen + __popc(vote & ((1u << lane) - 1u)) < keep;
+          slots += __reduce_add_sync(0xffffffffu, in ? __popc(stage_groups[tile]) : 0);
+          seen += __popc(vote);
+        }
+        at += (slots + 7) / 8;
+        if (lane == 0) round_ptr[row + 1] = at;
+      }
+    }
+    if (!cta_barrier(barrier, 3u * (uint32_t)n_ctas, err)) return;
+  }
+  // ---- the list and its rounds
+  for (int piece = (int)blockIdx.x; piece < n_rows * parts; piece += n_ctas) {
+    const int row = piece / parts, part = piece % parts;
+    const int t0 = __ldcg(row_ptr + row), keep = __ldcg(row_ptr + row + 1) - t0;
+    int rho = __ldcg(round_ptr + row), seen = 0;
+    int pending = 0;  // slots carried over from the previous pass (fewer than eight)
+    const uint32_t *row_bitmap = stage_bitmap + (size_t)row * n_kt * kBitmapWords;
+    for (int base = 0; base < n_kt && seen < keep; base += kSeg) {
+      const int kt = base + r;
+      const size_t tile = (size_t)row * n_kt + kt;
+      const int count = kt < n_kt ? stage_count[tile] : 0;
+      const bool full = count == kTile * kTile;
+      int2 incl = make_int2(count > 0 ? 1 : 0, 0);
+      uint32_t gm = count > 0 ? stage_groups[tile] : 0u;
+      incl.y = __popc(gm);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, incl.x, o), y = __shfl_up_sync(0xffffffffu, incl.y, o);
+        if (lane >= o) incl.x += x, incl.y += y;
+      }
+      if (lane == 31) warp_sums[warp] = incl;
+      __syncthreads();
+      int2 total = make_int2(0, 0);
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        if (w < warp) incl.x += warp_sums[w].x, incl.y += warp_sums[w].y;
+        total.x += warp_sums[w].x, total.y += warp_sums[w].y;
+      }
+      const int rank = incl.x - 1;  // among the pass's stored tiles
+      const bool there = count > 0 && seen + rank < keep;
+      int s = pending + incl.y - __popc(gm);
+      if (there) {
+        seg_kt[rank] = kt;
+        if (part == 0) {
+          const int t = t0 + seen + rank;
+          col_idx[t] = kt;
+          flags[t] = full ? 1 : 0;
+          groups[t] = (uint8_t)gm;
+        }
+        for (uint32_t left = gm; left; left &= left - 1u)
+          slot_src[s++] = ((uint32_t)kt << 4) | ((uint32_t)(__ffs((int)left) - 1) << 1) | (full ? 1u : 0u);
+      }
+      const int n_here = min(total.x, keep - seen);
+      // (a row that is cut off ends with the slots of its last kept tile)
+      __shared__ int slots_s;
+      if (there && rank == n_here - 1) slots_s = s;
+      __syncthreads();
+      const int avail = n_here > 0 ? slots_s : pending;
+      for (int k0 = part; k0 < n_here; k0 += 4 * parts) {  // four tiles in flight
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (k0 + u * parts < n_here)
+            v[u] = reinterpret_cast<const uint4 *>(row_bitmap + (size_t)seg_kt[k0 + u * parts] * kBitmapWords)[r];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (k0 + u * parts < n_here)
+            reinterpret_cast<uint4 *>(bitmap + (size_t)(t0 + seen + k0 + u * parts) * kBitmapWords)[r] = v[u];
+      }
+      const bool last_pass = base + kSeg >= n_kt || seen + n_here >= keep;
+      const int n_emit = last_pass ? (avail + 7) / 8 : avail / 8;
+      for (int k = part; k < n_emit; k += parts) {
+        const int ng = min(8, avail - 8 * k);
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+        bool all_full = true;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          if (q >= ng) continue;
+          const uint32_t src = slot_src[8 * k + q];
+          uint32_t field = 0xffffu;
+          if (!(src & 1u)) {
+            const uint32_t g = (src >> 1) & 7u;
+            field = (row_bitmap[(size_t)(src >> 4) * kBitmapWords + r * 4 + (g >> 1)] >> (16u * (g & 1u))) & 0xffffu;
+            all_full = false;
+          }
+          w[q >> 1] |= field << (16 * (q & 1));
+        }
+        const int out = rho + k;
+        if (out < cap) {
+          reinterpret_cast<uint4 *>(round_bitmap + (size_t)out * kBitmapWords)[r] = make_uint4(w[0], w[1], w[2], w[3]);
+          if (r < 8) {
+            const uint32_t src = r < ng ? slot_src[8 * k + r] : 0u;
+            round_rows[(size_t)out * 8 + r] = r < ng ? (int)(src >> 4) * kTile + 16 * (int)((src >> 1) & 7u) : -1;
+          }
+          if (r == 0) round_info[out] = (uint8_t)(ng | ((all_full && ng == 8) ? 0x80 : 0));
+        }
+      }
+      rho += n_emit;
+      seen += n_here;
+      __syncthreads();
+      // fewer than eight slots are left over; they move to the front (no overlap: they start at or
+      // beyond index 8 unless nothing was written out, in which case they are in place already)
+      const int left = avail - 8 * n_emit;
+      if (!last_pass && n_emit > 0 && r < left) slot_src[r] = slot_src[8 * n_emit + r];
+      pending = last_pass ? 0 : left;
+      __syncthreads();
+    }
+    __syncthreads();
+  }
+}
+
 // ---- gathered rounds: a list row's active key columns, 128 per round ----------------------------
 
 // The 128-bit column summary of one stored tile (bit c: some row keeps column c), by one warp:
@@ -595,8 +817,11 @@ __global__ void clear_grounds_kernel(int32_t *__restrict__ ground_ptr, int n) {
 
 }  // namespace
 
-// Writes the round arrays of a finished tile list (row_ptr, col_idx, flags, groups, bitmap), and the
-// gathered rounds where the list has room for them (gathered == false: an empty gathered schedule).
+// What a list may carry beside its rounds: balanced units of work, and the gathered rounds (gathered == false: an empty
+// gathered schedule).
+static cudaError_t launch_options(const ap_tiles &t, cudaStream_t s, bool gathered);
+
+// Writes the round arrays of a finished tile list (row_ptr, col_idx, flags, groups, bitmap) and what else it carries.
 cudaError_t launch_build_rounds(const ap_tiles &t, cudaStream_t s, bool gathered) {
   const int n_rows = t.H * t.n_qt;
   count_rounds_kernel<<<ceil_div(n_rows, 4), 128, 0, s>>>(t.row_ptr, t.flags, t.groups, n_rows, t.round_ptr);
@@ -605,7 +830,12 @@ cudaError_t launch_build_rounds(const ap_tiles &t, cudaStream_t s, bool gathered
                                             t.round_rows, t.round_info, t.round_bitmap);
   count_launches(3);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  return e == cudaSuccess ? launch_options(t, s, gathered) : e;
+}
+
+static cudaError_t launch_options(const ap_tiles &t, cudaStream_t s, bool gathered) {
+  const int n_rows = t.H * t.n_qt;
+  cudaError_t e = cudaSuccess;
   if (t.unit_qt) {
     pair_units_kernel<<<t.H, 256, 0, s>>>(t.round_ptr, t.n_qt, t.unit_qt);
     count_launches(1);
@@ -653,6 +883,29 @@ cudaError_t launch_compact_tiles(const uint32_t *stage_bitmap, const int32_t *st
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_build_rounds(t, s, true);
+}
+
+cudaError_t launch_compact_staged(const uint32_t *stage_bitmap, const int32_t *stage_count, const uint32_t *stage_groups,
+                                  const ap_tiles &t, int2 *totals, size_t n_totals, uint32_t *barrier, cudaStream_t s) {
+  unsigned *err = device_error_word();
+  const int sms = sm_count();
+  if (!err || sms <= 0) return cudaErrorUnknown;
+  int n_rows = t.H * t.n_qt, n_kt = t.n_kt, cap = t.cap;
+  long long grid = (long long)kCompactCtasPerSm * sms;  // all of them resident; up to eight per list row have work
+  if (grid > (long long)n_rows * 8) grid = (long long)n_rows * 8;
+  if (grid > (long long)n_totals) grid = (long long)n_totals;
+  int parts = (int)(grid / n_rows);
+  parts = parts < 1 ? 1 : parts > 8 ? 8 : parts;
+  int32_t *row_ptr = t.row_ptr, *col_idx = t.col_idx, *round_ptr = t.round_ptr, *round_rows = t.round_rows;
+  uint8_t *flags = t.flags, *groups = t.groups, *round_info = t.round_info;
+  uint32_t *bitmap = t.bitmap, *round_bitmap = t.round_bitmap;
+  void *args[] = {&stage_bitmap, &stage_count, &stage_groups, &n_rows, &n_kt, &cap, &parts, &row_ptr, &col_idx, &flags,
+                  &bitmap, &groups, &round_ptr, &round_rows, &round_info, &round_bitmap, &totals, &barrier, &err};
+  cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(compact_kernel), dim3((unsigned)grid), dim3(128),
+                                              args, 0, s);
+  if (e != cudaSuccess) return e;
+  count_launches(1);
+  return launch_options(t, s, true);
 }
 
 cudaError_t launch_dense_tiles(const ap_tiles &t, int causal, cudaStream_t s) {
