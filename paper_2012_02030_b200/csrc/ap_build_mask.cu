@@ -466,7 +466,7 @@ select_kernel(const float *__restrict__ acc, int rows, int Lk, int period, int c
           for (int u = 0; u < 4; ++u) count(c[u].x - lo, c[u].y, x0 + u * kSelThreads < n_cand);
         }
       } else {
-        scan_domain(base, rows, Lk, period, causal, diag, (uint32_t)(rank * (kSelThreads / 32) + warp),
+        scan_domain(base, rows, Lk, period, causal, diag, (uint32_t)(warp * per_sel + rank),
                     (uint32_t)(per_sel * (kSelThreads / 32)), lane,
                     [&](float f, uint32_t index, bool there) { count(key_of(f), index, there); });
       }
