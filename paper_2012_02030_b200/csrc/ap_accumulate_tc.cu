@@ -52,16 +52,17 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kThreads = 320;
-constexpr int kSoftmaxThreads = 256;
-constexpr int kSoftmaxWarps = kSoftmaxThreads / 32;
+constexpr int kSoftmaxWarps = 16;
+constexpr int kProducer = kSoftmaxWarps, kIssuer = kSoftmaxWarps + 1;
+constexpr int kThreads = (kSoftmaxWarps + 2) * 32;
+constexpr int kRegThreads = 640;  // registers are handed out to whole sets of four warps: 20 warps' worth, 96 each
 constexpr int kSubBytes = 128 * 128;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSumCol = 256;    // running sum over b: 128 columns
-constexpr uint32_t kStatsCol = 384;  // (max, sum) pairs: 64 columns per column half, 2 per sample
-constexpr int kMaxB = 32;            // samples per launch (what the spare tensor-memory columns hold)
+constexpr uint32_t kStatsCol = 384;  // (max, sum) pairs: 32 columns per column quarter, 2 per sample
+constexpr int kMaxB = 16;            // samples per launch (what the spare tensor-memory columns hold)
 constexpr int kBiasBytes = 128 * 128 * 4;  // one fp32 bias tile: 4 boxes of 128 rows x 32 columns
-constexpr int kRedBytes = 32 * 128;        // per softmax warp: 32 rows x 32 fp32 columns on their way to the accumulator
+constexpr int kRedBytes = 32 * 64;         // per softmax warp: 32 rows x 16 fp32 columns on their way to the accumulator
 constexpr float kLog2e = 1.4426950408889634f;
 
 template <int D>
@@ -127,7 +128,7 @@ unsigned *turn_words() {
 // kChunked: the instantiation for launches whose samples are cut into chunks (see below); a
 // separate one so that its extra code costs the plain launches nothing.
 template <int D, bool kChunked>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kRegThreads, 1)
 accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_bias, const __grid_constant__ CUtensorMap map_acc,
                      int bias_by_tma, int acc_by_tma, float *__restrict__ acc, const float *__restrict__ bias, int b0,
@@ -173,7 +174,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     bars->abort_flag = 0;
     fence_mbar_init();
   }
-  if (warp == 9) {
+  if (warp == kIssuer) {
     tmem_alloc(&bars->tmem_base, kTmemCols);
     tmem_relinquish();
   }
@@ -184,7 +185,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   volatile int *abort_flag = &bars->abort_flag;
   const Waiter wait{abort_flag, err, max_polls};
 
-  if (warp == 8) {
+  if (warp == kProducer) {
     // ------------------------------------------------------------ TMA producer
     {
       if (lane == 0) {
@@ -233,7 +234,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (bias_loads > 0) mbar_wait(&bars->bias_full, (uint32_t)(bias_loads - 1) & 1u, max_polls);
       }
     }
-  } else if (warp == 9) {
+  } else if (warp == kIssuer) {
     // ------------------------------------------------------------ MMA issuer
     {
       const uint32_t idesc = idesc_bf16_f32(128, 128, false, false, f16 != 0);
@@ -260,7 +261,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       }
     }
   } else {
-    // ------------------------------------------------------------ softmax (256 threads)
+    // ------------------------------------------------------------ softmax (512 threads)
     const int wg = warp >> 2;
     const int r = (warp & 3) * 32 + lane;  // row of the tile == TMEM lane
     const int i = qt * kTile + r;
@@ -268,40 +269,37 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const int jend = causal ? min(Lk, i + 1 + off) : Lk;  // first key outside this row's domain
     const bool vec = (Lk & 3) == 0;
-    const uint32_t s_addr = tmem + lane_addr + 64 * wg;                   // + 128 * buf
-    const uint32_t sum_addr = tmem + lane_addr + kSumCol + 64 * wg;       // + 32 * c
-    const uint32_t my_stats = tmem + lane_addr + kStatsCol + 64 * wg;     // + 2 * b
-    const uint32_t other_stats = tmem + lane_addr + kStatsCol + 64 * (1 - wg);
-    // this warp's 32 rows x 32 columns on their way to the accumulator, and the rows' place in it
+    const uint32_t s_addr = tmem + lane_addr + 32 * wg;             // + 128 * buf
+    const uint32_t sum_addr = tmem + lane_addr + kSumCol + 32 * wg;
+    const uint32_t stats = tmem + lane_addr + kStatsCol;            // + 32 * quarter + 2 * b
+    const uint32_t my_stats = stats + 32 * wg;
+    // this warp's 32 rows x 16 columns on their way to the accumulator, and the rows' place in it
     unsigned char *red_s = smem + C::kRedOffset + warp * kRedBytes;
     const int red_y = qt * kTile + (warp & 3) * 32;
     const int red_jend = causal ? min(Lk, red_y + 32 + off) : Lk;  // first key outside the domain of all 32 rows
 
     for (int b = 0; b < Bc; ++b) tmem_st2(my_stats + 2 * b, __float_as_uint(-CUDART_INF_F), 0u);
 
-    float bias2[64];  // bias * log2(e) of this thread's 64 columns of the current key tile
+    float bias2[32];  // bias * log2(e) of this thread's 32 columns of the current key tile
     bool ok = true;
     // the bias slice of key tile kt (tl: how many tiles were staged before it), once for all samples
     auto fetch_bias = [&](int kt, int tl) {
-      const int j0 = kt * kTile + 64 * wg;
+      const int j0 = kt * kTile + 32 * wg;
       if (bias_by_tma) {
         ok = wait(&bars->bias_full, (uint32_t)tl & 1u);
         if (!ok) return;
+        const unsigned char *box = bias_s + wg * (kBiasBytes / 4) + r * 128;
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const unsigned char *box = bias_s + (2 * wg + q) * (kBiasBytes / 4) + r * 128;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {  // 16-byte chunk k of the row sits at position k ^ (r % 8)
-            const float4 t = *reinterpret_cast<const float4 *>(box + ((k ^ (r & 7)) << 4));
-            bias2[32 * q + 4 * k] = t.x * kLog2e; bias2[32 * q + 4 * k + 1] = t.y * kLog2e;
-            bias2[32 * q + 4 * k + 2] = t.z * kLog2e; bias2[32 * q + 4 * k + 3] = t.w * kLog2e;
-          }
+        for (int k = 0; k < 8; ++k) {  // 16-byte chunk k of the row sits at position k ^ (r % 8)
+          const float4 t = *reinterpret_cast<const float4 *>(box + ((k ^ (r & 7)) << 4));
+          bias2[4 * k] = t.x * kLog2e; bias2[4 * k + 1] = t.y * kLog2e;
+          bias2[4 * k + 2] = t.z * kLog2e; bias2[4 * k + 3] = t.w * kLog2e;
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars->bias_empty);
       } else {
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
+        for (int c = 0; c < 8; ++c) {
           float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
           const int j = j0 + 4 * c;
           if (bias && row_ok) {
@@ -316,16 +314,15 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         }
       }
     };
-    // S of visit v is ready: copy this thread's 64 columns to registers and hand S back.  The MMA of
+    // S of visit v is ready: copy this thread's 32 columns to registers and hand S back.  The MMA of
     // visit v + 2 may then overwrite the buffer while the arithmetic on the copy is still going on
-    // (one arrival per warp: 256 threads arriving one by one would take longer than a visit's MMAs).
-    auto take_s = [&](int v, uint32_t (&xs)[64]) {
+    // (one arrival per warp: 512 threads arriving one by one would take longer than a visit's MMAs).
+    auto take_s = [&](int v, uint32_t (&xs)[32]) {
       const int buf = v & 1;
       ok = wait(&bars->s_full[buf], (uint32_t)(v >> 1) & 1u);
       if (!ok) return;
       tc_fence_after_sync();
       tmem_ld32(s_addr + 128 * buf, xs);
-      tmem_ld32(s_addr + 128 * buf + 32, xs + 32);
     };
     auto release_s = [&](int v) {
       tc_fence_before_sync();
@@ -339,29 +336,29 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       fetch_bias(kt, kt);
       if (!ok) break;
       // columns of this slice inside the row's domain; whole warp inside => no masking
-      const int n_valid = max(0, min(64, jend - (kt * kTile + 64 * wg)));
-      const bool interior = __all_sync(0xffffffffu, n_valid == 64);
+      const int n_valid = max(0, min(32, jend - (kt * kTile + 32 * wg)));
+      const bool interior = __all_sync(0xffffffffu, n_valid == 32);
       for (int b = 0; b < Bc; ++b, ++v) {
-        uint32_t xs[64], sv[2];
+        uint32_t xs[32], sv[2];
         take_s(v, xs);
         if (!ok) break;
         tmem_wait_st();  // this sample's pair as the previous key tile left it
         tmem_ld2(my_stats + 2 * b, sv);
         tmem_wait_ld();
         release_s(v);
-        float t[64];
+        float t[32];
 #pragma unroll
-        for (int e = 0; e < 64; e += 2)
+        for (int e = 0; e < 32; e += 2)
           ffma2(t[e], t[e + 1], __uint_as_float(xs[e]), __uint_as_float(xs[e + 1]), scale_log2, bias2[e], bias2[e + 1]);
         if (!interior) {
 #pragma unroll
-          for (int e = 0; e < 64; ++e) t[e] = e < n_valid ? t[e] : -CUDART_INF_F;
+          for (int e = 0; e < 32; ++e) t[e] = e < n_valid ? t[e] : -CUDART_INF_F;
         }
         const float m_old = __uint_as_float(sv[0]);
         // four independent chains each for the maximum and for the sum
         float m0 = m_old, m1 = -CUDART_INF_F, m2 = -CUDART_INF_F, m3 = -CUDART_INF_F;
 #pragma unroll
-        for (int e = 0; e < 64; e += 8) {  // three-input maxima: half the instructions
+        for (int e = 0; e < 32; e += 8) {  // three-input maxima: half the instructions
           m0 = fmax3(m0, t[e], t[e + 4]);
           m1 = fmax3(m1, t[e + 1], t[e + 5]);
           m2 = fmax3(m2, t[e + 2], t[e + 6]);
@@ -372,7 +369,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         float z0 = __uint_as_float(sv[1]) * ex2_approx(m_old - cm_safe), z1 = 0.f, z2 = 0.f, z3 = 0.f;
         const float neg_cm = -cm_safe;
 #pragma unroll
-        for (int e = 0; e < 64; e += 4) {
+        for (int e = 0; e < 32; e += 4) {
           float a0, a1, a2, a3;
           fadd2(a0, a1, t[e], t[e + 1], neg_cm, neg_cm);
           fadd2(a2, a3, t[e + 2], t[e + 3], neg_cm, neg_cm);
@@ -383,7 +380,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       }
     }
     if (ok) {
-      // every statistic of sweep 1 is final once both column halves of every row are done
+      // every statistic of sweep 1 is final once all column quarters of every row are done
       tmem_wait_st();
       tc_fence_before_sync();
       __syncwarp();
@@ -396,41 +393,43 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     for (int kt = 0; kt < n_k && ok; ++kt) {
       fetch_bias(kt, n_k + kt);
       if (!ok) break;
-      const int j0 = kt * kTile + 64 * wg;  // first column of this thread's slice
-      const int n_valid = max(0, min(64, jend - j0));
-      const bool interior = __all_sync(0xffffffffu, n_valid == 64);
+      const int j0 = kt * kTile + 32 * wg;  // first column of this thread's slice
+      const int n_valid = max(0, min(32, jend - j0));
+      const bool interior = __all_sync(0xffffffffu, n_valid == 32);
       for (int b = 0; b < Bc; ++b, ++v) {
-        uint32_t xs[64], s0[2], s1[2];
+        uint32_t xs[32], st[4][2];
         take_s(v, xs);
         if (!ok) break;
-        tmem_ld2(my_stats + 2 * b, s0);
-        tmem_ld2(other_stats + 2 * b, s1);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tmem_ld2(stats + 32 * q + 2 * b, st[q]);
         tmem_wait_ld();
         release_s(v);
-        // both column halves' statistics of sample b combined: max + log2(sum).  A row without any key
+        // the column quarters' statistics of sample b combined: max + log2(sum).  A row without any key
         // in its domain (possible when Lk < Lq) gets weight 0 everywhere.
-        const float mm = fmaxf(__uint_as_float(s0[0]), __uint_as_float(s1[0]));
-        const float z = __uint_as_float(s0[1]) * ex2_approx(__uint_as_float(s0[0]) - mm) +
-                        __uint_as_float(s1[1]) * ex2_approx(__uint_as_float(s1[0]) - mm);
+        const float mm = fmaxf(fmaxf(__uint_as_float(st[0][0]), __uint_as_float(st[1][0])),
+                               fmaxf(__uint_as_float(st[2][0]), __uint_as_float(st[3][0])));
+        float z = 0.f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) z += __uint_as_float(st[q][1]) * ex2_approx(__uint_as_float(st[q][0]) - mm);
         const float neg_ref = jend > 0 ? -(mm + lg2_approx(z)) : -CUDART_INF_F;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          float p[32];
+          float p[16];
 #pragma unroll
-          for (int e = 0; e < 32; e += 2)
-            ffma2(p[e], p[e + 1], __uint_as_float(xs[32 * c + e]), __uint_as_float(xs[32 * c + e + 1]), scale_log2,
-                  bias2[32 * c + e], bias2[32 * c + e + 1]);
+          for (int e = 0; e < 16; e += 2)
+            ffma2(p[e], p[e + 1], __uint_as_float(xs[16 * c + e]), __uint_as_float(xs[16 * c + e + 1]), scale_log2,
+                  bias2[16 * c + e], bias2[16 * c + e + 1]);
           if (!interior) {
 #pragma unroll
-            for (int e = 0; e < 32; ++e) p[e] = 32 * c + e < n_valid ? p[e] : -CUDART_INF_F;
+            for (int e = 0; e < 16; ++e) p[e] = 16 * c + e < n_valid ? p[e] : -CUDART_INF_F;
           }
-          uint32_t ps[32];
+          uint32_t ps[16];
           if (b > 0) {
-            tmem_ld32(sum_addr + 32 * c, ps);
+            tmem_ld16(sum_addr + 16 * c, ps);
             tmem_wait_ld();
           }
 #pragma unroll
-          for (int e = 0; e < 32; e += 2) {
+          for (int e = 0; e < 16; e += 2) {
             float a0, a1;
             fadd2(a0, a1, p[e], p[e + 1], neg_ref, neg_ref);
             float p0 = ex2_approx(a0), p1 = ex2_approx(a1);
@@ -439,22 +438,22 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             ps[e + 1] = __float_as_uint(p1);
           }
           if (b < Bc - 1) {
-            tmem_st32(sum_addr + 32 * c, ps);
+            tmem_st16(sum_addr + 16 * c, ps);
           } else if (acc_by_tma) {
             // last sample of this key tile: one addition per accumulator entry and launch, performed
-            // in L2 by a TMA reduction of this warp's 32 x 32 block
+            // in L2 by a TMA reduction of this warp's 32 x 16 block
             if (lane == 0) bulk_wait_group_read0();  // the block staged before has been read
             __syncwarp();
 #pragma unroll
-            for (int k = 0; k < 8; ++k)  // 16-byte chunk k of row `lane` goes to position k ^ (lane % 8)
-              *reinterpret_cast<uint4 *>(red_s + lane * 128 + ((k ^ (lane & 7)) << 4)) =
+            for (int k = 0; k < 4; ++k)  // 16-byte chunk k of row `lane` goes to position k ^ (lane / 2 % 4)
+              *reinterpret_cast<uint4 *>(red_s + lane * 64 + ((k ^ ((lane >> 1) & 3)) << 4)) =
                   make_uint4(ps[4 * k], ps[4 * k + 1], ps[4 * k + 2], ps[4 * k + 3]);
             fence_proxy_async_smem();
             __syncwarp();
-            const int x = j0 + 32 * c;
+            const int x = j0 + 16 * c;
             if (kChunked && c == 0) {
-              // this key tile's entries have received the sums of all lower chunks once their eight
-              // warps each have counted themselves in (bounded wait)
+              // this key tile's entries have received the sums of all lower chunks once their
+              // warps have counted themselves in (bounded wait)
               if (lane == 0) {
                 const unsigned *flag = turn + ((size_t)h * n_qt + qt) * n_kt + kt;
                 const unsigned want = (unsigned)chunk * kSoftmaxWarps;
@@ -487,10 +486,10 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           } else if (row_ok) {
             // accumulator rows that are no 16-byte multiples: one red per entry (entries outside the
             // domain are not touched)
-            float *arow = acc + ((size_t)h * Lq + i) * Lk + j0 + 32 * c;
-            const int nv = n_valid - 32 * c;
+            float *arow = acc + ((size_t)h * Lq + i) * Lk + j0 + 16 * c;
+            const int nv = n_valid - 16 * c;
 #pragma unroll
-            for (int g = 0; g < 8; ++g) {
+            for (int g = 0; g < 4; ++g) {
               const int jj = 4 * g;
               if (jj >= nv) break;
               if (vec && jj + 4 <= nv) {
@@ -516,7 +515,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   }
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == 9) tmem_dealloc(tmem, kTmemCols);
+  if (warp == kIssuer) tmem_dealloc(tmem, kTmemCols);
 }
 
 template <int D>
@@ -575,10 +574,10 @@ cudaError_t launch_accumulate_tc(float *acc, const void *Q, const void *K, const
   CUtensorMap mb = mq;
   const int bias_by_tma = (bias && (Lk & 3) == 0) ? 1 : 0;
   if (bias_by_tma && !make_tile_map_f32(&mb, bias, H, Lq, Lk)) return cudaErrorUnknown;
-  // so does the accumulator's update (32-row boxes, one per softmax warp)
+  // so does the accumulator's update (boxes of 32 rows x 16 columns, one softmax warp's half)
   CUtensorMap ma = mq;
   const int acc_by_tma = (Lk & 3) == 0 ? 1 : 0;
-  if (acc_by_tma && !make_tile_map_f32(&ma, acc, H, Lq, Lk, 32)) return cudaErrorUnknown;
+  if (acc_by_tma && !make_tile_map_f32(&ma, acc, H, Lq, Lk, 32, 16)) return cudaErrorUnknown;
   return d == 64
              ? launch<64>(mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, B, H, Lq, Lk, causal, f16, scale, err, s)
              : launch<128>(mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, B, H, Lq, Lk, causal, f16, scale, err, s);
