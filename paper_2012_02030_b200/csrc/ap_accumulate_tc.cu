@@ -123,6 +123,20 @@ unsigned *turn_words() {
   return base[dev] + (size_t)(next.fetch_add(1) % kTurnSets) * kTurnWords;
 }
 
+// Key tiles of a query tile (memory: keys before the segment under a causal mask; -1: no mask).
+__host__ __device__ inline int key_tiles(int qt, int n_kt, int memory) {
+  if (memory < 0) return n_kt;
+  const int n = (qt * kTile + kTile - 1 + memory) / kTile + 1;
+  return n < n_kt ? n : n_kt;
+}
+// Chunks that a query tile's B samples are cut into, for about `visits` visits each: at least kMinChunk samples a chunk,
+// at most kMaxB.
+__host__ __device__ inline int chunks_of(int visits, int n_k, int B) {
+  int per = visits / n_k;
+  per = per < kMinChunk ? kMinChunk : per > kMaxB ? kMaxB : per;
+  return (B + per - 1) / per;
+}
+
 // dbg_skip != 0 (test hook): the copies of the first visit are never issued, so the MMA issuer's
 // first wait runs out and the CTA leaves through its error path.
 // kChunked: the instantiation for launches whose samples are cut into chunks (see below); a
@@ -132,7 +146,7 @@ __global__ void __launch_bounds__(kRegThreads, 1)
 accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_bias, const __grid_constant__ CUtensorMap map_acc,
                      int bias_by_tma, int acc_by_tma, float *__restrict__ acc, const float *__restrict__ bias, int b0,
-                     int Bc_all, int chunk_samples, unsigned *__restrict__ turn, int H, int Lq, int Lk, int n_qt,
+                     int Bc_all, int chunk_visits, unsigned *__restrict__ turn, int H, int Lq, int Lk, int n_qt,
                      int n_kt, int causal, int f16, float scale_log2, unsigned *err, uint32_t max_polls, int dbg_skip) {
   using C = Cfg<D>;
   extern __shared__ unsigned char smem_raw[];
@@ -142,20 +156,30 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   Barriers *bars = reinterpret_cast<Barriers *>(smem + C::kBarOffset);
 
   // Small shapes have fewer (head, query tile) pairs than the GPU has SMs; the launch's samples are
-  // then cut into chunks, CTA (chunk, head, query tile) takes chunk_samples of them, and the chunks'
-  // sums are added to the accumulator in ascending order of the chunks (turn[], see below), so that
+  // then cut into chunks of about chunk_visits (sample, key tile) visits, one CTA per (chunk, head, query tile), and the
+  // chunks' sums are added to the accumulator in ascending order of the chunks (turn[], see below), so that
   // the result does not depend on which CTA finishes first.  Lower chunks have lower block indices.
-  const int unit = kChunked ? (int)blockIdx.x % (H * n_qt) : (int)blockIdx.x;
-  const int chunk = kChunked ? (int)blockIdx.x / (H * n_qt) : 0;
-  if (kChunked) b0 += chunk * chunk_samples;
-  const int Bc = kChunked ? min(chunk_samples, Bc_all - chunk * chunk_samples) : Bc_all;
   // late query tiles (most key tiles under a causal mask) first
-  const int qt = n_qt - 1 - unit / H;
-  const int h = unit % H;
+  int qt = n_qt - 1 - (int)blockIdx.x / H, h = (int)blockIdx.x % H, chunk = 0, Bc = Bc_all;
+  if (kChunked) {
+    int left = (int)blockIdx.x;
+    for (qt = n_qt - 1; qt > 0; --qt) {
+      const int here = H * chunks_of(chunk_visits, key_tiles(qt, n_kt, causal ? Lk - Lq : -1), Bc_all);
+      if (left < here) break;
+      left -= here;
+    }
+    // the samples of a query tile are dealt out evenly over its chunks
+    const int chunks = chunks_of(chunk_visits, key_tiles(qt, n_kt, causal ? Lk - Lq : -1), Bc_all);
+    h = left % H;
+    chunk = left / H;
+    const int first = chunk * Bc_all / chunks;
+    Bc = (chunk + 1) * Bc_all / chunks - first;
+    b0 += first;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // causal: row i looks at keys j <= i + (Lk - Lq), i.e. Lk - Lq memory keys, then its own segment
   const int off = causal ? Lk - Lq : 0;
-  const int n_k = causal ? min(n_kt, (qt * kTile + kTile - 1 + off) / kTile + 1) : n_kt;  // key tiles of this query tile
+  const int n_k = key_tiles(qt, n_kt, causal ? off : -1);
   const int visits_per_sweep = n_k * Bc;
   const int n_visits = 2 * visits_per_sweep;
 
@@ -530,30 +554,33 @@ cudaError_t launch(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorM
   if (e != cudaSuccess) return e;
   const int n_qt = ceil_div(Lq, kTile), n_kt = ceil_div(Lk, kTile);
   const DebugKnobs knobs = debug_knobs();
-  // Shapes with at most half as many (head, query tile) pairs as SMs: several CTAs per pair, each with
-  // a chunk of the samples, taking turns at the accumulator (one wave of CTAs, one per SM).
+  // Shapes with fewer (head, query tile) pairs than SMs: several CTAs per pair, each with a chunk of the samples, taking
+  // turns at the accumulator (one wave of CTAs, one per SM).  The smallest number of visits per chunk is taken for
+  // which they fit, so that the query tiles with many key tiles are cut into more chunks: with the same number for all,
+  // the longest CTA of 16 x 16 heads x 512 (causal) had 64 visits where 35 would be the mean (now 48: 77 -> 64 us).
   const int n_units = H * n_qt, sms = sm_count();
-  int max_chunks = 1;
   unsigned *turn = nullptr;
-  if (acc_by_tma && !knobs.skip_arrive && sms > 0 && 2 * n_units <= sms && (size_t)n_units * n_kt <= kTurnWords) {
+  if (acc_by_tma && !knobs.skip_arrive && n_units < sms && B >= 2 * kMinChunk && (size_t)n_units * n_kt <= kTurnWords)
     turn = turn_words();
-    if (turn) max_chunks = sms / n_units;
-  }
-  // samples in ascending order, at most kMaxB per CTA and launch; launches on one stream run in order
+  // samples in ascending order, at most kMaxB per CTA; launches on one stream run in order
   for (int b0 = 0; b0 < B;) {
-    const int left = B - b0;
-    int chunks = 1, per = left < kMaxB ? left : kMaxB;
-    if (max_chunks > 1 && left >= 2 * kMinChunk) {
-      chunks = left / kMinChunk < max_chunks ? left / kMinChunk : max_chunks;
-      per = ceil_div(left, chunks);
-      if (per > kMaxB) per = kMaxB;
-      chunks = ceil_div(left < chunks * per ? left : chunks * per, per);
+    int Bc = B - b0 < kMaxB ? B - b0 : kMaxB, visits = 0, grid = n_units;
+    if (turn) {
+      const int all = B - b0, memory = causal ? Lk - Lq : -1;
+      int total = 0;
+      for (int qt = 0; qt < n_qt; ++qt) total += H * key_tiles(qt, n_kt, memory) * all;
+      for (visits = (total + sms - 1) / sms;; visits += 1 + visits / 16) {
+        grid = 0;
+        for (int qt = 0; qt < n_qt; ++qt) grid += H * chunks_of(visits, key_tiles(qt, n_kt, memory), all);
+        if (grid <= sms || visits >= kMaxB * n_kt) break;
+      }
+      if (grid <= sms && grid > n_units) Bc = all;  // all the samples in one launch
+      else visits = 0, grid = n_units;
     }
-    const int Bc = left < chunks * per ? left : chunks * per;
-    unsigned *t = chunks > 1 ? turn : nullptr;
+    unsigned *t = visits ? turn : nullptr;
     if (t && (e = cudaMemsetAsync(t, 0, (size_t)n_units * n_kt * sizeof(unsigned), s)) != cudaSuccess) return e;
-    (t ? kern_chunked : kern)<<<knobs.skip_arrive ? 1 : n_units * chunks, kThreads, Cfg<D>::kSmemBytes, s>>>(
-        mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, b0, Bc, per, t, H, Lq, Lk, n_qt, n_kt, causal, f16,
+    (t ? kern_chunked : kern)<<<knobs.skip_arrive ? 1 : grid, kThreads, Cfg<D>::kSmemBytes, s>>>(
+        mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, b0, Bc, visits, t, H, Lq, Lk, n_qt, n_kt, causal, f16,
         scale * kLog2e, err, knobs.max_polls, knobs.skip_arrive);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
