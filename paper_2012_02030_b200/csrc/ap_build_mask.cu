@@ -89,6 +89,25 @@ __host__ __device__ inline long long cand_capacity(long long n_rest) {
   return n_rest >= kShortcutMinEntries ? n_rest / 16 : 0;
 }
 
+// 16 consecutive floats, from a 32-byte boundary (kVec = 8: two loads of a whole sector per lane) or a 16-byte one.
+template <int kVec>
+__device__ __forceinline__ void ldg_f16(const float *p, float v[16]) {
+  static_assert(kVec == 8 || kVec == 4, "floats per load");
+#pragma unroll
+  for (int e = 0; e < 16; e += kVec) {
+    if (kVec == 8) {
+      asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                   : "=f"(v[e]), "=f"(v[e + 1]), "=f"(v[e + 2]), "=f"(v[e + 3]), "=f"(v[e + 4]), "=f"(v[e + 5]),
+                     "=f"(v[e + 6]), "=f"(v[e + 7])
+                   : "l"(p + e));
+    } else {
+      asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(v[e]), "=f"(v[e + 1]), "=f"(v[e + 2]), "=f"(v[e + 3])
+                   : "l"(p + e));
+    }
+  }
+}
+
 __host__ __device__ inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 // Loads 4 consecutive entries of a row starting at column j0 (j0 % 4 == 0).
@@ -338,7 +357,8 @@ constexpr int kSelCtasPerSm = 2;
 
 // fn(value, linear index, whether the lane's entry is one of the selection's) for the selection's entries, spread over
 // `n_warps` warps of which this is the `warp`-th: four 128-column pieces of rows at a time, a lane four consecutive
-// entries of each.  Called by whole warps, fn by all lanes together.
+// entries of each (also where rows start anywhere: neighbouring entries often fall into the same bin, and a warp that
+// counts 32 neighbours at once, although its loads are contiguous then, is 5 us slower at 16 heads x 375 x 759).  Called by whole warps, fn by all lanes together.
 template <class F>
 __device__ __forceinline__ void scan_domain(const float *__restrict__ base, int rows, int Lk, int period, int causal,
                                             int diag, uint32_t warp, uint32_t n_warps, int lane, F fn) {
@@ -356,7 +376,15 @@ __device__ __forceinline__ void scan_domain(const float *__restrict__ base, int 
       own[u] = i % period + off;
       jend[u] = i >= rows ? 0 : causal ? min(Lk, own[u] + 1) : Lk;
       v[u][0] = v[u][1] = v[u][2] = v[u][3] = 0.f;
-      if (col[u] < jend[u]) load4(base + (size_t)i * Lk, col[u], jend[u], vec, v[u]);
+      const float *from = base + (size_t)i * Lk + col[u];
+      if (vec && col[u] + 4 <= jend[u]) {
+        const float4 t = *reinterpret_cast<const float4 *>(from);
+        v[u][0] = t.x, v[u][1] = t.y, v[u][2] = t.z, v[u][3] = t.w;
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (col[u] + c < jend[u]) v[u][c] = from[c];
+      }
       if (++kt == n_kt) {
         kt = 0;
         ++i;
@@ -539,37 +567,31 @@ select_kernel(const float *__restrict__ acc, int rows, int Lk, int period, int c
   }
 }
 
-// A warp's way into a selection's buffer of collected entries: staged in shared memory and appended
-// with one reservation per flush (an entry that finds the stage full goes straight to the buffer).
+// A warp's way into a selection's buffer of collected entries: staged in shared memory and appended with one reservation
+// per flush.  By the whole warp; the number staged is the same in all lanes.
 struct Collector {
-  uint2 *stage;        // this warp's kWarpStage entries of shared memory
-  uint32_t *stage_n;   // entries pushed since the last flush (may run past the stage)
-  uint2 *out;          // the selection's buffer
-  uint32_t *n_cand;    // entries reserved in it so far (may exceed the capacity: then the shortcut fails)
+  uint2 *stage;      // this warp's kWarpStage entries of shared memory
+  uint32_t staged;
+  uint2 *out;        // the selection's buffer
+  uint32_t *n_cand;  // entries reserved in it so far (may exceed the capacity: then the shortcut fails)
   uint32_t cap;
-  __device__ __forceinline__ void push(float f, uint32_t index) {
-    const uint2 entry = make_uint2(key_of(f), index);
-    const uint32_t pos = atomicAdd(stage_n, 1u);
-    if (pos < (uint32_t)kWarpStage) {
-      stage[pos] = entry;
-    } else {
-      const uint32_t g = atomicAdd(n_cand, 1u);
-      if (g < cap) out[g] = entry;
-    }
+  // the lane's entries go to stage[at ...]; `total` <= kWarpStage is the warp's number of them
+  __device__ __forceinline__ uint32_t reserve(uint32_t before_me, uint32_t total, int lane) {
+    if (staged + total > (uint32_t)kWarpStage) flush(lane);
+    const uint32_t at = staged + before_me;
+    staged += total;
+    return at;
   }
-  __device__ __forceinline__ void flush(uint32_t at_least, int lane) {  // by the whole warp
+  __device__ __forceinline__ void flush(int lane) {
+    if (staged == 0u) return;
     __syncwarp();
-    const uint32_t n = min(*stage_n, (uint32_t)kWarpStage);
-    if (n >= at_least && n > 0u) {
-      uint32_t dst = 0u;
-      if (lane == 0) dst = atomicAdd(n_cand, n);
-      dst = __shfl_sync(0xffffffffu, dst, 0);
-      for (uint32_t e = lane; e < n; e += 32)
-        if (dst + e < cap) out[dst + e] = stage[e];
-      __syncwarp();
-      if (lane == 0) *stage_n = 0u;
-      __syncwarp();
-    }
+    uint32_t dst = 0u;
+    if (lane == 0) dst = atomicAdd(n_cand, staged);
+    dst = __shfl_sync(0xffffffffu, dst, 0);
+    for (uint32_t e = lane; e < staged; e += 32)
+      if (dst + e < cap) out[dst + e] = stage[e];
+    __syncwarp();
+    staged = 0u;
   }
 };
 
@@ -581,117 +603,180 @@ struct EmitSel {
   uint32_t first_row;  // of this head in the tie order
 };
 
-// The rows of one tile, kCtaWarps warps; returns this lane's share of the tile's popcount (lanes 0, 8, 16, 24) and adds
-// the bitmap words it has written to `any` (same lanes).
-// kInterior: every row and column of the tile exists and lies in the domain and none is forced,
-// so nothing is checked per entry.
-// kClassify: the classifying pass of the one-pass shortcut instead of the emit pass proper.  Entries
-// above the bracket are kept, entries inside it are collected (col) and left out for the select
-// to decide, entries above the bracket are counted (above).
-template <bool kInterior, bool kClassify, int kCtaWarps>
-__device__ __forceinline__ int emit_tile_rows(const float *__restrict__ acc, int Lq, int Lk, int h, int qt, int kt,
-                                              int tile, int causal, int diag, const EmitSel &sel,
-                                              uint8_t *__restrict__ mask, uint32_t *__restrict__ stage_bitmap,
-                                              Collector &col, uint32_t &above, uint32_t &any) {
+// The two ways over the rows of one tile, each by kCtaWarps warps.  Both write the mask and the bitmap and return what
+// the lane has seen: `count` kept entries (to be added up over the lanes), `groups` of 16 columns with a kept entry (to be
+// combined), `above` entries above the bracket (kClassify; to be added up).
+// kClassify: the classifying pass of the one-pass shortcut instead of the emit pass proper.  Entries above the bracket are
+// kept, entries inside it are collected (col) and left out for the select to decide, entries above the bracket are counted.
+//
+// What bounds them: instructions, not memory.  With four columns per lane (a test of each, three shuffles to a bitmap word
+// and a four-byte mask store per row) the classifying pass issued 121 instructions per row of a tile and reached 2.6 TB/s.
+struct TileSums {
+  int count;
+  uint32_t groups, above;
+};
+
+// Tiles all of whose rows and columns exist, lie in the domain and are not forced.  kVec = 8: in arrays whose rows start on
+// 32-byte (scores) and 16-byte (mask) boundaries; 4: on 16-byte and 4-byte ones.  A lane takes 16 consecutive columns of one row, i.e. one group of the
+// tile: its bits are half a bitmap word, its mask bytes one 16-byte store, and where all 16 lie below the bracket (most of
+// them do: it sits near the top of the values) one comparison of their maximum says so.  A warp has four rows under way and
+// the next four loaded ahead.
+template <bool kClassify, int kCtaWarps, int kVec>
+__device__ __forceinline__ void emit_rows_by_group(const float *__restrict__ acc, int Lq, int Lk, int h, int qt, int kt,
+                                                   int tile, const EmitSel &sel, uint8_t *__restrict__ mask,
+                                                   uint32_t *__restrict__ stage_bitmap, Collector &col, TileSums &sums) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool vec = (Lk & 3) == 0;
-  const int j0 = kt * kTile + 4 * lane;
+  const int j0 = kt * kTile + 16 * (lane & 7), r_lane = lane >> 3;
   const float thr_f = sel.thr_f;
-  // the lowest value that needs a closer look: the threshold, or the bracket's lower pivot
+  const float floor_f = kClassify ? sel.lo_f : thr_f;  // the lowest value that needs a closer look
+  const int r_first = 4 * warp + r_lane;
+  size_t at = ((size_t)h * Lq + qt * kTile + r_first) * Lk + j0;
+  const size_t step = (size_t)(4 * kCtaWarps) * Lk;
+  float v[16], ahead[16];
+  ldg_f16<kVec>(acc + at, ahead);
+  uint32_t first = (sel.first_row + (uint32_t)(qt * kTile + r_first)) * (uint32_t)Lk + (uint32_t)j0;
+  size_t bits_at = (size_t)tile * (2 * kBitmapWords) + 8 * r_first + (lane & 7);  // in half-words
+#pragma unroll 1
+  for (int r0 = 4 * warp; r0 < kTile; r0 += 4 * kCtaWarps) {
+#pragma unroll
+    for (int c = 0; c < 16; ++c) v[c] = ahead[c];
+    if (r0 + 4 * kCtaWarps < kTile) ldg_f16<kVec>(acc + at + step, ahead);
+    uint32_t kept = 0u, ties = 0u;
+    // (written so that a value that is not a number gets the closer look as well)
+    bool below = true;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) below = below && v[c] < floor_f;
+    if (!below) {
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        const bool gt = v[c] > thr_f;
+        kept |= (gt ? 1u : 0u) << c;
+        ties |= ((kClassify ? !(v[c] < floor_f) && !gt : v[c] == thr_f) ? 1u : 0u) << c;
+      }
+      if (kClassify) {
+        sums.above += (uint32_t)__popc(kept);
+      } else if (ties && first <= sel.tie_cut) {  // entries equal to the threshold, up to the last kept one
+        const uint32_t last = sel.tie_cut - first;
+        kept |= last >= 15u ? ties : ties & ((2u << last) - 1u);
+      }
+    }
+    if (kClassify && __any_sync(0xffffffffu, ties != 0u)) {
+      const uint32_t mine = (uint32_t)__popc(ties);
+      uint32_t incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      uint32_t pos = col.reserve(incl - mine, __shfl_sync(0xffffffffu, incl, 31), lane);
+#pragma unroll
+      for (int c = 0; c < 16; ++c)
+        if ((ties >> c) & 1u) col.stage[pos++] = make_uint2(key_of(v[c]), first + c);
+    }
+    if (mask) {
+      uint4 bytes;  // four bits to four bytes: the products of the shifted copies do not meet
+      bytes.x = ((kept & 15u) * 0x00204081u) & 0x01010101u;
+      bytes.y = (((kept >> 4) & 15u) * 0x00204081u) & 0x01010101u;
+      bytes.z = (((kept >> 8) & 15u) * 0x00204081u) & 0x01010101u;
+      bytes.w = ((kept >> 12) * 0x00204081u) & 0x01010101u;
+      if (kVec == 8) {
+        *reinterpret_cast<uint4 *>(mask + at) = bytes;
+      } else {
+        uint32_t *words = reinterpret_cast<uint32_t *>(mask + at);
+        words[0] = bytes.x, words[1] = bytes.y, words[2] = bytes.z, words[3] = bytes.w;
+      }
+    }
+    if (stage_bitmap) reinterpret_cast<uint16_t *>(stage_bitmap)[bits_at] = (uint16_t)kept;
+    sums.count += __popc(kept);
+    sums.groups |= kept ? 1u << (lane & 7) : 0u;
+    at += step;
+    first += (uint32_t)(4 * kCtaWarps) * (uint32_t)Lk;
+    bits_at += 8 * 4 * kCtaWarps;
+  }
+}
+
+// Every other tile: a lane takes the columns lane, lane + 32, ... of a row, so that loads and mask stores of a warp are
+// contiguous wherever the row starts, and a vote of the warp is a bitmap word.  Four rows loaded ahead.
+// kInterior: as for emit_rows_by_group (rows that start anywhere), nothing is checked per entry and a row all of whose
+// entries lie below the bracket takes one vote.
+template <bool kClassify, int kCtaWarps, bool kInterior>
+__device__ __forceinline__ void emit_rows_by_column(const float *__restrict__ acc, int Lq, int Lk, int h, int qt, int kt,
+                                                    int tile, int causal, int diag, const EmitSel &sel,
+                                                    uint8_t *__restrict__ mask, uint32_t *__restrict__ stage_bitmap,
+                                                    Collector &col, TileSums &sums) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float thr_f = sel.thr_f;
   const float floor_f = kClassify ? sel.lo_f : thr_f;
   const int off = (causal || diag) ? Lk - Lq : 0;  // row i's own position is key i + off
-  int count = 0;
-  for (int r0 = warp; r0 < kTile; r0 += 4 * kCtaWarps) {
+  const int j_lane = kt * kTile + lane;
+  const int rows = kInterior ? kTile : min(kTile, Lq - qt * kTile);
+  int count = 0;  // the same in all lanes
+  uint32_t any[4] = {0u, 0u, 0u, 0u};
+#pragma unroll 1
+  for (int r0 = warp; r0 < rows; r0 += 4 * kCtaWarps) {
     float v[4][4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {  // four loads in flight
+    for (int u = 0; u < 4; ++u) {
       const int i = qt * kTile + r0 + kCtaWarps * u;
-      if (kInterior) {
-        const float4 t = *reinterpret_cast<const float4 *>(acc + ((size_t)h * Lq + i) * Lk + j0);
-        v[u][0] = t.x; v[u][1] = t.y; v[u][2] = t.z; v[u][3] = t.w;
-      } else {
-        v[u][0] = v[u][1] = v[u][2] = v[u][3] = 0.f;
-        if (i < Lq) {
-          const int jend = causal ? min(Lk, i + 1 + off) : Lk;
-          if (j0 < jend) load4(acc + ((size_t)h * Lq + i) * Lk, j0, jend, vec, v[u]);
-        }
-      }
+      const int jend = i >= Lq ? 0 : causal ? min(Lk, i + 1 + off) : Lk;
+      const float *row = acc + ((size_t)h * Lq + i) * Lk + j_lane;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[u][q] = kInterior || j_lane + 32 * q < jend ? row[32 * q] : 0.f;
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int r = r0 + kCtaWarps * u;
-      const int i = qt * kTile + r;
-      uint32_t nib = 0u;
-      bool close = false;  // some lane of the warp has an entry that needs a closer look
-      if (kInterior) {
-        // (most pieces of a row lie wholly below: one test for the warp, and zeros are written)
-        close = __any_sync(0xffffffffu, !(v[u][0] < floor_f && v[u][1] < floor_f && v[u][2] < floor_f && v[u][3] < floor_f));
-      } else {
-        close = i < Lq;
-      }
-      if (close) {  // warp-uniform
-        uint32_t tie_bits = 0u, gt_bits = 0u, forced_bits = 0u;
-        const int jend = kInterior ? j0 + 4 : causal ? min(Lk, i + 1 + off) : Lk;
+      const int r = r0 + kCtaWarps * u, i = qt * kTile + r;
+      if (r >= rows) break;
+      uint32_t w[4] = {0u, 0u, 0u, 0u};
+      if (!kInterior ||
+          __any_sync(0xffffffffu, !(v[u][0] < floor_f && v[u][1] < floor_f && v[u][2] < floor_f && v[u][3] < floor_f))) {
+        const int jend = causal ? min(Lk, i + 1 + off) : Lk;
+        const int own = diag ? i + off : -1;
+        const uint32_t first = (sel.first_row + (uint32_t)i) * (uint32_t)Lk + (uint32_t)j_lane;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int j = j0 + c;
-          if (kInterior || j < jend) {
-            if (!kInterior && diag && j == i + off) {
-              forced_bits |= 1u << c;
-            } else {
-              gt_bits |= (v[u][c] > thr_f ? 1u : 0u) << c;
-              tie_bits |= ((kClassify ? !(v[u][c] < floor_f) && !(v[u][c] > thr_f) : v[u][c] == thr_f) ? 1u : 0u) << c;
+        for (int q = 0; q < 4; ++q) {
+          const int j = j_lane + 32 * q;
+          const bool forced = !kInterior && j == own;
+          const bool in = kInterior || (j < jend && !forced);
+          const bool gt = in && v[u][q] > thr_f;
+          bool keep = gt || forced;
+          if (kClassify) {
+            const bool tie = in && !gt && !(v[u][q] < floor_f);
+            sums.above += gt ? 1u : 0u;
+            const uint32_t inside = __ballot_sync(0xffffffffu, tie);
+            if (inside) {
+              const uint32_t pos = col.reserve(__popc(inside & ((1u << lane) - 1u)), (uint32_t)__popc(inside), lane);
+              if (tie) col.stage[pos] = make_uint2(key_of(v[u][q]), first + 32u * q);
             }
+          } else {
+            keep = keep || (in && v[u][q] == thr_f && first + 32u * q <= sel.tie_cut);
           }
+          w[q] = __ballot_sync(0xffffffffu, keep);
+          count += __popc(w[q]);
+          any[q] |= w[q];
         }
-        nib = gt_bits | forced_bits;
-        if (kClassify) above += (uint32_t)__popc(gt_bits);
-        if (tie_bits) {
-          const uint32_t first = (sel.first_row + (uint32_t)i) * (uint32_t)Lk + (uint32_t)j0;
+      }
+      if (mask) {
+        uint8_t *mrow = mask + ((size_t)h * Lq + i) * Lk + j_lane;
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-            if (tie_bits & (1u << c)) {
-              if (kClassify)
-                col.push(v[u][c], first + c);
-              else if (first + c <= sel.tie_cut)
-                nib |= 1u << c;
-            }
-        }
+        for (int q = 0; q < 4; ++q)
+          if (kInterior || j_lane + 32 * q < Lk) mrow[32 * q] = (w[q] >> lane) & 1u;
       }
-      if ((kInterior || i < Lq) && mask) {
-        uint8_t *mrow = mask + ((size_t)h * Lq + i) * Lk;
-        if (kInterior || (vec && j0 + 4 <= Lk)) {
-          *reinterpret_cast<uchar4 *>(mrow + j0) =
-              make_uchar4(nib & 1u, (nib >> 1) & 1u, (nib >> 2) & 1u, (nib >> 3) & 1u);
-        } else {
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            if (j0 + c < Lk) mrow[j0 + c] = (nib >> c) & 1u;
-        }
-      }
-      uint32_t w = 0u;
-      if (close) {
-        // 8 lanes x 4 bits -> one bitmap word, complete in the first lane of each group of eight
-        w = nib << (4 * (lane & 7));
-        w |= __shfl_xor_sync(0xffffffffu, w, 1);
-        w |= __shfl_xor_sync(0xffffffffu, w, 2);
-        w |= __shfl_xor_sync(0xffffffffu, w, 4);
-      }
-      if ((lane & 7) == 0) {
-        count += __popc(w);
-        any |= w;
-        if (stage_bitmap) stage_bitmap[(size_t)tile * kBitmapWords + 4 * r + (lane >> 3)] = w;
-      }
+      if (stage_bitmap && lane == 0)
+        *reinterpret_cast<uint4 *>(stage_bitmap + (size_t)tile * kBitmapWords + 4 * r) = make_uint4(w[0], w[1], w[2], w[3]);
     }
-    if (kClassify) col.flush(kWarpStage / 2, lane);
   }
-  if (kClassify) col.flush(1u, lane);
-  return count;
+  if (!kInterior && stage_bitmap)  // rows beyond the last query keep nothing
+    for (int x = rows + (int)threadIdx.x; x < kTile; x += 32 * kCtaWarps)
+      *reinterpret_cast<uint4 *>(stage_bitmap + (size_t)tile * kBitmapWords + 4 * x) = make_uint4(0u, 0u, 0u, 0u);
+  if (lane == 0) {
+    sums.count += count;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sums.groups |= ((any[q] & 0xffffu ? 1u : 0u) | (any[q] >> 16 ? 2u : 0u)) << (2 * q);
+  }
 }
 
-// A CTA per tile of the (h, qt, kt) grid (a CTA takes several in turn where the grid is smaller); warp w takes tile rows
-// w, w + kCtaWarps, ... (four rows loaded ahead) and each lane four consecutive columns.  Writes the
-// element mask, the tile's bitmap, popcount and group summary into the staging area.  Values are
+// A CTA per tile of the (h, qt, kt) grid (a CTA takes several in turn where the grid is smaller).  Writes the element mask, the tile's bitmap, popcount and group summary into the staging area.  Values are
 // compared with the threshold as floats (the same order as their keys).  per_layer:
 // all heads share selection 0, ties are ordered by (h*Lq + i)*Lk + j, and the
 // tiles' popcounts are added up into nnz[h].  keep_ties: every entry equal to the threshold is
@@ -702,7 +787,7 @@ __device__ __forceinline__ int emit_tile_rows(const float *__restrict__ acc, int
 // left out, and the select adds the collected entries that turn out to be kept.  Only for exact
 // per-head selections (the kept count is known beforehand, nothing is counted here).
 template <bool kClassify, int kCtaWarps>
-__global__ void __launch_bounds__(32 * kCtaWarps) emit_kernel(const float *__restrict__ acc, int Lq, int Lk, int n_qt,
+__global__ void __launch_bounds__(32 * kCtaWarps, kCtaWarps == 4 ? 8 : 2) emit_kernel(const float *__restrict__ acc, int Lq, int Lk, int n_qt,
                                                               int n_kt, int n_tiles, int causal, int diag, int per_layer,
                                                               int keep_ties, SelectState *state,
                                                               uint8_t *__restrict__ mask,
@@ -714,8 +799,10 @@ __global__ void __launch_bounds__(32 * kCtaWarps) emit_kernel(const float *__res
   __shared__ int warp_count[kCtaWarps];
   __shared__ uint32_t warp_groups[kCtaWarps];
   __shared__ uint2 stage_all[kClassify ? kCtaWarps : 1][kClassify ? kWarpStage : 1];
-  __shared__ uint32_t stage_n_all[kCtaWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // rows of the scores start on 32-byte boundaries and rows of the mask on 16-byte ones
+  const bool aligned4 = (Lk & 3) == 0 && ((reinterpret_cast<uintptr_t>(acc) & 15) | (reinterpret_cast<uintptr_t>(mask) & 3)) == 0;
+  const bool aligned = (Lk & 15) == 0 && ((reinterpret_cast<uintptr_t>(acc) & 31) | (reinterpret_cast<uintptr_t>(mask) & 15)) == 0;
   for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     const int kt = tile % n_kt;
     const int qt = (tile / n_kt) % n_qt;
@@ -726,18 +813,17 @@ __global__ void __launch_bounds__(32 * kCtaWarps) emit_kernel(const float *__res
     const int own_lo = qt * kTile + ((causal || diag) ? Lk - Lq : 0), own_hi = own_lo + kTile - 1;
     if (causal && kt * kTile > own_hi) {
       // the whole tile lies above the diagonal: nothing is kept, nothing needs to be read
-      const bool vec = (Lk & 3) == 0;
-      const int j0 = kt * kTile + 4 * lane;
-      for (int r = warp; r < kTile; r += kCtaWarps) {
-        const int i = qt * kTile + r;
-        if (i < Lq && mask) {
-          uint8_t *mrow = mask + ((size_t)h * Lq + i) * Lk;
-          if (vec && j0 + 4 <= Lk) {
-            *reinterpret_cast<uchar4 *>(mrow + j0) = make_uchar4(0, 0, 0, 0);
-          } else {
-            for (int c = 0; c < 4; ++c)
-              if (j0 + c < Lk) mrow[j0 + c] = 0;
-          }
+      if (mask && aligned) {
+        const int j0 = kt * kTile + 16 * (lane & 7);
+        for (int r = 4 * warp + (lane >> 3); r < kTile; r += 4 * kCtaWarps) {
+          const int i = qt * kTile + r;
+          if (i < Lq && j0 < Lk) *reinterpret_cast<uint4 *>(mask + ((size_t)h * Lq + i) * Lk + j0) = make_uint4(0u, 0u, 0u, 0u);
+        }
+      } else if (mask) {
+        for (int r = warp; r < kTile; r += kCtaWarps) {
+          const int i = qt * kTile + r;
+          if (i >= Lq) break;
+          for (int j = kt * kTile + lane; j < min(Lk, (kt + 1) * kTile); j += 32) mask[((size_t)h * Lq + i) * Lk + j] = 0;
         }
       }
       // (the bitmap of an empty tile is not read)
@@ -754,29 +840,33 @@ __global__ void __launch_bounds__(32 * kCtaWarps) emit_kernel(const float *__res
     sel.first_row = per_layer ? (uint32_t)h * (uint32_t)Lq : 0u;
     Collector col;
     col.stage = stage_all[kClassify ? warp : 0];
-    col.stage_n = &stage_n_all[warp];
+    col.staged = 0u;
     col.out = cand + (size_t)(per_layer ? 0 : h) * cand_cap;
     col.n_cand = &st.n_cand;
     col.cap = cand_cap;
-    if (kClassify && lane == 0) stage_n_all[warp] = 0u;
-    __syncwarp();
-    uint32_t above = 0u, any = 0u;
+    TileSums sums = {0, 0u, 0u};
     const bool below = !causal || kt * kTile + kTile - 1 <= own_lo;  // every column in every row's domain
     const bool has_diag = diag && own_lo <= kt * kTile + kTile - 1 && own_hi >= kt * kTile;
-    const bool interior = (qt + 1) * kTile <= Lq && (kt + 1) * kTile <= Lk && (Lk & 3) == 0 && below && !has_diag;
-    int count = interior ? emit_tile_rows<true, kClassify, kCtaWarps>(acc, Lq, Lk, h, qt, kt, tile, causal, diag, sel,
-                                                                      mask, stage_bitmap, col, above, any)
-                         : emit_tile_rows<false, kClassify, kCtaWarps>(acc, Lq, Lk, h, qt, kt, tile, causal, diag, sel,
-                                                                       mask, stage_bitmap, col, above, any);
+    if ((qt + 1) * kTile <= Lq && (kt + 1) * kTile <= Lk && below && !has_diag) {
+      if (aligned)
+        emit_rows_by_group<kClassify, kCtaWarps, 8>(acc, Lq, Lk, h, qt, kt, tile, sel, mask, stage_bitmap, col, sums);
+      else if (aligned4)
+        emit_rows_by_group<kClassify, kCtaWarps, 4>(acc, Lq, Lk, h, qt, kt, tile, sel, mask, stage_bitmap, col, sums);
+      else
+        emit_rows_by_column<kClassify, kCtaWarps, true>(acc, Lq, Lk, h, qt, kt, tile, causal, diag, sel, mask, stage_bitmap,
+                                                        col, sums);
+    } else {
+      emit_rows_by_column<kClassify, kCtaWarps, false>(acc, Lq, Lk, h, qt, kt, tile, causal, diag, sel, mask, stage_bitmap,
+                                                       col, sums);
+    }
     if (kClassify) {
-      above = __reduce_add_sync(0xffffffffu, above);
+      col.flush(lane);
+      const uint32_t above = __reduce_add_sync(0xffffffffu, sums.above);
       if (lane == 0 && above) atomicAdd(&st.above_hi, (unsigned long long)above);
     }
     if (!stage_bitmap && !(nnz && !kClassify && (per_layer || keep_ties))) continue;
-    count = __reduce_add_sync(0xffffffffu, count);
-    // groups 2q and 2q + 1 of the tile are the halves of word q, which lane 8q has seen
-    const uint32_t bits = ((any & 0xffffu) ? 1u : 0u) | ((any >> 16) ? 2u : 0u);
-    const uint32_t groups = __reduce_or_sync(0xffffffffu, (lane & 7) == 0 ? bits << (2 * (lane >> 3)) : 0u);
+    const int count = __reduce_add_sync(0xffffffffu, sums.count);
+    const uint32_t groups = __reduce_or_sync(0xffffffffu, sums.groups);
     if (lane == 0) {
       warp_count[warp] = count;
       warp_groups[warp] = groups;
