@@ -24,12 +24,16 @@
 // One threshold for the whole layer (Eq. 2 as stated) is the same selection run
 // once over a virtual head of H*Lq rows: row i' = h*Lq + i has the domain of row
 // i, and the linear index i'*Lk + j is the layer-wide tie order.
+#include <cooperative_groups.h>
+
 #include "ap_common.cuh"
 #include "ap_grid.cuh"
 
 namespace ap {
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int kThreads = 256;  // collect_kernel
 constexpr int kWarps = kThreads / 32;
@@ -85,6 +89,7 @@ constexpr long long kShortcutMinEntries = 1ll << 20;
 constexpr long long kDirectEntries = 12ll << 20;
 constexpr int kSamples = 16384;  // draws per selection; those of forced entries are dropped (with memory keys, those outside
                                  // the domain too)
+constexpr int kSampleCtas = 8;   // CTAs (one cluster) that make them
 __host__ __device__ inline long long cand_capacity(long long n_rest) {
   return n_rest >= kShortcutMinEntries ? n_rest / 16 : 0;
 }
@@ -129,15 +134,15 @@ __device__ __forceinline__ void load4(const float *__restrict__ row, int j0, int
 
 // ---- the one-pass shortcut ------------------------------------------------------------------
 
-__device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
-  x += 0x9e3779b97f4a7c15ull;
-  x = (x ^ (x >> 30)) * 0xbf58476d1ce4e5b9ull;
-  x = (x ^ (x >> 27)) * 0x94d049bb133111ebull;
-  return x ^ (x >> 31);
+// A bijection of 32-bit words all of whose output bits depend on all input bits (the finaliser of MurmurHash3).
+__device__ __forceinline__ uint32_t mix32(uint32_t x) {
+  x = (x ^ (x >> 16)) * 0x85ebca6bu;
+  x = (x ^ (x >> 13)) * 0xc2b2ae35u;
+  return x ^ (x >> 16);
 }
 
-// CTA-wide (1024 threads): the leading 22 bits of the key of rank `rank` (1 = largest) among keys[0..n),
-// 1 <= rank <= n.  hist: kBins words of shared memory; xch: 2 words.
+// CTA-wide (1024 threads): the leading 22 bits of the key of rank `rank` (1 = largest) among keys[0..n) that are not 0,
+// at least `rank` of them.  hist: kBins words of shared memory; xch: 2 words.
 __device__ uint32_t block_select22(const uint32_t *keys, uint32_t n, uint32_t rank, uint32_t *hist, uint32_t *xch) {
   __shared__ uint32_t warp_sums[32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -153,7 +158,7 @@ __device__ uint32_t block_select22(const uint32_t *keys, uint32_t n, uint32_t ra
       for (int u = 0; u < 8; ++u) kk[u] = idx0 + u * 1024 < n ? keys[idx0 + u * 1024] : 0u;
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (idx0 + u * 1024 < n && (kk[u] & above_digit(pass)) == prefix)
+        if (kk[u] != 0u && (kk[u] & above_digit(pass)) == prefix)
           atomicAdd(&hist[(kk[u] >> shift) & digit_mask(pass)], 1u);
     }
     __syncthreads();
@@ -183,33 +188,38 @@ __device__ uint32_t block_select22(const uint32_t *keys, uint32_t n, uint32_t ra
   return prefix;
 }
 
-// Two CTAs per selection (blockIdx.y = 0: upper pivot, 1: lower pivot), each of which samples the
-// selection's entries (the same draws) and sets its end of the bracket [lo, hi] around the
-// expected threshold (rounded outwards to 22 bits: a third digit would not narrow it noticeably).
-__global__ void __launch_bounds__(1024) sample_pivots_kernel(const float *__restrict__ acc, int rows, int Lk, int period,
-                                                             int causal, int diag, unsigned long long k_rest,
-                                                             unsigned long long n_rest, SelectState *state) {
+// A cluster of CTAs per selection samples its entries and sets the bracket [lo, hi] around the expected threshold (rounded
+// outwards to 22 bits: a third digit would not narrow it noticeably).  The draws of all CTAs go to the shared memory of the
+// first two, which pick the upper and the lower pivot.
+//
+// What bounds it: the draws, each a sector of its own from somewhere in the selection, of which an SM has only so many under
+// way, and then the histograms (most keys fall into a few bins).  A pair of CTAs that made all draws, in no order: 28 us for 16
+// heads x 2048, 14 of them the draws; 16 x 4096 as a whole 265 us, 259 with a cluster.  32768 draws: 263.
+__global__ void __cluster_dims__(kSampleCtas, 1, 1) __launch_bounds__(1024)
+sample_pivots_kernel(const float *__restrict__ acc, int rows, int Lk, int period, int causal, int diag,
+                     unsigned long long k_rest, unsigned long long n_rest, SelectState *state) {
   extern __shared__ uint32_t sm_dyn[];
-  uint32_t *keys = sm_dyn;               // kSamples
+  uint32_t *keys = sm_dyn;               // kSamples; 0 where a draw was dropped
   uint32_t *hist = sm_dyn + kSamples;    // kBins
   __shared__ uint32_t xch[2];
   __shared__ uint32_t n_valid_s;
-  const int h = blockIdx.x, t = threadIdx.x, lane = t & 31;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int h = blockIdx.x / kSampleCtas, part = blockIdx.x % kSampleCtas, t = threadIdx.x, lane = t & 31;
   if (t == 0) n_valid_s = 0u;
-  __syncthreads();
   const int off = (causal || diag) ? Lk - period : 0;
-  constexpr int kDraws = kSamples / 1024;  // per thread, all loads in flight at once
+  constexpr int kDraws = kSamples / (1024 * kSampleCtas);  // per thread, all loads in flight at once
   float drawn[kDraws];
   bool valid[kDraws];
 #pragma unroll
   for (int u = 0; u < kDraws; ++u) {
-    const int s = t + 1024 * u;
-    // row and column from the two halves of one 64-bit draw, scaled by multiplication (64-bit
-    // divisions, emulated in dozens of instructions each, made up most of this kernel's time)
-    const unsigned long long m = mix64(((unsigned long long)h << 32) | (unsigned)s);
-    int i = (int)(((m >> 32) * (unsigned long long)rows) >> 32);
-    int j = (int)(((m & 0xffffffffull) * (unsigned long long)Lk) >> 32);
-    int r = i % period;
+    const int s = t + 1024 * (u + kDraws * part);
+    // The rows are drawn in order (draw s from the s-th part of the selection's rows), which narrows the sample's spread if
+    // anything and lets a warp's draws share a page; the column is a hash of the draw's number, scaled by multiplication.
+    const uint32_t m = mix32((uint32_t)s + (uint32_t)h * (uint32_t)kSamples);
+    constexpr uint32_t kSpan = (uint32_t)((1ull << 32) / kSamples);
+    int i = (int)__umulhi((uint32_t)s * kSpan + (mix32(m ^ 0x9e3779b9u) & (kSpan - 1u)), (uint32_t)rows);
+    int r = rows == period ? i : i % period;
+    int j = (int)__umulhi(m, (uint32_t)Lk);
     if (causal && off == 0 && j > r) {
       // The part of the rectangle above the diagonal, turned by half a circle, covers the part below it once: no draw is
       // lost.  (The diagonal itself, which is usually forced anyway, is drawn half as often as the rest.)
@@ -221,15 +231,20 @@ __global__ void __launch_bounds__(1024) sample_pivots_kernel(const float *__rest
     valid[u] = !((causal && j > own) || (diag && j == own));
     drawn[u] = valid[u] ? acc[((size_t)h * rows + i) * Lk + j] : 0.f;
   }
+  uint32_t mine = 0u;
 #pragma unroll
-  for (int u = 0; u < kDraws; ++u) {  // one reservation per warp
-    const uint32_t vote = __ballot_sync(0xffffffffu, valid[u]);
-    uint32_t at = 0u;
-    if (lane == 0) at = atomicAdd(&n_valid_s, (uint32_t)__popc(vote));
-    at = __shfl_sync(0xffffffffu, at, 0) + __popc(vote & ((1u << lane) - 1u));
-    if (valid[u]) keys[at] = key_of(drawn[u]);
+  for (int u = 0; u < kDraws; ++u) mine += valid[u] ? 1u : 0u;
+  mine = __reduce_add_sync(0xffffffffu, mine);
+  cluster.sync();  // every CTA has started and cleared its count
+#pragma unroll
+  for (int to = 0; to < 2; ++to) {
+    uint32_t *there = cluster.map_shared_rank(keys, to);
+#pragma unroll
+    for (int u = 0; u < kDraws; ++u) there[t + 1024 * (u + kDraws * part)] = valid[u] ? key_of(drawn[u]) : 0u;
+    if (lane == 0) atomicAdd(cluster.map_shared_rank(&n_valid_s, to), mine);
   }
-  __syncthreads();
+  cluster.sync();
+  if (part >= 2) return;
   const uint32_t nv = n_valid_s;
   if (nv < 1024u) return;  // too few draws landed in the domain: no shortcut for this head
   // Expected rank of the threshold inside the sample and a bracket of 4.5 standard deviations: a selection that misses it
@@ -240,13 +255,13 @@ __global__ void __launch_bounds__(1024) sample_pivots_kernel(const float *__rest
   const double r = frac * nv;
   const double dev = 4.5 * sqrt(fmax(r * (1.0 - frac), 1.0)) + 16.0;
   const long long r_hi = (long long)floor(r - dev), r_lo = (long long)ceil(r + dev);
-  if (blockIdx.y == 0) {
+  if (part == 0) {
     uint32_t hi = 0xffffffffu;
-    if (r_hi >= 1) hi = block_select22(keys, nv, (uint32_t)r_hi, hist, xch) | 0x3ffu;
+    if (r_hi >= 1) hi = block_select22(keys, (uint32_t)kSamples, (uint32_t)r_hi, hist, xch) | 0x3ffu;
     if (t == 0) state[h].hi = hi;
   } else {
     uint32_t lo = 0u;
-    if (r_lo <= (long long)nv) lo = block_select22(keys, nv, (uint32_t)r_lo, hist, xch);
+    if (r_lo <= (long long)nv) lo = block_select22(keys, (uint32_t)kSamples, (uint32_t)r_lo, hist, xch);
     if (t == 0) state[h].lo = lo;
   }
   if (t == 0) state[h].use_shortcut = 1u;  // both CTAs take the same decision
@@ -357,8 +372,9 @@ constexpr int kSelCtasPerSm = 2;
 
 // fn(value, linear index, whether the lane's entry is one of the selection's) for the selection's entries, spread over
 // `n_warps` warps of which this is the `warp`-th: four 128-column pieces of rows at a time, a lane four consecutive
-// entries of each (also where rows start anywhere: neighbouring entries often fall into the same bin, and a warp that
-// counts 32 neighbours at once, although its loads are contiguous then, is 5 us slower at 16 heads x 375 x 759).  Called by whole warps, fn by all lanes together.
+// entries of each (also where rows start anywhere: neighbours often fall into the same bin, and counting 32 of them at once,
+// although the loads are contiguous then, is slower: 63 instead of 58 us at 16 heads x 375 x 759).  Called by whole warps, fn
+// by all lanes together.
 template <class F>
 __device__ __forceinline__ void scan_domain(const float *__restrict__ base, int rows, int Lk, int period, int causal,
                                             int diag, uint32_t warp, uint32_t n_warps, int lane, F fn) {
@@ -610,7 +626,9 @@ struct EmitSel {
 // kept, entries inside it are collected (col) and left out for the select to decide, entries above the bracket are counted.
 //
 // What bounds them: instructions, not memory.  With four columns per lane (a test of each, three shuffles to a bitmap word
-// and a four-byte mask store per row) the classifying pass issued 121 instructions per row of a tile and reached 2.6 TB/s.
+// and a four-byte mask store per row) the classifying pass issued 121 instructions per row of a tile and reached 2.6 TB/s at
+// 16 heads x 2048 (causal).  Whole selections then and now: 16 x 4096 causal 304 -> 268 us; rows that start anywhere
+// (16 x 2501) 240 -> 202 us, one threshold for the layer 260 -> 200 us.
 struct TileSums {
   int count;
   uint32_t groups, above;
@@ -803,6 +821,12 @@ __global__ void __launch_bounds__(32 * kCtaWarps, kCtaWarps == 4 ? 8 : 2) emit_k
   // rows of the scores start on 32-byte boundaries and rows of the mask on 16-byte ones
   const bool aligned4 = (Lk & 3) == 0 && ((reinterpret_cast<uintptr_t>(acc) & 15) | (reinterpret_cast<uintptr_t>(mask) & 3)) == 0;
   const bool aligned = (Lk & 15) == 0 && ((reinterpret_cast<uintptr_t>(acc) & 31) | (reinterpret_cast<uintptr_t>(mask) & 15)) == 0;
+  if (!kClassify && !per_layer) {  // as a rule a classified selection has its mask by now: one look at all of them
+    bool pending = false;
+    const int H = n_tiles / (n_qt * n_kt);
+    for (int x = lane; x < H; x += 32) pending |= state[x].emitted == 0u;
+    if (!__any_sync(0xffffffffu, pending)) return;
+  }
   for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     const int kt = tile % n_kt;
     const int qt = (tile / n_kt) % n_qt;
@@ -958,7 +982,7 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
     const size_t smem = (kSamples + kBins) * sizeof(uint32_t);
     e = cudaFuncSetAttribute(sample_pivots_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    sample_pivots_kernel<<<dim3(n_sel, 2), 1024, smem, s>>>(a.acc, rows, a.Lk, period, a.causal, diag,
+    sample_pivots_kernel<<<n_sel * kSampleCtas, 1024, smem, s>>>(a.acc, rows, a.Lk, period, a.causal, diag,
                                                             (unsigned long long)a.k_rest, (unsigned long long)n_rest,
                                                             sc.state);
     if (classify) {
