@@ -754,7 +754,12 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
       l = l * alpha + (sum0 + sum1);
       o_started = true;
       tmem_wait_st();
-      }  // n_mine > 0
+      } else {
+        // No chunk of this round: the group still waits for its S, so that it does not run ahead of the other group (two
+        // rounds on it would arrive at the same p_full a second time; that round's S comes after O += P V of this one).
+        ok = wait(&sh->s_full[sb], (g >> 1) & 1u);
+        if (!ok) break;
+      }
       // one arrival per warp (32 lanes arriving one by one would take hundreds of cycles)
       tc_fence_before_sync();
       __syncwarp();
