@@ -789,7 +789,9 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
     }
   } else if (warp >= 11) {
     // ------------------------------------------------------------ epilogue
-    // Per item: merge the two groups' accumulators and write O / l, rounded once to bf16.
+    // Per item: merge the two groups' accumulators and write O / l, rounded once to bf16.  A thread writes its row in 32-byte
+    // pieces, i.e. whole sectors (with 16-byte ones: 4 x 16 heads x 4096 x 128, 5 % kept, 81.6 us instead of 78.3).
+    const bool wide = (reinterpret_cast<uintptr_t>(O) & 31) == 0;
     const int r = (warp & 3) * 32 + lane;    // row of the query tile == TMEM lane
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     bool ok = true;
@@ -825,18 +827,23 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
         }
         if (i < Lq) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            uint32_t pk[4];
+          for (int q = 0; q < 2; ++q) {
+            uint32_t pk[8];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
+            for (int e = 0; e < 8; ++e) {
               // a row without kept entries has l = 0 and P = 0 throughout: write exact zeros
-              const int j = 8 * q + 2 * e;
+              const int j = 16 * q + 2 * e;
               const float x0 = (f0 > 0.f ? __uint_as_float(o0[j]) * f0 : 0.f) + (f1 > 0.f ? __uint_as_float(o1[j]) * f1 : 0.f);
               const float x1 = (f0 > 0.f ? __uint_as_float(o0[j + 1]) * f0 : 0.f) +
                                (f1 > 0.f ? __uint_as_float(o1[j + 1]) * f1 : 0.f);
               pk[e] = pack2<kF16>(x0, x1);
             }
-            *reinterpret_cast<uint4 *>(orow + 32 * c + 8 * q) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            if (wide) {
+              stg_v8(orow + 32 * c + 16 * q, pk);
+            } else {
+              *reinterpret_cast<uint4 *>(orow + 32 * c + 16 * q) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+              *reinterpret_cast<uint4 *>(orow + 32 * c + 16 * q + 8) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+            }
           }
         }
       }

@@ -206,6 +206,13 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// 32 bytes to a 32-byte boundary: a whole sector with one store.
+__device__ __forceinline__ void stg_v8(void *p, const uint32_t v[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+               "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+
 // Read-only global loads that are issued where they are written: a plain load of read-only data may
 // be moved by the compiler down to its first use, which defeats a load meant as a prefetch into
 // registers (issued one loop iteration ahead of the use).
