@@ -682,7 +682,7 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
         if (lane == 0) mbar_arrive(which ? &sh->dk_free[ab] : &sh->dv_free[ab]);
 #pragma unroll
         for (int x = 0; x < D / 32; ++x)
-          store_rows<32>(out_s, lane, &pk[16 * x], [&](int rr) -> uint16_t * {
+          store_rows(out_s, lane, &pk[16 * x], [&](int rr) -> uint16_t * {
             const int j = (rr < 16 ? j0 : j1 - 16) + rr;
             return j < Lk ? out + (size_t)j * D + 32 * x : nullptr;
           });

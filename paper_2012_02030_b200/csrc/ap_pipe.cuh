@@ -92,22 +92,19 @@ __device__ __forceinline__ int run_of_slots(int lane, int ng, int row) {
   return head ? (later ? __ffs((int)later) : ng - lane) : 0;
 }
 
-// A warp's 32 accumulator rows, kCols columns of them (32 or 64) packed to 16 bits in pk (lane = row), to global memory
-// in whole 64- or 128-byte pieces: through 64 kCols bytes of shared memory, swizzled so that neither side has bank
-// conflicts.  (One 16-byte store per lane straight from the registers touches 32 lines per instruction and every
-// 32-byte sector twice.)  row_out(r): address of those columns of row r of the warp, or null.
-template <int kCols, class F>
+// A warp's 32 accumulator rows, 32 columns of them packed to 16 bits in pk (lane = row), to global memory in whole 64-byte
+// pieces: through 2 KB of shared memory, swizzled so that neither side has bank conflicts.  row_out(r): address of those columns
+// of row r of the warp, or null.
+template <class F>
 __device__ __forceinline__ void store_rows(unsigned char *stage, int lane, const uint32_t *pk, F row_out) {
-  constexpr int kPieces = kCols / 8;                      // of 16 bytes per row
-  auto place = [](int r, int p) { return kCols == 64 ? r * 8 + (p ^ (r & 7)) : r * 4 + (p ^ ((r >> 1) & 3)); };
+  auto place = [](int r, int p) { return r * 4 + (p ^ ((r >> 1) & 3)); };
   uint4 *s = reinterpret_cast<uint4 *>(stage);
 #pragma unroll
-  for (int p = 0; p < kPieces; ++p)
-    s[place(lane, p)] = make_uint4(pk[4 * p], pk[4 * p + 1], pk[4 * p + 2], pk[4 * p + 3]);
+  for (int p = 0; p < 4; ++p) s[place(lane, p)] = make_uint4(pk[4 * p], pk[4 * p + 1], pk[4 * p + 2], pk[4 * p + 3]);
   __syncwarp();
 #pragma unroll
-  for (int k = 0; k < kPieces; ++k) {
-    const int r = (32 / kPieces) * k + lane / kPieces, p = lane % kPieces;
+  for (int k = 0; k < 4; ++k) {
+    const int r = 8 * k + lane / 4, p = lane % 4;
     uint16_t *out = row_out(r);
     if (out) *reinterpret_cast<uint4 *>(out + 8 * p) = s[place(r, p)];
   }
