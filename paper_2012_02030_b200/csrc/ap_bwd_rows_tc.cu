@@ -649,15 +649,7 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
           // 128-byte ones took 355 instead of 346 us at 4 x 16 heads x 4096 x 128, 5 % kept, both passes)
           uint16_t *out = rows_out + (size_t)lane * D + 64 * x;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (wide) {
-              stg_v8(out + 16 * q, pk + 8 * q);
-            } else {
-              *reinterpret_cast<uint4 *>(out + 16 * q) = make_uint4(pk[8 * q], pk[8 * q + 1], pk[8 * q + 2], pk[8 * q + 3]);
-              *reinterpret_cast<uint4 *>(out + 16 * q + 8) =
-                  make_uint4(pk[8 * q + 4], pk[8 * q + 5], pk[8 * q + 6], pk[8 * q + 7]);
-            }
-          }
+          for (int q = 0; q < 4; ++q) store_sector(out + 16 * q, pk + 8 * q, wide);
         }
       }
     }

@@ -558,15 +558,15 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
           tmem_ld32(tmem + 128 * kSBufs + wg * (D / 2) + 32 * c + lane_addr, o);
           tmem_wait_ld();
           if (row_ok) {
-            uint4 *dst = reinterpret_cast<uint4 *>(O + ((size_t)bh * Lq + i) * D + wg * (D / 2) + 32 * c);
+            uint16_t *dst = O + ((size_t)bh * Lq + i) * D + wg * (D / 2) + 32 * c;
+            const bool wide = (reinterpret_cast<uintptr_t>(O) & 31) == 0;
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              uint4 pkt;
-              pkt.x = pack2<kF16>(__uint_as_float(o[8 * g]) * inv, __uint_as_float(o[8 * g + 1]) * inv);
-              pkt.y = pack2<kF16>(__uint_as_float(o[8 * g + 2]) * inv, __uint_as_float(o[8 * g + 3]) * inv);
-              pkt.z = pack2<kF16>(__uint_as_float(o[8 * g + 4]) * inv, __uint_as_float(o[8 * g + 5]) * inv);
-              pkt.w = pack2<kF16>(__uint_as_float(o[8 * g + 6]) * inv, __uint_as_float(o[8 * g + 7]) * inv);
-              dst[g] = pkt;
+            for (int g = 0; g < 2; ++g) {
+              uint32_t pk[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e)
+                pk[e] = pack2<kF16>(__uint_as_float(o[16 * g + 2 * e]) * inv, __uint_as_float(o[16 * g + 2 * e + 1]) * inv);
+              store_sector(dst + 16 * g, pk, wide);
             }
           }
         }

@@ -838,12 +838,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
                                (f1 > 0.f ? __uint_as_float(o1[j + 1]) * f1 : 0.f);
               pk[e] = pack2<kF16>(x0, x1);
             }
-            if (wide) {
-              stg_v8(orow + 32 * c + 16 * q, pk);
-            } else {
-              *reinterpret_cast<uint4 *>(orow + 32 * c + 16 * q) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-              *reinterpret_cast<uint4 *>(orow + 32 * c + 16 * q + 8) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-            }
+            store_sector(orow + 32 * c + 16 * q, pk, wide);
           }
         }
       }

@@ -213,6 +213,16 @@ __device__ __forceinline__ void stg_v8(void *p, const uint32_t v[8]) {
                : "memory");
 }
 
+// 32 bytes of an output row; wide: rows start on 32-byte boundaries (else on 16-byte ones).
+__device__ __forceinline__ void store_sector(uint16_t *p, const uint32_t v[8], bool wide) {
+  if (wide) {
+    stg_v8(p, v);
+  } else {
+    reinterpret_cast<uint4 *>(p)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<uint4 *>(p)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+  }
+}
+
 // Read-only global loads that are issued where they are written: a plain load of read-only data may
 // be moved by the compiler down to its first use, which defeats a load meant as a prefetch into
 // registers (issued one loop iteration ahead of the use).
