@@ -7,6 +7,7 @@ import torch
 from oracle import ap_oracle as orc
 from paper_2012_02030_b200 import inputs
 from tests import parity_util as pu
+from tests import test_gpu_parity as tp
 
 pytestmark = pytest.mark.gpu
 
@@ -59,3 +60,100 @@ def test_forward_rounds_that_one_softmax_group_sits_out(ap, dtype, d, columns):
     assert np.abs(ref).max() < 4.0
     pu.assert_close_attention(out, ref, dtype, str(columns))
     assert np.all(out[:, :, 7].float().cpu().numpy() == 0.0)
+
+
+def _scores(H, Lq, Lk, seed):
+    """One head each of distinct, quantised (ties by the thousand), skewed and, last, constant values."""
+    acc = np.random.default_rng(seed).random((H, Lq, Lk), dtype=np.float32)
+    acc[1] = np.round(acc[1] * 32) / 32
+    acc[2] = acc[2] ** 8
+    acc[-1] = 0.75
+    return acc
+
+
+@pytest.mark.parametrize("layer", [False, True])
+@pytest.mark.parametrize("H,Lq,Lk,causal", [(4, 1792, 1792, False),    # rows on 32-byte boundaries
+                                            (8, 1801, 1804, True),     # rows on 16-byte boundaries, four memory keys
+                                            (4, 1800, 1801, False)])   # rows anywhere
+def test_build_mask_from_drawn_pivots(ap, H, Lq, Lk, causal, layer):
+    """More than 12 * 2^20 entries in all: pivots from drawn entries, one pass between them, the select over the collected
+    entries; the constant head overflows its buffer and is selected over the accumulator."""
+    acc = _scores(H, Lq, Lk, 503)
+    w = W["tiny"].scaled(H=H, Lq=Lq, Lk=Lk, causal=causal, keep_diag=causal, keep_frac=0.07)
+    mask, tiles, nnz = pu.gpu_build_mask(ap, torch.from_numpy(acc).cuda(), w, layer=layer)
+    want, want_nnz = (orc.build_mask_layer if layer else orc.build_mask)(acc, 0.07, causal, causal)
+    np.testing.assert_array_equal(mask.cpu().numpy(), want)
+    np.testing.assert_array_equal(nnz.cpu().numpy(), want_nnz)
+    pu.assert_tiles_equal(tiles.to_host(), orc.mask_to_tiles(want))
+
+
+def test_build_mask_scores_16_bytes_past_a_sector(ap):
+    H, L = 3, 256
+    acc = _scores(H, L, L, 504)
+    want, _ = orc.build_mask(acc, 0.2, True, True)
+    acc_dev = torch.zeros(H * L * L + 4, device="cuda")[4:].view(H, L, L).copy_(torch.from_numpy(acc))
+    mask = torch.full((H, L, L), 7, dtype=torch.uint8, device="cuda")
+    ap.ap_build_mask(acc_dev, 0.2, True, True, mask=mask)
+    assert ap.ap_device_status() == ap.AP_OK
+    np.testing.assert_array_equal(mask.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("B,H,Lq,Lk,causal", [(7, 2, 512, 512, True),    # chunks of samples, an odd number of them
+                                              (5, 1, 260, 388, True),    # memory keys, ragged
+                                              (16, 3, 130, 64, False),   # one key tile, a query tile of two rows
+                                              (3, 1, 70, 301, False)])   # rows that no tensor map can describe
+def test_accumulate_chunks_of_samples(ap, B, H, Lq, Lk, causal):
+    """Fewer units of work than SMs: each query tile's samples are cut into chunks of about equal numbers of visits."""
+    w = W["tiny"].scaled(B=B, H=H, Lq=Lq, Lk=Lk, d=64, dtype="bf16", causal=causal)
+    bias = inputs.calib_bias(w)
+    acc = pu.gpu_accumulate(ap, w, 2, bias.cuda())
+    assert ap.ap_device_status() == ap.AP_OK
+    assert torch.equal(acc, pu.gpu_accumulate(ap, w, 2, bias.cuda()))
+    want = pu.oracle_accumulate(w, 2, bias)
+    tol = tp._acc_tolerance(w.dtype)
+    np.testing.assert_allclose(acc.cpu().numpy(), want, rtol=tol["rtol"], atol=tol["atol"] * 2 * B)
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 64), ("f16", 64), ("bf16", 128)])
+def test_forward_three_query_tiles(ap, dtype, d):
+    """A pair and a lone query tile per head, over more units than SMs: the grid has no factor in common with a head's units."""
+    B, H, Lq, Lk = 16, 8, 300, 333
+    w = W["tiny"].scaled(B=B, H=H, Lq=Lq, Lk=Lk, d=d, dtype=dtype)
+    mask = inputs.random_mask(H, Lq, Lk, 0.2, seed=505, empty_rows=(299,))
+    q, k, v = inputs.eval_qkv(w)
+    v = v * 0.5  # |O| below 4, see above
+    tiles = ap.Tiles(H, Lq, Lk)
+    ap.ap_mask_to_tiles(mask.cuda(), tiles)
+    # an output that starts 16 bytes past a 32-byte boundary is written in 16-byte pieces
+    plain = torch.full_like(q, float("nan"), device="cuda")
+    odd = torch.full((q.numel() + 8,), float("nan"), dtype=q.dtype, device="cuda")[8:].view(q.shape)
+    for out in (plain, odd):
+        ap.ap_sparse_attention_fwd(q.cuda(), k.cuda(), v.cuda(), tiles, out)
+    assert ap.ap_device_status() == ap.AP_OK
+    assert torch.equal(plain, odd)
+    ref = orc.attention_fwd(inputs.widen(q), inputs.widen(k), inputs.widen(v), mask.numpy())
+    assert np.abs(ref).max() < 4.0
+    pu.assert_close_attention(plain, ref, dtype)
+
+
+@pytest.mark.parametrize("dtype,d,tol", [("bf16", 64, 1e-2), ("bf16", 128, 1e-2), ("f16", 64, 2e-3), ("f16", 128, 2e-3)])
+@pytest.mark.parametrize("Lq,Lk", [(1024, 1024), (1030, 901)])
+def test_backward_gathered_key_blocks(ap, dtype, d, tol, Lq, Lk):
+    """Heavy key groups (sinks, strided columns, the last, partial group) among a band: they come last in the key order and
+    blocks gather them from several tiles.  The second head keeps the band alone and a key tile that nobody keeps."""
+    w = W["tiny"].scaled(B=1, H=2, Lq=Lq, Lk=Lk, d=d, dtype=dtype)
+    i, j = torch.arange(Lq)[:, None], torch.arange(Lk)[None, :]
+    band = (i * Lk // Lq - j).abs() <= 20
+    mask = torch.stack([band | (j < 3) | (j % 200 == 150) | (j == Lk - 1), band & (j // 128 != 2)]).to(torch.uint8)
+    tp._bwd_case(ap, w, mask, tol)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("spread", [0.0, 1e-3, 1.0])
+def test_entmax_forward_candidate_lists(ap, dtype, spread):
+    """More kept entries per row than a candidate list holds: equal scores (every entry is a candidate, no list can be
+    pruned), scores within 1e-3 of one another (the same), and spread-out ones (pruned once or more)."""
+    w = W["tiny"].scaled(B=1, H=2, Lq=200, Lk=520, d=64, dtype=dtype)
+    mask = inputs.random_mask(w.H, w.Lq, w.Lk, 0.9, seed=506, empty_rows=(9,))
+    mask[1, :, 60:] = 0                            # the second head: lists that just fit or just do not
+    tp._entmax_fwd_case(ap, w, mask, scale=spread / 8 if spread else 1e-30)
