@@ -591,10 +591,10 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
         for (int k = 0; k < 8; ++k) {
           const float4 nl = *reinterpret_cast<const float4 *>(&sh->neg_l[st][32 * ch + 4 * k]);
           // (a pruned score may exceed L: masked as packed bits)
-          const float p0 = ex2_approx(fmaf(__uint_as_float(p[x][4 * k]), c, nl.x));
-          const float p1 = ex2_approx(fmaf(__uint_as_float(p[x][4 * k + 1]), c, nl.y));
-          const float p2 = ex2_approx(fmaf(__uint_as_float(p[x][4 * k + 2]), c, nl.z));
-          const float p3 = ex2_approx(fmaf(__uint_as_float(p[x][4 * k + 3]), c, nl.w));
+          float a0, a1, a2, a3;
+          ffma2(a0, a1, __uint_as_float(p[x][4 * k]), __uint_as_float(p[x][4 * k + 1]), c, nl.x, nl.y);
+          ffma2(a2, a3, __uint_as_float(p[x][4 * k + 2]), __uint_as_float(p[x][4 * k + 3]), c, nl.z, nl.w);
+          const float p0 = ex2_approx(a0), p1 = ex2_approx(a1), p2 = ex2_approx(a2), p3 = ex2_approx(a3);
           uint32_t lo, hi;
           masks(w[x], k, lo, hi);
           pk[2 * k] = pack2<kF16>(p0, p1) & lo;
@@ -629,10 +629,11 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
         for (int k = 0; k < 4; ++k) {
           const float4 dd = *reinterpret_cast<const float4 *>(&sh->dsum[st][32 * ch + q0 + 4 * k]);
           const uint32_t *pp = &p[x >> 1][q0 + 4 * k];
-          const float v0 = __uint_as_float(pp[0]) * (__uint_as_float(y[4 * k]) - dd.x);
-          const float v1 = __uint_as_float(pp[1]) * (__uint_as_float(y[4 * k + 1]) - dd.y);
-          const float v2 = __uint_as_float(pp[2]) * (__uint_as_float(y[4 * k + 2]) - dd.z);
-          const float v3 = __uint_as_float(pp[3]) * (__uint_as_float(y[4 * k + 3]) - dd.w);
+          float v0, v1, v2, v3;  // p (dP - D)
+          ffma2(v0, v1, dd.x, dd.y, -1.f, __uint_as_float(y[4 * k]), __uint_as_float(y[4 * k + 1]));
+          ffma2(v2, v3, dd.z, dd.w, -1.f, __uint_as_float(y[4 * k + 2]), __uint_as_float(y[4 * k + 3]));
+          fmul2(v0, v1, __uint_as_float(pp[0]), __uint_as_float(pp[1]), v0, v1);
+          fmul2(v2, v3, __uint_as_float(pp[2]), __uint_as_float(pp[3]), v2, v3);
           uint32_t lo, hi;
           masks(w[x >> 1], 4 * (x & 1) + k, lo, hi);
           pk[2 * k] = pack2<kF16>(v0, v1) & lo;

@@ -487,9 +487,10 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
         float s0 = 0.f, s1 = 0.f;
 #pragma unroll
         for (int e = 0; e < 32; e += 2) {
-          const float p0 = ex2_approx(fmaf(__uint_as_float(xs[e]), c, neg_ref));
-          const float p1 = ex2_approx(fmaf(__uint_as_float(xs[e + 1]), c, neg_ref));
-          if (!kF16 || stats) s0 += p0, s1 += p1;
+          float a0, a1;
+          ffma2(a0, a1, __uint_as_float(xs[e]), __uint_as_float(xs[e + 1]), c, neg_ref, neg_ref);
+          const float p0 = ex2_approx(a0), p1 = ex2_approx(a1);
+          if (!kF16 || stats) fadd2(s0, s1, s0, s1, p0, p1);
           xs[e] = __float_as_uint(p0);
           xs[e + 1] = __float_as_uint(p1);
         }
@@ -515,8 +516,9 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             // a pruned entry has p = 0; a column beyond the round's slots is never read by the product
-            const float d0 = __uint_as_float(xs[16 * x + 2 * e]) * (__uint_as_float(y[2 * e]) - dsum);
-            const float d1 = __uint_as_float(xs[16 * x + 2 * e + 1]) * (__uint_as_float(y[2 * e + 1]) - dsum);
+            float d0, d1;
+            fadd2(d0, d1, __uint_as_float(y[2 * e]), __uint_as_float(y[2 * e + 1]), -dsum, -dsum);
+            fmul2(d0, d1, __uint_as_float(xs[16 * x + 2 * e]), __uint_as_float(xs[16 * x + 2 * e + 1]), d0, d1);
             pk[e] = pack2<kF16>(d0, d1);
           }
           tmem_st8(tmem_s + 8 * x, pk);

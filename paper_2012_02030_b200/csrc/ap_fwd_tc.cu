@@ -742,12 +742,11 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
         uint32_t pk[16];
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
-          const float p0 = ex2_approx(fmaf(__uint_as_float(xs[32 * c + 2 * e]), scale_log2, neg_mc));
-          const float p1 = ex2_approx(fmaf(__uint_as_float(xs[32 * c + 2 * e + 1]), scale_log2, neg_mc));
-          pk[e] = pack2<kF16>(p0, p1);
+          float a0, a1;
+          ffma2(a0, a1, __uint_as_float(xs[32 * c + 2 * e]), __uint_as_float(xs[32 * c + 2 * e + 1]), scale_log2, neg_mc, neg_mc);
+          pk[e] = pack2<kF16>(ex2_approx(a0), ex2_approx(a1));
           const float2 pr = unpack2<kF16>(pk[e]);
-          sum0 += pr.x;
-          sum1 += pr.y;
+          fadd2(sum0, sum1, sum0, sum1, pr.x, pr.y);
         }
         tmem_st16(tmem_s + lane_addr + 32 * (grp + 2 * c), pk);
       }
