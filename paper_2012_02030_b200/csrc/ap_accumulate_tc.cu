@@ -1,6 +1,6 @@
 // Eq. 1 as a running sum for bf16 and fp16 tensors, on the tcgen05 tensor cores.
 //
-// One CTA owns one (head, 128-row query tile) and adds, for up to 32 samples b per launch,
+// One CTA owns one (head, 128-row query tile) and adds, for up to 16 samples b per launch,
 // the normalised softmax rows to the accumulator.  A softmax row needs its
 // maximum and its sum of exponentials over ALL keys before any entry can be
 // normalised, and the sum over b needs each sample normalised separately, so
@@ -23,22 +23,23 @@
 // of lower chunks have finished their addition, and a CTA waits (bounded) for its turn
 // before it issues its own.  Where the accumulator's rows are
 // 16-byte multiples that addition is a TMA reduction: each softmax warp stages its
-// 32 rows x 32 columns in shared memory (128-byte swizzle again) and one lane issues
+// 32 rows x 32 columns in shared memory (16 columns at a time, 64-byte swizzle) and one lane issues
 // cp.reduce.async.bulk.tensor ... add, which updates whole 128-byte lines in L2;
 // a lane per row adding 16 bytes at a time would touch 32 lines per instruction.  Inside
 // a tile that straddles the edge of a causal domain the reduction adds exact zeros to the
 // entries outside the domain (boxes wholly outside are skipped).  Other shapes keep the
 // per-row red.global.add.
 //
-// Warp roles (320 threads, one CTA per SM): warps 0-7 softmax; thread (wg, r)
-// with wg = warp / 4 owns row r of the tile and columns [64 wg, 64 wg + 64) of
-// every key tile; warp 8 TMA producer; warp 9 MMA issuer and TMEM owner.  S is
-// double-buffered in TMEM (2 x 128 columns) so the MMA of the next visit runs
-// under the softmax of the current one; a visit's 64 columns are copied to registers in one
-// go and S is handed back before the arithmetic starts.  TMEM columns 256-383 hold the running
-// sum over b, columns 384-511 the per-sample (maximum, sum) pairs of both column halves, which
-// a thread reads back for its own row (lane) at the start of sweep 2.  Every mbarrier wait is
-// bounded.
+// Warp roles (576 threads, one CTA per SM): warps 0-15 softmax; thread (wg, r) with wg = warp / 4 owns row r of the tile and
+// columns [32 wg, 32 wg + 32) of every key tile; warp 16 TMA producer; warp 17 MMA issuer and TMEM owner.  S is
+// double-buffered in TMEM (2 x 128 columns) so the MMA of the next visit runs under the softmax of the current one; a
+// visit's 32 columns are copied to registers in one go and S is handed back before the arithmetic starts.  TMEM columns
+// 256-383 hold the running sum over b, columns 384-511 the per-sample (maximum, sum) pairs of the four column quarters,
+// which a thread reads back for its own row (lane) at the start of sweep 2.  Every mbarrier wait is bounded.
+//
+// What bounds it: the threads' chain per visit (S -> maximum -> exponentials, 1 024 cycles of them, -> sums: some 1 850
+// cycles) and, at d = 128, the 64 KB of operands and the bias that a visit brings.  Sixteen softmax warps instead of eight
+// with 64 columns each hide the chain's latency better (77 against 84 us at 16 x 16 heads x 512, causal; the same at 4096).
 #include <math_constants.h>
 
 #include <atomic>
@@ -213,9 +214,9 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // ------------------------------------------------------------ TMA producer
     {
       if (lane == 0) {
-      prefetch_tensormap(&map_q);
-      prefetch_tensormap(&map_k);
-      if (bias_by_tma) prefetch_tensormap(&map_bias);
+        prefetch_tensormap(&map_q);
+        prefetch_tensormap(&map_k);
+        if (bias_by_tma) prefetch_tensormap(&map_bias);
       }
       int v = 0, bias_loads = 0;
       for (; v < n_visits; ++v) {
@@ -229,10 +230,10 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           const int tl = v / Bc;
           if (!wait(&bars->bias_empty, ((uint32_t)tl & 1u) ^ 1u)) break;
           if (lane == 0) {
-          mbar_arrive_expect_tx(&bars->bias_full, kBiasBytes);
+            mbar_arrive_expect_tx(&bars->bias_full, kBiasBytes);
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            tma_load_3d(bias_s + q * (kBiasBytes / 4), &map_bias, &bars->bias_full, kt * kTile + 32 * q, qt * kTile, h);
+            for (int q = 0; q < 4; ++q)
+              tma_load_3d(bias_s + q * (kBiasBytes / 4), &map_bias, &bars->bias_full, kt * kTile + 32 * q, qt * kTile, h);
           }
           __syncwarp();
           bias_loads = tl + 1;
@@ -241,12 +242,12 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (dbg_skip != 0 && v == 0) continue;
         unsigned char *q_s = smem + (2 * st) * C::kTileBytes, *k_s = q_s + C::kTileBytes;
         if (lane == 0) {
-        mbar_arrive_expect_tx(&bars->in_full[st], 2 * C::kTileBytes);
+          mbar_arrive_expect_tx(&bars->in_full[st], 2 * C::kTileBytes);
 #pragma unroll
-        for (int s = 0; s < C::kSub; ++s) {
-          tma_load_3d(q_s + s * kSubBytes, &map_q, &bars->in_full[st], 64 * s, qt * kTile, b * H + h);
-          tma_load_3d(k_s + s * kSubBytes, &map_k, &bars->in_full[st], 64 * s, kt * kTile, b * H + h);
-        }
+          for (int s = 0; s < C::kSub; ++s) {
+            tma_load_3d(q_s + s * kSubBytes, &map_q, &bars->in_full[st], 64 * s, qt * kTile, b * H + h);
+            tma_load_3d(k_s + s * kSubBytes, &map_k, &bars->in_full[st], 64 * s, kt * kTile, b * H + h);
+          }
         }
         __syncwarp();
       }
@@ -271,15 +272,15 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (!wait(&bars->s_empty[buf], ((uint32_t)(v >> 1) & 1u) ^ 1u)) break;
         tc_fence_after_sync();
         if (elect_one()) {
-        const uint32_t q_lo = desc0 + 2 * st * (C::kTileBytes >> 4), k_lo = q_lo + (C::kTileBytes >> 4);
-        constexpr uint32_t kHi = smem_desc_hi_sw128(1024);
+          const uint32_t q_lo = desc0 + 2 * st * (C::kTileBytes >> 4), k_lo = q_lo + (C::kTileBytes >> 4);
+          constexpr uint32_t kHi = smem_desc_hi_sw128(1024);
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t step = (ks / 4) * (kSubBytes >> 4) + (ks % 4) * 2;
-          mma_ss<kHi, kHi>(tmem + 128 * buf, q_lo + step, k_lo + step, idesc, ks > 0);
-        }
-        mma_commit(&bars->in_empty[st]);
-        mma_commit(&bars->s_full[buf]);
+          for (int ks = 0; ks < D / 16; ++ks) {
+            const uint32_t step = (ks / 4) * (kSubBytes >> 4) + (ks % 4) * 2;
+            mma_ss<kHi, kHi>(tmem + 128 * buf, q_lo + step, k_lo + step, idesc, ks > 0);
+          }
+          mma_commit(&bars->in_empty[st]);
+          mma_commit(&bars->s_full[buf]);
         }
         __syncwarp();
       }
