@@ -8,6 +8,10 @@
 // and adds the normalised row to the accumulator with coalesced read-modify-
 // writes.  Used for fp32 inputs, where tensor-core precision would not do.
 //
+// What bounds it: the key rows' loads (a lane per row: as many lines per load as lanes) and the latency of a sample's
+// phases.  With 16-byte loads four at a time, the exponentials computed twice and one load of the accumulator under way:
+// 168 us at 16 x 8 heads x 256 x 64, 122 now; 34 -> 26 us at 3 x 16 heads x 194 x 64 (causal).
+//
 // kEntmax: the same sum with 1.5-entmax as the normaliser (the section on sparse normalisation),
 // p_j = max(s_j / 2 - tau, 0)^2 with tau such that the row sums to 1.  The row's scores are in
 // shared memory, so the warp iterates on tau there: from max/2 - 0.625 (the root lies in [max/2 - 1, max/2)) to the
@@ -25,31 +29,31 @@ namespace {
 
 constexpr int kRows = 8;
 constexpr int kThreads = 256;
+constexpr int kPiece = 64;  // elements of a key row loaded at once
 
-template <typename T>
-__device__ __forceinline__ void load8(const T *p, float v[8]);
-
-template <>
-__device__ __forceinline__ void load8<float>(const float *p, float v[8]) {
-  float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
-  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-  v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-}
-
-template <>
-__device__ __forceinline__ void load8<__nv_bfloat16>(const __nv_bfloat16 *p, float v[8]) {
-  uint4 u = *reinterpret_cast<const uint4 *>(p);
-  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+// kPiece elements of a key row, from a 32-byte boundary (wide) or a 16-byte one.  A thread reads a row of its own, so that
+// a load touches as many lines as the warp has lanes whatever its size: twice the size, half the lines' cycles.  (Volatile: all
+// loads are under way before the first product.)
+__device__ __forceinline__ void load_piece(const float *p, float v[kPiece], bool wide) {
+  if (wide) {
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    v[2 * c] = __uint_as_float(w[c] << 16);
-    v[2 * c + 1] = __uint_as_float(w[c] & 0xffff0000u);
+    for (int t = 0; t < kPiece; t += 8)
+      asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                   : "=f"(v[t]), "=f"(v[t + 1]), "=f"(v[t + 2]), "=f"(v[t + 3]), "=f"(v[t + 4]), "=f"(v[t + 5]),
+                     "=f"(v[t + 6]), "=f"(v[t + 7])
+                   : "l"(p + t));
+  } else {
+#pragma unroll
+    for (int t = 0; t < kPiece; t += 4)
+      asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(v[t]), "=f"(v[t + 1]), "=f"(v[t + 2]), "=f"(v[t + 3])
+                   : "l"(p + t));
   }
 }
 
-template <typename T, int D, bool kEntmax>
-__global__ void __launch_bounds__(kThreads) accumulate_simt_kernel(float *__restrict__ acc, const T *__restrict__ Q,
-                                                                   const T *__restrict__ K,
+template <int D, bool kEntmax>
+__global__ void __launch_bounds__(kThreads) accumulate_simt_kernel(float *__restrict__ acc, const float *__restrict__ Q,
+                                                                   const float *__restrict__ K,
                                                                    const float *__restrict__ bias, int B, int H,
                                                                    int Lq, int Lk, int rows, int causal,
                                                                    float scale) {
@@ -64,32 +68,32 @@ __global__ void __launch_bounds__(kThreads) accumulate_simt_kernel(float *__rest
   const int off = causal ? Lk - Lq : 0;  // causal: row i looks at keys j <= i + (Lk - Lq)
   const int jmax = causal ? min(Lk, i0 + n_rows + off) : Lk;
 
+  const bool wide = (reinterpret_cast<uintptr_t>(K) & 31) == 0;
   for (int b = 0; b < B; ++b) {
-    const T *Qb = Q + (((size_t)b * H + h) * Lq + i0) * D;
-    const T *Kb = K + ((size_t)b * H + h) * (size_t)Lk * D;
+    const float *Qb = Q + (((size_t)b * H + h) * Lq + i0) * D;
+    const float *Kb = K + ((size_t)b * H + h) * (size_t)Lk * D;
     for (int e = threadIdx.x; e < kRows * D; e += kThreads) {
       const int r = e / D;
-      q_s[e] = r < n_rows ? (float)Qb[e] : 0.f;
+      q_s[e] = r < n_rows ? Qb[e] : 0.f;
     }
     __syncthreads();
     for (int j = threadIdx.x; j < jmax; j += kThreads) {
       float dot[kRows];
 #pragma unroll
       for (int r = 0; r < kRows; ++r) dot[r] = 0.f;
-      const T *krow = Kb + (size_t)j * D;
-#pragma unroll 2
-      for (int t = 0; t < D; t += 8) {
-        float kv[8];
-        load8<T>(krow + t, kv);
+      const float *krow = Kb + (size_t)j * D;
+#pragma unroll 1
+      for (int t0 = 0; t0 < D; t0 += kPiece) {
+        float kv[kPiece];
+        load_piece(krow + t0, kv, wide);
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) {
-          const float4 qa = *reinterpret_cast<const float4 *>(q_s + r * D + t);
-          const float4 qb = *reinterpret_cast<const float4 *>(q_s + r * D + t + 4);
-          dot[r] = fmaf(qa.x, kv[0], dot[r]); dot[r] = fmaf(qa.y, kv[1], dot[r]);
-          dot[r] = fmaf(qa.z, kv[2], dot[r]); dot[r] = fmaf(qa.w, kv[3], dot[r]);
-          dot[r] = fmaf(qb.x, kv[4], dot[r]); dot[r] = fmaf(qb.y, kv[5], dot[r]);
-          dot[r] = fmaf(qb.z, kv[6], dot[r]); dot[r] = fmaf(qb.w, kv[7], dot[r]);
-        }
+        for (int t = 0; t < kPiece; t += 4)
+#pragma unroll
+          for (int r = 0; r < kRows; ++r) {
+            const float4 q = *reinterpret_cast<const float4 *>(q_s + r * D + t0 + t);
+            dot[r] = fmaf(q.x, kv[t], dot[r]); dot[r] = fmaf(q.y, kv[t + 1], dot[r]);
+            dot[r] = fmaf(q.z, kv[t + 2], dot[r]); dot[r] = fmaf(q.w, kv[t + 3], dot[r]);
+          }
       }
 #pragma unroll
       for (int r = 0; r < kRows; ++r) {
@@ -105,7 +109,7 @@ __global__ void __launch_bounds__(kThreads) accumulate_simt_kernel(float *__rest
     for (int r = warp; r < n_rows; r += kThreads / 32) {
       const int i = i0 + r;
       const int jend = causal ? min(Lk, i + 1 + off) : Lk;
-      const float *srow = s_s + (size_t)r * Lk;
+      float *srow = s_s + (size_t)r * Lk;
       float m = -CUDART_INF_F;
       for (int j = lane; j < jend; j += 32) m = fmaxf(m, srow[j]);
 #pragma unroll
@@ -141,16 +145,27 @@ __global__ void __launch_bounds__(kThreads) accumulate_simt_kernel(float *__rest
         continue;
       }
       float z = 0.f;
-      for (int j = lane; j < jend; j += 32) z += expf(srow[j] - m);
+      for (int j = lane; j < jend; j += 32) {
+        const float e = expf(srow[j] - m);
+        srow[j] = e;
+        z += e;
+      }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-      for (int j = lane; j < jend; j += 32) arow[j] += expf(srow[j] - m) / z;
+      for (int j0 = lane; j0 < jend; j0 += 128) {  // four of the accumulator's loads under way
+        float a[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] = j0 + 32 * u < jend ? arow[j0 + 32 * u] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (j0 + 32 * u < jend) arow[j0 + 32 * u] = a[u] + srow[j0 + 32 * u] / z;
+      }
     }
     __syncthreads();
   }
 }
 
-template <typename T, int D, bool kEntmax>
+template <int D, bool kEntmax>
 cudaError_t launch(float *acc, const void *Q, const void *K, const float *bias, int B, int H, int Lq, int Lk,
                    int causal, float scale, cudaStream_t s) {
   // as many rows per CTA (up to 8) as the score rows allow in shared memory
@@ -159,11 +174,11 @@ cudaError_t launch(float *acc, const void *Q, const void *K, const float *bias, 
   while (rows > 1 && (size_t)(kRows * D + (size_t)rows * Lk) * sizeof(float) > budget) rows >>= 1;
   const size_t smem = (size_t)(kRows * D + (size_t)rows * Lk) * sizeof(float);
   if (smem > budget) return cudaErrorInvalidValue;
-  auto kern = accumulate_simt_kernel<T, D, kEntmax>;
+  auto kern = accumulate_simt_kernel<D, kEntmax>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid(ceil_div(Lq, rows), H);
-  kern<<<grid, kThreads, smem, s>>>(acc, static_cast<const T *>(Q), static_cast<const T *>(K), bias, B, H, Lq, Lk,
+  kern<<<grid, kThreads, smem, s>>>(acc, static_cast<const float *>(Q), static_cast<const float *>(K), bias, B, H, Lq, Lk,
                                     rows, causal, scale);
   count_launches(1);
   return cudaGetLastError();
@@ -172,18 +187,13 @@ cudaError_t launch(float *acc, const void *Q, const void *K, const float *bias, 
 }  // namespace
 
 cudaError_t launch_accumulate_simt(float *acc, const void *Q, const void *K, const float *bias, int B, int H,
-                                   int Lq, int Lk, int d, ap_dtype dt, int causal, float scale,
+                                   int Lq, int Lk, int d, int causal, float scale,
                                    cudaStream_t s, int entmax) {
-  if (entmax) {  // fp32 tensors only
-    return d == 64 ? launch<float, 64, true>(acc, Q, K, bias, B, H, Lq, Lk, causal, scale, s)
-                   : launch<float, 128, true>(acc, Q, K, bias, B, H, Lq, Lk, causal, scale, s);
-  }
-  if (dt == AP_F32) {
-    return d == 64 ? launch<float, 64, false>(acc, Q, K, bias, B, H, Lq, Lk, causal, scale, s)
-                   : launch<float, 128, false>(acc, Q, K, bias, B, H, Lq, Lk, causal, scale, s);
-  }
-  return d == 64 ? launch<__nv_bfloat16, 64, false>(acc, Q, K, bias, B, H, Lq, Lk, causal, scale, s)
-                 : launch<__nv_bfloat16, 128, false>(acc, Q, K, bias, B, H, Lq, Lk, causal, scale, s);
+  if (entmax)
+    return d == 64 ? launch<64, true>(acc, Q, K, bias, B, H, Lq, Lk, causal, scale, s)
+                   : launch<128, true>(acc, Q, K, bias, B, H, Lq, Lk, causal, scale, s);
+  return d == 64 ? launch<64, false>(acc, Q, K, bias, B, H, Lq, Lk, causal, scale, s)
+                 : launch<128, false>(acc, Q, K, bias, B, H, Lq, Lk, causal, scale, s);
 }
 
 }  // namespace ap

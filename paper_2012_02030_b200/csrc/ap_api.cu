@@ -143,7 +143,7 @@ ap_status ap_accumulate_attention(float *acc, const void *Q, const void *K, cons
   const float sc = scale == 0.f ? (float)(1.0 / sqrt((double)d)) : scale;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (dt != AP_F32 && !device_error_word()) return AP_ERR_CUDA;
-  cudaError_t e = dt == AP_F32 ? launch_accumulate_simt(acc, Q, K, bias, B, H, Lq, Lk, d, dt, causal ? 1 : 0, sc, s)
+  cudaError_t e = dt == AP_F32 ? launch_accumulate_simt(acc, Q, K, bias, B, H, Lq, Lk, d, causal ? 1 : 0, sc, s)
                                : launch_accumulate_tc(acc, Q, K, bias, B, H, Lq, Lk, d, causal ? 1 : 0,
                                                       dt == AP_F16 ? 1 : 0, sc, s);
   if (e == cudaErrorInvalidValue) return AP_ERR_UNSUPPORTED;  // key length beyond the shared-memory budget
@@ -162,7 +162,7 @@ ap_status ap_accumulate_attention_entmax15(float *acc, const void *Q, const void
   const float sc = scale == 0.f ? (float)(1.0 / sqrt((double)d)) : scale;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = dt == AP_F32
-                      ? launch_accumulate_simt(acc, Q, K, bias, B, H, Lq, Lk, d, dt, causal ? 1 : 0, sc, s, 1)
+                      ? launch_accumulate_simt(acc, Q, K, bias, B, H, Lq, Lk, d, causal ? 1 : 0, sc, s, 1)
                       : launch_accumulate_entmax_tc(acc, Q, K, bias, B, H, Lq, Lk, d, causal ? 1 : 0,
                                                     dt == AP_F16 ? 1 : 0, sc, s);
   if (e == cudaErrorInvalidValue) return AP_ERR_UNSUPPORTED;  // key length beyond the shared-memory budget

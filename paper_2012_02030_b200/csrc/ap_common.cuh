@@ -126,7 +126,7 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s);
 
 // (entmax: the 1.5-entmax normaliser instead of the softmax; fp32 tensors)
 cudaError_t launch_accumulate_simt(float *acc, const void *Q, const void *K, const float *bias, int B,
-                                   int H, int Lq, int Lk, int d, ap_dtype dt, int causal, float scale,
+                                   int H, int Lq, int Lk, int d, int causal, float scale,
                                    cudaStream_t s, int entmax = 0);
 
 // fp32 tensors: CUDA-core kernel

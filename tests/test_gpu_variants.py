@@ -157,3 +157,20 @@ def test_entmax_forward_candidate_lists(ap, dtype, spread):
     mask = inputs.random_mask(w.H, w.Lq, w.Lk, 0.9, seed=506, empty_rows=(9,))
     mask[1, :, 60:] = 0                            # the second head: lists that just fit or just do not
     tp._entmax_fwd_case(ap, w, mask, scale=spread / 8 if spread else 1e-30)
+
+
+@pytest.mark.parametrize("Lk", [33, 260])
+def test_fp32_accumulate_key_rows_16_bytes_past_a_sector(ap, Lk):
+    """Key rows that start on 32-byte boundaries are read with wider loads: the same numbers either way."""
+    w = W["tiny"].scaled(B=3, H=2, Lq=29, Lk=Lk, d=64, dtype="f32", causal=False)
+    q, k = (t.cuda() for t in inputs.calib_qk(w, 0))
+    odd = torch.zeros(k.numel() + 4, device="cuda")[4:].view(k.shape).copy_(k)
+    got = [torch.zeros((w.H, w.Lq, w.Lk), device="cuda") for _ in range(2)]
+    for acc, keys in zip(got, (k, odd)):
+        ap.ap_accumulate_attention(acc, q, keys, None, causal=False)
+    assert ap.ap_device_status() == ap.AP_OK
+    assert torch.equal(*got)
+    want = np.zeros((w.H, w.Lq, w.Lk))
+    orc.accumulate(want, inputs.widen(q.cpu()), inputs.widen(k.cpu()), None, causal=False)
+    tol = tp._acc_tolerance("f32")
+    np.testing.assert_allclose(got[0].cpu().numpy(), want, rtol=tol["rtol"], atol=tol["atol"] * w.B)
