@@ -464,18 +464,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           }
           if (b < Bc - 1) {
             tmem_st16(sum_addr + 16 * c, ps);
-          } else if (acc_by_tma) {
-            // last sample of this key tile: one addition per accumulator entry and launch, performed
-            // in L2 by a TMA reduction of this warp's 32 x 16 block
-            if (lane == 0) bulk_wait_group_read0();  // the block staged before has been read
-            __syncwarp();
-#pragma unroll
-            for (int k = 0; k < 4; ++k)  // 16-byte chunk k of row `lane` goes to position k ^ (lane / 2 % 4)
-              *reinterpret_cast<uint4 *>(red_s + lane * 64 + ((k ^ ((lane >> 1) & 3)) << 4)) =
-                  make_uint4(ps[4 * k], ps[4 * k + 1], ps[4 * k + 2], ps[4 * k + 3]);
-            fence_proxy_async_smem();
-            __syncwarp();
-            const int x = j0 + 16 * c;
+          } else {
             if (kChunked && c == 0) {
               // this key tile's entries have received the sums of all lower chunks once their
               // warps have counted themselves in (bounded wait)
@@ -497,38 +486,53 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
               }
               ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
               if (!ok) break;
+              __syncwarp();
             }
-            if (lane == 0 && red_y < Lq && x < red_jend) {
-              tma_reduce_add_3d(&map_acc, red_s, x, red_y, h);
-              bulk_commit_group();
-            }
-            if (kChunked && c == 1 && lane == 0) {
-              // both blocks of this warp are in the accumulator: count this warp in for the next chunk
-              bulk_wait_group0();
-              __threadfence();
-              atomicAdd(turn + ((size_t)h * n_qt + qt) * n_kt + kt, 1u);
-            }
-          } else if (row_ok) {
-            // accumulator rows that are no 16-byte multiples: one red per entry (entries outside the
-            // domain are not touched)
-            float *arow = acc + ((size_t)h * Lq + i) * Lk + j0 + 16 * c;
-            const int nv = n_valid - 16 * c;
+            if (acc_by_tma) {
+              // last sample of this key tile: one addition per accumulator entry and launch, performed
+              // in L2 by a TMA reduction of this warp's 32 x 16 block
+              if (lane == 0) bulk_wait_group_read0();  // the block staged before has been read
+              __syncwarp();
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              const int jj = 4 * g;
-              if (jj >= nv) break;
-              if (vec && jj + 4 <= nv) {
-                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(arow + jj),
-                             "f"(__uint_as_float(ps[jj])), "f"(__uint_as_float(ps[jj + 1])),
-                             "f"(__uint_as_float(ps[jj + 2])), "f"(__uint_as_float(ps[jj + 3]))
-                             : "memory");
-              } else {
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                  if (jj + e < nv)
-                    asm volatile("red.global.add.f32 [%0], %1;" ::"l"(arow + jj + e), "f"(__uint_as_float(ps[jj + e]))
-                                 : "memory");
+              for (int k = 0; k < 4; ++k)  // 16-byte chunk k of row `lane` goes to position k ^ (lane / 2 % 4)
+                *reinterpret_cast<uint4 *>(red_s + lane * 64 + ((k ^ ((lane >> 1) & 3)) << 4)) =
+                    make_uint4(ps[4 * k], ps[4 * k + 1], ps[4 * k + 2], ps[4 * k + 3]);
+              fence_proxy_async_smem();
+              __syncwarp();
+              const int x = j0 + 16 * c;
+              if (lane == 0 && red_y < Lq && x < red_jend) {
+                tma_reduce_add_3d(&map_acc, red_s, x, red_y, h);
+                bulk_commit_group();
               }
+            } else if (row_ok) {
+              // accumulator rows that are no 16-byte multiples: one red per entry (entries outside the
+              // domain are not touched)
+              float *arow = acc + ((size_t)h * Lq + i) * Lk + j0 + 16 * c;
+              const int nv = n_valid - 16 * c;
+#pragma unroll
+              for (int g = 0; g < 4; ++g) {
+                const int jj = 4 * g;
+                if (jj >= nv) break;
+                if (vec && jj + 4 <= nv) {
+                  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(arow + jj),
+                               "f"(__uint_as_float(ps[jj])), "f"(__uint_as_float(ps[jj + 1])),
+                               "f"(__uint_as_float(ps[jj + 2])), "f"(__uint_as_float(ps[jj + 3]))
+                               : "memory");
+                } else {
+#pragma unroll
+                  for (int e = 0; e < 4; ++e)
+                    if (jj + e < nv)
+                      asm volatile("red.global.add.f32 [%0], %1;" ::"l"(arow + jj + e), "f"(__uint_as_float(ps[jj + e]))
+                                   : "memory");
+                }
+              }
+            }
+            if (kChunked && c == 1) {
+              // both blocks of this warp are in the accumulator: count this warp in for the next chunk
+              if (acc_by_tma && lane == 0) bulk_wait_group0();
+              __threadfence();
+              __syncwarp();
+              if (lane == 0) atomicAdd(turn + ((size_t)h * n_qt + qt) * n_kt + kt, 1u);
             }
           }
         }
@@ -559,9 +563,14 @@ cudaError_t launch(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorM
   // turns at the accumulator (one wave of CTAs, one per SM).  The smallest number of visits per chunk is taken for
   // which they fit, so that the query tiles with many key tiles are cut into more chunks: with the same number for all,
   // the longest CTA of 16 x 16 heads x 512 (causal) had 64 visits where 35 would be the mean (now 48: 77 -> 64 us).
+  // Accumulator rows that no tensor map describes are added to with one instruction per entry, several microseconds per tile,
+  // and a chunk's turn waits for those of all lower ones: worth it from three key tiles and 48 visits per sweep and pair on
+  // (19 x 2 heads x 975 x 1950: 1 147 -> 532 us, 20 x 333: 170 -> 147; but 9 x 333, 27 visits: 85 -> 117, and 40 x 2 x 130 x
+  // 130, two key tiles: 216 -> 232).
   const int n_units = H * n_qt, sms = sm_count();
   unsigned *turn = nullptr;
-  if (acc_by_tma && !knobs.skip_arrive && n_units < sms && B >= 2 * kMinChunk && (size_t)n_units * n_kt <= kTurnWords)
+  const bool long_enough = acc_by_tma || (n_kt >= 3 && n_kt * B >= 48);
+  if (long_enough && !knobs.skip_arrive && n_units < sms && B >= 2 * kMinChunk && (size_t)n_units * n_kt <= kTurnWords)
     turn = turn_words();
   // samples in ascending order, at most kMaxB per CTA; launches on one stream run in order
   for (int b0 = 0; b0 < B;) {

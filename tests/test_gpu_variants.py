@@ -101,7 +101,8 @@ def test_build_mask_scores_16_bytes_past_a_sector(ap):
 @pytest.mark.parametrize("B,H,Lq,Lk,causal", [(7, 2, 512, 512, True),    # chunks of samples, an odd number of them
                                               (5, 1, 260, 388, True),    # memory keys, ragged
                                               (16, 3, 130, 64, False),   # one key tile, a query tile of two rows
-                                              (3, 1, 70, 301, False)])   # rows that no tensor map can describe
+                                              (3, 1, 70, 301, False),    # rows that no tensor map can describe, ...
+                                              (18, 2, 200, 387, True)])  # ... in chunks
 def test_accumulate_chunks_of_samples(ap, B, H, Lq, Lk, causal):
     """Fewer units of work than SMs: each query tile's samples are cut into chunks of about equal numbers of visits."""
     w = W["tiny"].scaled(B=B, H=H, Lq=Lq, Lk=Lk, d=64, dtype="bf16", causal=causal)
