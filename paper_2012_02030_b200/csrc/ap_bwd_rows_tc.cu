@@ -1,7 +1,7 @@
 // Backward of the masked attention, rows kernel: dQ and the row statistics.
 //
-// Persistent, one CTA per SM; a work item is one (b, h, query tile), handed out through a counter (late query
-// tiles of a head first, heads in order, so that concurrent CTAs share a few heads' K and V in L2).
+// Persistent, one CTA per SM; a work item is one (b, h, query tile) and a block of the grid, taken over by a running
+// CTA (late query tiles of a head first, heads in order, so that concurrent CTAs share a few heads' K and V in L2).
 // An item follows the query tile's rounds (up to eight non-empty 16-column groups each).  Per round:
 //   S  = Q K^T, dP = dO V^T   tcgen05.mma, fp32 accumulators in TMEM
 //   dS = 2^(c S - r) (dP - D) by four threads per query row (a 32-column chunk each), written as 16-bit values
@@ -66,6 +66,7 @@ struct Shared {
   uint64_t o_free;              // dQ of the item read out
   uint64_t ml_ready[4], d_ready[2], item_ready[kItemRing];
   uint64_t quad[4];             // the four warps that share 32 rows
+  TakeOver more;                // the next item
   int32_t item_bh[kItemRing], item_qt[kItemRing];  // qt = -1: no more items
   uint32_t item_last[4];        // [item % 4]: its last round
   uint32_t info[kRing + 1];
@@ -88,7 +89,7 @@ struct Cfg {
 template <int D, bool kSplit, bool kF16>
 __global__ void __launch_bounds__(kThreads, 1)
 rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ O, const uint16_t *__restrict__ dO,
-            uint16_t *__restrict__ dQ, float *__restrict__ neg_l, float *__restrict__ stat_d, int32_t *__restrict__ next,
+            uint16_t *__restrict__ dQ, float *__restrict__ neg_l, float *__restrict__ stat_d,
             const int32_t *__restrict__ round_ptr, const int32_t *__restrict__ round_rows,
             const uint8_t *__restrict__ round_info, const uint32_t *__restrict__ round_bitmap, int n_items, int H,
             int Lq, int n_qt, float scale, unsigned *err, uint32_t max_polls, int dbg_skip) {
@@ -129,6 +130,7 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
       mbar_init(&sh->quad[i], 4);
     }
     for (int i = 0; i < kItemRing; ++i) mbar_init(&sh->item_ready[i], 1);
+    mbar_init(&sh->more.answered, 1);
     sh->abort_flag = 0;
     fence_mbar_init();
   }
@@ -153,11 +155,16 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
     }
     bool ok = dbg_skip == 0;  // (test hook: nothing is copied, the other roles' waits run out)
     uint32_t g = 0, n = 0;    // rounds / non-empty items so far
-    // the next item's number is drawn while the current one is under way, its rounds looked up with it
-    auto draw = [&]() {
-      int x = 0;
-      if (lane == 0) x = atomicAdd(next, 1);  // (every CTA begins with the item of its own number)
-      return (int)gridDim.x + __shfl_sync(0xffffffffu, x, 0);
+    // The next item is asked for when the current one begins (every CTA begins with the item of its own number) and looked up
+    // once its second round's copies are under way: one item ahead, no more, or the last ones would pile up on the CTAs
+    // that happen to be first.
+    uint32_t asked = 0, heard = 0;
+    bool blocks_left = true;
+    auto ask = [&]() {
+      if (!blocks_left) return;
+      if (lane == 0) ask_block(&sh->more);
+      __syncwarp();
+      ++asked;
     };
     struct Item {
       int bh, qt, r0, r1;
@@ -204,16 +211,29 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
       __syncwarp();
       ++published;
     };
+    auto hear = [&]() {  // (none where nothing was asked for)
+      int k = -1;
+      if (asked != heard) {
+        ok = wait(&sh->more.answered, heard & 1u);
+        if (ok) {
+          ++heard;
+          k = taken_block(&sh->more);
+          __syncwarp();
+          blocks_left = k >= 0;
+        }
+      }
+      return look_up(k >= 0 ? k : n_items);
+    };
     Item cur = look_up((int)blockIdx.x);
-    int k_next = ok ? draw() : n_items;
     while (ok && cur.qt >= 0) {
       const Item it = cur;
-      cur = look_up(k_next);
-      if (cur.qt >= 0) k_next = draw();
+      ask();
+      bool known = false;  // the next item
       if (it.r0 == it.r1) {  // nothing kept: dQ is zero, and no key block visits the tile
         const int rows = min(kTile, Lq - it.qt * kTile);
         uint4 *dst = reinterpret_cast<uint4 *>(dQ + ((size_t)it.bh * Lq + (size_t)it.qt * kTile) * D);
         for (int x = lane; x < rows * (D / 8); x += 32) dst[x] = make_uint4(0u, 0u, 0u, 0u);
+        cur = hear();
         continue;
       }
       if (published == n) publish(it);
@@ -280,7 +300,8 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
             __syncwarp();
           }
           // the item after this one, as soon as it is known (the finishing warps form its D ahead)
-          if (published == n + 1u && cur.qt >= 0 && cur.r0 < cur.r1) publish(cur);
+          if (ok && !known && (v > it.r0 || it.r0 + 1 == it.r1)) cur = hear(), known = true;
+          if (known && published == n + 1u && cur.qt >= 0 && cur.r0 < cur.r1) publish(cur);
           ++g;
           v_pending = true, v_used = sweep == 1;
           v_row = my_row, v_run = run, v_bh = it.bh, v_slots = ng;
@@ -303,7 +324,14 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
       }
     }
     if (!ok && dbg_skip == 0 && lane == 0) {
-      // winding down: wait (bounded) for the copies armed most recently
+      // winding down: the items left are taken and dropped (their waits would run out one after the other), then a bounded
+      // wait for the copies armed most recently
+      while (asked != heard && mbar_wait(&sh->more.answered, heard & 1u, 1u << 16)) {
+        ++heard;
+        if (taken_block(&sh->more) < 0) break;
+        ask_block(&sh->more);
+        ++asked;
+      }
       if (q_armed >= 0) mbar_wait(&sh->q_full[q_armed % kQBufs], ((uint32_t)q_armed / kQBufs) & 1u, 1u << 16);
       if (do_armed >= 0) mbar_wait(&sh->do_full[do_armed % kQBufs], ((uint32_t)do_armed / kQBufs) & 1u, 1u << 16);
       for (uint32_t a = g > kRing ? g - kRing : 0; a <= g; ++a) {
@@ -670,10 +698,11 @@ cudaError_t launch(const RowsMaps &maps, const Args &a) {
   const int sms = sm_count();
   if (sms <= 0) return cudaErrorUnknown;
   const DebugKnobs knobs = debug_knobs();
-  const int n_items = a.B * a.H * a.t->n_qt, grid = n_items < sms ? n_items : sms;
+  // (the test hook runs on the first wave only: none of its CTAs takes over another's item)
+  const int n_items = a.B * a.H * a.t->n_qt, grid = knobs.skip_arrive && n_items > sms ? sms : n_items;
   kern<<<grid, kThreads, C::kSmemBytes, a.s>>>(
       maps, static_cast<const uint16_t *>(a.O), static_cast<const uint16_t *>(a.dO), static_cast<uint16_t *>(a.dQ),
-      a.plan.neg_l, a.plan.dsum, a.plan.next, a.t->round_ptr, a.t->round_rows, a.t->round_info, a.t->round_bitmap,
+      a.plan.neg_l, a.plan.dsum, a.t->round_ptr, a.t->round_rows, a.t->round_info, a.t->round_bitmap,
       n_items, a.H, a.Lq, a.t->n_qt, a.scale, a.err, knobs.max_polls, knobs.skip_arrive);
   count_launches(1);
   return cudaGetLastError();

@@ -7,8 +7,6 @@
 // Three kernels: the (query tile, key tile) table (here), the rows kernel (dQ and the row statistics
 // L = log2 sum 2^(c S), c = scale log2 e, and D; ap_bwd_rows_tc.cu) and the columns kernel (dK, dV;
 // ap_bwd_cols_tc.cu).
-#include <atomic>
-
 #include "ap_bwd_tc.cuh"
 
 namespace ap {
@@ -16,33 +14,13 @@ namespace bwd {
 
 namespace {
 
-// Item counters of the calls in flight (rows kernel, columns kernel), set to zero by a call's first kernel.  Calls
-// take the pairs in rotation, so calls on different streams do not share one.
-constexpr unsigned kCounters = 1024;
-__device__ int32_t g_next[kCounters][2];
-
-int32_t *next_items() {
-  static std::atomic<unsigned> turn{0};
-  static std::atomic<int32_t *> base[64];
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-  int32_t *b = base[dev].load(std::memory_order_relaxed);
-  if (!b) {
-    void *p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_next) != cudaSuccess) return nullptr;
-    base[dev].store(b = static_cast<int32_t *>(p), std::memory_order_relaxed);
-  }
-  return b + 2 * (turn.fetch_add(1) % kCounters);
-}
-
 // One CTA per list row (h, query tile).
 __global__ void __launch_bounds__(128) table_kernel(const int32_t *__restrict__ row_ptr,
                                                     const int32_t *__restrict__ col_idx,
                                                     const uint8_t *__restrict__ flags,
                                                     const uint8_t *__restrict__ groups, int n_kt,
-                                                    uint32_t *__restrict__ table, int32_t *__restrict__ next) {
+                                                    uint32_t *__restrict__ table) {
   uint32_t *row = table + (size_t)blockIdx.x * n_kt;
-  if (blockIdx.x == 0 && threadIdx.x < 2) next[threadIdx.x] = 0;
   for (int kt = threadIdx.x; kt < n_kt; kt += blockDim.x) row[kt] = 0u;
   __syncthreads();
   const int t1 = row_ptr[blockIdx.x + 1];
@@ -64,8 +42,7 @@ cudaError_t launch_bwd_tc(const void *Q, const void *K, const void *V, const voi
                           const ap_tiles &t, void *dQ, void *dK, void *dV, void *workspace, int B, int H, int Lq,
                           int Lk, int d, int f16, float scale, cudaStream_t s) {
   unsigned *err = device_error_word();
-  int32_t *next = bwd::next_items();
-  if (!err || !next) return cudaErrorUnknown;
+  if (!err) return cudaErrorUnknown;
   const bool split = d == 128 && Lk % 8 == 0;
   bwd::RowsMaps rows;
   bwd::ColsMaps cols;
@@ -90,12 +67,11 @@ cudaError_t launch_bwd_tc(const void *Q, const void *K, const void *V, const voi
   a.plan.neg_l = static_cast<float *>(workspace);
   a.plan.dsum = a.plan.neg_l + (size_t)B * H * Lq;
   a.plan.table = reinterpret_cast<uint32_t *>(static_cast<char *>(workspace) + bwd::stats_bytes(B, H, Lq));
-  a.plan.next = next;
   a.B = B, a.H = H, a.Lq = Lq, a.Lk = Lk, a.d = d, a.f16 = f16, a.split = split ? 1 : 0;
   a.scale = scale;
   a.err = err;
   a.s = s;
-  bwd::table_kernel<<<H * t.n_qt, 128, 0, s>>>(t.row_ptr, t.col_idx, t.flags, t.groups, t.n_kt, a.plan.table, next);
+  bwd::table_kernel<<<H * t.n_qt, 128, 0, s>>>(t.row_ptr, t.col_idx, t.flags, t.groups, t.n_kt, a.plan.table);
   count_launches(1);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = bwd::launch_rows(rows, a);

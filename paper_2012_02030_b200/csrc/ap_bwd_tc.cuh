@@ -11,7 +11,6 @@ struct Plan {
   float *neg_l;     // [B*H][Lq]        -log2 of the row's sum of 2^(c S); -inf: no kept entry
   float *dsum;      // [B*H][Lq]        D_i = dO_i . O_i
   uint32_t *table;  // [H][n_qt][n_kt]  bits 0..23: list position of a tile; 24..31: its groups that keep an entry (0: not stored)
-  int32_t *next;    // [2]              next item to hand out (rows kernel, columns kernel)
 };
 
 struct RowsMaps {

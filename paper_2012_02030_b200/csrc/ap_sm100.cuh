@@ -124,6 +124,44 @@ struct Waiter {
   }
 };
 
+// Work items of a persistent kernel: the grid has a block per item, and a running block takes over blocks that have not
+// started (cluster launch control) instead of drawing numbers from a counter in global memory.  The hardware keeps
+// account, so calls share nothing, whatever streams or graphs they run in.
+struct alignas(16) TakeOver {
+  uint32_t answer[4];
+  uint64_t answered;  // an mbarrier of one arrival
+};
+
+// By one thread: asks for another block.  No request may follow an answer without a block.
+__device__ __forceinline__ void ask_block(TakeOver *t) {
+  mbar_arrive_expect_tx(&t->answered, 16);
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+                   smem_u32(t->answer)),
+               "r"(smem_u32(&t->answered))
+               : "memory");
+}
+
+// The block's index, or -1 where none was left; by any threads once `answered` has completed.  The fence puts these reads
+// before the answer to the next request.
+__device__ __forceinline__ int taken_block(TakeOver *t) {
+  uint32_t got, x;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      ".reg .b128 a;\n"
+      "ld.shared.b128 a, [%2];\n"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "mov.u32 %1, 0;\n"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, a;\n"
+      "fence.proxy.async.shared::cta;\n"
+      "}\n"
+      : "=r"(got), "=r"(x)
+      : "r"(smem_u32(t->answer))
+      : "memory");
+  return got ? (int)x : -1;
+}
+
 // True in exactly one lane of a fully converged warp.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;

@@ -1,0 +1,54 @@
+"""Calls that overlap: several streams, captured graphs, threads."""
+import pytest
+import torch
+
+from paper_2012_02030_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ap():
+    from paper_2012_02030_b200 import binding
+
+    assert torch.cuda.is_available()
+    return binding
+
+
+def _attention(ap, B, H, L, d, seed, keep=0.1, dtype=torch.bfloat16):
+    """Inputs of a backward call, its output buffers and its workspace."""
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    q, k, v, d_o = (torch.randn((B, H, L, d), generator=gen, device="cuda").to(dtype) for _ in range(4))
+    tiles = ap.Tiles(H, L, L)
+    ap.ap_mask_to_tiles(inputs.random_mask(H, L, L, keep, seed=seed, causal=True).cuda(), tiles)
+    out = ap.ap_sparse_attention_fwd(q, k, v, tiles)
+    ws = torch.empty(ap.ap_sparse_attention_bwd_workspace_bytes(B, H, L, L), dtype=torch.uint8, device="cuda")
+    return (q, k, v, out, d_o, tiles), [torch.empty_like(q) for _ in range(3)], ws
+
+
+def test_backward_replayed_beside_eager_calls(ap):
+    """A captured backward is replayed on one stream while an eager one runs on another, after enough calls in between that
+    any state handed out in rotation has come round: both give the bits that they give alone."""
+    side = torch.cuda.Stream()
+    args, grads, ws = _attention(ap, 8, 8, 1024, 64, 1)
+    args2, grads2, ws2 = _attention(ap, 8, 8, 1024, 64, 2)
+    tiny, tiny_grads, tiny_ws = _attention(ap, 1, 1, 16, 64, 3)
+    want = [t.clone() for t in ap.ap_sparse_attention_bwd(*args, *grads, workspace=ws)]
+    want2 = [t.clone() for t in ap.ap_sparse_attention_bwd(*args2, *grads2, workspace=ws2)]
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ap.ap_sparse_attention_bwd(*args, *grads, workspace=ws)
+    for _ in range(8):
+        for _ in range(1023):
+            ap.ap_sparse_attention_bwd(*tiny, *tiny_grads, workspace=tiny_ws)
+        for t in grads + grads2:
+            t.fill_(float("nan"))
+        torch.cuda.synchronize()
+        graph.replay()
+        with torch.cuda.stream(side):
+            ap.ap_sparse_attention_bwd(*args2, *grads2, workspace=ws2)
+        torch.cuda.synchronize()
+        for got, ref in zip(grads + grads2, want + want2):
+            assert torch.equal(got, ref)
+    assert ap.ap_device_status() == ap.AP_OK
