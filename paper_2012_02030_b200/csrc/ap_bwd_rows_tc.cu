@@ -345,7 +345,7 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
     const uint32_t base = smem_u32(smem);
     constexpr uint32_t idesc_dq = idesc_bf16_f32(128, D, false, true, kF16);
     uint32_t n_front = 0, n_back = 0;  // items finished by dP / by dQ
-    uint32_t info_front = 0u;
+    uint32_t info_front = 0u, sweep_round = 0u;
     bool ok = true;
     // C[128 x 16 ng] = A B^T
     auto issue_abt = [&](uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, int ng) {
@@ -393,8 +393,11 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
     // dQ of round g
     auto back = [&](uint32_t g, uint32_t info) {
       const bool stats = kF16 && (info & kInfoStats), first = (info & kInfoFirst) != 0u;
-      // the first round of an item overwrites dQ: the previous item's must have been read
-      if (first && !stats && n_back > 0) ok = wait(&sh->o_free, (n_back - 1u) & 1u);
+      // The first round of an item overwrites dQ: the previous item's must have been read.  A first sweep (fp16) writes no
+      // dQ, but its kRing-th round completes the barrier on which the finishing warps wait for the previous item's last dQ a
+      // second time: unless they have been there, that phase is lost to them.
+      sweep_round = first ? 0u : sweep_round + 1u;
+      if (sweep_round == (stats ? kRing - 1u : 0u) && n_back > 0) ok = wait(&sh->o_free, (n_back - 1u) & 1u);
       if (ok) ok = wait(&sh->ds_full[g & 1u], (g >> 1) & 1u);
       if (!ok) return;
       tc_fence_after_sync();

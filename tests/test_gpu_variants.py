@@ -175,3 +175,27 @@ def test_fp32_accumulate_key_rows_16_bytes_past_a_sector(ap, Lk):
     orc.accumulate(want, inputs.widen(q.cpu()), inputs.widen(k.cpu()), None, causal=False)
     tol = tp._acc_tolerance("f32")
     np.testing.assert_allclose(got[0].cpu().numpy(), want, rtol=tol["rtol"], atol=tol["atol"] * w.B)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_fp16_backward_many_items_of_few_rounds(ap, d):
+    """fp16 tensors sweep an item's rounds twice, the first time without a dQ: many items of one round each beside items of
+    several, so that a first sweep runs ahead of what reads out the item before."""
+    B, H, L = 24, 4, 640
+    w = W["tiny"].scaled(B=B, H=H, Lq=L, Lk=L, d=d, dtype="f16")
+    i, j = torch.arange(L)[:, None], torch.arange(L)[None, :]
+    few = (j < 4) | (i == j)                           # one or two rounds
+    many = (j % 8 == i % 8) & (i // 128 % 2 == 1) | few  # every other query tile: five rounds
+    mask = torch.stack([few, many, few, many]).to(torch.uint8)
+    q, k, v = (t.cuda() for t in inputs.eval_qkv(w))
+    d_o = torch.randn(q.shape, generator=torch.Generator(device="cuda").manual_seed(507), device="cuda").to(q.dtype)
+    tiles = ap.Tiles(H, L, L)
+    ap.ap_mask_to_tiles(mask.cuda(), tiles)
+    out = ap.ap_sparse_attention_fwd(q, k, v, tiles)
+    for _ in range(20):
+        got = ap.ap_sparse_attention_bwd(q, k, v, out, d_o, tiles)
+    assert ap.ap_device_status() == ap.AP_OK
+    for b in (0, B - 1):
+        want = orc.attention_bwd(*(inputs.widen(t[b:b + 1].cpu()) for t in (q, k, v, d_o)), mask.numpy())
+        for x, ref in zip(got, want):
+            assert np.linalg.norm(x[b].float().cpu().numpy() - ref[0]) <= 2e-3 * np.linalg.norm(ref)
