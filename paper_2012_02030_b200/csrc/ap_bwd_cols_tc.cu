@@ -98,18 +98,6 @@ struct Cfg {
   static_assert(kSmemBytes > 114 * 1024, "one CTA per SM: all of TMEM is taken");
 };
 
-// 32 x 32 bit transpose across a warp: lane i's bit j becomes lane j's bit i.
-__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) {
-    const uint32_t low = s == 16 ? 0x0000ffffu : s == 8 ? 0x00ff00ffu : s == 4 ? 0x0f0f0f0fu : s == 2 ? 0x33333333u
-                                                                                                  : 0x55555555u;
-    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
-    x = (lane & s) ? ((y >> s) & low) | (x & ~low) : (x & low) | ((y & low) << s);
-  }
-  return x;
-}
-
 // 4 bytes global -> shared memory, asynchronously.
 __device__ __forceinline__ void cp_async4(void *smem_dst, const void *gmem_src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(smem_dst)), "l"(gmem_src) : "memory");

@@ -62,6 +62,18 @@ struct DebugKnobs {
 };
 DebugKnobs debug_knobs();
 
+// 32 x 32 bit transpose across a warp: lane i's bit j becomes lane j's bit i.
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const uint32_t low = s == 16 ? 0x0000ffffu : s == 8 ? 0x00ff00ffu : s == 4 ? 0x0f0f0f0fu : s == 2 ? 0x33333333u
+                                                                                                  : 0x55555555u;
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
+    x = (lane & s) ? ((y >> s) & low) | (x & ~low) : (x & low) | ((y & low) << s);
+  }
+  return x;
+}
+
 // SMs of the current device (0 if it cannot be queried).
 int sm_count();
 

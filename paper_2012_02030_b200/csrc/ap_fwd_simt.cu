@@ -1,18 +1,22 @@
 // Masked attention of Section 3.2 on CUDA cores (fp32 FMA), for fp32 tensors.
 //
-// fwd_simt_kernel: one CTA takes R query rows of one (b, h) through the stored tiles of their list row.
-// Per tile: S = Q K^T with a register tile per thread, S (pruned entries -inf) to shared memory, a warp
-// per row for maximum, weights and sum, O += P V with a register tile per thread and the tile's keys
-// split over groups of threads (summed once, at the end).  K and V rows arrive by asynchronous 16-byte
-// copies; the next tile's K is copied during the softmax and P V, its V during the next S.  Pruned entries
-// get weight exactly 0; rows that never see a kept entry output zeros.
+// fwd_simt_kernel: one CTA takes R query rows of one (b, h) through the keys that any of them keeps.  Planning: the R rows'
+// words of the next two tiles' bitmaps, transposed by shuffles, give every key the rows that keep it; keys kept by none
+// are left out, the others are appended to a list in shared memory.  Work: a batch of 64 or 128 listed keys at a time, whatever
+// tiles they come from.  S = Q K^T with a register tile per thread, S to shared memory, a warp's share of the rows for maxima,
+// weights and sums, O += P V with a register tile per thread and the batch's keys split over groups of threads (summed
+// once, at the end).  K and V rows arrive by asynchronous 16-byte copies; the next batch's K is copied during the
+// softmax and P V, this one's V during its S, and the next batch is planned meanwhile.  Pruned entries get weight exactly 0;
+// rows that never see a kept entry output zeros.
 //
-// What bounds it: at small shapes the chain copy -> S -> softmax -> P V of one tile (a few
-// microseconds), so R goes down to 8 until the SMs are covered; at large ones shared-memory bandwidth
-// (S: KT + RT 16-byte reads per 4 KT RT FMAs).  The version with two threads per query row that walked the
-// kept keys one by one took 24 us where a toy model's 4 (head, sequence) pairs of 128 x 128 gave it 4
-// CTAs of 128 dependent steps each; see kRowsRule for what R measured.
+// What bounds it: at small shapes the chain plan -> copy -> S -> softmax -> P V of one batch (a few microseconds), so R
+// goes down to 8 until the SMs are covered; at large ones the products, at half of the FMA rate, and the reductions of
+// the softmax.  Without the list, every key of a stored tile copied and multiplied: 32 x 16 heads x 512 x 64 causal 600 us at
+// 5 % kept, 729 at 50 %, 737 unpruned (170, 452, 642 now); with two threads per query row that walked the kept keys one by
+// one: 227, 792, 1069.
 #include <math_constants.h>
+
+#include <type_traits>
 
 #include "ap_common.cuh"
 
@@ -20,7 +24,7 @@ namespace ap {
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kEntmaxThreads = 256;
 
 template <typename T>
 __device__ __forceinline__ float4 load4(const T *p);
@@ -54,189 +58,316 @@ __device__ __forceinline__ float4 *chunk_at(float *base, int r, int c) {
   return reinterpret_cast<float4 *>(base + r * D) + (c ^ (r & 7));
 }
 
-template <int D, int R>
-struct SimtCfg {
-  // S: a warp computes (4 RT) x (8 KT) of the R x 128 scores, lane = 4 row lanes x 8 key lanes
-  static constexpr int RT = R == 32 ? 4 : 2;
-  static constexpr int KT = R == 8 ? 2 : 4;
-  static_assert((R / (4 * RT)) * (kTile / (8 * KT)) == kThreads / 32, "eight warps cover S");
-  // P V: a thread owns PR rows x 4 columns; D/4 column lanes, R/PR row groups, the rest splits the keys
-  static constexpr int PR = R == 32 ? 4 : 2;
-  static constexpr int kSplit = kThreads / ((D / 4) * (R / PR));
-  static_assert(kSplit >= 1 && kTile % (4 * kSplit) == 0, "keys split evenly");
-  static constexpr int kPitch = kTile + 4;  // floats per row of S
-  static constexpr int kKOff = R * D, kVOff = kKOff + kTile * D, kSOff = kVOff + kTile * D,
-                       kAlphaOff = kSOff + R * kPitch, kFloats = kAlphaOff + 2 * R;
-  static_assert(kSplit * R * D <= 2 * kTile * D, "the partial outputs fit over K and V");
+// N values per lane, each combined over the 32 lanes by op: every lane gets the result of value lane / (32 / N).  (One by one they
+// would take 5 N exchanges, this way N - 1 + log2(32 / N).)
+template <int N, class Op>
+__device__ __forceinline__ float reduce_rows(float (&v)[N], int lane, Op op) {
+#pragma unroll
+  for (int n = N, o = 16; o > 0; o >>= 1) {
+    if (n > 1) {
+      n >>= 1;
+#pragma unroll
+      for (int x = 0; x < N / 2; ++x)
+        if (x < n) {
+          const bool upper = (lane & o) != 0;
+          const float there = __shfl_xor_sync(0xffffffffu, upper ? v[x] : v[x + n], o);
+          v[x] = op(upper ? v[x + n] : v[x], there);
+        }
+    } else {
+      v[0] = op(v[0], __shfl_xor_sync(0xffffffffu, v[0], o));
+    }
+  }
+  return v[0];
+}
+
+template <class T, int N>
+struct alignas(sizeof(T) * N) Run {
+  T v[N];
 };
 
 template <int D, int R>
-__global__ void __launch_bounds__(kThreads) fwd_simt_kernel(const float *__restrict__ Q, const float *__restrict__ K,
-                                                            const float *__restrict__ V,
-                                                            const int32_t *__restrict__ row_ptr,
-                                                            const int32_t *__restrict__ col_idx,
-                                                            const uint8_t *__restrict__ flags,
-                                                            const uint32_t *__restrict__ bitmap,
-                                                            float *__restrict__ O, int H, int Lq, int Lk, int n_qt,
-                                                            int n_rt, float scale) {
+struct SimtCfg {
+  // Four CTAs of four warps with 64 keys at a time fill an SM better than two of eight with 128, but d = 128 has no registers
+  // for that and eight rows (a grid that does not fill the GPU) are done sooner by eight warps: 8 x 12 heads x 512 x 64, 5 and
+  // 50 % kept, 63 and 257 us with eight warps and 128 keys, 47 and 263 with 64 keys, 45 and 250 with four warps (before the
+  // reductions over rows were combined: 41 and 224 now).
+  static constexpr int kThreads = D == 64 && R > 8 ? 128 : 256, kWarps = kThreads / 32;
+  static constexpr int kBatch = D == 64 && R == 8 ? 128 : 64;  // keys worked on at a time
+  static constexpr int kCtas = D == 64 && R > 8 ? 4 : 2;       // per SM
+  // S: a warp computes (4 RT) x (8 KT) of the R x kBatch scores, lane = 4 row lanes x 8 key lanes
+  static constexpr int RT = R == 32 ? 4 : 2;
+  static constexpr int KT = (R / (4 * RT)) * (kBatch / 8) / kWarps;
+  static_assert((R / (4 * RT)) * (kBatch / (8 * KT)) == kWarps, "the warps cover S");
+  static constexpr int kMyKeys = kBatch / 32;  // softmax: consecutive keys of a lane
+  // P V: a thread owns PR rows x 4 columns; D/4 column lanes, R/PR row groups, the rest splits the keys
+  static constexpr int PR = R == 32 ? 4 : 2;
+  static constexpr int kSplit = kThreads / ((D / 4) * (R / PR));
+  static_assert(kSplit >= 1 && kBatch % (4 * kSplit) == 0, "keys split evenly");
+  static constexpr int kPitch = kBatch + 4;  // floats per row of S
+  // a planning step adds up to 256 keys to at most 2 kBatch - 1
+  static constexpr int kList = 512;
+  static_assert(2 * kBatch - 1 + 256 <= kList && kList % kBatch == 0, "the list holds what is planned ahead");
+  static constexpr int kKOff = R * D, kVOff = kKOff + kBatch * D, kSOff = kVOff + kBatch * D,
+                       kAlphaOff = kSOff + R * kPitch, kListOff = kAlphaOff + 2 * R, kFloats = kListOff + 2 * kList;
+  static_assert(kSplit * R * D <= 2 * kBatch * D, "the partial outputs fit over K and V");
+};
+
+template <int D, int R>
+__global__ void __launch_bounds__((SimtCfg<D, R>::kThreads), (SimtCfg<D, R>::kCtas))
+fwd_simt_kernel(const float *__restrict__ Q, const float *__restrict__ K, const float *__restrict__ V,
+                const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col_idx,
+                const uint8_t *__restrict__ flags, const uint32_t *__restrict__ bitmap, float *__restrict__ O, int H,
+                int Lq, int Lk, int n_qt, int n_rt, float scale) {
   using C = SimtCfg<D, R>;
+  constexpr int kThreads = C::kThreads;
   constexpr int CH = D / 4;  // 16-byte chunks per row
   extern __shared__ __align__(16) float smem[];
+  __shared__ int counts[2][8];
   float *q_s = smem, *k_s = smem + C::kKOff, *v_s = smem + C::kVOff, *s_s = smem + C::kSOff,
         *alpha_s = smem + C::kAlphaOff, *l_s = alpha_s + R;
+  // the kept keys of these rows in list order: the key, and a bit for each row that keeps it
+  uint32_t *list_key = reinterpret_cast<uint32_t *>(smem + C::kListOff), *list_rows = list_key + C::kList;
   const int rt = blockIdx.x % n_rt;
   const size_t bh = blockIdx.x / n_rt;
   const int i0 = rt * R, qt = i0 / kTile, h = (int)(bh % H);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t_begin = row_ptr[h * n_qt + qt], t_end = row_ptr[h * n_qt + qt + 1];
 
-  auto copy_tile = [&](float *dst, const float *src, int kt) {
-    for (int e = threadIdx.x; e < kTile * CH; e += kThreads) {
-      const int jj = e / CH, c = e % CH, j = kt * kTile + jj;
-      const bool valid = j < Lk;
-      copy16(reinterpret_cast<float *>(chunk_at<D>(dst, jj, c)), src + (bh * Lk + (valid ? j : 0)) * D + 4 * c, valid);
-    }
-  };
-  int kt_next = t_begin < t_end ? col_idx[t_begin] : 0;
   for (int e = threadIdx.x; e < R * CH; e += kThreads) {
     const int r = e / CH, c = e % CH, i = i0 + r;
     const bool valid = i < Lq;
     copy16(reinterpret_cast<float *>(chunk_at<D>(q_s, r, c)), Q + (bh * Lq + (valid ? i : 0)) * D + 4 * c, valid);
   }
-  if (t_begin < t_end) copy_tile(k_s, K, kt_next);
-  copy_commit();
-
   // scores: this thread's rows sr + 4 x and keys sk + 8 y
-  constexpr int kKeyWarps = kTile / (8 * C::KT);
-  const int sr = (warp / kKeyWarps) * 4 * C::RT + (lane >> 3), sk = (warp % kKeyWarps) * 8 * C::KT + (lane & 7);
-  // softmax: this warp's rows, R / 8 of them; a lane owns four consecutive keys
-  constexpr int kMyRows = R / 8;
-  float m[kMyRows], l[kMyRows];
-#pragma unroll
-  for (int x = 0; x < kMyRows; ++x) m[x] = -CUDART_INF_F, l[x] = 0.f;
+  constexpr int kKeyWarps = C::kBatch / (8 * C::KT);
+  const int s_key0 = (warp % kKeyWarps) * 8 * C::KT;  // first key of the warp
+  const int sr = (warp / kKeyWarps) * 4 * C::RT + (lane >> 3), sk = s_key0 + (lane & 7);
+  constexpr int kMyRows = R / C::kWarps, kRowLanes = 32 / kMyRows;  // softmax: rows of a warp
   // P V: column chunk pc, rows pr .. pr + PR - 1, keys of split part ps
   const int pc = threadIdx.x % CH, pr = (threadIdx.x / CH) % (R / C::PR) * C::PR, ps = threadIdx.x / (CH * (R / C::PR));
-  float4 o[C::PR];
-#pragma unroll
-  for (int x = 0; x < C::PR; ++x) o[x] = make_float4(0.f, 0.f, 0.f, 0.f);
 
-  for (int t = t_begin; t < t_end; ++t) {
-    const int kt = kt_next;
-    copy_tile(v_s, V, kt);  // (every thread is past the last P V, see the barrier at the loop's end)
-    copy_commit();
-    if (t + 1 < t_end) kt_next = col_idx[t + 1];
-    const bool full = flags[t] & 1;
-    uint32_t keep[kMyRows];
+  // A pruned entry's weight is -0 (a kept one's that underflows is +0).  Where V holds infinities or NaNs, its product is
+  // not zero: a CTA that finds a NaN among its outputs works them out once more with `careful`, which leaves the products
+  // of pruned entries out.
+  bool careful = false;
+#pragma unroll 1
+  while (true) {
+    // Planning: two tiles a step, a warp a 32-column word of one of them (or of both), lane = row; transposed, lane = column.
+    constexpr int kWords = 256 / kThreads;  // per warp
+    int t_plan = t_begin, tail = 0, step = 0, ahead_kt[kWords];
+    uint32_t ahead_word[kWords];
+    auto look_ahead = [&]() {  // (raw loads, used a step later)
 #pragma unroll
-    for (int x = 0; x < kMyRows; ++x) {
-      const int r = (i0 & (kTile - 1)) + warp * kMyRows + x;
-      const uint32_t w = full ? 0xffffffffu : bitmap[(size_t)t * kBitmapWords + 4 * r + (lane >> 3)];
-      keep[x] = w >> (4 * (lane & 7)) & 15u;
-    }
-    copy_wait<1>();  // K of this tile (and Q)
-    __syncthreads();
-    float s[C::RT][C::KT];
-#pragma unroll
-    for (int x = 0; x < C::RT; ++x)
-#pragma unroll
-      for (int y = 0; y < C::KT; ++y) s[x][y] = 0.f;
-#pragma unroll 4
-    for (int c = 0; c < CH; ++c) {
-      float4 qv[C::RT], kv[C::KT];
-#pragma unroll
-      for (int x = 0; x < C::RT; ++x) qv[x] = *chunk_at<D>(q_s, sr + 4 * x, c);
-#pragma unroll
-      for (int y = 0; y < C::KT; ++y) kv[y] = *chunk_at<D>(k_s, sk + 8 * y, c);
-#pragma unroll
-      for (int x = 0; x < C::RT; ++x)
-#pragma unroll
-        for (int y = 0; y < C::KT; ++y) {
-          s[x][y] = fmaf(qv[x].x, kv[y].x, s[x][y]);
-          s[x][y] = fmaf(qv[x].y, kv[y].y, s[x][y]);
-          s[x][y] = fmaf(qv[x].z, kv[y].z, s[x][y]);
-          s[x][y] = fmaf(qv[x].w, kv[y].w, s[x][y]);
-        }
-    }
-#pragma unroll
-    for (int x = 0; x < C::RT; ++x)
-#pragma unroll
-      for (int y = 0; y < C::KT; ++y) s_s[(sr + 4 * x) * C::kPitch + sk + 8 * y] = s[x][y] * scale;
-    __syncthreads();
-    if (t + 1 < t_end) copy_tile(k_s, K, kt_next);
-    copy_commit();
-#pragma unroll
-    for (int x = 0; x < kMyRows; ++x) {
-      const int r = warp * kMyRows + x;
-      float4 *cell = reinterpret_cast<float4 *>(s_s + r * C::kPitch + 4 * lane);
-      float4 v = *cell;
-      v.x = keep[x] & 1u ? v.x : -CUDART_INF_F;
-      v.y = keep[x] & 2u ? v.y : -CUDART_INF_F;
-      v.z = keep[x] & 4u ? v.z : -CUDART_INF_F;
-      v.w = keep[x] & 8u ? v.w : -CUDART_INF_F;
-      float top = fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
-      const float m_new = fmaxf(m[x], top);
-      const float ref = m_new == -CUDART_INF_F ? 0.f : m_new;
-      const float alpha = expf(m[x] - ref);  // exp(-inf) = 0 before the row's first kept entry
-      m[x] = m_new;
-      v.x = expf(v.x - ref), v.y = expf(v.y - ref), v.z = expf(v.z - ref), v.w = expf(v.w - ref);
-      *cell = v;
-      float sum = (v.x + v.y) + (v.z + v.w);
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
-      l[x] = l[x] * alpha + sum;
-      if (lane == 0) alpha_s[r] = alpha;
-    }
-    copy_wait<1>();  // V of this tile
-    __syncthreads();
-#pragma unroll
-    for (int x = 0; x < C::PR; ++x) {
-      const float alpha = alpha_s[pr + x];
-      o[x].x *= alpha, o[x].y *= alpha, o[x].z *= alpha, o[x].w *= alpha;
-    }
-    constexpr int kPart = kTile / C::kSplit;
-#pragma unroll 2
-    for (int j = ps * kPart; j < (ps + 1) * kPart; j += 4) {
-      float4 p[C::PR];
-#pragma unroll
-      for (int x = 0; x < C::PR; ++x) p[x] = *reinterpret_cast<const float4 *>(s_s + (pr + x) * C::kPitch + j);
-#pragma unroll
-      for (int y = 0; y < 4; ++y) {
-        const float4 v = *chunk_at<D>(v_s, j + y, pc);
-#pragma unroll
-        for (int x = 0; x < C::PR; ++x) {
-          const float w = y == 0 ? p[x].x : y == 1 ? p[x].y : y == 2 ? p[x].z : p[x].w;
-          o[x].x = fmaf(w, v.x, o[x].x), o[x].y = fmaf(w, v.y, o[x].y);
-          o[x].z = fmaf(w, v.z, o[x].z), o[x].w = fmaf(w, v.w, o[x].w);
+      for (int u = 0; u < kWords; ++u) {
+        const int t = t_plan + (warp >> 2) + u;
+        ahead_word[u] = 0u;
+        ahead_kt[u] = 0;
+        if (t < t_end) {
+          ahead_kt[u] = col_idx[t];
+          const bool full = flags[t] & 1;
+          if (lane < R)
+            ahead_word[u] = full ? 0xffffffffu : bitmap[(size_t)t * kBitmapWords + 4 * ((i0 & (kTile - 1)) + lane) + (warp & 3)];
         }
       }
+    };
+    auto plan = [&]() {
+      uint32_t key[kWords], rows[kWords], vote[kWords];
+      int *n = counts[step++ & 1];
+#pragma unroll
+      for (int u = 0; u < kWords; ++u) {
+        rows[u] = transpose32(ahead_word[u], lane);
+        key[u] = (uint32_t)(ahead_kt[u] * kTile + 32 * (warp & 3) + lane);
+        vote[u] = __ballot_sync(0xffffffffu, rows[u] != 0u);
+        if (lane == 0) n[warp + 4 * u] = __popc(vote[u]);
+      }
+      t_plan += 2;
+      look_ahead();
+      __syncthreads();
+      int before[kWords] = {}, all = 0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) {
+#pragma unroll
+        for (int u = 0; u < kWords; ++u) before[u] += w < warp + 4 * u ? n[w] : 0;
+        all += n[w];
+      }
+#pragma unroll
+      for (int u = 0; u < kWords; ++u)
+        if (rows[u] != 0u) {
+          const int at = (tail + before[u] + __popc(vote[u] & ((1u << lane) - 1u))) & (C::kList - 1);
+          list_key[at] = key[u];
+          list_rows[at] = rows[u];
+        }
+      tail += all;
+    };
+    look_ahead();
+    // Rows of `src` that belong to the n keys from list position `first` on; rows [n, n_zero) become zeros.
+    auto copy_rows = [&](float *dst, const float *src, int first, int n, int n_zero) {
+      const int c = threadIdx.x % CH, j0 = threadIdx.x / CH;
+      const float *from = src + bh * Lk * D + 4 * c;
+      constexpr int kStep = kThreads / CH;
+      if (n == C::kBatch) {
+        const uint32_t *keys = list_key + (first & (C::kList - 1)) + j0;
+#pragma unroll
+        for (int x = 0; x < C::kBatch / kStep; ++x)
+          copy16(reinterpret_cast<float *>(chunk_at<D>(dst, j0 + x * kStep, c)), from + (size_t)keys[x * kStep] * D, true);
+      } else {
+        for (int jj = j0; jj < n_zero; jj += kStep) {
+          const bool valid = jj < n;
+          const size_t j = valid ? list_key[(first + jj) & (C::kList - 1)] : 0u;
+          copy16(reinterpret_cast<float *>(chunk_at<D>(dst, jj, c)), from + j * D, valid);
+        }
+      }
+    };
+    while (tail < C::kBatch && t_plan < t_end) plan();
+    __syncthreads();
+    int head = 0, nb = min(C::kBatch, tail);
+    copy_rows(k_s, K, 0, nb, nb);
+    copy_commit();
+
+    float m = -CUDART_INF_F, l = 0.f;  // of row lane / kRowLanes of the warp's
+    float4 o[C::PR];
+#pragma unroll
+    for (int x = 0; x < C::PR; ++x) o[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+
+#pragma unroll 1
+    while (nb > 0) {
+      const int part = (nb + 4 * C::kSplit - 1) / (4 * C::kSplit) * 4;  // keys of a split part of P V
+      copy_rows(v_s, V, head, nb, part * C::kSplit);  // (every thread is past the last P V, see the barrier at the loop's end)
+      copy_commit();
+      while (tail - head - nb < C::kBatch && t_plan < t_end) plan();  // the next batch
+      copy_wait<1>();  // K of this batch (and Q)
+      __syncthreads();
+      if (s_key0 < nb) {
+        float s[C::RT][C::KT];
+#pragma unroll
+        for (int x = 0; x < C::RT; ++x)
+#pragma unroll
+          for (int y = 0; y < C::KT; ++y) s[x][y] = 0.f;
+#pragma unroll 4
+        for (int c = 0; c < CH; ++c) {
+          float4 qv[C::RT], kv[C::KT];
+#pragma unroll
+          for (int x = 0; x < C::RT; ++x) qv[x] = *chunk_at<D>(q_s, sr + 4 * x, c);
+#pragma unroll
+          for (int y = 0; y < C::KT; ++y) kv[y] = *chunk_at<D>(k_s, sk + 8 * y, c);
+#pragma unroll
+          for (int x = 0; x < C::RT; ++x)
+#pragma unroll
+            for (int y = 0; y < C::KT; ++y) {
+              s[x][y] = fmaf(qv[x].x, kv[y].x, s[x][y]);
+              s[x][y] = fmaf(qv[x].y, kv[y].y, s[x][y]);
+              s[x][y] = fmaf(qv[x].z, kv[y].z, s[x][y]);
+              s[x][y] = fmaf(qv[x].w, kv[y].w, s[x][y]);
+            }
+        }
+#pragma unroll
+        for (int x = 0; x < C::RT; ++x)
+#pragma unroll
+          for (int y = 0; y < C::KT; ++y) s_s[(sr + 4 * x) * C::kPitch + sk + 8 * y] = s[x][y] * scale;
+      }
+      __syncthreads();
+      const int n_next = min(C::kBatch, tail - head - nb);
+      copy_rows(k_s, K, head + nb, n_next, n_next);
+      copy_commit();
+      using Rows = Run<uint32_t, C::kMyKeys>;
+      using Keys = Run<float, C::kMyKeys>;
+      const int my_key = C::kMyKeys * lane;  // (batches start at multiples of their size)
+      Rows rows = *reinterpret_cast<const Rows *>(list_rows + (head & (C::kList - 1)) + my_key);
+#pragma unroll
+      for (int y = 0; y < C::kMyKeys; ++y) rows.v[y] = my_key + y < nb ? rows.v[y] : 0u;
+      float *my_s = s_s + warp * kMyRows * C::kPitch + my_key;
+      Keys w[kMyRows];
+      float top[kMyRows], sum[kMyRows];
+#pragma unroll
+      for (int x = 0; x < kMyRows; ++x) {
+        w[x] = *reinterpret_cast<const Keys *>(my_s + x * C::kPitch);
+        top[x] = -CUDART_INF_F;
+#pragma unroll
+        for (int y = 0; y < C::kMyKeys; ++y) {
+          w[x].v[y] = (rows.v[y] >> (warp * kMyRows + x)) & 1u ? w[x].v[y] : -CUDART_INF_F;
+          top[x] = fmaxf(top[x], w[x].v[y]);
+        }
+      }
+      const float m_new = fmaxf(m, reduce_rows<kMyRows>(top, lane, [](float a, float b) { return fmaxf(a, b); }));
+      const float ref = m_new == -CUDART_INF_F ? 0.f : m_new;
+      const float alpha = expf(m - ref);  // exp(-inf) = 0 before the row's first kept entry
+      m = m_new;
+#pragma unroll
+      for (int x = 0; x < kMyRows; ++x) {
+        const float ref_x = __shfl_sync(0xffffffffu, ref, x * kRowLanes);
+        sum[x] = 0.f;
+#pragma unroll
+        for (int y = 0; y < C::kMyKeys; ++y) {
+          w[x].v[y] = (rows.v[y] >> (warp * kMyRows + x)) & 1u ? expf(w[x].v[y] - ref_x) : -0.f;
+          sum[x] += w[x].v[y];
+        }
+        *reinterpret_cast<Keys *>(my_s + x * C::kPitch) = w[x];
+      }
+      l = l * alpha + reduce_rows<kMyRows>(sum, lane, [](float a, float b) { return a + b; });
+      if (lane % kRowLanes == 0) alpha_s[warp * kMyRows + lane / kRowLanes] = alpha;
+      copy_wait<1>();  // V of this batch
+      __syncthreads();
+#pragma unroll
+      for (int x = 0; x < C::PR; ++x) {
+        const float alpha = alpha_s[pr + x];
+        o[x].x *= alpha, o[x].y *= alpha, o[x].z *= alpha, o[x].w *= alpha;
+      }
+      auto add = [&](auto with_care, int from, int n) {
+#pragma unroll 2
+        for (int j = from; j < from + n; j += 4) {
+          float4 p[C::PR];
+#pragma unroll
+          for (int x = 0; x < C::PR; ++x) p[x] = *reinterpret_cast<const float4 *>(s_s + (pr + x) * C::kPitch + j);
+#pragma unroll
+          for (int y = 0; y < 4; ++y) {
+            const float4 v = *chunk_at<D>(v_s, j + y, pc);
+#pragma unroll
+            for (int x = 0; x < C::PR; ++x) {
+              const float w = y == 0 ? p[x].x : y == 1 ? p[x].y : y == 2 ? p[x].z : p[x].w;
+              if (decltype(with_care)::value && signbit(w)) continue;
+              o[x].x = fmaf(w, v.x, o[x].x), o[x].y = fmaf(w, v.y, o[x].y);
+              o[x].z = fmaf(w, v.z, o[x].z), o[x].w = fmaf(w, v.w, o[x].w);
+            }
+          }
+        }
+      };
+      constexpr int kPart = C::kBatch / C::kSplit;
+      if (careful)
+        add(std::true_type{}, ps * part, part);
+      else if (nb == C::kBatch)
+        add(std::false_type{}, ps * kPart, kPart);
+      else
+        add(std::false_type{}, ps * part, part);
+      __syncthreads();  // S, alpha, V and this batch's place in the list are read
+      head += nb;
+      nb = n_next;
     }
-    __syncthreads();  // S, alpha and V of this tile are read
-  }
-  // sums of the key parts (over K and V), then the division by l
-  copy_wait<0>();
-  float *part = k_s;
+    // sums of the key parts (over K and V), then the division by l
+    copy_wait<0>();
+    float *part = k_s;
 #pragma unroll
-  for (int x = 0; x < C::PR; ++x)
-    *reinterpret_cast<float4 *>(part + ((ps * R) + pr + x) * D + 4 * pc) = o[x];
+    for (int x = 0; x < C::PR; ++x)
+      *reinterpret_cast<float4 *>(part + ((ps * R) + pr + x) * D + 4 * pc) = o[x];
+    if (lane % kRowLanes == 0) l_s[warp * kMyRows + lane / kRowLanes] = l;
+    __syncthreads();
+    bool nan = false;
+    for (int e = threadIdx.x; e < R * CH; e += kThreads) {
+      const int r = e / CH, c = e % CH;
+      if (i0 + r >= Lq) continue;
+      float4 sum = *reinterpret_cast<const float4 *>(part + r * D + 4 * c);
 #pragma unroll
-  for (int x = 0; x < kMyRows; ++x)
-    if (lane == 0) l_s[warp * kMyRows + x] = l[x];
-  __syncthreads();
-  for (int e = threadIdx.x; e < R * CH; e += kThreads) {
-    const int r = e / CH, c = e % CH;
-    if (i0 + r >= Lq) continue;
-    float4 sum = *reinterpret_cast<const float4 *>(part + r * D + 4 * c);
-#pragma unroll
-    for (int y = 1; y < C::kSplit; ++y) {
-      const float4 v = *reinterpret_cast<const float4 *>(part + (y * R + r) * D + 4 * c);
-      sum.x += v.x, sum.y += v.y, sum.z += v.z, sum.w += v.w;
+      for (int y = 1; y < C::kSplit; ++y) {
+        const float4 v = *reinterpret_cast<const float4 *>(part + (y * R + r) * D + 4 * c);
+        sum.x += v.x, sum.y += v.y, sum.z += v.z, sum.w += v.w;
+      }
+      const float lr = l_s[r];
+      float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (lr > 0.f) out = make_float4(sum.x / lr, sum.y / lr, sum.z / lr, sum.w / lr);
+      nan = nan || out.x != out.x || out.y != out.y || out.z != out.z || out.w != out.w;
+      *reinterpret_cast<float4 *>(O + (bh * Lq + i0 + r) * D + 4 * c) = out;
     }
-    const float lr = l_s[r];
-    float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (lr > 0.f) out = make_float4(sum.x / lr, sum.y / lr, sum.z / lr, sum.w / lr);
-    *reinterpret_cast<float4 *>(O + (bh * Lq + i0 + r) * D + 4 * c) = out;
+    if (careful || !__syncthreads_or(nan ? 1 : 0)) break;
+    careful = true;
   }
 }
 
@@ -250,7 +381,7 @@ __global__ void __launch_bounds__(kThreads) fwd_simt_kernel(const float *__restr
 // 5e-7 max(1, |tau|) (at most 30 sweeps), then the sweep that forms the weights and adds p V.
 // Both threads of a row see the same scores and keep the same statistics.
 template <typename T, int D>
-__global__ void __launch_bounds__(kThreads) fwd_entmax_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K,
+__global__ void __launch_bounds__(kEntmaxThreads) fwd_entmax_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K,
                                                                    const T *__restrict__ V,
                                                                    const int32_t *__restrict__ row_ptr,
                                                                    const int32_t *__restrict__ col_idx,
@@ -283,7 +414,7 @@ __global__ void __launch_bounds__(kThreads) fwd_entmax_simt_kernel(const T *__re
     for (int t = t_begin; t < t_end; ++t) {
       const int kt = col_idx[t];
       __syncthreads();  // previous tile fully consumed
-      for (int e = threadIdx.x; e < kTile * D / 4; e += kThreads) {
+      for (int e = threadIdx.x; e < kTile * D / 4; e += kEntmaxThreads) {
         const int jj = e / (D / 4), c = e % (D / 4);
         const int j = kt * kTile + jj;
         float4 kv = make_float4(0.f, 0.f, 0.f, 0.f), vv = kv;
@@ -374,7 +505,7 @@ cudaError_t launch_entmax(const void *Q, const void *K, const void *V, const ap_
   auto kern = fwd_entmax_simt_kernel<T, D>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<B * H * t.n_qt, kThreads, smem, s>>>(static_cast<const T *>(Q), static_cast<const T *>(K),
+  kern<<<B * H * t.n_qt, kEntmaxThreads, smem, s>>>(static_cast<const T *>(Q), static_cast<const T *>(K),
                                               static_cast<const T *>(V), t.row_ptr, t.col_idx, t.flags, t.bitmap,
                                               static_cast<T *>(O), H, Lq, Lk, t.n_qt, 0.5f * scale);
   count_launches(1);
@@ -389,7 +520,7 @@ cudaError_t launch_rows(const void *Q, const void *K, const void *V, const ap_ti
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int n_rt = ceil_div(Lq, R);
-  kern<<<(unsigned)((int64_t)B * H * n_rt), kThreads, smem, s>>>(
+  kern<<<(unsigned)((int64_t)B * H * n_rt), SimtCfg<D, R>::kThreads, smem, s>>>(
       static_cast<const float *>(Q), static_cast<const float *>(K), static_cast<const float *>(V), t.row_ptr, t.col_idx,
       t.flags, t.bitmap, static_cast<float *>(O), H, Lq, Lk, t.n_qt, n_rt, scale);
   count_launches(1);

@@ -199,3 +199,42 @@ def test_fp16_backward_many_items_of_few_rounds(ap, d):
         want = orc.attention_bwd(*(inputs.widen(t[b:b + 1].cpu()) for t in (q, k, v, d_o)), mask.numpy())
         for x, ref in zip(got, want):
             assert np.linalg.norm(x[b].float().cpu().numpy() - ref[0]) <= 2e-3 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,Lq,Lk,causal,keep", [(4, 16, 256, 700, True, 0.02),   # 32 rows per block, few keys of many tiles
+                                                   (4, 16, 200, 200, True, 1.0),    # ... every key of the domain
+                                                   (5, 16, 33, 1030, False, 0.01),  # 8 rows: most blocks keep less than a batch
+                                                   (9, 16, 40, 129, False, 0.5)])   # 16 rows, one key in a tile of its own
+def test_fp32_forward_batches_of_kept_keys(ap, d, B, H, Lq, Lk, causal, keep):
+    """Keys kept by a block of rows, gathered from several tiles into batches: sparse and dense lists, partial batches."""
+    w = W["tiny"].scaled(B=B, H=H, Lq=Lq, Lk=Lk, d=d, dtype="f32")
+    mask = inputs.random_mask(H, Lq, Lk, keep, seed=508, empty_rows=(5,), causal=causal)
+    mask[:, :, -1] = mask[:, :, -2]
+    q, k, v = inputs.eval_qkv(w)
+    tiles = ap.Tiles(H, Lq, Lk)
+    ap.ap_mask_to_tiles(mask.cuda(), tiles)
+    out = ap.ap_sparse_attention_fwd(q.cuda(), k.cuda(), v.cuda(), tiles, torch.full_like(q, float("nan"), device="cuda"))
+    assert ap.ap_device_status() == ap.AP_OK
+    ref = orc.attention_fwd(inputs.widen(q), inputs.widen(k), inputs.widen(v), mask.numpy())
+    pu.assert_close_attention(out, ref, "f32", str((B, H, Lq, Lk)))
+    assert np.all(out[:, :, 5].cpu().numpy() == 0.0)
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_fp32_forward_pruned_values_are_not_looked_at(ap, bad):
+    """A value row of infinities or NaNs reaches the queries that keep its key and no other."""
+    w = W["tiny"].scaled(B=2, H=2, Lq=70, Lk=200, d=64, dtype="f32")
+    mask = inputs.random_mask(w.H, w.Lq, w.Lk, 0.3, seed=509)
+    mask[:, ::2, 150] = 1
+    mask[:, 1::2, 150] = 0
+    q, k, v = inputs.eval_qkv(w)
+    tiles = ap.Tiles(w.H, w.Lq, w.Lk)
+    ap.ap_mask_to_tiles(mask.cuda(), tiles)
+    ref = orc.attention_fwd(inputs.widen(q), inputs.widen(k), inputs.widen(v), mask.numpy())
+    v = v.clone()
+    v[:, :, 150] = bad
+    out = ap.ap_sparse_attention_fwd(q.cuda(), k.cuda(), v.cuda(), tiles)
+    assert ap.ap_device_status() == ap.AP_OK
+    assert not torch.isfinite(out[:, :, ::2]).any()
+    pu.assert_close_attention(out[:, :, 1::2].contiguous(), ref[:, :, 1::2], "f32")
