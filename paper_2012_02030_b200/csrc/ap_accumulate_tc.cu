@@ -30,8 +30,9 @@
 // entries outside the domain (boxes wholly outside are skipped).  Other shapes keep the
 // per-row red.global.add.
 //
-// Warp roles (576 threads, one CTA per SM): warps 0-15 softmax; thread (wg, r) with wg = warp / 4 owns row r of the tile and
-// columns [32 wg, 32 wg + 32) of every key tile; warp 16 TMA producer; warp 17 MMA issuer and TMEM owner.  S is
+// Warp roles (576 threads, one CTA per SM; kGroups = 4): warps 0-15 softmax; thread (wg, r) with wg = warp / 4 owns row r of
+// the tile and columns [32 wg, 32 wg + 32) of every key tile; warp 16 TMA producer; warp 17 MMA issuer and TMEM owner.  With
+// kGroups = 2 eight softmax warps take 64 columns per thread, which leaves room for the statistics of 32 samples.  S is
 // double-buffered in TMEM (2 x 128 columns) so the MMA of the next visit runs under the softmax of the current one; a
 // visit's 32 columns are copied to registers in one go and S is handed back before the arithmetic starts.  TMEM columns
 // 256-383 hold the running sum over b, columns 384-511 the per-sample (maximum, sum) pairs of the four column quarters,
@@ -53,15 +54,10 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kSoftmaxWarps = 16;
-constexpr int kProducer = kSoftmaxWarps, kIssuer = kSoftmaxWarps + 1;
-constexpr int kThreads = (kSoftmaxWarps + 2) * 32;
-constexpr int kRegThreads = 640;  // registers are handed out to whole sets of four warps: 20 warps' worth, 96 each
 constexpr int kSubBytes = 128 * 128;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSumCol = 256;    // running sum over b: 128 columns
-constexpr uint32_t kStatsCol = 384;  // (max, sum) pairs: 32 columns per column quarter, 2 per sample
-constexpr int kMaxB = 16;            // samples per launch (what the spare tensor-memory columns hold)
+constexpr uint32_t kStatsCol = 384;  // (max, sum) pairs: as many columns per group of columns as it has, 2 per sample
 constexpr int kBiasBytes = 128 * 128 * 4;  // one fp32 bias tile: 4 boxes of 128 rows x 32 columns
 constexpr int kRedBytes = 32 * 64;         // per softmax warp: 32 rows x 16 fp32 columns on their way to the accumulator
 constexpr float kLog2e = 1.4426950408889634f;
@@ -73,9 +69,20 @@ struct Cfg {
   static constexpr int kStages = D == 64 ? 4 : 2;        // (Q, K) pairs in flight
   static constexpr int kBiasOffset = 2 * kStages * kTileBytes;
   static constexpr int kRedOffset = kBiasOffset + kBiasBytes;
-  static constexpr int kBarOffset = kRedOffset + kSoftmaxWarps * kRedBytes;
+  static constexpr int kBarOffset = kRedOffset + 16 * kRedBytes;
   static constexpr int kSmemBytes = kBarOffset + 256 + 1024;
   static_assert(kSmemBytes <= 227 * 1024, "within the shared memory of one CTA");
+};
+
+// kGroups groups of four softmax warps share a key tile's columns.
+template <int kGroups>
+struct Roles {
+  static constexpr int kSoftmaxWarps = 4 * kGroups, kProducer = kSoftmaxWarps, kIssuer = kSoftmaxWarps + 1;
+  static constexpr int kThreads = (kSoftmaxWarps + 2) * 32;
+  // registers are handed out to whole sets of four warps (sixteen softmax warps: 20 warps' worth, 96 each)
+  static constexpr int kRegThreads = (kSoftmaxWarps + 4) * 32;
+  static constexpr int kCols = 128 / kGroups;   // of a thread
+  static constexpr int kMaxB = 64 / kGroups;    // samples per CTA (what the spare tensor-memory columns hold)
 };
 
 struct Barriers {
@@ -131,10 +138,10 @@ __host__ __device__ inline int key_tiles(int qt, int n_kt, int memory) {
   return n < n_kt ? n : n_kt;
 }
 // Chunks that a query tile's B samples are cut into, for about `visits` visits each: at least kMinChunk samples a chunk,
-// at most kMaxB.
-__host__ __device__ inline int chunks_of(int visits, int n_k, int B) {
+// at most max_b.
+__host__ __device__ inline int chunks_of(int visits, int n_k, int B, int max_b) {
   int per = visits / n_k;
-  per = per < kMinChunk ? kMinChunk : per > kMaxB ? kMaxB : per;
+  per = per < kMinChunk ? kMinChunk : per > max_b ? max_b : per;
   return (B + per - 1) / per;
 }
 
@@ -142,14 +149,16 @@ __host__ __device__ inline int chunks_of(int visits, int n_k, int B) {
 // first wait runs out and the CTA leaves through its error path.
 // kChunked: the instantiation for launches whose samples are cut into chunks (see below); a
 // separate one so that its extra code costs the plain launches nothing.
-template <int D, bool kChunked>
-__global__ void __launch_bounds__(kRegThreads, 1)
+template <int D, bool kChunked, int kGroups>
+__global__ void __launch_bounds__(Roles<kGroups>::kRegThreads, 1)
 accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_bias, const __grid_constant__ CUtensorMap map_acc,
                      int bias_by_tma, int acc_by_tma, float *__restrict__ acc, const float *__restrict__ bias, int b0,
                      int Bc_all, int chunk_visits, unsigned *__restrict__ turn, int H, int Lq, int Lk, int n_qt,
                      int n_kt, int causal, int f16, float scale_log2, unsigned *err, uint32_t max_polls, int dbg_skip) {
   using C = Cfg<D>;
+  constexpr int kSoftmaxWarps = Roles<kGroups>::kSoftmaxWarps, kProducer = Roles<kGroups>::kProducer,
+                kIssuer = Roles<kGroups>::kIssuer, kCols = Roles<kGroups>::kCols, kMaxB = Roles<kGroups>::kMaxB;
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem =
       reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -165,12 +174,12 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   if (kChunked) {
     int left = (int)blockIdx.x;
     for (qt = n_qt - 1; qt > 0; --qt) {
-      const int here = H * chunks_of(chunk_visits, key_tiles(qt, n_kt, causal ? Lk - Lq : -1), Bc_all);
+      const int here = H * chunks_of(chunk_visits, key_tiles(qt, n_kt, causal ? Lk - Lq : -1), Bc_all, kMaxB);
       if (left < here) break;
       left -= here;
     }
     // the samples of a query tile are dealt out evenly over its chunks
-    const int chunks = chunks_of(chunk_visits, key_tiles(qt, n_kt, causal ? Lk - Lq : -1), Bc_all);
+    const int chunks = chunks_of(chunk_visits, key_tiles(qt, n_kt, causal ? Lk - Lq : -1), Bc_all, kMaxB);
     h = left % H;
     chunk = left / H;
     const int first = chunk * Bc_all / chunks;
@@ -286,7 +295,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       }
     }
   } else {
-    // ------------------------------------------------------------ softmax (512 threads)
+    // ------------------------------------------------------------ softmax (256 or 512 threads)
     const int wg = warp >> 2;
     const int r = (warp & 3) * 32 + lane;  // row of the tile == TMEM lane
     const int i = qt * kTile + r;
@@ -294,10 +303,10 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const int jend = causal ? min(Lk, i + 1 + off) : Lk;  // first key outside this row's domain
     const bool vec = (Lk & 3) == 0;
-    const uint32_t s_addr = tmem + lane_addr + 32 * wg;             // + 128 * buf
-    const uint32_t sum_addr = tmem + lane_addr + kSumCol + 32 * wg;
-    const uint32_t stats = tmem + lane_addr + kStatsCol;            // + 32 * quarter + 2 * b
-    const uint32_t my_stats = stats + 32 * wg;
+    const uint32_t s_addr = tmem + lane_addr + kCols * wg;          // + 128 * buf
+    const uint32_t sum_addr = tmem + lane_addr + kSumCol + kCols * wg;
+    const uint32_t stats = tmem + lane_addr + kStatsCol;            // + kCols * group + 2 * b
+    const uint32_t my_stats = stats + kCols * wg;
     // this warp's 32 rows x 16 columns on their way to the accumulator, and the rows' place in it
     unsigned char *red_s = smem + C::kRedOffset + warp * kRedBytes;
     const int red_y = qt * kTile + (warp & 3) * 32;
@@ -305,18 +314,18 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
     for (int b = 0; b < Bc; ++b) tmem_st2(my_stats + 2 * b, __float_as_uint(-CUDART_INF_F), 0u);
 
-    float bias2[32];  // bias * log2(e) of this thread's 32 columns of the current key tile
+    float bias2[kCols];  // bias * log2(e) of this thread's columns of the current key tile
     bool ok = true;
     // the bias slice of key tile kt (tl: how many tiles were staged before it), once for all samples
     auto fetch_bias = [&](int kt, int tl) {
-      const int j0 = kt * kTile + 32 * wg;
+      const int j0 = kt * kTile + kCols * wg;
       if (bias_by_tma) {
         ok = wait(&bars->bias_full, (uint32_t)tl & 1u);
         if (!ok) return;
-        const unsigned char *box = bias_s + wg * (kBiasBytes / 4) + r * 128;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {  // 16-byte chunk k of the row sits at position k ^ (r % 8)
-          const float4 t = *reinterpret_cast<const float4 *>(box + ((k ^ (r & 7)) << 4));
+        for (int k = 0; k < kCols / 4; ++k) {  // 16-byte chunk k of a box's row sits at position k ^ (r % 8)
+          const unsigned char *box = bias_s + (wg * (kCols / 32) + k / 8) * (kBiasBytes / 4) + r * 128;
+          const float4 t = *reinterpret_cast<const float4 *>(box + (((k & 7) ^ (r & 7)) << 4));
           bias2[4 * k] = t.x * kLog2e; bias2[4 * k + 1] = t.y * kLog2e;
           bias2[4 * k + 2] = t.z * kLog2e; bias2[4 * k + 3] = t.w * kLog2e;
         }
@@ -324,7 +333,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (lane == 0) mbar_arrive(&bars->bias_empty);
       } else {
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
+        for (int c = 0; c < kCols / 4; ++c) {
           float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
           const int j = j0 + 4 * c;
           if (bias && row_ok) {
@@ -339,15 +348,16 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         }
       }
     };
-    // S of visit v is ready: copy this thread's 32 columns to registers and hand S back.  The MMA of
+    // S of visit v is ready: copy this thread's columns to registers and hand S back.  The MMA of
     // visit v + 2 may then overwrite the buffer while the arithmetic on the copy is still going on
-    // (one arrival per warp: 512 threads arriving one by one would take longer than a visit's MMAs).
-    auto take_s = [&](int v, uint32_t (&xs)[32]) {
+    // (one arrival per warp: all threads arriving one by one would take longer than a visit's MMAs).
+    auto take_s = [&](int v, uint32_t (&xs)[kCols]) {
       const int buf = v & 1;
       ok = wait(&bars->s_full[buf], (uint32_t)(v >> 1) & 1u);
       if (!ok) return;
       tc_fence_after_sync();
-      tmem_ld32(s_addr + 128 * buf, xs);
+#pragma unroll
+      for (int c = 0; c < kCols; c += 32) tmem_ld32(s_addr + 128 * buf + c, xs + c);
     };
     auto release_s = [&](int v) {
       tc_fence_before_sync();
@@ -361,29 +371,29 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       fetch_bias(kt, kt);
       if (!ok) break;
       // columns of this slice inside the row's domain; whole warp inside => no masking
-      const int n_valid = max(0, min(32, jend - (kt * kTile + 32 * wg)));
-      const bool interior = __all_sync(0xffffffffu, n_valid == 32);
+      const int n_valid = max(0, min(kCols, jend - (kt * kTile + kCols * wg)));
+      const bool interior = __all_sync(0xffffffffu, n_valid == kCols);
       for (int b = 0; b < Bc; ++b, ++v) {
-        uint32_t xs[32], sv[2];
+        uint32_t xs[kCols], sv[2];
         take_s(v, xs);
         if (!ok) break;
         tmem_wait_st();  // this sample's pair as the previous key tile left it
         tmem_ld2(my_stats + 2 * b, sv);
         tmem_wait_ld();
         release_s(v);
-        float t[32];
+        float t[kCols];
 #pragma unroll
-        for (int e = 0; e < 32; e += 2)
+        for (int e = 0; e < kCols; e += 2)
           ffma2(t[e], t[e + 1], __uint_as_float(xs[e]), __uint_as_float(xs[e + 1]), scale_log2, bias2[e], bias2[e + 1]);
         if (!interior) {
 #pragma unroll
-          for (int e = 0; e < 32; ++e) t[e] = e < n_valid ? t[e] : -CUDART_INF_F;
+          for (int e = 0; e < kCols; ++e) t[e] = e < n_valid ? t[e] : -CUDART_INF_F;
         }
         const float m_old = __uint_as_float(sv[0]);
         // four independent chains each for the maximum and for the sum
         float m0 = m_old, m1 = -CUDART_INF_F, m2 = -CUDART_INF_F, m3 = -CUDART_INF_F;
 #pragma unroll
-        for (int e = 0; e < 32; e += 8) {  // three-input maxima: half the instructions
+        for (int e = 0; e < kCols; e += 8) {  // three-input maxima: half the instructions
           m0 = fmax3(m0, t[e], t[e + 4]);
           m1 = fmax3(m1, t[e + 1], t[e + 5]);
           m2 = fmax3(m2, t[e + 2], t[e + 6]);
@@ -394,7 +404,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         float z0 = __uint_as_float(sv[1]) * ex2_approx(m_old - cm_safe), z1 = 0.f, z2 = 0.f, z3 = 0.f;
         const float neg_cm = -cm_safe;
 #pragma unroll
-        for (int e = 0; e < 32; e += 4) {
+        for (int e = 0; e < kCols; e += 4) {
           float a0, a1, a2, a3;
           fadd2(a0, a1, t[e], t[e + 1], neg_cm, neg_cm);
           fadd2(a2, a3, t[e + 2], t[e + 3], neg_cm, neg_cm);
@@ -405,7 +415,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       }
     }
     if (ok) {
-      // every statistic of sweep 1 is final once all column quarters of every row are done
+      // every statistic of sweep 1 is final once all groups of columns of every row are done
       tmem_wait_st();
       tc_fence_before_sync();
       __syncwarp();
@@ -418,27 +428,28 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     for (int kt = 0; kt < n_k && ok; ++kt) {
       fetch_bias(kt, n_k + kt);
       if (!ok) break;
-      const int j0 = kt * kTile + 32 * wg;  // first column of this thread's slice
-      const int n_valid = max(0, min(32, jend - j0));
-      const bool interior = __all_sync(0xffffffffu, n_valid == 32);
+      const int j0 = kt * kTile + kCols * wg;  // first column of this thread's slice
+      const int n_valid = max(0, min(kCols, jend - j0));
+      const bool interior = __all_sync(0xffffffffu, n_valid == kCols);
       for (int b = 0; b < Bc; ++b, ++v) {
-        uint32_t xs[32], st[4][2];
+        uint32_t xs[kCols], st[kGroups][2];
         take_s(v, xs);
         if (!ok) break;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) tmem_ld2(stats + 32 * q + 2 * b, st[q]);
+        for (int q = 0; q < kGroups; ++q) tmem_ld2(stats + kCols * q + 2 * b, st[q]);
         tmem_wait_ld();
         release_s(v);
-        // the column quarters' statistics of sample b combined: max + log2(sum).  A row without any key
+        // the groups' statistics of sample b combined: max + log2(sum).  A row without any key
         // in its domain (possible when Lk < Lq) gets weight 0 everywhere.
-        const float mm = fmaxf(fmaxf(__uint_as_float(st[0][0]), __uint_as_float(st[1][0])),
-                               fmaxf(__uint_as_float(st[2][0]), __uint_as_float(st[3][0])));
+        float mm = __uint_as_float(st[0][0]);
+#pragma unroll
+        for (int q = 1; q < kGroups; ++q) mm = fmaxf(mm, __uint_as_float(st[q][0]));
         float z = 0.f;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) z += __uint_as_float(st[q][1]) * ex2_approx(__uint_as_float(st[q][0]) - mm);
+        for (int q = 0; q < kGroups; ++q) z += __uint_as_float(st[q][1]) * ex2_approx(__uint_as_float(st[q][0]) - mm);
         const float neg_ref = jend > 0 ? -(mm + lg2_approx(z)) : -CUDART_INF_F;
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
+        for (int c = 0; c < kCols / 16; ++c) {
           float p[16];
 #pragma unroll
           for (int e = 0; e < 16; e += 2)
@@ -527,8 +538,8 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 }
               }
             }
-            if (kChunked && c == 1) {
-              // both blocks of this warp are in the accumulator: count this warp in for the next chunk
+            if (kChunked && c == kCols / 16 - 1) {
+              // all blocks of this warp are in the accumulator: count this warp in for the next chunk
               if (acc_by_tma && lane == 0) bulk_wait_group0();
               __threadfence();
               __syncwarp();
@@ -547,54 +558,95 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   if (warp == kIssuer) tmem_dealloc(tmem, kTmemCols);
 }
 
-template <int D>
+// How a call's samples are spread over launches and CTAs.
+//
+// One CTA takes up to max_b samples of a (head, query tile) pair: 16 with sixteen softmax warps, 32 with eight, which are
+// slower per visit (84 instead of 77 us at 16 x 16 heads x 512, causal) but save launches and additions.  Shapes with fewer
+// pairs than SMs: several CTAs per pair, each with a chunk of the samples, taking turns at the accumulator, all in one wave
+// (one CTA per SM).  Fewer visits per chunk keep more SMs busy, but the chunks' additions wait for one another; of all numbers
+// of visits per chunk the one with the lowest estimate is taken.  Query tiles with more key tiles are cut into more chunks:
+// with the same number for all, the longest CTA of 16 x 16 heads x 512 (causal) had 64 visits (77 us, now 48: 64 us).
+// The estimates, in units of a visit (some 1.0 us with sixteen warps), are fitted to these measurements (us; chunks of as many
+// samples): 300 x 2 heads x 128 60 x 5 210, 19 x 16 90; 20 x 2 heads x 333, rows added by entry, one CTA per pair 176, 10 x 2
+// 176, 4 x 5 122; 7 x 4 heads x 250 x 231, by entry, one CTA 67, 2 x 4 73.
+struct Shape {
+  int B, H, n_qt, n_kt, memory, sms;  // memory: as for key_tiles
+  bool by_tma;                        // accumulator rows have a tensor map
+};
+constexpr double kLaunch = 6.0;      // a launch
+constexpr double kTurn = 3.3;        // an addition to a key tile that others wait for
+constexpr double kTurnByEntry = 18.0, kAddByEntry = 13.0;  // by entry, with and without others waiting
+
+// Estimate for n samples in one launch: chunks of about `visits` visits, or (0) one CTA per pair.
+double estimate(const Shape &p, int n, int visits, int max_b) {
+  const double visit = max_b == 16 ? 1.0 : 1.12, turn = !p.by_tma ? kTurnByEntry : kTurn;
+  if (!visits) {  // whole rounds of CTAs; nobody waits, and the reductions of a tensor map run beside the next tile
+    const int rounds = (p.H * p.n_qt + p.sms - 1) / p.sms;
+    return kLaunch + rounds * p.n_kt * (2.0 * n * visit + (p.by_tma ? 0.0 : kAddByEntry));
+  }
+  double worst = 0.0;
+  for (int qt = 0; qt < p.n_qt; ++qt) {
+    const int n_k = key_tiles(qt, p.n_kt, p.memory), chunks = chunks_of(visits, n_k, n, max_b), per = (n + chunks - 1) / chunks;
+    const double t = 2.0 * n_k * per * visit + chunks * turn + (n_k - 1) * (turn > per * visit ? turn - per * visit : 0.0);
+    worst = t > worst ? t : worst;
+  }
+  return kLaunch + worst;
+}
+
+struct Launch {
+  int samples, visits, grid;  // visits = 0: no chunks
+  double time;
+};
+
+// The next launch of a call with `left` samples to go.
+Launch plan_launch(const Shape &p, int left, int max_b, bool chunks) {
+  const int n_units = p.H * p.n_qt;
+  Launch best = {left < max_b ? left : max_b, 0, n_units, 0.0};
+  best.time = estimate(p, best.samples, 0, max_b);
+  if (!chunks) return best;
+  const int most = max_b * (p.sms / n_units), n = left < most ? left : most;  // as many as one wave can take
+  int total = 0;
+  for (int qt = 0; qt < p.n_qt; ++qt) total += p.H * key_tiles(qt, p.n_kt, p.memory) * n;
+  for (int visits = (total + p.sms - 1) / p.sms; visits <= max_b * p.n_kt; visits += 1 + visits / 16) {
+    int grid = 0;
+    for (int qt = 0; qt < p.n_qt; ++qt) grid += p.H * chunks_of(visits, key_tiles(qt, p.n_kt, p.memory), n, max_b);
+    if (grid > p.sms || grid <= n_units) continue;
+    const double time = estimate(p, n, visits, max_b);
+    if (time * best.samples < best.time * n) best = {n, visits, grid, time};  // (per sample)
+  }
+  return best;
+}
+
+// Estimate for a whole call: launches of the first one's size, then what is left.
+double plan_call(const Shape &p, int max_b, bool chunks) {
+  const Launch first = plan_launch(p, p.B, max_b, chunks);
+  const int full = p.B / first.samples, rest = p.B % first.samples;
+  return full * first.time + (rest ? plan_launch(p, rest, max_b, chunks).time : 0.0);
+}
+
+template <int D, int kGroups>
 cudaError_t launch(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mb, const CUtensorMap &ma,
-                   int bias_by_tma, int acc_by_tma, float *acc, const float *bias, int B, int H, int Lq, int Lk,
-                   int causal, int f16, float scale, unsigned *err, cudaStream_t s) {
-  auto kern = accumulate_tc_kernel<D, false>;
-  auto kern_chunked = accumulate_tc_kernel<D, true>;
+                   int bias_by_tma, int acc_by_tma, float *acc, const float *bias, const Shape &p, unsigned *turn, int Lq,
+                   int Lk, int causal, int f16, float scale, unsigned *err, cudaStream_t s) {
+  using R = Roles<kGroups>;
+  auto kern = accumulate_tc_kernel<D, false, kGroups>;
+  auto kern_chunked = accumulate_tc_kernel<D, true, kGroups>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(kern_chunked, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
   if (e != cudaSuccess) return e;
-  const int n_qt = ceil_div(Lq, kTile), n_kt = ceil_div(Lk, kTile);
   const DebugKnobs knobs = debug_knobs();
-  // Shapes with fewer (head, query tile) pairs than SMs: several CTAs per pair, each with a chunk of the samples, taking
-  // turns at the accumulator (one wave of CTAs, one per SM).  The smallest number of visits per chunk is taken for
-  // which they fit, so that the query tiles with many key tiles are cut into more chunks: with the same number for all,
-  // the longest CTA of 16 x 16 heads x 512 (causal) had 64 visits where 35 would be the mean (now 48: 77 -> 64 us).
-  // Accumulator rows that no tensor map describes are added to with one instruction per entry, several microseconds per tile,
-  // and a chunk's turn waits for those of all lower ones: worth it from three key tiles and 48 visits per sweep and pair on
-  // (19 x 2 heads x 975 x 1950: 1 147 -> 532 us, 20 x 333: 170 -> 147; but 9 x 333, 27 visits: 85 -> 117, and 40 x 2 x 130 x
-  // 130, two key tiles: 216 -> 232).
-  const int n_units = H * n_qt, sms = sm_count();
-  unsigned *turn = nullptr;
-  const bool long_enough = acc_by_tma || (n_kt >= 3 && n_kt * B >= 48);
-  if (long_enough && !knobs.skip_arrive && n_units < sms && B >= 2 * kMinChunk && (size_t)n_units * n_kt <= kTurnWords)
-    turn = turn_words();
-  // samples in ascending order, at most kMaxB per CTA; launches on one stream run in order
-  for (int b0 = 0; b0 < B;) {
-    int Bc = B - b0 < kMaxB ? B - b0 : kMaxB, visits = 0, grid = n_units;
-    if (turn) {
-      const int all = B - b0, memory = causal ? Lk - Lq : -1;
-      int total = 0;
-      for (int qt = 0; qt < n_qt; ++qt) total += H * key_tiles(qt, n_kt, memory) * all;
-      for (visits = (total + sms - 1) / sms;; visits += 1 + visits / 16) {
-        grid = 0;
-        for (int qt = 0; qt < n_qt; ++qt) grid += H * chunks_of(visits, key_tiles(qt, n_kt, memory), all);
-        if (grid <= sms || visits >= kMaxB * n_kt) break;
-      }
-      if (grid <= sms && grid > n_units) Bc = all;  // all the samples in one launch
-      else visits = 0, grid = n_units;
-    }
-    unsigned *t = visits ? turn : nullptr;
-    if (t && (e = cudaMemsetAsync(t, 0, (size_t)n_units * n_kt * sizeof(unsigned), s)) != cudaSuccess) return e;
-    (t ? kern_chunked : kern)<<<knobs.skip_arrive ? 1 : grid, kThreads, Cfg<D>::kSmemBytes, s>>>(
-        mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, b0, Bc, visits, t, H, Lq, Lk, n_qt, n_kt, causal, f16,
-        scale * kLog2e, err, knobs.max_polls, knobs.skip_arrive);
+  // samples in ascending order; launches on one stream run in order
+  for (int b0 = 0; b0 < p.B;) {
+    const Launch l = plan_launch(p, p.B - b0, R::kMaxB, turn != nullptr);
+    unsigned *t = l.visits ? turn : nullptr;
+    if (t && (e = cudaMemsetAsync(t, 0, (size_t)p.H * p.n_qt * p.n_kt * sizeof(unsigned), s)) != cudaSuccess) return e;
+    (t ? kern_chunked : kern)<<<knobs.skip_arrive ? 1 : l.grid, R::kThreads, Cfg<D>::kSmemBytes, s>>>(
+        mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, b0, l.samples, l.visits, t, p.H, Lq, Lk, p.n_qt, p.n_kt, causal,
+        f16, scale * kLog2e, err, knobs.max_polls, knobs.skip_arrive);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    b0 += Bc;
+    b0 += l.samples;
   }
   return cudaSuccess;
 }
@@ -615,9 +667,19 @@ cudaError_t launch_accumulate_tc(float *acc, const void *Q, const void *K, const
   CUtensorMap ma = mq;
   const int acc_by_tma = (Lk & 3) == 0 ? 1 : 0;
   if (acc_by_tma && !make_tile_map_f32(&ma, acc, H, Lq, Lk, 32, 16)) return cudaErrorUnknown;
-  return d == 64
-             ? launch<64>(mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, B, H, Lq, Lk, causal, f16, scale, err, s)
-             : launch<128>(mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, B, H, Lq, Lk, causal, f16, scale, err, s);
+  const Shape p = {B, H, ceil_div(Lq, kTile), ceil_div(Lk, kTile), causal ? Lk - Lq : -1, sm_count(), acc_by_tma != 0};
+  if (p.sms <= 0) return cudaErrorUnknown;
+  const int n_units = H * p.n_qt;
+  unsigned *turn = nullptr;
+  if (!debug_knobs().skip_arrive && n_units < p.sms && B >= 2 * kMinChunk && (size_t)n_units * p.n_kt <= kTurnWords)
+    turn = turn_words();
+  const bool eight = B > Roles<4>::kMaxB &&
+                     plan_call(p, Roles<2>::kMaxB, turn != nullptr) < plan_call(p, Roles<4>::kMaxB, turn != nullptr);
+  auto go = [&](auto fn) {
+    return fn(mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, p, turn, Lq, Lk, causal, f16, scale, err, s);
+  };
+  if (d == 64) return eight ? go(launch<64, 2>) : go(launch<64, 4>);
+  return eight ? go(launch<128, 2>) : go(launch<128, 4>);
 }
 
 }  // namespace ap

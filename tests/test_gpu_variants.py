@@ -238,3 +238,19 @@ def test_fp32_forward_pruned_values_are_not_looked_at(ap, bad):
     assert ap.ap_device_status() == ap.AP_OK
     assert not torch.isfinite(out[:, :, ::2]).any()
     pu.assert_close_attention(out[:, :, 1::2].contiguous(), ref[:, :, 1::2], "f32")
+
+
+@pytest.mark.parametrize("B,H,Lq,Lk", [(33, 2, 130, 130),    # eight softmax warps, rows added by entry, chunks
+                                       (35, 1, 200, 132),    # ... rows with a tensor map
+                                       (150, 12, 64, 64),    # more samples than one wave of CTAs takes: a second launch
+                                       (20, 160, 33, 36)])   # more (head, query tile) pairs than SMs
+def test_accumulate_many_samples(ap, B, H, Lq, Lk):
+    """More samples than a CTA of sixteen softmax warps holds the statistics of."""
+    w = W["tiny"].scaled(B=B, H=H, Lq=Lq, Lk=Lk, d=64, dtype="bf16", causal=False)
+    bias = inputs.calib_bias(w)
+    acc = pu.gpu_accumulate(ap, w, 1, bias.cuda())
+    assert ap.ap_device_status() == ap.AP_OK
+    assert torch.equal(acc, pu.gpu_accumulate(ap, w, 1, bias.cuda()))
+    want = pu.oracle_accumulate(w, 1, bias)
+    tol = tp._acc_tolerance(w.dtype)
+    np.testing.assert_allclose(acc.cpu().numpy(), want, rtol=tol["rtol"], atol=tol["atol"] * B)
