@@ -863,10 +863,14 @@ cudaError_t launch_kernel(const FwdMaps &maps, const void *K, const void *V, voi
   const int n_half = (t.n_qt + 1) / 2, n_units = B * H * n_half;  // pairs of query tiles, see the producer
   // A CTA takes every ctas-th unit.  If that shares a factor with the units of a head, a CTA meets only some of them: with
   // three query tiles (a pair and a lone one) and 148 CTAs, half of the CTAs got all the pairs (16 x 16 heads, 375 queries,
-  // 759 keys: 29.5 us, 23.8 with 147).
+  // 759 keys: 29.5 us, 23.8 with 147).  A smaller grid may take one unit more, though, which is worth it only where the
+  // units are uneven: the query tiles of the CTA with the most must not become more (74 heads x 500: one unit per CTA with
+  // 148, two for one of 147, 20.0 against 26.9 us).
   int ctas = sms;
   for (int d = 2; d <= n_half && d <= 64; ++d)
     if (n_half % d == 0 && ctas % d == 0) --ctas, d = 1;
+  const int most_units = ceil_div(n_units, ctas), lone_units = t.n_qt % 2 ? most_units / n_half : 0;
+  if (2 * most_units - lone_units > 2 * ceil_div(n_units, sms)) ctas = sms;
   const float scale_log2 = scale * 1.4426950408889634f;
   Gathered gth = {nullptr, nullptr, nullptr, nullptr, static_cast<const uint16_t *>(K), static_cast<const uint16_t *>(V),
                   Lk, dbg.schedule, kPairs ? t.unit_qt : nullptr};
