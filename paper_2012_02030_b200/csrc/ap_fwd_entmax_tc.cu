@@ -24,7 +24,7 @@
 //                    weights, so that O is an exact convex combination of V rows.
 // Warps 0-7 normalise (thread (wg, r) owns row r and columns [64 wg, 64 wg + 64) of every round),
 // warp 8 copies with TMA (Q once; the rounds' K rows every sweep, in boxes of 16 rows per group or
-// one box of 128 rows for eight adjacent groups, into a ring of 4 to 6 stages; V rows in the last
+// one box of 128 rows for eight adjacent groups, into a ring of two or three stages; V rows in the last
 // sweep), warp 9 issues the products.
 // Every mbarrier wait is bounded.
 //
@@ -53,18 +53,18 @@ constexpr int kMaxNewton = 30;
 // either side of it the iteration lands on the other side or on the root).
 constexpr float kFirstGap = 0.625f;
 
-template <int D>
+// kCtasPerSm: at d = 64 two, or one where the grid has no second one for an SM.
+template <int D, int kCtasPerSm>
 struct Cfg {
   static constexpr int kSub = D / 64;
   static constexpr int kTileBytes = kSub * kSubBytes;
-  // K is copied again in every sweep and a list row is a few rounds long: a ring deep enough to hold
-  // a short row whole keeps the copies several visits ahead of the products.  V is needed once.
+  // K is copied again in every sweep, through a ring; V is needed once.
   // d = 64: two CTAs share an SM and fill each other's waits (a list row is a few rounds long, so most of a CTA's
   // time is one chain), each with half of TMEM: one S buffer.  d = 128: one CTA, three S buffers in flight.
-  static constexpr int kCtas = D == 64 ? 2 : 1;
-  static constexpr int kSBufs = D == 64 ? 1 : 3;
-  static constexpr uint32_t kTmemCols = D == 64 ? 256 : 512;  // S x kSBufs, then O
-  static constexpr int kStages = D == 64 ? 2 : 3;         // K ring
+  static constexpr int kCtas = kCtasPerSm;
+  static constexpr int kSBufs = kCtas == 2 ? 1 : 3;
+  static constexpr uint32_t kTmemCols = 512 / kCtas;      // S x kSBufs, then O
+  static constexpr int kStages = kCtas == 2 ? 2 : 3;      // K ring
   static constexpr int kVStages = 1;                      // V ring (last sweep)
   static constexpr int kKOffset = kTileBytes;             // after Q
   static constexpr int kVOffset = kKOffset + kStages * kTileBytes;
@@ -159,13 +159,13 @@ __device__ __forceinline__ float2 unpack2(uint32_t v) {
   }
 }
 
-template <int D, bool kF16>
-__global__ void __launch_bounds__(kThreads, Cfg<D>::kCtas)
+template <int D, int kCtas, bool kF16>
+__global__ void __launch_bounds__(kThreads, kCtas)
 fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, const int32_t *__restrict__ round_ptr,
                   const int32_t *__restrict__ round_rows, const uint8_t *__restrict__ round_info,
                   const uint32_t *__restrict__ round_bitmap, int BH, int H, int Lq, int n_qt, float half_scale,
                   unsigned *err) {
-  using C = Cfg<D>;
+  using C = Cfg<D, kCtas>;
   constexpr int kSBufs = C::kSBufs;
   constexpr uint32_t kTmemCols = C::kTmemCols;
   extern __shared__ unsigned char smem_raw[];
@@ -344,7 +344,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         ++v;
         return true;
       };
-      // O += P V of visit u = round j of the last sweep: P is in S[u & 1] once the normalising
+      // O += P V of visit u = round j of the last sweep: P is in S[u % kSBufs] once the normalising
       // threads have arrived; one contraction step of 16 keys per group; then the V stage is free
       auto issue_pv = [&](int u, int j) -> bool {
         const int sb = u % kSBufs, sv = j % C::kVStages, ng_u = ng_of(j);
@@ -399,21 +399,22 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     float cnt = 0.f;
     float *list = reinterpret_cast<float *>(smem + C::kListOffset) + 144 * wg + r;  // entry k at list[k * kListPitch]
     int n_list = 0;
-    bool overflow = false;
-    // This thread's list without the entries that cannot lie above tau: three Newton steps on the list from `thr`, a
-    // lower bound of its root; they stay below it (the sum is convex in tau).
+    bool listing = true;  // of the whole warp
+    // A Newton step from a lower bound of the root of some of the row's entries, whose sums are S1 and S2: it stays below that root
+    // (the sum is convex in tau), which is no higher than the row's.
+    auto raise = [](float thr, float S1, float S2) {
+      return S2 > 1.f ? thr + 0.999f * (S2 - 1.f) / (2.f * S1) : thr;  // (0.999: never above the root by rounding)
+    };
+    // This thread's list without the entries that cannot lie above tau: one such step on the list from `thr`.
     auto prune = [&](float thr) {
-#pragma unroll 1
-      for (int it = 0; it < 1; ++it) {
-        float S1 = 0.f, S2 = 0.f;
+      float S1 = 0.f, S2 = 0.f;
 #pragma unroll 4
-        for (int k = 0; k < n_list; ++k) {
-          const float u = __saturatef(list[k * kListPitch] - thr);
-          S1 += u;
-          S2 = fmaf(u, u, S2);
-        }
-        if (S2 > 1.f) thr += 0.999f * (S2 - 1.f) / (2.f * S1);  // (0.999: never above the root by rounding)
+      for (int k = 0; k < n_list; ++k) {
+        const float u = __saturatef(list[k * kListPitch] - thr);
+        S1 += u;
+        S2 = fmaf(u, u, S2);
       }
+      thr = raise(thr, S1, S2);
       int kept = 0;
       for (int k = 0; k < n_list; ++k) {
         const float x = list[k * kListPitch];
@@ -423,8 +424,9 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
         }
       }
       n_list = kept;
-      if (n_list > kListCap) {
-        overflow = true;
+      if (__any_sync(0xffffffffu, n_list > kListCap)) {  // no list of the CTA is used then
+        *reinterpret_cast<volatile int *>(&bars->more[0]) = 1;
+        listing = false;
         n_list = 0;
       }
       return thr;
@@ -485,7 +487,25 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
               m3 = fmax3(m3, t[e + 3], t[e + 7]);
             }
             st.x = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
+            if (!listing) continue;
             list_thr = fmaxf(list_thr, st.x - 1.f);
+            if (__any_sync(0xffffffffu, n_list + (full ? 32 : __popc(w)) > kListCap)) {
+              // a list could fill up: two steps on the chunk itself first, in registers, or most of it would go through the lists
+              // (unless one of the CTA's has overflowed: then the others are not needed either)
+              listing = !__any_sync(0xffffffffu, *reinterpret_cast<volatile int *>(&bars->more[0]) != 0);
+              if (!listing) continue;
+#pragma unroll 1
+              for (int it = 0; it < 2; ++it) {
+                float a0 = 0.f, a1 = 0.f, q0 = 0.f, q1 = 0.f;
+#pragma unroll
+                for (int e = 0; e < 32; e += 2) {
+                  const float u0 = __saturatef(t[e] - list_thr), u1 = __saturatef(t[e + 1] - list_thr);
+                  fadd2(a0, a1, a0, a1, u0, u1);
+                  ffma2v(q0, q1, u0, u1, u0, u1, q0, q1);
+                }
+                list_thr = raise(list_thr, a0 + a1, q0 + q1);
+              }
+            }
 #pragma unroll
             for (int half = 0; half < 4; ++half) {
 #pragma unroll
@@ -495,6 +515,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
                   ++n_list;
                 }
               if (__any_sync(0xffffffffu, n_list > kListCap)) list_thr = prune(list_thr);
+              if (!listing) break;
             }
           } else if (kind == 1) {
             float a0 = st.x, a1 = 0.f, a2 = 0.f, a3 = 0.f, q0 = st.y, q1 = 0.f, q2 = 0.f, q3 = 0.f;
@@ -538,7 +559,6 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
       if (!ok) break;
       *my_stats = st;
       cnts[wg * 128 + r] = sw == 0 ? __int_as_float(n_list) : cnt;
-      if (sw == 0 && overflow) *reinterpret_cast<volatile int *>(&bars->more[0]) = 1;
       // ---- end of a sweep: the two halves of every row meet
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->sweep_done);
@@ -636,13 +656,13 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
   if (warp == 9) tmem_dealloc(tmem, kTmemCols);
 }
 
-template <int D, bool kF16>
+template <int D, int kCtas, bool kF16>
 cudaError_t launch(const Maps &maps, const ap_tiles &t, void *O, int B, int H, int Lq, float scale, unsigned *err,
                    cudaStream_t s) {
-  auto kern = fwd_entmax_kernel<D, kF16>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
+  auto kern = fwd_entmax_kernel<D, kCtas, kF16>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D, kCtas>::kSmemBytes);
   if (e != cudaSuccess) return e;
-  kern<<<B * H * t.n_qt, kThreads, Cfg<D>::kSmemBytes, s>>>(maps, static_cast<uint16_t *>(O), t.round_ptr, t.round_rows,
+  kern<<<B * H * t.n_qt, kThreads, Cfg<D, kCtas>::kSmemBytes, s>>>(maps, static_cast<uint16_t *>(O), t.round_ptr, t.round_rows,
                                                            t.round_info, t.round_bitmap, B * H, H, Lq, t.n_qt,
                                                            0.5f * scale, err);
   count_launches(1);
@@ -660,9 +680,12 @@ cudaError_t launch_fwd_entmax_tc(const void *Q, const void *K, const void *V, co
       !make_tile_map_bf16(&maps.k128, K, B * H, Lk, d, 128) || !make_tile_map_bf16(&maps.v16, V, B * H, Lk, d, 16) ||
       !make_tile_map_bf16(&maps.v128, V, B * H, Lk, d, 128))
     return cudaErrorUnknown;
+  // d = 64: where there is no second CTA for an SM, one with all of tensor memory (4 heads x 512 x 1024, half kept: 117 -> 87 us)
+  if (d == 64 && (int64_t)B * H * t.n_qt > sm_count())
+    return f16 ? launch<64, 2, true>(maps, t, O, B, H, Lq, scale, err, s) : launch<64, 2, false>(maps, t, O, B, H, Lq, scale, err, s);
   if (d == 64)
-    return f16 ? launch<64, true>(maps, t, O, B, H, Lq, scale, err, s) : launch<64, false>(maps, t, O, B, H, Lq, scale, err, s);
-  return f16 ? launch<128, true>(maps, t, O, B, H, Lq, scale, err, s) : launch<128, false>(maps, t, O, B, H, Lq, scale, err, s);
+    return f16 ? launch<64, 1, true>(maps, t, O, B, H, Lq, scale, err, s) : launch<64, 1, false>(maps, t, O, B, H, Lq, scale, err, s);
+  return f16 ? launch<128, 1, true>(maps, t, O, B, H, Lq, scale, err, s) : launch<128, 1, false>(maps, t, O, B, H, Lq, scale, err, s);
 }
 
 }  // namespace ap

@@ -254,3 +254,13 @@ def test_accumulate_many_samples(ap, B, H, Lq, Lk):
     want = pu.oracle_accumulate(w, 1, bias)
     tol = tp._acc_tolerance(w.dtype)
     np.testing.assert_allclose(acc.cpu().numpy(), want, rtol=tol["rtol"], atol=tol["atol"] * B)
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 64), ("f16", 128)])
+@pytest.mark.parametrize("B", [1, 60])     # one CTA per SM at d = 64, or two
+@pytest.mark.parametrize("keep", [0.3, 1.0])
+def test_entmax_forward_dense_rows(ap, dtype, d, B, keep):
+    """Rows with many kept, spread-out entries: the threshold is raised by a chunk's own sums, and some lists overflow."""
+    w = W["tiny"].scaled(B=B, H=1, Lq=260, Lk=700 if B == 1 else 300, d=d, dtype=dtype)
+    mask = inputs.random_mask(1, w.Lq, w.Lk, keep, seed=511, empty_rows=(9,))
+    tp._entmax_fwd_case(ap, w, mask)
