@@ -103,6 +103,17 @@ void want(Py_ssize_t n, Py_ssize_t expected) {
   if (n != expected) fail(PyExc_TypeError, "wrong number of arguments");
 }
 
+// The interpreter lock is released while f allocates and launches: a launch waits where the stream's queue is full.  f uses C++
+// values only.
+template <class F>
+auto unlocked(F f) {
+  struct Lock {
+    PyThreadState *state = PyEval_SaveThread();
+    ~Lock() { PyEval_RestoreThread(state); }
+  } lock;
+  return f();
+}
+
 struct Shape {
   int B, H, Lq, Lk, d;
 };
@@ -146,10 +157,16 @@ PyObject *py_accumulate(PyObject *, PyObject *const *a, Py_ssize_t n) {
       if (!scores(b)) fail(PyExc_ValueError, "bias must be float32 [H,Lq,Lk]");
       bias = static_cast<const float *>(b.data_ptr());
     }
+    float *out = static_cast<float *>(acc.data_ptr());
+    const void *pq = q.data_ptr(), *pk = k.data_ptr();
+    const ap_dtype dt = dtype_code(q);
+    const int causal = truth(a[4]);
+    const float scale = (float)number(a[5]);
+    void *stream = stream_of(a[6]);
     const auto fn = kEntmax ? g_fn.accumulate_entmax : g_fn.accumulate;
-    return done(fn(static_cast<float *>(acc.data_ptr()), q.data_ptr(), k.data_ptr(), bias, s.B, s.H, s.Lq, s.Lk, s.d,
-                   dtype_code(q), truth(a[4]), (float)number(a[5]), stream_of(a[6])),
-                kEntmax ? "ap_accumulate_attention_entmax15" : "ap_accumulate_attention", none());
+    const ap_status st =
+        unlocked([&] { return fn(out, pq, pk, bias, s.B, s.H, s.Lq, s.Lk, s.d, dt, causal, scale, stream); });
+    return done(st, kEntmax ? "ap_accumulate_attention_entmax15" : "ap_accumulate_attention", none());
   });
 }
 
@@ -165,10 +182,8 @@ PyObject *py_build_mask(PyObject *, PyObject *const *a, Py_ssize_t n) {
     if (acc.scalar_type() != at::kFloat) fail(PyExc_ValueError, "acc must be float32");
     const int H = (int)acc.size(0), Lq = (int)acc.size(1), Lk = (int)acc.size(2);
     at::Tensor ws;
-    if (a[9] == Py_None)
-      ws = at::empty({(int64_t)g_fn.build_mask_workspace(H, Lq, Lk)}, acc.options().dtype(at::kByte));
-    else
-      ws = tensor(a[9], "workspace");
+    if (a[9] != Py_None) ws = tensor(a[9], "workspace");
+    const at::TensorOptions bytes = acc.options().dtype(at::kByte);
     const float *in = static_cast<const float *>(acc.data_ptr());
     const double keep = number(a[2]);
     const int causal = truth(a[3]), diag = truth(a[4]);
@@ -176,12 +191,15 @@ PyObject *py_build_mask(PyObject *, PyObject *const *a, Py_ssize_t n) {
     ap_tiles *tiles = tiles_at(a[7]);
     int64_t *nnz = static_cast<int64_t *>(address(a[8], "nnz_per_head"));
     void *s = stream_of(a[10]);
-    if (rule == 2)
-      return done(g_fn.build_mask_ex(in, H, Lq, Lk, keep, causal, diag, (int)flags, mask, tiles, nnz, ws.data_ptr(),
-                                     (size_t)ws.numel(), s), "ap_build_mask_ex", none());
     const auto fn = rule == 1 ? g_fn.build_mask_layer : g_fn.build_mask;
-    return done(fn(in, H, Lq, Lk, keep, causal, diag, mask, tiles, nnz, ws.data_ptr(), (size_t)ws.numel(), s),
-                rule == 1 ? "ap_build_mask_layer" : "ap_build_mask", none());
+    const ap_status st = unlocked([&] {
+      if (!ws.defined()) ws = at::empty({(int64_t)g_fn.build_mask_workspace(H, Lq, Lk)}, bytes);
+      void *p = ws.data_ptr();
+      const size_t n = (size_t)ws.numel();
+      return rule == 2 ? g_fn.build_mask_ex(in, H, Lq, Lk, keep, causal, diag, (int)flags, mask, tiles, nnz, p, n, s)
+                       : fn(in, H, Lq, Lk, keep, causal, diag, mask, tiles, nnz, p, n, s);
+    });
+    return done(st, rule == 2 ? "ap_build_mask_ex" : rule == 1 ? "ap_build_mask_layer" : "ap_build_mask", none());
   });
 }
 
@@ -193,13 +211,20 @@ PyObject *py_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
     const at::Tensor &q = device_tensor(a[0], "Q"), &k = device_tensor(a[1], "K"), &v = device_tensor(a[2], "V");
     const Shape s = shape_of(q, k);
     like(v, k);
-    at::Tensor fresh;
-    if (a[4] == Py_None) fresh = at::empty_like(q);
-    void *o = a[4] == Py_None ? fresh.data_ptr() : device_tensor(a[4], "O").data_ptr();
+    at::Tensor o;
+    if (a[4] != Py_None) o = device_tensor(a[4], "O");
+    const void *pq = q.data_ptr(), *pk = k.data_ptr(), *pv = v.data_ptr();
+    ap_tiles *tiles = tiles_at(a[3]);
+    const ap_dtype dt = dtype_code(q);
+    const float scale = (float)number(a[5]);
+    void *stream = stream_of(a[6]);
     const auto fn = kEntmax ? g_fn.fwd_entmax : g_fn.fwd;
-    const ap_status st = fn(q.data_ptr(), k.data_ptr(), v.data_ptr(), tiles_at(a[3]), o, s.B, s.H, s.Lq, s.Lk, s.d,
-                            dtype_code(q), (float)number(a[5]), stream_of(a[6]));
-    PyObject *out = a[4] == Py_None ? THPVariable_Wrap(std::move(fresh)) : Py_NewRef(a[4]);
+    const ap_status st = unlocked([&] {
+      if (!o.defined()) o = at::empty_like(q);
+      return fn(pq, pk, pv, tiles, o.data_ptr(), s.B, s.H, s.Lq, s.Lk, s.d, dt, scale, stream);
+    });
+    PyObject *out = a[4] == Py_None ? THPVariable_Wrap(std::move(o)) : Py_NewRef(a[4]);
+    if (!out) return nullptr;
     return done(st, kEntmax ? "ap_sparse_attention_entmax15_fwd" : "ap_sparse_attention_fwd", out);
   });
 }
@@ -212,17 +237,25 @@ PyObject *py_bwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
                      &o = device_tensor(a[3], "O"), &g = device_tensor(a[4], "dO");
     const Shape s = shape_of(q, k);
     like(v, k), like(o, q), like(g, q);
-    const at::Tensor dq = a[6] == Py_None ? at::empty_like(q) : device_tensor(a[6], "dQ"),
-                     dk = a[7] == Py_None ? at::empty_like(k) : device_tensor(a[7], "dK"),
-                     dv = a[8] == Py_None ? at::empty_like(v) : device_tensor(a[8], "dV");
-    at::Tensor ws;
-    if (a[10] == Py_None)
-      ws = at::empty({(int64_t)g_fn.bwd_workspace(s.B, s.H, s.Lq, s.Lk)}, q.options().dtype(at::kByte));
-    else
-      ws = tensor(a[10], "workspace");
-    const ap_status st = g_fn.bwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), g.data_ptr(), tiles_at(a[5]),
-                                  dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), s.B, s.H, s.Lq, s.Lk, s.d, dtype_code(q),
-                                  (float)number(a[9]), ws.data_ptr(), (size_t)ws.numel(), stream_of(a[11]));
+    at::Tensor dq, dk, dv, ws;
+    if (a[6] != Py_None) dq = device_tensor(a[6], "dQ");
+    if (a[7] != Py_None) dk = device_tensor(a[7], "dK");
+    if (a[8] != Py_None) dv = device_tensor(a[8], "dV");
+    if (a[10] != Py_None) ws = tensor(a[10], "workspace");
+    const void *pq = q.data_ptr(), *pk = k.data_ptr(), *pv = v.data_ptr(), *po = o.data_ptr(), *pg = g.data_ptr();
+    ap_tiles *tiles = tiles_at(a[5]);
+    const ap_dtype dt = dtype_code(q);
+    const float scale = (float)number(a[9]);
+    void *stream = stream_of(a[11]);
+    const ap_status st = unlocked([&] {
+      if (!dq.defined()) dq = at::empty_like(q);
+      if (!dk.defined()) dk = at::empty_like(k);
+      if (!dv.defined()) dv = at::empty_like(v);
+      if (!ws.defined())
+        ws = at::empty({(int64_t)g_fn.bwd_workspace(s.B, s.H, s.Lq, s.Lk)}, q.options().dtype(at::kByte));
+      return g_fn.bwd(pq, pk, pv, po, pg, tiles, dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), s.B, s.H, s.Lq, s.Lk, s.d, dt,
+                      scale, ws.data_ptr(), (size_t)ws.numel(), stream);
+    });
     PyObject *out = Py_BuildValue("(NNN)", THPVariable_Wrap(dq), THPVariable_Wrap(dk), THPVariable_Wrap(dv));
     if (!out) return nullptr;
     return done(st, "ap_sparse_attention_bwd", out);

@@ -1,4 +1,7 @@
 """Calls that overlap: several streams, captured graphs, threads."""
+import threading
+import time
+
 import pytest
 import torch
 
@@ -52,3 +55,36 @@ def test_backward_replayed_beside_eager_calls(ap):
         for got, ref in zip(grads + grads2, want + want2):
             assert torch.equal(got, ref)
     assert ap.ap_device_status() == ap.AP_OK
+
+
+def _busy(stream, seconds=0.2):
+    """Keeps `stream` busy for about that long (a bounded loop on the device)."""
+    with torch.cuda.stream(stream):
+        torch.cuda._sleep(int(seconds * 1.9e9))
+
+
+def test_other_threads_run_while_a_launch_waits(ap):
+    """A launch that waits for room in its stream's queue does not hold the interpreter lock."""
+    args, _, _ = _attention(ap, 1, 1, 64, 64, 7)
+    side = torch.cuda.Stream()
+    out = torch.empty_like(args[0])
+    torch.cuda.synchronize()
+    done = threading.Event()
+
+    def launches():
+        for _ in range(4000):
+            ap.ap_sparse_attention_fwd(*args[:3], args[5], out, stream=side)
+        done.set()
+
+    _busy(side, 1.0)
+    thread = threading.Thread(target=launches)
+    began = last = time.perf_counter()
+    gap = 0.0
+    thread.start()
+    while not done.wait(0.001):
+        now = time.perf_counter()
+        gap, last = max(gap, now - last), now
+    thread.join()
+    gap, took = max(gap, time.perf_counter() - last), time.perf_counter() - began
+    torch.cuda.synchronize()
+    assert took < 0.5 or gap < 0.25  # (a queue without end would never make a launch wait)
