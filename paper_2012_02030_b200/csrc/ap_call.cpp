@@ -6,6 +6,7 @@
 // Why native: a small forward runs for 10 to 15 us on the device, and the same steps written in Python
 // (attribute look-ups on four tensors, argument conversion by ctypes, the stream look-up) took about as
 // long on the host, so back-to-back calls waited for the host.
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAStream.h>
@@ -134,8 +135,8 @@ PyObject *guarded(F f) {
     return f();
   } catch (const Error &) {
     return nullptr;
-  } catch (const std::exception &e) {
-    if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
+  } catch (...) {  // to the exceptions that torch's own functions raise (out of memory among them)
+    torch::translate_exception_to_python(std::current_exception());
     return nullptr;
   }
 }

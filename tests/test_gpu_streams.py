@@ -88,3 +88,17 @@ def test_other_threads_run_while_a_launch_waits(ap):
     gap, took = max(gap, time.perf_counter() - last), time.perf_counter() - began
     torch.cuda.synchronize()
     assert took < 0.5 or gap < 0.25  # (a queue without end would never make a launch wait)
+
+
+def test_out_of_memory_is_raised_as_such(ap):
+    H, L = 16, 1024
+    acc = torch.zeros((H, L, L), device="cuda")
+    mask = torch.empty((H, L, L), dtype=torch.uint8, device="cuda")
+    torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    torch.cuda.set_per_process_memory_fraction(torch.cuda.memory_reserved() / total)
+    try:
+        with pytest.raises(torch.cuda.OutOfMemoryError):
+            ap.ap_build_mask(acc, 0.1, True, True, mask=mask)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
