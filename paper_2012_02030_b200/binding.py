@@ -150,6 +150,20 @@ def _dtype_code(t: torch.Tensor) -> int:
     raise TypeError("dtype must be float32, bfloat16 or float16, got %s" % t.dtype)
 
 
+def _empty(shape, dtype, device, stream) -> torch.Tensor:
+    """Memory for a call on `stream`, allocated for it where it is not the current one (the kernels run after the call
+    has returned, and a block of the current stream could be handed out again by then)."""
+    current = torch.cuda.current_stream(device)
+    if stream is None or int(stream.cuda_stream) == current.cuda_stream:
+        return torch.empty(shape, dtype=dtype, device=device)
+    if not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(int(stream.cuda_stream), device=device)
+    with torch.cuda.stream(stream):
+        t = torch.empty(shape, dtype=dtype, device=device)
+    t.record_stream(current)
+    return t
+
+
 def _check(status: int, where: str) -> None:
     if status != AP_OK:
         raise ApError(status, where)
@@ -272,8 +286,7 @@ def ap_pool_scores(acc, block: int, causal=False, pooled=None, stream=None):
     if acc.dtype != torch.float32:
         raise ValueError("acc must be float32")
     if pooled is None:
-        pooled = torch.empty((H, max(Lq // max(block, 1), 1), max(Lk // max(block, 1), 1)), dtype=torch.float32,
-                             device=acc.device)
+        pooled = _empty((H, max(Lq // max(block, 1), 1), max(Lk // max(block, 1), 1)), torch.float32, acc.device, stream)
     _check(lib.ap_pool_scores(_ptr(acc), H, Lq, Lk, int(block), int(bool(causal)), _ptr(pooled), _stream(stream)),
            "ap_pool_scores")
     return pooled
@@ -285,7 +298,7 @@ def ap_expand_block_mask(block_mask, block: int, causal=False, mask=None, stream
     if block_mask.dtype != torch.uint8:
         raise ValueError("block_mask must be uint8")
     if mask is None:
-        mask = torch.empty((H, R * block, C * block), dtype=torch.uint8, device=block_mask.device)
+        mask = _empty((H, R * block, C * block), torch.uint8, block_mask.device, stream)
     _check(lib.ap_expand_block_mask(_ptr(block_mask), H, R * block, C * block, int(block), int(bool(causal)),
                                     _ptr(mask), _stream(stream)), "ap_expand_block_mask")
     return mask
@@ -306,7 +319,7 @@ def ap_mask_to_tiles(mask, tiles: Tiles, workspace=None, stream=None) -> None:
     if mask.dtype != torch.uint8:
         raise ValueError("mask must be uint8")
     if workspace is None:
-        workspace = torch.empty(ap_mask_to_tiles_workspace_bytes(H, Lq, Lk), dtype=torch.uint8, device=mask.device)
+        workspace = _empty(ap_mask_to_tiles_workspace_bytes(H, Lq, Lk), torch.uint8, mask.device, stream)
     _check(lib.ap_mask_to_tiles(_ptr(mask), H, Lq, Lk, ctypes.byref(tiles.c), _ptr(workspace),
                                 workspace.numel(), _stream(stream)), "ap_mask_to_tiles")
 

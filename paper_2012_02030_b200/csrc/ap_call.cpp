@@ -9,8 +9,10 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 
+#include <optional>
 #include <string>
 
 #include "ap.h"
@@ -115,6 +117,29 @@ auto unlocked(F f) {
   return f();
 }
 
+// Memory for a call on `stream`.  Where that is not the current stream, the memory is allocated for `stream`: it is not
+// handed out again before the call's kernels have run, nor does the call use memory that earlier work of the current
+// stream still reads.  What the caller gets to see is also held for the current stream.
+class Memory {
+ public:
+  Memory(const at::Tensor &like, void *stream) : current_(c10::cuda::getCurrentCUDAStream(like.device().index())) {
+    if (current_.stream() != stream)
+      guard_.emplace(c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream), like.device().index()));
+  }
+  at::Tensor output(const at::Tensor &like) const {
+    at::Tensor t = at::empty_like(like);
+    if (guard_) t.record_stream(current_.unwrap());
+    return t;
+  }
+  at::Tensor bytes(size_t n, const at::Tensor &like) const {
+    return at::empty({(int64_t)n}, like.options().dtype(at::kByte));
+  }
+
+ private:
+  c10::cuda::CUDAStream current_;
+  std::optional<c10::cuda::CUDAStreamGuard> guard_;
+};
+
 struct Shape {
   int B, H, Lq, Lk, d;
 };
@@ -184,7 +209,6 @@ PyObject *py_build_mask(PyObject *, PyObject *const *a, Py_ssize_t n) {
     const int H = (int)acc.size(0), Lq = (int)acc.size(1), Lk = (int)acc.size(2);
     at::Tensor ws;
     if (a[9] != Py_None) ws = tensor(a[9], "workspace");
-    const at::TensorOptions bytes = acc.options().dtype(at::kByte);
     const float *in = static_cast<const float *>(acc.data_ptr());
     const double keep = number(a[2]);
     const int causal = truth(a[3]), diag = truth(a[4]);
@@ -194,7 +218,7 @@ PyObject *py_build_mask(PyObject *, PyObject *const *a, Py_ssize_t n) {
     void *s = stream_of(a[10]);
     const auto fn = rule == 1 ? g_fn.build_mask_layer : g_fn.build_mask;
     const ap_status st = unlocked([&] {
-      if (!ws.defined()) ws = at::empty({(int64_t)g_fn.build_mask_workspace(H, Lq, Lk)}, bytes);
+      if (!ws.defined()) ws = Memory(acc, s).bytes(g_fn.build_mask_workspace(H, Lq, Lk), acc);
       void *p = ws.data_ptr();
       const size_t n = (size_t)ws.numel();
       return rule == 2 ? g_fn.build_mask_ex(in, H, Lq, Lk, keep, causal, diag, (int)flags, mask, tiles, nnz, p, n, s)
@@ -221,7 +245,7 @@ PyObject *py_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
     void *stream = stream_of(a[6]);
     const auto fn = kEntmax ? g_fn.fwd_entmax : g_fn.fwd;
     const ap_status st = unlocked([&] {
-      if (!o.defined()) o = at::empty_like(q);
+      if (!o.defined()) o = Memory(q, stream).output(q);
       return fn(pq, pk, pv, tiles, o.data_ptr(), s.B, s.H, s.Lq, s.Lk, s.d, dt, scale, stream);
     });
     PyObject *out = a[4] == Py_None ? THPVariable_Wrap(std::move(o)) : Py_NewRef(a[4]);
@@ -249,11 +273,13 @@ PyObject *py_bwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
     const float scale = (float)number(a[9]);
     void *stream = stream_of(a[11]);
     const ap_status st = unlocked([&] {
-      if (!dq.defined()) dq = at::empty_like(q);
-      if (!dk.defined()) dk = at::empty_like(k);
-      if (!dv.defined()) dv = at::empty_like(v);
-      if (!ws.defined())
-        ws = at::empty({(int64_t)g_fn.bwd_workspace(s.B, s.H, s.Lq, s.Lk)}, q.options().dtype(at::kByte));
+      {
+        const Memory memory(q, stream);
+        if (!dq.defined()) dq = memory.output(q);
+        if (!dk.defined()) dk = memory.output(k);
+        if (!dv.defined()) dv = memory.output(v);
+        if (!ws.defined()) ws = memory.bytes(g_fn.bwd_workspace(s.B, s.H, s.Lq, s.Lk), q);
+      }
       return g_fn.bwd(pq, pk, pv, po, pg, tiles, dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), s.B, s.H, s.Lq, s.Lk, s.d, dt,
                       scale, ws.data_ptr(), (size_t)ws.numel(), stream);
     });

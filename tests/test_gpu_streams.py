@@ -102,3 +102,34 @@ def test_out_of_memory_is_raised_as_such(ap):
             ap.ap_build_mask(acc, 0.1, True, True, mask=mask)
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
+
+
+def test_memory_of_calls_on_another_stream(ap):
+    """Workspaces and outputs that the binding allocates for a call on a stream that is not the current one: the memory is not
+    handed out to the current stream before the call has run."""
+    side = torch.cuda.Stream()
+    H, L = 4, 512
+    acc = torch.rand((H, L, L), generator=torch.Generator(device="cuda").manual_seed(5), device="cuda")
+    args, _, _ = _attention(ap, 2, H, L, 64, 6)
+    mask = torch.empty((H, L, L), dtype=torch.uint8, device="cuda")
+    tiles = ap.Tiles(H, L, L)
+
+    def calls(stream):
+        ap.ap_build_mask(acc, 0.1, True, True, mask=mask, tiles=tiles, stream=stream)
+        ap.ap_mask_to_tiles(mask, tiles, stream=stream)
+        out = ap.ap_sparse_attention_fwd(*args[:3], tiles, stream=stream)
+        return (out,) + tuple(ap.ap_sparse_attention_bwd(*args[:3], out, args[4], tiles, stream=stream)) + (
+            ap.ap_pool_scores(acc, 32, True, stream=stream),)
+
+    want = [t.clone() for t in calls(None)] + [mask.clone()]
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    _busy(side)
+    got = calls(side)
+    # the current stream, meanwhile: memory of every size that the calls used, overwritten at once
+    junk = [torch.full((n,), 0x7f, dtype=torch.uint8, device="cuda") for n in [1 << k for k in range(9, 26)] * 4]
+    torch.cuda.synchronize()
+    del junk
+    assert ap.ap_device_status() == ap.AP_OK
+    for a, b in zip(list(got) + [mask], want):
+        assert torch.equal(a, b)
