@@ -174,6 +174,9 @@ try:
 except ImportError as e:
     raise ImportError("_ap_call.so is missing or does not match this torch: build it with "
                       "`python -m paper_2012_02030_b200.build` (there is no fallback implementation)") from e
+if _call.built_for != "torch " + torch.__version__:
+    raise ImportError("_ap_call.so was built for %s, this is torch %s: build it again with `python -m "
+                      "paper_2012_02030_b200.build`" % (_call.built_for, torch.__version__))
 _call.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in EXPORTS}, _check)
 
 

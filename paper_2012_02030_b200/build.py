@@ -44,10 +44,19 @@ def call_command(target: str):
     cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
     return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
             "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+            '-DAP_TORCH_VERSION="%s"' % torch.__version__,
             "-I", os.path.join(ROOT, "include"), "-isystem", sysconfig.get_paths()["include"],
             "-isystem", os.path.join(base, "include"), "-isystem", os.path.join(cuda, "include"),
             CALL_SRC, "-o", target, "-L", libs, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python",
             "-Wl,-rpath," + libs]
+
+
+def _other_torch(target: str) -> bool:
+    """Whether the call path at `target` was compiled with another torch's headers (it names the one it was)."""
+    import torch
+
+    with open(target, "rb") as f:
+        return b"torch %s\0" % torch.__version__.encode() not in f.read()
 
 
 def _stale(target: str, deps) -> bool:
@@ -77,7 +86,8 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
             raise RuntimeError("nvcc failed:\n%s\n%s\n%s" % (" ".join(cmd), r.stdout, r.stderr))
         return r.stdout + r.stderr
 
-    if force or _stale(CALL_LIB, [CALL_SRC, os.path.join(ROOT, "include", "ap.h"), os.path.abspath(__file__)]):
+    if (force or _stale(CALL_LIB, [CALL_SRC, os.path.join(ROOT, "include", "ap.h"), os.path.abspath(__file__)])
+            or _other_torch(CALL_LIB)):
         call_tmp = CALL_LIB + ".%d.tmp" % os.getpid()
         run(call_command(call_tmp))
         os.replace(call_tmp, CALL_LIB)

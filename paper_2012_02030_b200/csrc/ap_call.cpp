@@ -328,4 +328,9 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_ap_call", "Native call path of 
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__ap_call(void) { return PyModule_Create(&g_module); }
+// The torch whose headers this was compiled with: binding.py loads it beside no other, build.py looks for it in the file.
+PyMODINIT_FUNC PyInit__ap_call(void) {
+  PyObject *m = PyModule_Create(&g_module);
+  if (m && PyModule_AddStringConstant(m, "built_for", "torch " AP_TORCH_VERSION) < 0) Py_CLEAR(m);
+  return m;
+}

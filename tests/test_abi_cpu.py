@@ -174,3 +174,15 @@ def test_no_cpu_fallback_without_a_device():
     with pytest.raises(ValueError):
         ap.ap_sparse_attention_fwd(torch.zeros(1, 2, 128, 64), torch.zeros(1, 2, 128, 64),
                                    torch.zeros(1, 2, 128, 64), None)
+
+
+def test_call_path_names_the_torch_it_was_built_for(tmp_path):
+    import torch
+
+    from paper_2012_02030_b200 import build
+
+    assert ap._call.built_for == "torch " + torch.__version__
+    assert not build._other_torch(build.CALL_LIB)
+    other = tmp_path / "other.so"
+    other.write_bytes(b"torch 0.0\0")
+    assert build._other_torch(str(other))
