@@ -436,10 +436,10 @@ __device__ __forceinline__ void patch(const uint2 *__restrict__ cand, uint32_t n
     if (keep && mask) mask[((size_t)h * Lq + i) * Lk + j] = 1;
     if (stage_bitmap) {
       const uint32_t tile = (uint32_t)((h * n_qt + (int)(i >> 7)) * n_kt + (int)(j >> 7));
-      const uint32_t word = tile * (uint32_t)kBitmapWords + 4u * (i & 127u) + ((j & 127u) >> 5);
+      const size_t word = (size_t)tile * kBitmapWords + 4u * (i & 127u) + ((j & 127u) >> 5);
       const unsigned voters = __ballot_sync(0xffffffffu, keep);
       if (keep) {
-        const unsigned same_word = __match_any_sync(voters, word);
+        const unsigned same_word = __match_any_sync(voters, (unsigned long long)word);
         const uint32_t all_bits = __reduce_or_sync(same_word, 1u << (j & 31u));
         if (lane == __ffs((int)same_word) - 1) atomicOr(stage_bitmap + word, all_bits);
         const unsigned same_tile = __match_any_sync(voters, tile);

@@ -264,3 +264,23 @@ def test_entmax_forward_dense_rows(ap, dtype, d, B, keep):
     w = W["tiny"].scaled(B=B, H=1, Lq=260, Lk=700 if B == 1 else 300, d=d, dtype=dtype)
     mask = inputs.random_mask(1, w.Lq, w.Lk, keep, seed=511, empty_rows=(9,))
     tp._entmax_fwd_case(ap, w, mask)
+
+
+def test_build_mask_more_tiles_than_bitmap_words_in_32_bits(ap):
+    """2^23 tiles hold 2^32 bitmap words: the entries that the select adds to the bitmaps of the last heads stay with them."""
+    H, Lk, k = 1030, 1 << 20, 20
+    acc = torch.rand((H, 1, Lk), generator=torch.Generator(device="cuda").manual_seed(510), device="cuda")
+    tiles = ap.Tiles(H, 1, Lk, cap=1 << 15)
+    ap.ap_build_mask(acc, k / Lk, False, False, tiles=tiles)
+    assert ap.ap_device_status() == ap.AP_OK
+    row_ptr = tiles.row_ptr.cpu().numpy()
+    for h in (0, 3, 1023, 1024, H - 1):
+        cols = []
+        for t in range(row_ptr[h], row_ptr[h + 1]):
+            words = tiles.bitmap[t].cpu().numpy().view(np.uint32)
+            assert not words[1:].any()
+            bits = np.unpackbits(words[0].view(np.uint8), bitorder="little")
+            cols += [int(tiles.col_idx[t]) * 128 + int(c) for c in np.flatnonzero(bits)]
+        assert len(cols) == k
+        got = acc[h, 0, torch.tensor(cols, device="cuda")].sort(descending=True).values
+        assert torch.equal(got, acc[h, 0].topk(k).values)
