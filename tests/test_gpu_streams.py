@@ -69,24 +69,30 @@ def test_other_threads_run_while_a_launch_waits(ap):
     side = torch.cuda.Stream()
     out = torch.empty_like(args[0])
     torch.cuda.synchronize()
-    done = threading.Event()
+    done, errors = threading.Event(), []
 
     def launches():
-        for _ in range(4000):
-            ap.ap_sparse_attention_fwd(*args[:3], args[5], out, stream=side)
-        done.set()
+        try:
+            torch.zeros(1, device="cuda")  # the thread's first CUDA call
+            for _ in range(4000):
+                ap.ap_sparse_attention_fwd(*args[:3], args[5], out, stream=side)
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+        finally:
+            done.set()
 
     _busy(side, 1.0)
     thread = threading.Thread(target=launches)
     began = last = time.perf_counter()
     gap = 0.0
     thread.start()
-    while not done.wait(0.001):
+    while not done.wait(0.001) and last - began < 20.0:
         now = time.perf_counter()
         gap, last = max(gap, now - last), now
-    thread.join()
+    thread.join(20.0)
     gap, took = max(gap, time.perf_counter() - last), time.perf_counter() - began
     torch.cuda.synchronize()
+    assert done.is_set() and not errors, errors
     assert took < 0.5 or gap < 0.25  # (a queue without end would never make a launch wait)
 
 
