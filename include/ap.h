@@ -207,6 +207,10 @@ size_t ap_mask_to_tiles_workspace_bytes(int H, int Lq, int Lk);
  *   Q, K   [B,H,Lq,d], [B,H,Lk,d] of type dt (AP_BF16 and AP_F16 run on the tensor cores)
  *   bias   [H,Lq,Lk] fp32 added after scaling, or NULL
  *   scale  multiplier of Q.K^T; 0 selects 1/sqrt(d)
+ * Several streams: 16-bit calls with fewer (head, 128-row query tile) pairs than the GPU has SMs share eight
+ * sets of counters in device memory, taken in rotation.  A call must not overlap on the GPU with the eighth
+ * call after it (or a multiple), on whatever streams they are; a captured call keeps its set, so replays of its
+ * graph must not overlap with other such calls.
  */
 ap_status ap_accumulate_attention(float *acc, const void *Q, const void *K, const float *bias,
                                   int B, int H, int Lq, int Lk, int d, ap_dtype dt, int causal,

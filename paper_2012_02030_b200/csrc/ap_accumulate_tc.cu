@@ -112,7 +112,7 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p) {
 }
 
 // Turn counters of the chunked launches: one word per (head, query tile, key tile), zeroed before every
-// such launch.  Launches that overlap on the GPU (different streams) take different sets.
+// such launch.  Calls take the sets in rotation: two launches that share one must not overlap on the GPU (see ap.h).
 constexpr size_t kTurnWords = 8192;
 constexpr int kTurnSets = 8;
 constexpr int kMinChunk = 2;  // samples per CTA at least
