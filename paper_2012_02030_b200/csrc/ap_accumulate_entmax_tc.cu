@@ -245,6 +245,7 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                 hbias[32 * q + 4 * k + 2] = t.z * 0.5f; hbias[32 * q + 4 * k + 3] = t.w * 0.5f;
               }
             }
+            fence_proxy_async_smem();  // the reads are over before the next tile's copy may write
             mbar_arrive(&bars->bias_empty);
           } else {
 #pragma unroll

@@ -329,6 +329,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           bias2[4 * k] = t.x * kLog2e; bias2[4 * k + 1] = t.y * kLog2e;
           bias2[4 * k + 2] = t.z * kLog2e; bias2[4 * k + 3] = t.w * kLog2e;
         }
+        fence_proxy_async_smem();  // the reads are over before the next tile's copy may write
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars->bias_empty);
       } else {

@@ -239,7 +239,9 @@ __device__ __forceinline__ void bulk_wait_group_read0() {
 // all of this thread's bulk groups are complete
 __device__ __forceinline__ void bulk_wait_group0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// generic-proxy writes to shared memory -> visible to the async proxy (TMA / tcgen05)
+// Orders the calling thread's accesses to shared memory before what the async proxy (TMA / tcgen05) does after it: writes
+// become visible to it, and reads have taken place before a copy overwrites the place.  An arrival on an mbarrier alone does
+// not hold the copy back: loads whose values are not used yet may still be under way when it is counted.
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
