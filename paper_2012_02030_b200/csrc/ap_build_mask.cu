@@ -7,8 +7,9 @@
 // first three give the threshold; the last three, the index of the last kept entry equal to it,
 // run only where some of those entries are kept and others are not.
 //
-// Small inputs (up to kDirectEntries in all, a few times less than L2 holds) select straight over the
-// accumulator, one pass over it per digit.  Larger ones take a shortcut that reads it once: a
+// Inputs that fit into the shared memory of the SMs are read once and held there (held_kernel: select, mask and bitmaps in one).
+// Larger ones of up to kDirectEntries in all, a few times less than L2 holds, select straight over the
+// accumulator, one pass over it per digit.  Still larger ones take a shortcut that reads it once: a
 // random sample of the selection brackets the threshold between two pivot keys, one
 // pass counts the keys above the upper pivot and collects those between the
 // pivots, and the select runs over the collected entries; it is exact whenever the bracket holds
@@ -915,6 +916,296 @@ __global__ void __launch_bounds__(32 * kCtaWarps, kCtaWarps == 4 ? 8 : 2) emit_k
   }
 }
 
+// ---- inputs that fit into shared memory --------------------------------------------------------
+
+constexpr int kHeldThreads = 1024;
+constexpr int kUnitRows = 32, kUnitWords = kUnitRows * kTile;  // a quarter of a 128 x 128 tile: a row per warp
+constexpr int kHeldUnits = 12;                                 // per CTA at most, one CTA per SM
+constexpr int kHeldSels = kHeldUnits / 4 + 1;                  // selections that these belong to (at least four units each), at most
+
+// The units of the domain's tiles, selection by selection, dealt out evenly to the CTAs of the grid.
+struct Held {
+  int H, Lq, Lk, n_qt, n_kt, causal, per_layer;
+  int per_head;  // units of a head's domain
+  __host__ __device__ int total() const { return H * per_head; }
+  __device__ int first_of(int cta, int ctas) const { return (int)((long long)cta * total() / ctas); }
+  __device__ int owner_of(int u, int ctas) const { return (int)(((long long)(u + 1) * ctas - 1) / total()); }
+  __device__ int sel_of(int u) const { return per_layer ? 0 : u / per_head; }
+  // the CTAs that hold a unit of the selection: `first` and how many
+  __device__ int2 ctas_of(int sel, int ctas) const {
+    const int n = per_layer ? total() : per_head, first = owner_of(sel * n, ctas);
+    return make_int2(first, owner_of((sel + 1) * n - 1, ctas) - first + 1);
+  }
+};
+
+// Cooperative.  The whole of a call but the compaction in one kernel: every CTA copies its units into shared memory as keys,
+// takes part in the select of the selections they belong to, and writes their mask and bitmaps.
+//
+// What bounds it: latency, three times a histogram, its merging into global memory, a barrier of the selection's CTAs and the pick of
+// a digit.  The accumulator is read once; with a scan of it per digit and an emit pass of its own one layer of 16 heads x 512
+// took 60 us, 39 with this kernel, some 20 of them its own (59 with whole tiles instead of quarters, of which a few CTAs then have two).  The first histogram's
+// counts fall into few bins (a digit is little more than the exponent), so a warp takes entries of different rows and columns:
+// neighbours, which are alike, would queue for the same bin.
+__global__ void __launch_bounds__(kHeldThreads, 1)
+held_kernel(const float *__restrict__ acc, const Held p, int diag, unsigned long long k_rest, SelectState *state,
+            uint32_t *hist, int keep_ties, long long nnz_init, int64_t *__restrict__ nnz, uint8_t *__restrict__ mask,
+            uint32_t *__restrict__ stage_bitmap, int32_t *__restrict__ stage_count, uint32_t *__restrict__ stage_groups,
+            unsigned *err) {
+  extern __shared__ __align__(16) uint32_t held_smem[];
+  uint32_t *counts_s = held_smem;                     // [kHeldSels][kBins]: a histogram per selection of the CTA
+  uint32_t *keys_s = held_smem + kHeldSels * kBins;   // [units][32][128]; 0: not one of the selection's
+  struct Unit {
+    int h, row0, kt, tile;
+  };
+  struct Sel {  // the select's progress
+    unsigned long long rest;
+    uint32_t prefix, thr, tie_cut, count;
+    int going, sharers, rank;
+  };
+  __shared__ Unit units[kHeldUnits];
+  __shared__ Sel sels[kHeldSels];
+  __shared__ uint32_t warp_sums[kHeldThreads / 32], unit_votes[kHeldUnits];
+  __shared__ int unit_count[kHeldUnits], ok_s;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, ctas = (int)gridDim.x, cta = (int)blockIdx.x;
+  const int Lq = p.Lq, Lk = p.Lk, off = (p.causal || diag) ? Lk - Lq : 0;
+  const int u0 = p.first_of(cta, ctas), n_units = p.first_of(cta + 1, ctas) - u0;
+  const int sel0 = p.sel_of(u0), n_sel = p.sel_of(u0 + n_units - 1) - sel0 + 1;
+  if (t < n_units) {
+    const int h = (u0 + t) / p.per_head, in_head = (u0 + t) - h * p.per_head;
+    int qt = 0;
+    while (qt + 1 < p.n_qt && (int)dense_row_start(qt + 1, p.n_kt, Lq, Lk, p.causal) <= in_head / 4) ++qt;
+    const int kt = in_head / 4 - (int)dense_row_start(qt, p.n_kt, Lq, Lk, p.causal), tile = (h * p.n_qt + qt) * p.n_kt + kt;
+    units[t] = Unit{h, qt * kTile + kUnitRows * (in_head & 3), kt, tile};
+    unit_votes[t] = 0u;
+    unit_count[t] = 0;
+    // (added to by the CTAs of the selection, behind a barrier of theirs)
+    if (stage_count && (in_head & 3) == 0) {
+      stage_count[tile] = 0;
+      stage_groups[tile] = 0u;
+    }
+    if (nnz && in_head == 0) nnz[h] = nnz_init;
+  }
+  if (t < n_sel) {
+    const int2 c = p.ctas_of(sel0 + t, ctas);
+    sels[t] = Sel{k_rest, 0u, 0u, 0xffffffffu, 0u, 1, c.y, cta - c.x};
+  }
+  __syncthreads();
+  // ---- keys of this CTA's units
+  const bool vec = (Lk & 3) == 0 && (reinterpret_cast<uintptr_t>(acc) & 15) == 0;
+#pragma unroll 1
+  for (int x0 = 0; x0 < n_units; x0 += 4) {
+    float v[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      v[u][0] = v[u][1] = v[u][2] = v[u][3] = 0.f;
+      if (x0 + u < n_units) {
+        const Unit un = units[x0 + u];
+        const int i = un.row0 + warp;
+        if (i < Lq) load4(acc + ((size_t)un.h * Lq + i) * Lk, un.kt * kTile + 4 * lane, Lk, vec, v[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (x0 + u < n_units) {
+        const Unit un = units[x0 + u];
+        const int i = un.row0 + warp, own = i + off, j = un.kt * kTile + 4 * lane;
+        const int jend = i >= Lq ? 0 : p.causal ? min(Lk, own + 1) : Lk;
+        uint32_t k[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) k[c] = j + c < jend && !(diag && j + c == own) ? key_of(v[u][c]) : 0u;
+        reinterpret_cast<uint4 *>(keys_s + (x0 + u) * kUnitWords)[t] = make_uint4(k[0], k[1], k[2], k[3]);
+      }
+  }
+  // Tiles outside the domain: nothing is kept (their bitmaps are not read).  Written while the first digit's counts come in.
+  const bool mask4 = (Lk & 3) == 0 && (reinterpret_cast<uintptr_t>(mask) & 3) == 0;
+  auto clear_outside = [&]() {
+    const int n_rows = p.H * p.n_qt;
+    for (int x = cta; x < n_rows; x += ctas) {
+      const int h = x / p.n_qt, qt = x % p.n_qt, kt0 = dense_row_tiles(qt, p.n_kt, Lq, Lk, 1);
+      if (mask) {
+        const int j0 = kt0 * kTile;
+        for (int i = qt * kTile + warp; i < min(Lq, (qt + 1) * kTile); i += kHeldThreads / 32) {
+          uint8_t *m = mask + ((size_t)h * Lq + i) * Lk;
+          if (mask4) {
+            for (int j = j0 + 4 * lane; j < Lk; j += kTile) *reinterpret_cast<uint32_t *>(m + j) = 0u;
+          } else {
+            for (int j = j0 + lane; j < Lk; j += 32) m[j] = 0;
+          }
+        }
+      }
+      if (stage_count && t < p.n_kt - kt0) {
+        stage_count[x * p.n_kt + kt0 + t] = 0;
+        stage_groups[x * p.n_kt + kt0 + t] = 0u;
+      }
+    }
+  };
+  // ---- select
+  const uint32_t *my_keys = keys_s + ((warp + 11 * lane) & 31) * kTile + lane;  // + 32 e: this thread's four entries of a unit
+#pragma unroll 1
+  for (int digit = 0; digit < 2 * kPasses; ++digit) {
+    const int pass = digit % kPasses, shift = digit_shift(pass);
+    const bool of_index = digit >= kPasses;
+    const uint32_t dmask = digit_mask(pass), hi_mask = above_digit(pass);
+    for (int b = t; b < n_sel * kBins; b += kHeldThreads) counts_s[b] = 0u;
+    __syncthreads();  // (the keys are there, the last digit has been picked)
+    bool any = false;
+#pragma unroll 1
+    for (int q = 0; q < n_sel; ++q) {
+      if (!sels[q].going) continue;
+      any = true;
+      const uint32_t pre = sels[q].prefix, thr = sels[q].thr;
+      uint32_t *mine = counts_s + q * kBins;
+      const int n = p.per_layer ? p.total() : p.per_head;  // units of a selection
+      const int x0 = max((sel0 + q) * n - u0, 0), x1 = min((sel0 + q + 1) * n - u0, n_units);
+      if (!of_index) {
+#pragma unroll 2
+        for (int x = x0; x < x1; ++x) {
+          uint32_t k[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) k[e] = my_keys[x * kUnitWords + 32 * e];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (k[e] != 0u && (k[e] & hi_mask) == pre) atomicAdd(&mine[(k[e] >> shift) & dmask], 1u);
+        }
+      } else {
+        for (int x = x0; x < x1; ++x) {
+          const Unit un = units[x];
+          const uint32_t row = (p.per_layer ? (uint32_t)un.h * (uint32_t)Lq : 0u) + (uint32_t)(un.row0 + ((warp + 11 * lane) & 31));
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const uint32_t word = ~(row * (uint32_t)Lk + (uint32_t)(un.kt * kTile + lane + 32 * e));
+            if (my_keys[x * kUnitWords + 32 * e] == thr && (word & hi_mask) == pre)
+              atomicAdd(&mine[(word >> shift) & dmask], 1u);
+          }
+        }
+      }
+    }
+    if (!any) break;
+    __syncthreads();
+    // the histograms of selections that several CTAs share meet in global memory
+    for (int q = 0; q < n_sel; ++q) {
+      const int sharers = sels[q].sharers;
+      if (!sels[q].going || sharers == 1) continue;
+      uint32_t *all = hist + ((size_t)(sel0 + q) * kHistBuffers + digit % kHistBuffers) * kBins;
+      for (int b = t; b < kBins; b += kHeldThreads)
+        if (counts_s[q * kBins + b]) atomicAdd(all + b, counts_s[q * kBins + b]);
+      if (digit >= 2) {  // the buffer of two digits ago has been read by all: ready for the next digit but ...
+        uint32_t *old = hist + ((size_t)(sel0 + q) * kHistBuffers + (digit - 2) % kHistBuffers) * kBins;
+        for (int b = sels[q].rank * kHeldThreads + t; b < kBins; b += sharers * kHeldThreads) old[b] = 0u;
+      }
+    }
+    __syncthreads();
+    if (t == 0) {
+      __threadfence();
+      for (int q = 0; q < n_sel; ++q)
+        if (sels[q].going && sels[q].sharers > 1) atomicAdd(&state[sel0 + q].barrier, 1u);
+    }
+    if (digit == 0 && p.causal) clear_outside();
+    if (t == 0) {
+      bool ok = true;
+      for (int q = 0; q < n_sel; ++q)
+        if (sels[q].going && sels[q].sharers > 1)
+          ok = ok && reached(&state[sel0 + q].barrier, (uint32_t)sels[q].sharers * (uint32_t)(digit + 1));
+      __threadfence();
+      ok_s = ok;
+      if (!ok) atomicOr(err, kDevErrTimeout);
+    }
+    __syncthreads();
+    if (!ok_s) return;
+    for (int q = 0; q < n_sel; ++q) {
+      if (!sels[q].going) continue;
+      const unsigned long long rest = sels[q].rest;
+      // thread t owns bins 2047 - 2t and 2046 - 2t (descending); the owner of the wanted rank picks the digit
+      uint2 c;
+      if (sels[q].sharers > 1) {
+        const uint32_t *all = hist + ((size_t)(sel0 + q) * kHistBuffers + digit % kHistBuffers) * kBins;
+        c = __ldcg(reinterpret_cast<const uint2 *>(all) + (kBins / 2 - 1 - t));
+      } else {
+        c = reinterpret_cast<const uint2 *>(counts_s + q * kBins)[kBins / 2 - 1 - t];
+      }
+      const uint32_t sum = c.x + c.y;
+      uint32_t incl = sum;  // (fewer than 2^32 entries: at most kHeldUnits units per SM)
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      if (lane == 31) warp_sums[warp] = incl;
+      __syncthreads();
+      const unsigned long long before = incl - sum + __reduce_add_sync(0xffffffffu, lane < warp ? warp_sums[lane] : 0u);
+      if (before < rest && before + sum >= rest) {  // exactly one thread
+        Sel &st = sels[q];
+        const bool first = before + c.y >= rest;
+        const uint32_t bin = (uint32_t)(kBins - 1 - 2 * t - (first ? 0 : 1)), count = first ? c.y : c.x;
+        const uint32_t prefix = st.prefix | bin << shift;
+        st.rest = rest - before - (first ? 0u : c.y);
+        st.prefix = digit == kPasses - 1 ? 0u : prefix;
+        if (digit == kPasses - 1) {
+          st.thr = prefix;
+          if (keep_ties || st.rest == count) st.going = 0;  // every entry equal to the threshold is kept
+        } else if (digit == 2 * kPasses - 1) {
+          st.tie_cut = ~prefix;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  // ---- mask and bitmaps
+#pragma unroll 2
+  for (int x = 0; x < n_units; ++x) {
+    const Unit un = units[x];
+    const int q = p.sel_of(u0 + x) - sel0;
+    const uint32_t thr = sels[q].thr;
+    const int i = un.row0 + warp, j = un.kt * kTile + 4 * lane;
+    const uint4 k = reinterpret_cast<const uint4 *>(keys_s + x * kUnitWords)[t];
+    uint32_t kept = (k.x >= thr ? 1u : 0u) | (k.y >= thr ? 2u : 0u) | (k.z >= thr ? 4u : 0u) | (k.w >= thr ? 8u : 0u);
+    if (sels[q].tie_cut != 0xffffffffu) {  // entries equal to the threshold are kept up to the last kept one only
+      const uint32_t cut = sels[q].tie_cut;
+      const uint32_t ties = (k.x == thr ? 1u : 0u) | (k.y == thr ? 2u : 0u) | (k.z == thr ? 4u : 0u) | (k.w == thr ? 8u : 0u);
+      const uint32_t first = ((p.per_layer ? (uint32_t)un.h * (uint32_t)Lq : 0u) + (uint32_t)i) * (uint32_t)Lk + (uint32_t)j;
+      if (first > cut)
+        kept &= ~ties;
+      else if (cut - first < 3u)
+        kept &= ~(ties & ~((2u << (cut - first)) - 1u));
+    }
+    if (diag && i < Lq && (unsigned)(i + off - j) < 4u) kept |= 1u << (i + off - j);
+    if (mask && i < Lq) {
+      uint8_t *m = mask + ((size_t)un.h * Lq + i) * Lk + j;
+      if (mask4) {  // four bits to four bytes: the products of the shifted copies do not meet
+        if (j < Lk) *reinterpret_cast<uint32_t *>(m) = (kept * 0x00204081u) & 0x01010101u;
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (j + c < Lk) m[c] = (kept >> c) & 1u;
+      }
+    }
+    const int count = __reduce_add_sync(0xffffffffu, __popc(kept));
+    if (stage_bitmap) {  // eight lanes make a word
+      uint32_t w = kept << (4 * (lane & 7));
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) w |= __shfl_xor_sync(0xffffffffu, w, o);
+      const int r = un.row0 % kTile + warp;
+      if ((lane & 7) == 0) stage_bitmap[(size_t)un.tile * kBitmapWords + 4 * r + (lane >> 3)] = w;
+      const uint32_t vote = __ballot_sync(0xffffffffu, kept != 0u);
+      if (lane == 0 && vote) atomicOr(&unit_votes[x], vote);
+    }
+    if (lane == 0 && count) atomicAdd(&unit_count[x], count);
+  }
+  __syncthreads();
+  if (t < n_units && unit_count[t]) {
+    const Unit un = units[t];
+    if (stage_count) {
+      atomicAdd(stage_count + un.tile, unit_count[t]);
+      uint32_t groups = 0u;  // a group is four lanes
+#pragma unroll
+      for (int g = 0; g < 8; ++g) groups |= ((unit_votes[t] >> (4 * g)) & 15u ? 1u : 0u) << g;
+      atomicOr(stage_groups + un.tile, groups);
+    }
+    if (nnz && (p.per_layer || keep_ties))
+      atomicAdd(reinterpret_cast<unsigned long long *>(nnz + un.h), (unsigned long long)unit_count[t]);
+  }
+}
+
 // Where the arrays of the select scratch lie.  The header and the states (and the histograms, where the select shares
 // them between CTAs) are zeroed before the first kernel of a call.
 struct Header {
@@ -956,6 +1247,36 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
   Scratch sc = carve(a.scratch, a.H, &header);
   // the selections: one per head over Lq rows, or one over the H*Lq rows of the layer
   const int n_sel = a.per_layer ? 1 : a.H;
+  // per head nnz = k; per layer, or with all ties kept, it is counted
+  const bool count_nnz = a.per_layer || a.keep_ties;
+  // What fits into the shared memory of the SMs is read once and held there.
+  Held held = {a.H, a.Lq, a.Lk, n_qt, n_kt, a.causal, a.per_layer, 4 * (int)dense_row_start(n_qt, n_kt, a.Lq, a.Lk, a.causal)};
+  if ((long long)a.H * held.per_head <= (long long)kHeldUnits * sms && n_sel <= kMaxSharedSelections && a.k_rest > 0) {
+    cudaError_t e = cudaMemsetAsync(header, 0, (reinterpret_cast<char *>(sc.hist) - reinterpret_cast<char *>(header)) +
+                                                   (size_t)n_sel * kHistBuffers * kBins * sizeof(uint32_t), s);
+    if (e != cudaSuccess) return e;
+    const int grid = held.total() < sms ? held.total() : sms;
+    int diag_arg = diag, keep_ties = a.keep_ties;
+    auto smem_of = [](int units) { return (kHeldSels * kBins + units * kUnitWords) * sizeof(uint32_t); };
+    e = cudaFuncSetAttribute(held_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(kHeldUnits));
+    if (e != cudaSuccess) return e;
+    const size_t smem = smem_of(ceil_div(held.total(), grid));
+    unsigned long long k_rest = (unsigned long long)a.k_rest;
+    long long nnz_init = count_nnz ? 0ll : (long long)a.k;
+    const float *acc = a.acc;
+    int64_t *nnz = a.nnz;
+    uint8_t *mask = a.mask;
+    uint32_t *stage_bitmap = a.stage_bitmap, *stage_groups = a.stage_groups;
+    int32_t *stage_count = a.stage_count;
+    void *args[] = {&acc, &held, &diag_arg, &k_rest, &sc.state, &sc.hist, &keep_ties, &nnz_init, &nnz, &mask, &stage_bitmap,
+                    &stage_count, &stage_groups, &err};
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(held_kernel), dim3(grid), dim3(kHeldThreads), args, smem, s);
+    if (e != cudaSuccess) return e;
+    count_launches(1);
+    if (!a.tiles) return cudaSuccess;
+    return launch_compact_staged(a.stage_bitmap, a.stage_count, a.stage_groups, *a.tiles, reinterpret_cast<int2 *>(sc.hist),
+                                 (size_t)kHistBuffers * kBins * sizeof(uint32_t) / sizeof(int2), &header->compact_barrier, s);
+  }
   const int rows = a.per_layer ? a.H * a.Lq : a.Lq;
   const int period = a.Lq;
   // CTAs per selection: all that fit, as far as there is a row for each of their warps
@@ -967,8 +1288,6 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
   const size_t hist_bytes = per_sel > 1 ? (size_t)n_sel * kHistBuffers * kBins * sizeof(uint32_t) : 0;
   cudaError_t e = cudaMemsetAsync(header, 0, (reinterpret_cast<char *>(sc.hist) - reinterpret_cast<char *>(header)) + hist_bytes, s);
   if (e != cudaSuccess) return e;
-  // per head nnz = k; per layer, or with all ties kept, the emit pass counts it
-  const bool count_nnz = a.per_layer || a.keep_ties;
   const long long n_valid = domain_size(a.Lq, a.Lk, a.causal);
   const long long n_rest = (n_valid - (diag ? a.Lq : 0)) * (a.per_layer ? a.H : 1);
   const long long cap = cand_capacity(n_rest);

@@ -11,20 +11,25 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t *p) {
   return v;
 }
 
+// By one thread: waits (bounded) until `arrivals` has been counted up to `target`.
+__device__ __forceinline__ bool reached(const uint32_t *arrivals, uint32_t target) {
+  constexpr uint32_t kMaxPolls = 1u << 22;
+  uint32_t polls = 0;
+  while (ld_acquire_gpu(arrivals) < target)
+    if (++polls >= kMaxPolls) return false;
+  return true;
+}
+
 // By all threads of a CTA: returns once `arrivals` has been counted up to `target` (every participant adds one), with
 // everything the others wrote before it visible.  false, and the device status word raised, if that takes too long.
 __device__ __forceinline__ bool cta_barrier(uint32_t *arrivals, uint32_t target, unsigned *err) {
-  constexpr uint32_t kMaxPolls = 1u << 22;
   __shared__ int ok_s;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(arrivals, 1u);
-    uint32_t polls = 0;
-    while (ld_acquire_gpu(arrivals) < target && ++polls < kMaxPolls) {
-    }
-    ok_s = polls < kMaxPolls;
-    if (polls >= kMaxPolls) atomicOr(err, kDevErrTimeout);
+    ok_s = reached(arrivals, target);
+    if (!ok_s) atomicOr(err, kDevErrTimeout);
     __threadfence();
   }
   __syncthreads();

@@ -305,3 +305,32 @@ def test_averages_repeat_bit_for_bit(ap, entry, dtype):
         differ += (acc != want).any()
     assert ap.ap_device_status() == ap.AP_OK
     assert int(differ) == 0
+
+
+@pytest.mark.parametrize("H,Lq,Lk,causal", [(8, 1280, 1280, True), (8, 1281, 1284, True),   # 440 and 528 tiles: 444 are held in shared memory
+                                            (1, 384, 18944, False), (1, 385, 18944, False),  # 444 and 592
+                                            (127, 40, 50, False), (129, 33, 130, True),     # selections a CTA has several of; too many
+                                            (3, 130, 259, True), (1, 1, 1, False), (5, 257, 129, False)])
+@pytest.mark.parametrize("rule", ["head", "layer", "ties"])
+@pytest.mark.parametrize("distinct", [True, False])
+def test_build_mask_held_in_shared_memory(ap, H, Lq, Lk, causal, rule, distinct):
+    """The largest inputs that are held and the smallest that are not, ragged edges, rows that start anywhere, a CTA with units of
+    several selections; thresholds among many equal values (index digits) and among distinct ones."""
+    g = torch.Generator().manual_seed(509 + H)
+    acc = torch.rand((H, Lq, Lk), generator=g)
+    if not distinct:
+        acc = (acc * 7).floor() / 7
+    keep, diag = 0.23, causal
+    mask = torch.full(acc.shape, 7, dtype=torch.uint8, device="cuda")
+    nnz = torch.full((H,), -1, dtype=torch.int64, device="cuda")
+    tiles = ap.Tiles(H, Lq, Lk)
+    if rule == "ties":
+        ap.ap_build_mask_ex(acc.cuda(), keep, causal, diag, ap.AP_MASK_KEEP_TIES, mask, tiles, nnz)
+        want, want_nnz = orc.build_mask_ties(acc.numpy(), keep, causal, diag)
+    else:
+        (ap.ap_build_mask_layer if rule == "layer" else ap.ap_build_mask)(acc.cuda(), keep, causal, diag, mask, tiles, nnz)
+        want, want_nnz = (orc.build_mask_layer if rule == "layer" else orc.build_mask)(acc.numpy(), keep, causal, diag)
+    assert ap.ap_device_status() == ap.AP_OK
+    assert np.array_equal(mask.cpu().numpy(), want)
+    assert np.array_equal(nnz.cpu().numpy(), want_nnz)
+    pu.assert_tiles_equal(tiles.to_host(), orc.mask_to_tiles(want))
