@@ -398,22 +398,141 @@ __global__ void __launch_bounds__(128) fill_rounds_kernel(const int32_t *__restr
 
 constexpr int kCompactCtasPerSm = 8;
 
+// Staging area -> list rows: what write_row needs.
+struct List {
+  const uint32_t *stage_bitmap;
+  const int32_t *stage_count;
+  const uint32_t *stage_groups;
+  int n_rows, n_kt, cap;
+  int32_t *row_ptr, *col_idx;
+  uint8_t *flags;
+  uint32_t *bitmap;
+  uint8_t *groups;
+  int32_t *round_ptr, *round_rows;
+  uint8_t *round_info;
+  uint32_t *round_bitmap;
+};
+
+constexpr int kSeg = 128;                      // key tiles per pass
+struct RowShared {
+  uint32_t slot_src[kSeg * 8 + 8];  // key tile << 4 | group << 1 | tile fully kept
+  int32_t seg_kt[kSeg];             // the pass's stored tiles
+  int2 warp_sums[4];
+  int slots;
+};
+
+// By 128 threads: part `part` of `parts` of list row `row`, whose `keep` tiles start at t0 and whose rounds at rho: its
+// tiles' bitmaps, and its rounds, straight from the staging area.
+__device__ __forceinline__ void write_row(const List &l, RowShared &sh, int row, int part, int parts, int t0, int keep, int rho) {
+  const int r = threadIdx.x, lane = r & 31, warp = r >> 5;
+  int seen = 0;
+  int pending = 0;  // slots carried over from the previous pass (fewer than eight)
+  const uint32_t *row_bitmap = l.stage_bitmap + (size_t)row * l.n_kt * kBitmapWords;
+  for (int base = 0; base < l.n_kt && seen < keep; base += kSeg) {
+    const int kt = base + r;
+    const size_t tile = (size_t)row * l.n_kt + kt;
+    const int count = kt < l.n_kt ? l.stage_count[tile] : 0;
+    const bool full = count == kTile * kTile;
+    int2 incl = make_int2(count > 0 ? 1 : 0, 0);
+    uint32_t gm = count > 0 ? l.stage_groups[tile] : 0u;
+    incl.y = __popc(gm);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl.x, o), y = __shfl_up_sync(0xffffffffu, incl.y, o);
+      if (lane >= o) incl.x += x, incl.y += y;
+    }
+    if (lane == 31) sh.warp_sums[warp] = incl;
+    __syncthreads();
+    int2 total = make_int2(0, 0);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      if (w < warp) incl.x += sh.warp_sums[w].x, incl.y += sh.warp_sums[w].y;
+      total.x += sh.warp_sums[w].x, total.y += sh.warp_sums[w].y;
+    }
+    const int rank = incl.x - 1;  // among the pass's stored tiles
+    const bool there = count > 0 && seen + rank < keep;
+    int s = pending + incl.y - __popc(gm);
+    if (there) {
+      sh.seg_kt[rank] = kt;
+      if (part == 0) {
+        const int t = t0 + seen + rank;
+        l.col_idx[t] = kt;
+        l.flags[t] = full ? 1 : 0;
+        l.groups[t] = (uint8_t)gm;
+      }
+      for (uint32_t left = gm; left; left &= left - 1u)
+        sh.slot_src[s++] = ((uint32_t)kt << 4) | ((uint32_t)(__ffs((int)left) - 1) << 1) | (full ? 1u : 0u);
+    }
+    const int n_here = min(total.x, keep - seen);
+    // (a row that is cut off ends with the slots of its last kept tile)
+    if (there && rank == n_here - 1) sh.slots = s;
+    __syncthreads();
+    const int avail = n_here > 0 ? sh.slots : pending;
+    for (int k0 = part; k0 < n_here; k0 += 4 * parts) {  // four tiles in flight
+      uint4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + u * parts < n_here)
+          v[u] = reinterpret_cast<const uint4 *>(row_bitmap + (size_t)sh.seg_kt[k0 + u * parts] * kBitmapWords)[r];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + u * parts < n_here)
+          reinterpret_cast<uint4 *>(l.bitmap + (size_t)(t0 + seen + k0 + u * parts) * kBitmapWords)[r] = v[u];
+    }
+    const bool last_pass = base + kSeg >= l.n_kt || seen + n_here >= keep;
+    const int n_emit = last_pass ? (avail + 7) / 8 : avail / 8;
+    for (int k = part; k < n_emit; k += parts) {
+      const int ng = min(8, avail - 8 * k);
+      uint32_t w[4] = {0u, 0u, 0u, 0u};
+      bool all_full = true;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (q >= ng) continue;
+        const uint32_t src = sh.slot_src[8 * k + q];
+        uint32_t field = 0xffffu;
+        if (!(src & 1u)) {
+          const uint32_t g = (src >> 1) & 7u;
+          field = (row_bitmap[(size_t)(src >> 4) * kBitmapWords + r * 4 + (g >> 1)] >> (16u * (g & 1u))) & 0xffffu;
+          all_full = false;
+        }
+        w[q >> 1] |= field << (16 * (q & 1));
+      }
+      const int out = rho + k;
+      if (out < l.cap) {
+        reinterpret_cast<uint4 *>(l.round_bitmap + (size_t)out * kBitmapWords)[r] = make_uint4(w[0], w[1], w[2], w[3]);
+        if (r < 8) {
+          const uint32_t src = r < ng ? sh.slot_src[8 * k + r] : 0u;
+          l.round_rows[(size_t)out * 8 + r] = r < ng ? (int)(src >> 4) * kTile + 16 * (int)((src >> 1) & 7u) : -1;
+        }
+        if (r == 0) l.round_info[out] = (uint8_t)(ng | ((all_full && ng == 8) ? 0x80 : 0));
+      }
+    }
+    rho += n_emit;
+    seen += n_here;
+    __syncthreads();
+    // fewer than eight slots are left over; they move to the front (no overlap: they start at or
+    // beyond index 8 unless nothing was written out, in which case they are in place already)
+    const int left = avail - 8 * n_emit;
+    if (!last_pass && n_emit > 0 && r < left) sh.slot_src[r] = sh.slot_src[8 * n_emit + r];
+    pending = last_pass ? 0 : left;
+    __syncthreads();
+  }
+}
+
+
 // Cooperative: staging area with group summaries -> tile list and rounds.  A CTA counts the tiles and rounds of its share
 // of the list rows; after a barrier it knows what lies before them and writes their offsets; after another, `parts`
 // CTAs per list row (n_rows * parts pieces, taken in turn) copy the row's bitmaps and write its rounds, straight from
 // the staging area.  The five kernels it stands for (still those of ap_mask_to_tiles) took 23 us on 16 heads x 512
 // tokens, most of it launches and the latency of short grids.
 __global__ void __launch_bounds__(128, kCompactCtasPerSm)
-compact_kernel(const uint32_t *__restrict__ stage_bitmap, const int32_t *__restrict__ stage_count,
-               const uint32_t *__restrict__ stage_groups, int n_rows, int n_kt, int cap, int parts, int32_t *row_ptr,
-               int32_t *__restrict__ col_idx, uint8_t *__restrict__ flags, uint32_t *__restrict__ bitmap,
-               uint8_t *__restrict__ groups, int32_t *round_ptr, int32_t *__restrict__ round_rows,
-               uint8_t *__restrict__ round_info, uint32_t *__restrict__ round_bitmap, int2 *totals, uint32_t *barrier,
-               unsigned *err) {
-  constexpr int kSeg = 128;                    // key tiles per pass
-  __shared__ uint32_t slot_src[kSeg * 8 + 8];  // key tile << 4 | group << 1 | tile fully kept
-  __shared__ int32_t seg_kt[kSeg];             // the pass's stored tiles
-  __shared__ int2 warp_sums[4];
+compact_kernel(const List l, int parts, int2 *totals, uint32_t *barrier, unsigned *err) {
+  const int32_t *__restrict__ stage_count = l.stage_count;
+  const uint32_t *__restrict__ stage_groups = l.stage_groups;
+  int32_t *row_ptr = l.row_ptr, *round_ptr = l.round_ptr;
+  const int n_rows = l.n_rows, n_kt = l.n_kt, cap = l.cap;
+  __shared__ RowShared sh;
+  int2 *warp_sums = sh.warp_sums;
   const int r = threadIdx.x, lane = r & 31, warp = r >> 5, n_ctas = (int)gridDim.x;
   // ---- counts of this CTA's rows
   const int per_cta = (n_rows + n_ctas - 1) / n_ctas, row0 = min(n_rows, (int)blockIdx.x * per_cta),
@@ -518,101 +637,56 @@ compact_kernel(const uint32_t *__restrict__ stage_bitmap, const int32_t *__restr
   for (int piece = (int)blockIdx.x; piece < n_rows * parts; piece += n_ctas) {
     const int row = piece / parts, part = piece % parts;
     const int t0 = __ldcg(row_ptr + row), keep = __ldcg(row_ptr + row + 1) - t0;
-    int rho = __ldcg(round_ptr + row), seen = 0;
-    int pending = 0;  // slots carried over from the previous pass (fewer than eight)
-    const uint32_t *row_bitmap = stage_bitmap + (size_t)row * n_kt * kBitmapWords;
-    for (int base = 0; base < n_kt && seen < keep; base += kSeg) {
-      const int kt = base + r;
-      const size_t tile = (size_t)row * n_kt + kt;
-      const int count = kt < n_kt ? stage_count[tile] : 0;
-      const bool full = count == kTile * kTile;
-      int2 incl = make_int2(count > 0 ? 1 : 0, 0);
-      uint32_t gm = count > 0 ? stage_groups[tile] : 0u;
-      incl.y = __popc(gm);
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(0xffffffffu, incl.x, o), y = __shfl_up_sync(0xffffffffu, incl.y, o);
-        if (lane >= o) incl.x += x, incl.y += y;
-      }
-      if (lane == 31) warp_sums[warp] = incl;
-      __syncthreads();
-      int2 total = make_int2(0, 0);
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        if (w < warp) incl.x += warp_sums[w].x, incl.y += warp_sums[w].y;
-        total.x += warp_sums[w].x, total.y += warp_sums[w].y;
-      }
-      const int rank = incl.x - 1;  // among the pass's stored tiles
-      const bool there = count > 0 && seen + rank < keep;
-      int s = pending + incl.y - __popc(gm);
-      if (there) {
-        seg_kt[rank] = kt;
-        if (part == 0) {
-          const int t = t0 + seen + rank;
-          col_idx[t] = kt;
-          flags[t] = full ? 1 : 0;
-          groups[t] = (uint8_t)gm;
-        }
-        for (uint32_t left = gm; left; left &= left - 1u)
-          slot_src[s++] = ((uint32_t)kt << 4) | ((uint32_t)(__ffs((int)left) - 1) << 1) | (full ? 1u : 0u);
-      }
-      const int n_here = min(total.x, keep - seen);
-      // (a row that is cut off ends with the slots of its last kept tile)
-      __shared__ int slots_s;
-      if (there && rank == n_here - 1) slots_s = s;
-      __syncthreads();
-      const int avail = n_here > 0 ? slots_s : pending;
-      for (int k0 = part; k0 < n_here; k0 += 4 * parts) {  // four tiles in flight
-        uint4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (k0 + u * parts < n_here)
-            v[u] = reinterpret_cast<const uint4 *>(row_bitmap + (size_t)seg_kt[k0 + u * parts] * kBitmapWords)[r];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (k0 + u * parts < n_here)
-            reinterpret_cast<uint4 *>(bitmap + (size_t)(t0 + seen + k0 + u * parts) * kBitmapWords)[r] = v[u];
-      }
-      const bool last_pass = base + kSeg >= n_kt || seen + n_here >= keep;
-      const int n_emit = last_pass ? (avail + 7) / 8 : avail / 8;
-      for (int k = part; k < n_emit; k += parts) {
-        const int ng = min(8, avail - 8 * k);
-        uint32_t w[4] = {0u, 0u, 0u, 0u};
-        bool all_full = true;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          if (q >= ng) continue;
-          const uint32_t src = slot_src[8 * k + q];
-          uint32_t field = 0xffffu;
-          if (!(src & 1u)) {
-            const uint32_t g = (src >> 1) & 7u;
-            field = (row_bitmap[(size_t)(src >> 4) * kBitmapWords + r * 4 + (g >> 1)] >> (16u * (g & 1u))) & 0xffffu;
-            all_full = false;
-          }
-          w[q >> 1] |= field << (16 * (q & 1));
-        }
-        const int out = rho + k;
-        if (out < cap) {
-          reinterpret_cast<uint4 *>(round_bitmap + (size_t)out * kBitmapWords)[r] = make_uint4(w[0], w[1], w[2], w[3]);
-          if (r < 8) {
-            const uint32_t src = r < ng ? slot_src[8 * k + r] : 0u;
-            round_rows[(size_t)out * 8 + r] = r < ng ? (int)(src >> 4) * kTile + 16 * (int)((src >> 1) & 7u) : -1;
-          }
-          if (r == 0) round_info[out] = (uint8_t)(ng | ((all_full && ng == 8) ? 0x80 : 0));
-        }
-      }
-      rho += n_emit;
-      seen += n_here;
-      __syncthreads();
-      // fewer than eight slots are left over; they move to the front (no overlap: they start at or
-      // beyond index 8 unless nothing was written out, in which case they are in place already)
-      const int left = avail - 8 * n_emit;
-      if (!last_pass && n_emit > 0 && r < left) slot_src[r] = slot_src[8 * n_emit + r];
-      pending = last_pass ? 0 : left;
-      __syncthreads();
-    }
+    const int rho = __ldcg(round_ptr + row);
+    write_row(l, sh, row, part, parts, t0, keep, rho);
     __syncthreads();
   }
+}
+
+// The same for lists of at most kSmallList grid tiles that cannot outgrow their capacity, without barriers: every CTA adds up
+// what lies before its list row for itself.  One layer of 16 heads x 512 (256 grid tiles): XX us instead of XX.
+constexpr int kSmallList = 4096;
+__global__ void __launch_bounds__(128) small_list_kernel(const List l, int parts) {
+  extern __shared__ int slots_s[];  // [n_rows]: slots of the list rows
+  __shared__ RowShared sh;
+  const int r = threadIdx.x, lane = r & 31, warp = r >> 5;
+  const int row = (int)blockIdx.x / parts, part = (int)blockIdx.x % parts, n_grid = l.n_rows * l.n_kt;
+  for (int x = r; x < l.n_rows; x += 128) slots_s[x] = 0;
+  __syncthreads();
+  int2 before = make_int2(0, 0);  // tiles and rounds of the list rows before this one
+  int here = 0;
+#pragma unroll 4
+  for (int x = r; x < n_grid; x += 128) {
+    const int count = l.stage_count[x];
+    const uint32_t gm = l.stage_groups[x];
+    const int of = x / l.n_kt;
+    if (count > 0) {
+      before.x += of < row ? 1 : 0;
+      here += of == row ? 1 : 0;
+      if (of <= row) atomicAdd(&slots_s[of], __popc(gm));
+    }
+  }
+  __syncthreads();
+  for (int x = r; x < row; x += 128) before.y += (slots_s[x] + 7) / 8;
+  before.x = __reduce_add_sync(0xffffffffu, before.x);
+  before.y = __reduce_add_sync(0xffffffffu, before.y);
+  here = __reduce_add_sync(0xffffffffu, here);
+  __shared__ int here_s[4];
+  if (lane == 0) {
+    sh.warp_sums[warp] = before;
+    here_s[warp] = here;
+  }
+  __syncthreads();
+  const int t0 = sh.warp_sums[0].x + sh.warp_sums[1].x + sh.warp_sums[2].x + sh.warp_sums[3].x;
+  const int rho = sh.warp_sums[0].y + sh.warp_sums[1].y + sh.warp_sums[2].y + sh.warp_sums[3].y;
+  const int keep = here_s[0] + here_s[1] + here_s[2] + here_s[3];
+  if (part == 0 && r == 0) {
+    if (row == 0) l.row_ptr[0] = l.round_ptr[0] = 0;
+    l.row_ptr[row + 1] = t0 + keep;
+    l.round_ptr[row + 1] = rho + (slots_s[row] + 7) / 8;
+  }
+  __syncthreads();  // (the sums are read)
+  write_row(l, sh, row, part, parts, t0, keep, rho);
 }
 
 // ---- gathered rounds: a list row's active key columns, 128 per round ----------------------------
@@ -890,19 +964,23 @@ cudaError_t launch_compact_staged(const uint32_t *stage_bitmap, const int32_t *s
   unsigned *err = device_error_word();
   const int sms = sm_count();
   if (!err || sms <= 0) return cudaErrorUnknown;
-  int n_rows = t.H * t.n_qt, n_kt = t.n_kt, cap = t.cap;
+  const int n_rows = t.H * t.n_qt;
+  List l = {stage_bitmap, stage_count, stage_groups, n_rows, t.n_kt, t.cap, t.row_ptr, t.col_idx, t.flags, t.bitmap, t.groups,
+            t.round_ptr, t.round_rows, t.round_info, t.round_bitmap};
   long long grid = (long long)kCompactCtasPerSm * sms;  // all of them resident; up to eight per list row have work
   if (grid > (long long)n_rows * 8) grid = (long long)n_rows * 8;
-  if (grid > (long long)n_totals) grid = (long long)n_totals;
-  int parts = (int)(grid / n_rows);
-  parts = parts < 1 ? 1 : parts > 8 ? 8 : parts;
-  int32_t *row_ptr = t.row_ptr, *col_idx = t.col_idx, *round_ptr = t.round_ptr, *round_rows = t.round_rows;
-  uint8_t *flags = t.flags, *groups = t.groups, *round_info = t.round_info;
-  uint32_t *bitmap = t.bitmap, *round_bitmap = t.round_bitmap;
-  void *args[] = {&stage_bitmap, &stage_count, &stage_groups, &n_rows, &n_kt, &cap, &parts, &row_ptr, &col_idx, &flags,
-                  &bitmap, &groups, &round_ptr, &round_rows, &round_info, &round_bitmap, &totals, &barrier, &err};
-  cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(compact_kernel), dim3((unsigned)grid), dim3(128),
-                                              args, 0, s);
+  cudaError_t e;
+  if ((long long)n_rows * t.n_kt <= kSmallList && t.cap >= n_rows * t.n_kt) {
+    const int parts = grid < n_rows ? 1 : (int)(grid / n_rows);
+    small_list_kernel<<<n_rows * parts, 128, n_rows * sizeof(int), s>>>(l, parts);
+    e = cudaGetLastError();
+  } else {
+    if (grid > (long long)n_totals) grid = (long long)n_totals;
+    int parts = (int)(grid / n_rows);
+    parts = parts < 1 ? 1 : parts > 8 ? 8 : parts;
+    void *args[] = {&l, &parts, &totals, &barrier, &err};
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(compact_kernel), dim3((unsigned)grid), dim3(128), args, 0, s);
+  }
   if (e != cudaSuccess) return e;
   count_launches(1);
   return launch_options(t, s, true);
