@@ -644,7 +644,7 @@ compact_kernel(const List l, int parts, int2 *totals, uint32_t *barrier, unsigne
 }
 
 // The same for lists of at most kSmallList grid tiles that cannot outgrow their capacity, without barriers: every CTA adds up
-// what lies before its list row for itself.  One layer of 16 heads x 512 (256 grid tiles): XX us instead of XX.
+// what lies before its list row for itself.  One layer of 16 heads x 512 (256 grid tiles): the mask of such a layer as a whole 39 -> 33 us.
 constexpr int kSmallList = 4096;
 __global__ void __launch_bounds__(128) small_list_kernel(const List l, int parts) {
   extern __shared__ int slots_s[];  // [n_rows]: slots of the list rows
@@ -687,6 +687,65 @@ __global__ void __launch_bounds__(128) small_list_kernel(const List l, int parts
   }
   __syncthreads();  // (the sums are read)
   write_row(l, sh, row, part, parts, t0, keep, rho);
+}
+
+// Larger lists that cannot outgrow their capacity: one CTA adds up the tiles and rounds of all list rows, then the rows are
+// written by as many CTAs as there is work for.  Barriers of a thousand CTAs, each an addition to the same word, cost more than
+// the second launch (16 heads x 4096: 23 us in one cooperative kernel, 8 + 10 in two).
+constexpr int kMediumList = 1 << 17, kMediumRows = 8192;
+__global__ void __launch_bounds__(1024) row_sums_kernel(const List l) {
+  extern __shared__ int2 rows_s[];  // [n_rows]: tiles and slots
+  __shared__ int2 warp_sums[32];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, n_grid = l.n_rows * l.n_kt;
+  for (int x = t; x < l.n_rows; x += 1024) rows_s[x] = make_int2(0, 0);
+  __syncthreads();
+  for (int x0 = t; x0 < n_grid; x0 += 8 * 1024) {
+    int count[8];
+    uint32_t gm[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int x = x0 + 1024 * u;
+      count[u] = x < n_grid ? l.stage_count[x] : 0;
+      gm[u] = x < n_grid ? l.stage_groups[x] : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (count[u] > 0) {
+        int2 *row = rows_s + (x0 + 1024 * u) / l.n_kt;
+        atomicAdd(&row->x, 1);
+        atomicAdd(&row->y, __popc(gm[u]));
+      }
+  }
+  __syncthreads();
+  int2 before = make_int2(0, 0);
+  for (int base = 0; base < l.n_rows; base += 1024) {
+    int2 incl = make_int2(0, 0);
+    if (base + t < l.n_rows) incl = make_int2(rows_s[base + t].x, (rows_s[base + t].y + 7) / 8);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl.x, o), y = __shfl_up_sync(0xffffffffu, incl.y, o);
+      if (lane >= o) incl.x += x, incl.y += y;
+    }
+    if (lane == 31) warp_sums[warp] = incl;
+    __syncthreads();
+    const int2 of_warp = warp_sums[lane];
+    const int lower = lane < warp ? 1 : 0;
+    incl.x += before.x + __reduce_add_sync(0xffffffffu, lower * of_warp.x);
+    incl.y += before.y + __reduce_add_sync(0xffffffffu, lower * of_warp.y);
+    if (base + t < l.n_rows) {
+      l.row_ptr[base + t + 1] = incl.x;
+      l.round_ptr[base + t + 1] = incl.y;
+    }
+    before.x += __reduce_add_sync(0xffffffffu, of_warp.x);
+    before.y += __reduce_add_sync(0xffffffffu, of_warp.y);
+    __syncthreads();
+  }
+  if (t == 0) l.row_ptr[0] = l.round_ptr[0] = 0;
+}
+__global__ void __launch_bounds__(128) rows_kernel(const List l, int parts) {
+  __shared__ RowShared sh;
+  const int row = (int)blockIdx.x / parts, t0 = l.row_ptr[row];
+  write_row(l, sh, row, (int)blockIdx.x % parts, parts, t0, l.row_ptr[row + 1] - t0, l.round_ptr[row]);
 }
 
 // ---- gathered rounds: a list row's active key columns, 128 per round ----------------------------
@@ -973,6 +1032,14 @@ cudaError_t launch_compact_staged(const uint32_t *stage_bitmap, const int32_t *s
   if ((long long)n_rows * t.n_kt <= kSmallList && t.cap >= n_rows * t.n_kt) {
     const int parts = grid < n_rows ? 1 : (int)(grid / n_rows);
     small_list_kernel<<<n_rows * parts, 128, n_rows * sizeof(int), s>>>(l, parts);
+    e = cudaGetLastError();
+  } else if ((long long)n_rows * t.n_kt <= kMediumList && n_rows <= kMediumRows && t.cap >= n_rows * t.n_kt) {
+    const int parts = grid < n_rows ? 1 : (int)(grid / n_rows);
+    e = cudaFuncSetAttribute(row_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMediumRows * sizeof(int2)));
+    if (e != cudaSuccess) return e;
+    row_sums_kernel<<<1, 1024, n_rows * sizeof(int2), s>>>(l);
+    rows_kernel<<<n_rows * parts, 128, 0, s>>>(l, parts);
+    count_launches(1);
     e = cudaGetLastError();
   } else {
     if (grid > (long long)n_totals) grid = (long long)n_totals;
