@@ -89,6 +89,7 @@ struct Barriers {
   uint64_t s_full[2], s_empty[2];
   uint64_t in_full[4], in_empty[4];
   uint64_t sweep1_done;  // all softmax warps have stored their sweep-1 statistics
+  uint64_t stats_read;   // ... and have read them
   uint64_t bias_full, bias_empty;
   uint32_t tmem_base;
   int abort_flag;
@@ -203,6 +204,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       mbar_init(&bars->in_empty[s], 1);
     }
     mbar_init(&bars->sweep1_done, kSoftmaxWarps);
+    mbar_init(&bars->stats_read, kSoftmaxWarps);
     mbar_init(&bars->bias_full, 1);
     mbar_init(&bars->bias_empty, kSoftmaxWarps);
     bars->abort_flag = 0;
@@ -424,6 +426,39 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       ok = wait(&bars->sweep1_done, 0);
       tc_fence_after_sync();
     }
+    if (ok) {
+      // The groups' statistics of every sample combined, once for all visits of sweep 2: minus (max + log2(sum)), first to the
+      // columns of the running sum, then, when all have read the pairs, over this group's pairs.  A row without any key
+      // in its domain (possible when Lk < Lq) gets weight 0 everywhere.
+#pragma unroll 1
+      for (int b = 0; b < Bc; ++b) {
+        uint32_t st[kGroups][2];
+#pragma unroll
+        for (int q = 0; q < kGroups; ++q) tmem_ld2(stats + kCols * q + 2 * b, st[q]);
+        tmem_wait_ld();
+        float mm = __uint_as_float(st[0][0]);
+#pragma unroll
+        for (int q = 1; q < kGroups; ++q) mm = fmaxf(mm, __uint_as_float(st[q][0]));
+        float z = 0.f;
+#pragma unroll
+        for (int q = 0; q < kGroups; ++q) z += __uint_as_float(st[q][1]) * ex2_approx(__uint_as_float(st[q][0]) - mm);
+        tmem_st1(sum_addr + b, __float_as_uint(jend > 0 ? -(mm + lg2_approx(z)) : -CUDART_INF_F));
+      }
+      tmem_wait_st();
+      tc_fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->stats_read);
+      ok = wait(&bars->stats_read, 0);
+      tc_fence_after_sync();
+#pragma unroll 1
+      for (int b = 0; b < Bc; ++b) {
+        uint32_t ref;
+        tmem_ld1(sum_addr + b, ref);
+        tmem_wait_ld();
+        tmem_st1(my_stats + b, ref);
+      }
+      tmem_wait_st();
+    }
 
     // ---- sweep 2: normalised weights, summed over b in TMEM, added to the accumulator per key tile
     for (int kt = 0; kt < n_k && ok; ++kt) {
@@ -433,22 +468,13 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       const int n_valid = max(0, min(kCols, jend - j0));
       const bool interior = __all_sync(0xffffffffu, n_valid == kCols);
       for (int b = 0; b < Bc; ++b, ++v) {
-        uint32_t xs[kCols], st[kGroups][2];
+        uint32_t xs[kCols], ref;
         take_s(v, xs);
         if (!ok) break;
-#pragma unroll
-        for (int q = 0; q < kGroups; ++q) tmem_ld2(stats + kCols * q + 2 * b, st[q]);
+        tmem_ld1(my_stats + b, ref);
         tmem_wait_ld();
         release_s(v);
-        // the groups' statistics of sample b combined: max + log2(sum).  A row without any key
-        // in its domain (possible when Lk < Lq) gets weight 0 everywhere.
-        float mm = __uint_as_float(st[0][0]);
-#pragma unroll
-        for (int q = 1; q < kGroups; ++q) mm = fmaxf(mm, __uint_as_float(st[q][0]));
-        float z = 0.f;
-#pragma unroll
-        for (int q = 0; q < kGroups; ++q) z += __uint_as_float(st[q][1]) * ex2_approx(__uint_as_float(st[q][0]) - mm);
-        const float neg_ref = jend > 0 ? -(mm + lg2_approx(z)) : -CUDART_INF_F;
+        const float neg_ref = __uint_as_float(ref);
 #pragma unroll
         for (int c = 0; c < kCols / 16; ++c) {
           float p[16];
