@@ -430,19 +430,25 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       // The groups' statistics of every sample combined, once for all visits of sweep 2: minus (max + log2(sum)), first to the
       // columns of the running sum, then, when all have read the pairs, over this group's pairs.  A row without any key
       // in its domain (possible when Lk < Lq) gets weight 0 everywhere.
+      constexpr int kAhead = 16 / kGroups;  // samples at a time
 #pragma unroll 1
-      for (int b = 0; b < Bc; ++b) {
-        uint32_t st[kGroups][2];
+      for (int b0 = 0; b0 < Bc; b0 += kAhead) {
+        uint32_t st[kAhead][kGroups][2];
 #pragma unroll
-        for (int q = 0; q < kGroups; ++q) tmem_ld2(stats + kCols * q + 2 * b, st[q]);
+        for (int u = 0; u < kAhead; ++u)
+#pragma unroll
+          for (int q = 0; q < kGroups; ++q) tmem_ld2(stats + kCols * q + 2 * (b0 + u), st[u][q]);  // (beyond the last: not used)
         tmem_wait_ld();
-        float mm = __uint_as_float(st[0][0]);
 #pragma unroll
-        for (int q = 1; q < kGroups; ++q) mm = fmaxf(mm, __uint_as_float(st[q][0]));
-        float z = 0.f;
+        for (int u = 0; u < kAhead; ++u) {
+          float mm = __uint_as_float(st[u][0][0]);
 #pragma unroll
-        for (int q = 0; q < kGroups; ++q) z += __uint_as_float(st[q][1]) * ex2_approx(__uint_as_float(st[q][0]) - mm);
-        tmem_st1(sum_addr + b, __float_as_uint(jend > 0 ? -(mm + lg2_approx(z)) : -CUDART_INF_F));
+          for (int q = 1; q < kGroups; ++q) mm = fmaxf(mm, __uint_as_float(st[u][q][0]));
+          float z = 0.f;
+#pragma unroll
+          for (int q = 0; q < kGroups; ++q) z += __uint_as_float(st[u][q][1]) * ex2_approx(__uint_as_float(st[u][q][0]) - mm);
+          tmem_st1(sum_addr + b0 + u, __float_as_uint(jend > 0 ? -(mm + lg2_approx(z)) : -CUDART_INF_F));
+        }
       }
       tmem_wait_st();
       tc_fence_before_sync();
@@ -450,12 +456,12 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       if (lane == 0) mbar_arrive(&bars->stats_read);
       ok = wait(&bars->stats_read, 0);
       tc_fence_after_sync();
-#pragma unroll 1
-      for (int b = 0; b < Bc; ++b) {
-        uint32_t ref;
-        tmem_ld1(sum_addr + b, ref);
+#pragma unroll
+      for (int b0 = 0; b0 < kMaxB; b0 += 16) {
+        uint32_t ref[16];
+        tmem_ld16(sum_addr + b0, ref);
         tmem_wait_ld();
-        tmem_st1(my_stats + b, ref);
+        tmem_st16(my_stats + b0, ref);
       }
       tmem_wait_st();
     }
