@@ -133,10 +133,10 @@ __device__ __forceinline__ bool last_follows(const Barriers *bars, int s) {
   return s >= kMaxNewton || *reinterpret_cast<const volatile int *>(&bars->more[s]) == 0;
 }
 
-// v when sel < 0, -inf otherwise (one select instruction on the sign of an integer).
-__device__ __forceinline__ float keep_if_negative(float v, int sel) {
+// v when sel < 0, `other` otherwise (one select instruction on the sign of an integer).
+__device__ __forceinline__ float keep_if_negative(float v, int sel, float other) {
   float d;
-  asm("slct.f32.s32 %0, %1, %2, %3;" : "=f"(d) : "f"(-CUDART_INF_F), "f"(v), "r"(sel));
+  asm("slct.f32.s32 %0, %1, %2, %3;" : "=f"(d) : "f"(other), "f"(v), "r"(sel));
   return d;
 }
 
@@ -150,13 +150,15 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     return *reinterpret_cast<const uint32_t *>(&h);
   }
 }
+// (s0, s1) += the two 16-bit values of v.
 template <bool kF16>
-__device__ __forceinline__ float2 unpack2(uint32_t v) {
-  if constexpr (kF16) {
-    return __half22float2(*reinterpret_cast<const __half2 *>(&v));
-  } else {
-    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v));
-  }
+__device__ __forceinline__ void add_pair(float &s0, float &s1, uint32_t v) {
+  if constexpr (kF16)
+    asm("{\n .reg .b16 lo, hi;\n mov.b32 {lo, hi}, %2;\n add.f32.f16 %0, lo, %0;\n add.f32.f16 %1, hi, %1;\n}"
+        : "+f"(s0), "+f"(s1) : "r"(v));
+  else
+    asm("{\n .reg .b16 lo, hi;\n mov.b32 {lo, hi}, %2;\n add.f32.bf16 %0, lo, %0;\n add.f32.bf16 %1, hi, %1;\n}"
+        : "+f"(s0), "+f"(s1) : "r"(v));
 }
 
 template <int D, int kCtas, bool kF16>
@@ -398,7 +400,15 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     float *my_tau = taus + wg * 128 + r;
     float cnt = 0.f;
     float *list = reinterpret_cast<float *>(smem + C::kListOffset) + 144 * wg + r;  // entry k at list[k * kListPitch]
-    int n_list = 0;
+    constexpr uint32_t kListStep = 4 * kListPitch;
+    const uint32_t list_addr = smem_u32(list), list_full = list_addr + kListCap * kListStep;
+    uint32_t list_at = list_addr;  // the next entry's place
+    // v > thr: to the list (three instructions, no branch).  Whatever reads the list depends on list_at.
+    auto append = [&](float v, float thr) {
+      asm volatile(
+          "{\n .reg .pred p;\n setp.gt.f32 p, %1, %2;\n @p st.shared.f32 [%0], %1;\n @p add.u32 %0, %0, %3;\n}"
+          : "+r"(list_at) : "f"(v), "f"(thr), "n"(kListStep) : "memory");
+    };
     bool listing = true;  // of the whole warp
     // A Newton step from a lower bound of the root of some of the row's entries, whose sums are S1 and S2: it stays below that root
     // (the sum is convex in tau), which is no higher than the row's.
@@ -407,6 +417,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     };
     // This thread's list without the entries that cannot lie above tau: one such step on the list from `thr`.
     auto prune = [&](float thr) {
+      const int n_list = (int)((list_at - list_addr) / kListStep);
       float S1 = 0.f, S2 = 0.f;
 #pragma unroll 4
       for (int k = 0; k < n_list; ++k) {
@@ -423,11 +434,11 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
           ++kept;
         }
       }
-      n_list = kept;
-      if (__any_sync(0xffffffffu, n_list > kListCap)) {  // no list of the CTA is used then
+      list_at = list_addr + kListStep * (uint32_t)kept;
+      if (__any_sync(0xffffffffu, kept > kListCap)) {  // no list of the CTA is used then
         *reinterpret_cast<volatile int *>(&bars->more[0]) = 1;
         listing = false;
-        n_list = 0;
+        list_at = list_addr;
       }
       return thr;
     };
@@ -468,6 +479,25 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
           tmem_ld32(tmem + 128 * buf + 64 * wg + 32 * c + lane_addr, x);
           tmem_wait_ld();
           const uint32_t w = c == 0 ? bits.x : bits.y;
+          if (kind == 2) {
+            // P in the tensors' type over the first 16 columns of this chunk of S.  max(x - tau, 0) as a saturating
+            // multiply-add (see below); a pruned entry's is 0 by the sign of its bit
+            uint32_t pk[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              float u0 = __saturatef(fmaf(__uint_as_float(x[2 * e]), half_scale, neg_tau));
+              float u1 = __saturatef(fmaf(__uint_as_float(x[2 * e + 1]), half_scale, neg_tau));
+              if (!full) {
+                u0 = keep_if_negative(u0, (int)(w << (31 - 2 * e)), 0.f);
+                u1 = keep_if_negative(u1, (int)(w << (30 - 2 * e)), 0.f);
+              }
+              fmul2(u0, u1, u0, u1, u0, u1);
+              pk[e] = pack2<kF16>(u0, u1);
+              add_pair<kF16>(psum0, psum1, pk[e]);  // the weights the product will use
+            }
+            tmem_st16(tmem + 128 * buf + 64 * wg + 32 * c + lane_addr, pk);
+            continue;
+          }
           float t[32];  // x_j = scale * q.k_j / 2, -inf for pruned entries
 #pragma unroll
           for (int e = 0; e < 32; e += 2)
@@ -475,7 +505,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
           if (!full) {
             // bit e of w moved to the sign position selects between the score and -inf
 #pragma unroll
-            for (int e = 0; e < 32; ++e) t[e] = keep_if_negative(t[e], (int)(w << (31 - e)));
+            for (int e = 0; e < 32; ++e) t[e] = keep_if_negative(t[e], (int)(w << (31 - e)), -CUDART_INF_F);
           }
           if (kind == 0) {
             float m0 = st.x, m1 = -CUDART_INF_F, m2 = -CUDART_INF_F, m3 = -CUDART_INF_F;
@@ -489,7 +519,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
             st.x = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
             if (!listing) continue;
             list_thr = fmaxf(list_thr, st.x - 1.f);
-            if (__any_sync(0xffffffffu, n_list + (full ? 32 : __popc(w)) > kListCap)) {
+            if (__any_sync(0xffffffffu, list_at + kListStep * (full ? 32u : (uint32_t)__popc(w)) > list_full)) {
               // a list could fill up: two steps on the chunk itself first, in registers, or most of it would go through the lists
               // (unless one of the CTA's has overflowed: then the others are not needed either)
               listing = !__any_sync(0xffffffffu, *reinterpret_cast<volatile int *>(&bars->more[0]) != 0);
@@ -509,12 +539,8 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
 #pragma unroll
             for (int half = 0; half < 4; ++half) {
 #pragma unroll
-              for (int e = 8 * half; e < 8 * half + 8; ++e)
-                if (t[e] > list_thr) {
-                  list[n_list * kListPitch] = t[e];
-                  ++n_list;
-                }
-              if (__any_sync(0xffffffffu, n_list > kListCap)) list_thr = prune(list_thr);
+              for (int e = 8 * half; e < 8 * half + 8; ++e) append(t[e], list_thr);
+              if (__any_sync(0xffffffffu, list_at > list_full)) list_thr = prune(list_thr);
               if (!listing) break;
             }
           } else if (kind == 1) {
@@ -533,18 +559,6 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
               cnt += ((u0 > 0.f ? 1.f : 0.f) + (u1 > 0.f ? 1.f : 0.f)) + ((u2 > 0.f ? 1.f : 0.f) + (u3 > 0.f ? 1.f : 0.f));
             }
             st = make_float2((a0 + a1) + (a2 + a3), (q0 + q1) + (q2 + q3));
-          } else {
-            // P in the tensors' type over the first 16 columns of this chunk of S
-            uint32_t pk[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-              const float u0 = __saturatef(t[2 * e] + neg_tau), u1 = __saturatef(t[2 * e + 1] + neg_tau);
-              pk[e] = pack2<kF16>(u0 * u0, u1 * u1);
-              const float2 pr = unpack2<kF16>(pk[e]);  // the weights the product will use
-              psum0 += pr.x;
-              psum1 += pr.y;
-            }
-            tmem_st16(tmem + 128 * buf + 64 * wg + 32 * c + lane_addr, pk);
           }
         }
         if (kind == 2) {
@@ -558,7 +572,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
       }
       if (!ok) break;
       *my_stats = st;
-      cnts[wg * 128 + r] = sw == 0 ? __int_as_float(n_list) : cnt;
+      cnts[wg * 128 + r] = sw == 0 ? __int_as_float((int)((list_at - list_addr) / kListStep)) : cnt;
       // ---- end of a sweep: the two halves of every row meet
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->sweep_done);
