@@ -403,11 +403,12 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     constexpr uint32_t kListStep = 4 * kListPitch;
     const uint32_t list_addr = smem_u32(list), list_full = list_addr + kListCap * kListStep;
     uint32_t list_at = list_addr;  // the next entry's place
-    // v > thr: to the list (three instructions, no branch).  Whatever reads the list depends on list_at.
+    // v > thr: to the list (three instructions, no branch)
     auto append = [&](float v, float thr) {
-      asm volatile(
-          "{\n .reg .pred p;\n setp.gt.f32 p, %1, %2;\n @p st.shared.f32 [%0], %1;\n @p add.u32 %0, %0, %3;\n}"
-          : "+r"(list_at) : "f"(v), "f"(thr), "n"(kListStep) : "memory");
+      if (v > thr) {
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(list_at), "f"(v) : "memory");
+        list_at += kListStep;
+      }
     };
     bool listing = true;  // of the whole warp
     // A Newton step from a lower bound of the root of some of the row's entries, whose sums are S1 and S2: it stays below that root
