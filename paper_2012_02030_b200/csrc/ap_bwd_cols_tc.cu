@@ -108,7 +108,7 @@ template <int D, bool kF16>
 __global__ void __launch_bounds__(kThreads, 1)
 cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, uint16_t *__restrict__ dV,
             const float *__restrict__ neg_l, const float *__restrict__ stat_d,
-            const uint32_t *__restrict__ table, const uint32_t *__restrict__ bitmap, int BH, int H, int Lq, int Lk,
+            const uint32_t *__restrict__ table, const uint32_t *__restrict__ bitmap, int last_tile, int BH, int H, int Lq, int Lk,
             int n_qt, int n_kt, float scale, unsigned *err, uint32_t max_polls, int dbg_skip) {
   using C = Cfg<D>;
   using L = TileLayout<D, false>;
@@ -338,7 +338,8 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
         uint32_t pos[8];  // the groups' tiles in the list
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          pos[q] = __shfl_sync(0xffffffffu, it.word[q], src) & 0xffffffu;
+          // (never beyond the list, whatever a rows kernel that gave up has left in the table)
+          pos[q] = min(__shfl_sync(0xffffffffu, it.word[q], src) & 0xffffffu, (uint32_t)last_tile);
           if (it.plain) break;
         }
         last = !more();
@@ -728,7 +729,7 @@ cudaError_t launch(const ColsMaps &maps, const Args &a) {
   const int n_items = a.B * a.H * a.t->n_kt, grid = knobs.skip_arrive && n_items > sms ? sms : n_items;
   kern<<<grid, kThreads, C::kSmemBytes, a.s>>>(
       maps, static_cast<uint16_t *>(a.dK), static_cast<uint16_t *>(a.dV), a.plan.neg_l, a.plan.dsum, a.plan.table,
-      a.t->bitmap, a.B * a.H, a.H, a.Lq, a.Lk, a.t->n_qt, a.t->n_kt, a.scale, a.err, knobs.max_polls,
+      a.t->bitmap, a.t->cap > 0 ? a.t->cap - 1 : 0, a.B * a.H, a.H, a.Lq, a.Lk, a.t->n_qt, a.t->n_kt, a.scale, a.err, knobs.max_polls,
       knobs.skip_arrive);
   count_launches(1);
   return cudaGetLastError();

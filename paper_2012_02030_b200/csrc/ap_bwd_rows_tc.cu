@@ -1,4 +1,4 @@
-// Backward of the masked attention, rows kernel: dQ and the row statistics.
+// Backward of the masked attention, rows kernel: dQ, the row statistics and the columns kernel's (query tile, key tile) table.
 //
 // Persistent, one CTA per SM; a work item is one (b, h, query tile) and a block of the grid, taken over by a running
 // CTA (late query tiles of a head first, heads in order, so that concurrent CTAs share a few heads' K and V in L2).
@@ -13,7 +13,8 @@
 // rounds twice (kF16): S alone for r = log2 of the row's sum, then the above with that fixed reference.
 //
 // Warp roles (704 threads): warps 0-15 compute, 16 producer, 17 issues every MMA, 18-21 form D_i = dO_i . O_i of the
-// NEXT item straight from global memory and write the last item's dQ, -log2 sum and D.  Sixteen compute warps, because
+// NEXT item straight from global memory and write the last item's dQ, -log2 sum and D, and the item's row of the table (as a
+// launch of its own in front the table took 4 of 117 us at 64 x 8 heads, 250 queries, 231 keys, forward and backward).  Sixteen compute warps, because
 // what a round costs a warp is mostly latency (barriers, tensor-memory loads), which four warps per scheduler hide
 // better than two.  TMEM (512 columns): S[2], dP, dQ.  The issuer runs one round ahead: S(g+1) and dP(g+1) are under way
 // while the threads work on round g.  Slots: V of a round is free after its dP, K only after its dQ, so the K that
@@ -86,13 +87,30 @@ struct Cfg {
   static_assert(kSmemBytes > 114 * 1024, "one CTA per SM: all of TMEM is taken");
 };
 
+// What a list row holds, for the table of the columns kernel.
+struct ListRows {
+  const int32_t *row_ptr, *col_idx;
+  const uint8_t *flags, *groups;
+  uint32_t *table;  // see Plan
+  int n_kt;
+};
+// By one warp: list row lr of the table.
+__device__ __forceinline__ void write_table(const ListRows &l, int lr, int lane) {
+  uint32_t *row = l.table + (size_t)lr * l.n_kt;
+  for (int kt = lane; kt < l.n_kt; kt += 32) row[kt] = 0u;
+  __syncwarp();
+  const int t1 = l.row_ptr[lr + 1];
+  for (int t = l.row_ptr[lr] + lane; t < t1; t += 32)
+    row[l.col_idx[t]] = (uint32_t)t | (((l.flags[t] & 1u) ? 0xffu : (uint32_t)l.groups[t]) << 24);
+}
+
 template <int D, bool kSplit, bool kF16>
 __global__ void __launch_bounds__(kThreads, 1)
 rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ O, const uint16_t *__restrict__ dO,
             uint16_t *__restrict__ dQ, float *__restrict__ neg_l, float *__restrict__ stat_d,
             const int32_t *__restrict__ round_ptr, const int32_t *__restrict__ round_rows,
-            const uint8_t *__restrict__ round_info, const uint32_t *__restrict__ round_bitmap, int n_items, int H,
-            int Lq, int n_qt, float scale, unsigned *err, uint32_t max_polls, int dbg_skip) {
+            const uint8_t *__restrict__ round_info, const uint32_t *__restrict__ round_bitmap, const ListRows list, int n_items,
+            int H, int Lq, int n_qt, float scale, unsigned *err, uint32_t max_polls, int dbg_skip) {
   using C = Cfg<D, kSplit>;
   using L = TileLayout<D, kSplit>;
   constexpr uint32_t kRing = C::kRing, kQBufs = C::kQBufs;
@@ -233,6 +251,7 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
         const int rows = min(kTile, Lq - it.qt * kTile);
         uint4 *dst = reinterpret_cast<uint4 *>(dQ + ((size_t)it.bh * Lq + (size_t)it.qt * kTile) * D);
         for (int x = lane; x < rows * (D / 8); x += 32) dst[x] = make_uint4(0u, 0u, 0u, 0u);
+        if (it.bh < H) write_table(list, it.bh * n_qt + it.qt, lane);
         cur = hear();
         continue;
       }
@@ -641,6 +660,7 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
       if (wr + lane < rows) stat_d[(size_t)bh * Lq + qt * kTile + wr + lane] = sh->dsum[n & 1u][wr + lane];
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh->d_ready[n & 1u]);
+      if (wr == 0 && bh < H) write_table(list, bh * n_qt + qt, lane);  // (every list row is an item of the first batch element)
       return true;
     };
     bool there = form_d(0);
@@ -706,7 +726,7 @@ cudaError_t launch(const RowsMaps &maps, const Args &a) {
   kern<<<grid, kThreads, C::kSmemBytes, a.s>>>(
       maps, static_cast<const uint16_t *>(a.O), static_cast<const uint16_t *>(a.dO), static_cast<uint16_t *>(a.dQ),
       a.plan.neg_l, a.plan.dsum, a.t->round_ptr, a.t->round_rows, a.t->round_info, a.t->round_bitmap,
-      n_items, a.H, a.Lq, a.t->n_qt, a.scale, a.err, knobs.max_polls, knobs.skip_arrive);
+      ListRows{a.t->row_ptr, a.t->col_idx, a.t->flags, a.t->groups, a.plan.table, a.t->n_kt}, n_items, a.H, a.Lq, a.t->n_qt, a.scale, a.err, knobs.max_polls, knobs.skip_arrive);
   count_launches(1);
   return cudaGetLastError();
 }

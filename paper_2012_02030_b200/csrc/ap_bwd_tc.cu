@@ -4,29 +4,14 @@
 // With S = scale Q K^T, P = softmax of S over the kept entries of a row, O = P V and an incoming dO:
 //   dV = P^T dO,   dP = dO V^T,   dS = P o (dP - D),  D_i = dO_i . O_i,
 //   dQ = scale dS K,   dK = scale dS^T Q.
-// Three kernels: the (query tile, key tile) table (here), the rows kernel (dQ and the row statistics
-// L = log2 sum 2^(c S), c = scale log2 e, and D; ap_bwd_rows_tc.cu) and the columns kernel (dK, dV;
-// ap_bwd_cols_tc.cu).
+// Two kernels: the rows kernel (dQ, the row statistics L = log2 sum 2^(c S), c = scale log2 e, and D, and the (query tile,
+// key tile) table; ap_bwd_rows_tc.cu) and the columns kernel (dK, dV; ap_bwd_cols_tc.cu).
 #include "ap_bwd_tc.cuh"
 
 namespace ap {
 namespace bwd {
 
 namespace {
-
-// One CTA per list row (h, query tile).
-__global__ void __launch_bounds__(128) table_kernel(const int32_t *__restrict__ row_ptr,
-                                                    const int32_t *__restrict__ col_idx,
-                                                    const uint8_t *__restrict__ flags,
-                                                    const uint8_t *__restrict__ groups, int n_kt,
-                                                    uint32_t *__restrict__ table) {
-  uint32_t *row = table + (size_t)blockIdx.x * n_kt;
-  for (int kt = threadIdx.x; kt < n_kt; kt += blockDim.x) row[kt] = 0u;
-  __syncthreads();
-  const int t1 = row_ptr[blockIdx.x + 1];
-  for (int t = row_ptr[blockIdx.x] + (int)threadIdx.x; t < t1; t += blockDim.x)
-    row[col_idx[t]] = (uint32_t)t | (((flags[t] & 1u) ? 0xffu : (uint32_t)groups[t]) << 24);
-}
 
 size_t stats_bytes(int B, int H, int Lq) { return (2 * sizeof(float) * (size_t)B * H * Lq + 255) / 256 * 256; }
 
@@ -71,10 +56,7 @@ cudaError_t launch_bwd_tc(const void *Q, const void *K, const void *V, const voi
   a.scale = scale;
   a.err = err;
   a.s = s;
-  bwd::table_kernel<<<H * t.n_qt, 128, 0, s>>>(t.row_ptr, t.col_idx, t.flags, t.groups, t.n_kt, a.plan.table);
-  count_launches(1);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = bwd::launch_rows(rows, a);
+  cudaError_t e = bwd::launch_rows(rows, a);
   if (e == cudaSuccess) e = bwd::launch_cols(cols, a);
   return e;
 }
