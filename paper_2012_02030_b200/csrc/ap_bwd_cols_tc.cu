@@ -150,6 +150,7 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
     tmem_alloc(&sh->tmem_base, kTmemCols);
     tmem_relinquish();
   }
+  after_previous();
   const bool ordered = n_qt >= kMinOrderedTiles && H * n_kt <= kMaxHeavy && (int64_t)H * n_qt * n_kt <= kMaxTable;
   if (ordered) {
     for (int x = threadIdx.x; x < H * n_kt; x += kThreads) {
@@ -727,12 +728,12 @@ cudaError_t launch(const ColsMaps &maps, const Args &a) {
   const DebugKnobs knobs = debug_knobs();
   // (the test hook runs on the first wave only: none of its CTAs takes over another's item)
   const int n_items = a.B * a.H * a.t->n_kt, grid = knobs.skip_arrive && n_items > sms ? sms : n_items;
-  kern<<<grid, kThreads, C::kSmemBytes, a.s>>>(
-      maps, static_cast<uint16_t *>(a.dK), static_cast<uint16_t *>(a.dV), a.plan.neg_l, a.plan.dsum, a.plan.table,
+  e = launch_early(
+      kern, (unsigned)grid, kThreads, C::kSmemBytes, a.s, maps, static_cast<uint16_t *>(a.dK), static_cast<uint16_t *>(a.dV), a.plan.neg_l, a.plan.dsum, a.plan.table,
       a.t->bitmap, a.t->cap > 0 ? a.t->cap - 1 : 0, a.B * a.H, a.H, a.Lq, a.Lk, a.t->n_qt, a.t->n_kt, a.scale, a.err, knobs.max_polls,
       knobs.skip_arrive);
   count_launches(1);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace

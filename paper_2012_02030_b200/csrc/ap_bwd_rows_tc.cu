@@ -156,6 +156,7 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
     tmem_alloc(&sh->tmem_base, kTmemCols);
     tmem_relinquish();
   }
+  after_previous();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -723,12 +724,12 @@ cudaError_t launch(const RowsMaps &maps, const Args &a) {
   const DebugKnobs knobs = debug_knobs();
   // (the test hook runs on the first wave only: none of its CTAs takes over another's item)
   const int n_items = a.B * a.H * a.t->n_qt, grid = knobs.skip_arrive && n_items > sms ? sms : n_items;
-  kern<<<grid, kThreads, C::kSmemBytes, a.s>>>(
-      maps, static_cast<const uint16_t *>(a.O), static_cast<const uint16_t *>(a.dO), static_cast<uint16_t *>(a.dQ),
+  e = launch_early(
+      kern, (unsigned)grid, kThreads, C::kSmemBytes, a.s, maps, static_cast<const uint16_t *>(a.O), static_cast<const uint16_t *>(a.dO), static_cast<uint16_t *>(a.dQ),
       a.plan.neg_l, a.plan.dsum, a.t->round_ptr, a.t->round_rows, a.t->round_info, a.t->round_bitmap,
       ListRows{a.t->row_ptr, a.t->col_idx, a.t->flags, a.t->groups, a.plan.table, a.t->n_kt}, n_items, a.H, a.Lq, a.t->n_qt, a.scale, a.err, knobs.max_polls, knobs.skip_arrive);
   count_launches(1);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace

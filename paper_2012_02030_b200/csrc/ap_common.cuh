@@ -77,6 +77,29 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
 // SMs of the current device (0 if it cannot be queried).
 int sm_count();
 
+// Launches a kernel that begins with after_previous(): its blocks may take the SMs that the kernel before it in the stream has
+// left, set themselves up there and wait.
+template <class... Params, class... Args>
+cudaError_t launch_early(void (*kern)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, Args &&...args) {
+  cudaLaunchAttribute early;
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<Args &&>(args)...);
+}
+// By every thread, before it touches global memory: waits until the kernel before in the stream is over and its writes are
+// visible.  After it, the same is allowed to the kernel behind.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Kernels launched by this library in this process (see ap_launch_count in ap.h).
 void count_launches(int n);
 

@@ -180,6 +180,7 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
     tmem_alloc(&sh->tmem_base, kTmemCols);
     tmem_relinquish();
   }
+  after_previous();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -876,11 +877,11 @@ cudaError_t launch_kernel(const FwdMaps &maps, const void *K, const void *V, voi
                   Lk, dbg.schedule, kPairs ? t.unit_qt : nullptr};
   if (kGath) gth.ptr = t.ground_ptr, gth.keys = t.ground_keys, gth.info = t.ground_info, gth.bitmap = t.ground_bitmap;
   // the test hook runs on one CTA only (a tiny grid is all it is meant for)
-  kern<<<dbg.skip_arrive ? 1 : (n_units < sms ? n_units : ctas), kThreads, C::kSmemBytes, s>>>(
-      maps, static_cast<uint16_t *>(O), t.round_ptr, t.round_rows, t.round_info, t.round_bitmap, gth, B, H, Lq,
-      t.n_qt, scale_log2, err, dbg.max_polls, dbg.skip_arrive);
+  e = launch_early(kern, dbg.skip_arrive ? 1 : (n_units < sms ? n_units : ctas), kThreads, C::kSmemBytes, s, maps,
+                   static_cast<uint16_t *>(O), t.round_ptr, t.round_rows, t.round_info, t.round_bitmap, gth, B, H, Lq, t.n_qt,
+                   scale_log2, err, dbg.max_polls, dbg.skip_arrive);
   count_launches(1);
-  return cudaGetLastError();
+  return e;
 }
 
 // Lists that carry a gathered schedule get the instantiation that can follow it.
