@@ -214,6 +214,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     tmem_alloc(&bars->tmem_base, kTmemCols);
     tmem_relinquish();
   }
+  after_previous();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -674,11 +675,11 @@ cudaError_t launch(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorM
     const Launch l = plan_launch(p, p.B - b0, R::kMaxB, turn != nullptr);
     unsigned *t = l.visits ? turn : nullptr;
     if (t && (e = cudaMemsetAsync(t, 0, (size_t)p.H * p.n_qt * p.n_kt * sizeof(unsigned), s)) != cudaSuccess) return e;
-    (t ? kern_chunked : kern)<<<knobs.skip_arrive ? 1 : l.grid, R::kThreads, Cfg<D>::kSmemBytes, s>>>(
-        mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, b0, l.samples, l.visits, t, p.H, Lq, Lk, p.n_qt, p.n_kt, causal,
+    e = launch_early(
+        t ? kern_chunked : kern, (unsigned)(knobs.skip_arrive ? 1 : l.grid), R::kThreads, Cfg<D>::kSmemBytes, s, mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, b0, l.samples, l.visits, t, p.H, Lq, Lk, p.n_qt, p.n_kt, causal,
         f16, scale * kLog2e, err, knobs.max_polls, knobs.skip_arrive);
     count_launches(1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
     b0 += l.samples;
   }
   return cudaSuccess;

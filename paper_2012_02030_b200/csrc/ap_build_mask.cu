@@ -830,6 +830,7 @@ __global__ void __launch_bounds__(32 * kCtaWarps, kCtaWarps == 4 ? 8 : 2) emit_k
   __shared__ uint32_t warp_groups[kCtaWarps];
   __shared__ uint2 stage_all[kClassify ? kCtaWarps : 1][kClassify ? kWarpStage : 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  after_previous();
   // rows of the scores start on 32-byte boundaries and rows of the mask on 16-byte ones
   const bool aligned4 = (Lk & 3) == 0 && ((reinterpret_cast<uintptr_t>(acc) & 15) | (reinterpret_cast<uintptr_t>(mask) & 3)) == 0;
   const bool aligned = (Lk & 15) == 0 && ((reinterpret_cast<uintptr_t>(acc) & 31) | (reinterpret_cast<uintptr_t>(mask) & 15)) == 0;
@@ -1001,6 +1002,7 @@ held_kernel(const float *__restrict__ acc, const Held p, int diag, unsigned long
     sels[t] = Sel{k_rest, 0u, 0u, 0xffffffffu, 0u, 1, c.y, cta - c.x};
   }
   __syncthreads();
+  allow_next();  // (the list's blocks)
   // ---- keys of this CTA's units
   const bool vec = (Lk & 3) == 0 && (reinterpret_cast<uintptr_t>(acc) & 15) == 0;
 #pragma unroll 1
@@ -1316,9 +1318,8 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
                                                             (unsigned long long)a.k_rest, (unsigned long long)n_rest,
                                                             sc.state);
     if (classify) {
-      emit_kernel<true, 4><<<n_tiles, 128, 0, s>>>(a.acc, a.Lq, a.Lk, n_qt, n_kt, n_tiles, a.causal, diag, 0, 0, sc.state,
-                                                   a.mask, a.stage_bitmap, a.stage_count, a.stage_groups, a.nnz, sc.cand,
-                                                   (uint32_t)cap);
+      e = launch_early(emit_kernel<true, 4>, (unsigned)n_tiles, 128, 0, s, a.acc, a.Lq, a.Lk, n_qt, n_kt, n_tiles, a.causal, diag,
+                       0, 0, sc.state, a.mask, a.stage_bitmap, a.stage_count, a.stage_groups, a.nnz, sc.cand, (uint32_t)cap);
     } else {
       // one wave of CTAs (five fit an SM), so that no SM idles while a second, partial wave runs
       int collect_blocks = ceil_div(rows, kWarps);
@@ -1327,7 +1328,7 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
                                                                      sc.cand, (uint32_t)cap);
     }
     count_launches(2);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
   }
   {
     const int grid = per_sel > 1 ? n_sel * per_sel : n_sel < max_ctas ? n_sel : max_ctas;
@@ -1353,17 +1354,16 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
   // Few tiles: sixteen warps each, so that a tile's rows are all in flight at once.  With the mask written by then (the
   // usual end of a classified selection) the launch only has to look.
   if (n_tiles <= 4 * sms) {
-    emit_kernel<false, 16><<<n_tiles, 512, 0, s>>>(a.acc, a.Lq, a.Lk, n_qt, n_kt, n_tiles, a.causal, diag, a.per_layer,
-                                                   a.keep_ties, sc.state, a.mask, a.stage_bitmap, a.stage_count,
-                                                   a.stage_groups, a.nnz, nullptr, 0u);
+    e = launch_early(emit_kernel<false, 16>, (unsigned)n_tiles, 512, 0, s, a.acc, a.Lq, a.Lk, n_qt, n_kt, n_tiles, a.causal, diag,
+                     a.per_layer, a.keep_ties, sc.state, a.mask, a.stage_bitmap, a.stage_count, a.stage_groups, a.nnz, nullptr, 0u);
   } else {
     const int most = (classify ? 2 : 16) * sms;
-    emit_kernel<false, 4><<<n_tiles < most ? n_tiles : most, 128, 0, s>>>(
-        a.acc, a.Lq, a.Lk, n_qt, n_kt, n_tiles, a.causal, diag, a.per_layer, a.keep_ties, sc.state, a.mask, a.stage_bitmap,
-        a.stage_count, a.stage_groups, a.nnz, nullptr, 0u);
+    e = launch_early(emit_kernel<false, 4>, (unsigned)(n_tiles < most ? n_tiles : most), 128, 0, s, a.acc, a.Lq, a.Lk, n_qt, n_kt,
+                     n_tiles, a.causal, diag, a.per_layer, a.keep_ties, sc.state, a.mask, a.stage_bitmap, a.stage_count,
+                     a.stage_groups, a.nnz, nullptr, 0u);
   }
   count_launches(1);
-  if ((e = cudaGetLastError()) != cudaSuccess || !a.tiles) return e;
+  if (e != cudaSuccess || !a.tiles) return e;
   // the histograms are free by now: the compaction keeps its CTAs' totals there
   return launch_compact_staged(a.stage_bitmap, a.stage_count, a.stage_groups, *a.tiles, reinterpret_cast<int2 *>(sc.hist),
                                (size_t)kHistBuffers * kBins * sizeof(uint32_t) / sizeof(int2), &header->compact_barrier, s);

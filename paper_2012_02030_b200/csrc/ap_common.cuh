@@ -95,9 +95,10 @@ cudaError_t launch_early(void (*kern)(Params...), unsigned grid, unsigned block,
 }
 // By every thread, before it touches global memory: waits until the kernel before in the stream is over and its writes are
 // visible.  After it, the same is allowed to the kernel behind.
+__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  allow_next();
 }
 
 // Kernels launched by this library in this process (see ap_launch_count in ap.h).

@@ -182,9 +182,6 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
   const int qt = n_qt - 1 - (int)(blockIdx.x / BH);  // late query tiles (the longest list rows when causal) first
   const int h = bh % H;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t0 = round_ptr[h * n_qt + qt];
-  const int T = round_ptr[h * n_qt + qt + 1] - t0;  // rounds of this query tile: visits per sweep
-
   if (threadIdx.x == 0) {
     mbar_init(&bars->q_full, 1);
     for (int s = 0; s < kSBufs; ++s) {
@@ -210,6 +207,9 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     tmem_alloc(&bars->tmem_base, kTmemCols);
     tmem_relinquish();
   }
+  after_previous();
+  const int t0 = round_ptr[h * n_qt + qt];
+  const int T = round_ptr[h * n_qt + qt + 1] - t0;  // rounds of this query tile: visits per sweep
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -677,11 +677,10 @@ cudaError_t launch(const Maps &maps, const ap_tiles &t, void *O, int B, int H, i
   auto kern = fwd_entmax_kernel<D, kCtas, kF16>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D, kCtas>::kSmemBytes);
   if (e != cudaSuccess) return e;
-  kern<<<B * H * t.n_qt, kThreads, Cfg<D, kCtas>::kSmemBytes, s>>>(maps, static_cast<uint16_t *>(O), t.round_ptr, t.round_rows,
-                                                           t.round_info, t.round_bitmap, B * H, H, Lq, t.n_qt,
-                                                           0.5f * scale, err);
+  e = launch_early(kern, (unsigned)(B * H * t.n_qt), kThreads, Cfg<D, kCtas>::kSmemBytes, s, maps, static_cast<uint16_t *>(O),
+                   t.round_ptr, t.round_rows, t.round_info, t.round_bitmap, B * H, H, Lq, t.n_qt, 0.5f * scale, err);
   count_launches(1);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace

@@ -651,6 +651,7 @@ __global__ void __launch_bounds__(128) small_list_kernel(const List l, int parts
   __shared__ RowShared sh;
   const int r = threadIdx.x, lane = r & 31, warp = r >> 5;
   const int row = (int)blockIdx.x / parts, part = (int)blockIdx.x % parts, n_grid = l.n_rows * l.n_kt;
+  after_previous();
   for (int x = r; x < l.n_rows; x += 128) slots_s[x] = 0;
   __syncthreads();
   int2 before = make_int2(0, 0);  // tiles and rounds of the list rows before this one
@@ -698,6 +699,7 @@ __global__ void __launch_bounds__(1024) row_sums_kernel(const List l) {
   __shared__ int2 warp_sums[32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5, n_grid = l.n_rows * l.n_kt;
   for (int x = t; x < l.n_rows; x += 1024) rows_s[x] = make_int2(0, 0);
+  after_previous();
   __syncthreads();
   for (int x0 = t; x0 < n_grid; x0 += 8 * 1024) {
     int count[8];
@@ -744,6 +746,7 @@ __global__ void __launch_bounds__(1024) row_sums_kernel(const List l) {
 }
 __global__ void __launch_bounds__(128) rows_kernel(const List l, int parts) {
   __shared__ RowShared sh;
+  after_previous();
   const int row = (int)blockIdx.x / parts, t0 = l.row_ptr[row];
   write_row(l, sh, row, (int)blockIdx.x % parts, parts, t0, l.row_ptr[row + 1] - t0, l.round_ptr[row]);
 }
@@ -1031,16 +1034,14 @@ cudaError_t launch_compact_staged(const uint32_t *stage_bitmap, const int32_t *s
   cudaError_t e;
   if ((long long)n_rows * t.n_kt <= kSmallList && t.cap >= n_rows * t.n_kt) {
     const int parts = grid < n_rows ? 1 : (int)(grid / n_rows);
-    small_list_kernel<<<n_rows * parts, 128, n_rows * sizeof(int), s>>>(l, parts);
-    e = cudaGetLastError();
+    e = launch_early(small_list_kernel, (unsigned)(n_rows * parts), 128, n_rows * sizeof(int), s, l, parts);
   } else if ((long long)n_rows * t.n_kt <= kMediumList && n_rows <= kMediumRows && t.cap >= n_rows * t.n_kt) {
     const int parts = grid < n_rows ? 1 : (int)(grid / n_rows);
     e = cudaFuncSetAttribute(row_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMediumRows * sizeof(int2)));
     if (e != cudaSuccess) return e;
-    row_sums_kernel<<<1, 1024, n_rows * sizeof(int2), s>>>(l);
-    rows_kernel<<<n_rows * parts, 128, 0, s>>>(l, parts);
+    e = launch_early(row_sums_kernel, 1, 1024, n_rows * sizeof(int2), s, l);
+    if (e == cudaSuccess) e = launch_early(rows_kernel, (unsigned)(n_rows * parts), 128, 0, s, l, parts);
     count_launches(1);
-    e = cudaGetLastError();
   } else {
     if (grid > (long long)n_totals) grid = (long long)n_totals;
     int parts = (int)(grid / n_rows);
