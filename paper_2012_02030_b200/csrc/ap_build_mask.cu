@@ -205,6 +205,7 @@ sample_pivots_kernel(const float *__restrict__ acc, int rows, int Lk, int period
   __shared__ uint32_t xch[2];
   __shared__ uint32_t n_valid_s;
   cg::cluster_group cluster = cg::this_cluster();
+  after_previous();
   const int h = blockIdx.x / kSampleCtas, part = blockIdx.x % kSampleCtas, t = threadIdx.x, lane = t & 31;
   if (t == 0) n_valid_s = 0u;
   const int off = (causal || diag) ? Lk - period : 0;
@@ -484,6 +485,7 @@ select_kernel(const float *__restrict__ acc, int rows, int Lk, int period, int c
   __shared__ uint32_t pick_bin, pick_count;
   __shared__ unsigned long long pick_rest;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  after_previous();
   if (nnz)
     for (int x = blockIdx.x * kSelThreads + threadIdx.x; x < H; x += gridDim.x * kSelThreads) nnz[x] = nnz_init;
   const int rank = (int)blockIdx.x % per_sel;
@@ -982,6 +984,7 @@ held_kernel(const float *__restrict__ acc, const Held p, int diag, unsigned long
   const int Lq = p.Lq, Lk = p.Lk, off = (p.causal || diag) ? Lk - Lq : 0;
   const int u0 = p.first_of(cta, ctas), n_units = p.first_of(cta + 1, ctas) - u0;
   const int sel0 = p.sel_of(u0), n_sel = p.sel_of(u0 + n_units - 1) - sel0 + 1;
+  after_previous();
   if (t < n_units) {
     const int h = (u0 + t) / p.per_head, in_head = (u0 + t) - h * p.per_head;
     int qt = 0;
@@ -1002,7 +1005,6 @@ held_kernel(const float *__restrict__ acc, const Held p, int diag, unsigned long
     sels[t] = Sel{k_rest, 0u, 0u, 0xffffffffu, 0u, 1, c.y, cta - c.x};
   }
   __syncthreads();
-  allow_next();  // (the list's blocks)
   // ---- keys of this CTA's units
   const bool vec = (Lk & 3) == 0 && (reinterpret_cast<uintptr_t>(acc) & 15) == 0;
 #pragma unroll 1
@@ -1265,7 +1267,7 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
   // What fits into the shared memory of the SMs is read once and held there.
   Held held = {a.H, a.Lq, a.Lk, n_qt, n_kt, a.causal, a.per_layer, 4 * (int)dense_row_start(n_qt, n_kt, a.Lq, a.Lk, a.causal)};
   if ((long long)a.H * held.per_head <= (long long)kHeldUnits * sms && n_sel <= kMaxSharedSelections && a.k_rest > 0) {
-    cudaError_t e = cudaMemsetAsync(header, 0, (reinterpret_cast<char *>(sc.hist) - reinterpret_cast<char *>(header)) +
+    cudaError_t e = launch_clear(header, (reinterpret_cast<char *>(sc.hist) - reinterpret_cast<char *>(header)) +
                                                    (size_t)n_sel * kHistBuffers * kBins * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
     const int grid = held.total() < sms ? held.total() : sms;
@@ -1283,7 +1285,7 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
     int32_t *stage_count = a.stage_count;
     void *args[] = {&acc, &held, &diag_arg, &k_rest, &sc.state, &sc.hist, &keep_ties, &nnz_init, &nnz, &mask, &stage_bitmap,
                     &stage_count, &stage_groups, &err};
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(held_kernel), dim3(grid), dim3(kHeldThreads), args, smem, s);
+    e = launch_early_cooperative(reinterpret_cast<const void *>(held_kernel), grid, kHeldThreads, args, smem, s);
     if (e != cudaSuccess) return e;
     count_launches(1);
     if (!a.tiles) return cudaSuccess;
@@ -1299,7 +1301,7 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
   if ((long long)per_sel * (kSelThreads / 32) > pieces) per_sel = (int)((pieces + kSelThreads / 32 - 1) / (kSelThreads / 32));
   if (per_sel < 1 || n_sel > kMaxSharedSelections) per_sel = 1;
   const size_t hist_bytes = per_sel > 1 ? (size_t)n_sel * kHistBuffers * kBins * sizeof(uint32_t) : 0;
-  cudaError_t e = cudaMemsetAsync(header, 0, (reinterpret_cast<char *>(sc.hist) - reinterpret_cast<char *>(header)) + hist_bytes, s);
+  cudaError_t e = launch_clear(header, (reinterpret_cast<char *>(sc.hist) - reinterpret_cast<char *>(header)) + hist_bytes, s);
   if (e != cudaSuccess) return e;
   const long long n_valid = domain_size(a.Lq, a.Lk, a.causal);
   const long long n_rest = (n_valid - (diag ? a.Lq : 0)) * (a.per_layer ? a.H : 1);
@@ -1314,9 +1316,9 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
     const size_t smem = (kSamples + kBins) * sizeof(uint32_t);
     e = cudaFuncSetAttribute(sample_pivots_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    sample_pivots_kernel<<<n_sel * kSampleCtas, 1024, smem, s>>>(a.acc, rows, a.Lk, period, a.causal, diag,
-                                                            (unsigned long long)a.k_rest, (unsigned long long)n_rest,
-                                                            sc.state);
+    e = launch_early(sample_pivots_kernel, (unsigned)(n_sel * kSampleCtas), 1024, smem, s, a.acc, rows, a.Lk, period, a.causal, diag,
+                     (unsigned long long)a.k_rest, (unsigned long long)n_rest, sc.state);
+    if (e != cudaSuccess) return e;
     if (classify) {
       e = launch_early(emit_kernel<true, 4>, (unsigned)n_tiles, 128, 0, s, a.acc, a.Lq, a.Lk, n_qt, n_kt, n_tiles, a.causal, diag,
                        0, 0, sc.state, a.mask, a.stage_bitmap, a.stage_count, a.stage_groups, a.nnz, sc.cand, (uint32_t)cap);
@@ -1347,7 +1349,7 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
     void *args[] = {&acc, &rows_arg, &Lk, &period_arg, &causal, &diag_arg, &k_rest, &n_sel_arg, &per_sel_arg, &sc.state,
                     &sc.hist, &cand, &cap_arg, &keep_ties, &H, &nnz_init, &nnz, &classified, &Lq, &n_qt_arg, &n_kt_arg,
                     &mask, &stage_bitmap, &stage_count, &stage_groups, &err};
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(select_kernel), dim3(grid), dim3(kSelThreads), args, 0, s);
+    e = launch_early_cooperative(reinterpret_cast<const void *>(select_kernel), grid, kSelThreads, args, 0, s);
     if (e != cudaSuccess) return e;
     count_launches(1);
   }

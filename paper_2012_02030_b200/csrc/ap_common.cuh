@@ -79,20 +79,36 @@ int sm_count();
 
 // Launches a kernel that begins with after_previous(): its blocks may take the SMs that the kernel before it in the stream has
 // left, set themselves up there and wait.
+struct EarlyLaunch {
+  cudaLaunchAttribute attrs[2];
+  cudaLaunchConfig_t cfg = {};
+  EarlyLaunch(unsigned grid, unsigned block, size_t smem, cudaStream_t s, bool cooperative) {
+    attrs[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attrs[0].val.programmaticStreamSerializationAllowed = 1;
+    attrs[1].id = cudaLaunchAttributeCooperative;
+    attrs[1].val.cooperative = 1;
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attrs;
+    cfg.numAttrs = cooperative ? 2 : 1;
+  }
+};
 template <class... Params, class... Args>
 cudaError_t launch_early(void (*kern)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, Args &&...args) {
-  cudaLaunchAttribute early;
-  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  early.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = &early;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<Args &&>(args)...);
+  const EarlyLaunch l(grid, block, smem, s, false);
+  return cudaLaunchKernelEx(&l.cfg, kern, static_cast<Args &&>(args)...);
 }
+// The same for a cooperative kernel, arguments by address.
+inline cudaError_t launch_early_cooperative(const void *kern, unsigned grid, unsigned block, void **args, size_t smem,
+                                            cudaStream_t s) {
+  const EarlyLaunch l(grid, block, smem, s, true);
+  return cudaLaunchKernelExC(&l.cfg, kern, args);
+}
+// Zeroes a multiple of four bytes: a kernel, since a memset between two kernels would end what launch_early gains.
+cudaError_t launch_clear(void *p, size_t bytes, cudaStream_t s);
+
 // By every thread, before it touches global memory: waits until the kernel before in the stream is over and its writes are
 // visible.  After it, the same is allowed to the kernel behind.
 __device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
