@@ -125,6 +125,8 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     tmem_alloc(&bars->tmem_base, kTmemCols);
     tmem_relinquish();
   }
+  after_previous();
+  bias = from_here(bias);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -417,10 +419,10 @@ cudaError_t launch(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorM
   // samples in ascending order, at most kMaxB per launch; launches on one stream run in order
   for (int b0 = 0; b0 < B; b0 += kMaxB) {
     const int Bc = B - b0 < kMaxB ? B - b0 : kMaxB;
-    kern<<<H * n_qt, kThreads, Cfg<D>::kSmemBytes, s>>>(mq, mk, mb, bias_by_tma, acc, bias, b0, Bc, H, Lq, Lk, n_qt,
-                                                       n_kt, causal, f16, 0.5f * scale, err);
+    e = launch_early(kern, (unsigned)(H * n_qt), kThreads, Cfg<D>::kSmemBytes, s, mq, mk, mb, bias_by_tma, acc, bias, b0, Bc, H, Lq,
+                     Lk, n_qt, n_kt, causal, f16, 0.5f * scale, err);
     count_launches(1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }

@@ -68,6 +68,8 @@ __global__ void __launch_bounds__(kThreads) accumulate_simt_kernel(float *__rest
   const int off = causal ? Lk - Lq : 0;  // causal: row i looks at keys j <= i + (Lk - Lq)
   const int jmax = causal ? min(Lk, i0 + n_rows + off) : Lk;
 
+  after_previous();
+  Q = from_here(Q), K = from_here(K), bias = from_here(bias), acc = from_here(acc);
   const bool wide = (reinterpret_cast<uintptr_t>(K) & 31) == 0;
   for (int b = 0; b < B; ++b) {
     const float *Qb = Q + (((size_t)b * H + h) * Lq + i0) * D;
@@ -178,10 +180,10 @@ cudaError_t launch(float *acc, const void *Q, const void *K, const float *bias, 
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid(ceil_div(Lq, rows), H);
-  kern<<<grid, kThreads, smem, s>>>(acc, static_cast<const float *>(Q), static_cast<const float *>(K), bias, B, H, Lq, Lk,
-                                    rows, causal, scale);
+  e = launch_early(kern, grid, kThreads, smem, s, acc, static_cast<const float *>(Q), static_cast<const float *>(K), bias, B, H,
+                   Lq, Lk, rows, causal, scale);
   count_launches(1);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace

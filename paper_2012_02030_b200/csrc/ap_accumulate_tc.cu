@@ -215,6 +215,7 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     tmem_relinquish();
   }
   after_previous();
+  bias = from_here(bias);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();

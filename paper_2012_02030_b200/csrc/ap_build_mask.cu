@@ -206,6 +206,7 @@ sample_pivots_kernel(const float *__restrict__ acc, int rows, int Lk, int period
   __shared__ uint32_t n_valid_s;
   cg::cluster_group cluster = cg::this_cluster();
   after_previous();
+  acc = from_here(acc);
   const int h = blockIdx.x / kSampleCtas, part = blockIdx.x % kSampleCtas, t = threadIdx.x, lane = t & 31;
   if (t == 0) n_valid_s = 0u;
   const int off = (causal || diag) ? Lk - period : 0;
@@ -486,6 +487,8 @@ select_kernel(const float *__restrict__ acc, int rows, int Lk, int period, int c
   __shared__ unsigned long long pick_rest;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   after_previous();
+  acc = from_here(acc);
+  cand = from_here(cand);
   if (nnz)
     for (int x = blockIdx.x * kSelThreads + threadIdx.x; x < H; x += gridDim.x * kSelThreads) nnz[x] = nnz_init;
   const int rank = (int)blockIdx.x % per_sel;
@@ -833,6 +836,7 @@ __global__ void __launch_bounds__(32 * kCtaWarps, kCtaWarps == 4 ? 8 : 2) emit_k
   __shared__ uint2 stage_all[kClassify ? kCtaWarps : 1][kClassify ? kWarpStage : 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   after_previous();
+  acc = from_here(acc);
   // rows of the scores start on 32-byte boundaries and rows of the mask on 16-byte ones
   const bool aligned4 = (Lk & 3) == 0 && ((reinterpret_cast<uintptr_t>(acc) & 15) | (reinterpret_cast<uintptr_t>(mask) & 3)) == 0;
   const bool aligned = (Lk & 15) == 0 && ((reinterpret_cast<uintptr_t>(acc) & 31) | (reinterpret_cast<uintptr_t>(mask) & 15)) == 0;
@@ -985,6 +989,7 @@ held_kernel(const float *__restrict__ acc, const Held p, int diag, unsigned long
   const int u0 = p.first_of(cta, ctas), n_units = p.first_of(cta + 1, ctas) - u0;
   const int sel0 = p.sel_of(u0), n_sel = p.sel_of(u0 + n_units - 1) - sel0 + 1;
   after_previous();
+  acc = from_here(acc);
   if (t < n_units) {
     const int h = (u0 + t) / p.per_head, in_head = (u0 + t) - h * p.per_head;
     int qt = 0;

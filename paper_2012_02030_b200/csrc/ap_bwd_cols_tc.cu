@@ -151,6 +151,7 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
     tmem_relinquish();
   }
   after_previous();
+  table = from_here(table);
   const bool ordered = n_qt >= kMinOrderedTiles && H * n_kt <= kMaxHeavy && (int64_t)H * n_qt * n_kt <= kMaxTable;
   if (ordered) {
     for (int x = threadIdx.x; x < H * n_kt; x += kThreads) {

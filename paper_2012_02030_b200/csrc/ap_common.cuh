@@ -82,12 +82,12 @@ int sm_count();
 struct EarlyLaunch {
   cudaLaunchAttribute attrs[2];
   cudaLaunchConfig_t cfg = {};
-  EarlyLaunch(unsigned grid, unsigned block, size_t smem, cudaStream_t s, bool cooperative) {
+  EarlyLaunch(dim3 grid, unsigned block, size_t smem, cudaStream_t s, bool cooperative) {
     attrs[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attrs[0].val.programmaticStreamSerializationAllowed = 1;
     attrs[1].id = cudaLaunchAttributeCooperative;
     attrs[1].val.cooperative = 1;
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
@@ -96,7 +96,7 @@ struct EarlyLaunch {
   }
 };
 template <class... Params, class... Args>
-cudaError_t launch_early(void (*kern)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, Args &&...args) {
+cudaError_t launch_early(void (*kern)(Params...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, Args &&...args) {
   const EarlyLaunch l(grid, block, smem, s, false);
   return cudaLaunchKernelEx(&l.cfg, kern, static_cast<Args &&>(args)...);
 }
@@ -105,6 +105,13 @@ inline cudaError_t launch_early_cooperative(const void *kern, unsigned grid, uns
                                             cudaStream_t s) {
   const EarlyLaunch l(grid, block, smem, s, true);
   return cudaLaunchKernelExC(&l.cfg, kern, args);
+}
+// The same pointer, as the compiler sees it only known from here on: loads through a const __restrict__ parameter, which it may
+// take for loads of constant memory, stay behind after_previous().
+template <class T>
+__device__ __forceinline__ T *from_here(T *p) {
+  asm volatile("" : "+l"(p));
+  return p;
 }
 // Zeroes a multiple of four bytes: a kernel, since a memset between two kernels would end what launch_early gains.
 cudaError_t launch_clear(void *p, size_t bytes, cudaStream_t s);

@@ -208,6 +208,7 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     tmem_relinquish();
   }
   after_previous();
+  round_ptr = from_here(round_ptr);  // (the other loads depend on it)
   const int t0 = round_ptr[h * n_qt + qt];
   const int T = round_ptr[h * n_qt + qt + 1] - t0;  // rounds of this query tile: visits per sweep
   tc_fence_before_sync();

@@ -131,6 +131,9 @@ fwd_simt_kernel(const float *__restrict__ Q, const float *__restrict__ K, const 
   const size_t bh = blockIdx.x / n_rt;
   const int i0 = rt * R, qt = i0 / kTile, h = (int)(bh % H);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  after_previous();
+  Q = from_here(Q), K = from_here(K), V = from_here(V);
+  row_ptr = from_here(row_ptr);  // (the list's other arrays are read behind it)
   const int t_begin = row_ptr[h * n_qt + qt], t_end = row_ptr[h * n_qt + qt + 1];
 
   for (int e = threadIdx.x; e < R * CH; e += kThreads) {
@@ -400,6 +403,9 @@ __global__ void __launch_bounds__(kEntmaxThreads) fwd_entmax_simt_kernel(const T
   const int i = qt * kTile + r;
   const size_t bh = (size_t)b * H + h;
 
+  after_previous();
+  Q = from_here(Q), K = from_here(K), V = from_here(V);
+  row_ptr = from_here(row_ptr);  // (the list's other arrays are read behind it)
   float4 q[G], o[G];
 #pragma unroll
   for (int g = 0; g < G; ++g) {
@@ -505,11 +511,11 @@ cudaError_t launch_entmax(const void *Q, const void *K, const void *V, const ap_
   auto kern = fwd_entmax_simt_kernel<T, D>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<B * H * t.n_qt, kEntmaxThreads, smem, s>>>(static_cast<const T *>(Q), static_cast<const T *>(K),
-                                              static_cast<const T *>(V), t.row_ptr, t.col_idx, t.flags, t.bitmap,
-                                              static_cast<T *>(O), H, Lq, Lk, t.n_qt, 0.5f * scale);
+  e = launch_early(kern, (unsigned)(B * H * t.n_qt), kEntmaxThreads, smem, s, static_cast<const T *>(Q), static_cast<const T *>(K),
+                   static_cast<const T *>(V), t.row_ptr, t.col_idx, t.flags, t.bitmap, static_cast<T *>(O), H, Lq, Lk, t.n_qt,
+                   0.5f * scale);
   count_launches(1);
-  return cudaGetLastError();
+  return e;
 }
 
 template <int D, int R>
@@ -520,11 +526,11 @@ cudaError_t launch_rows(const void *Q, const void *K, const void *V, const ap_ti
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int n_rt = ceil_div(Lq, R);
-  kern<<<(unsigned)((int64_t)B * H * n_rt), SimtCfg<D, R>::kThreads, smem, s>>>(
-      static_cast<const float *>(Q), static_cast<const float *>(K), static_cast<const float *>(V), t.row_ptr, t.col_idx,
-      t.flags, t.bitmap, static_cast<float *>(O), H, Lq, Lk, t.n_qt, n_rt, scale);
+  e = launch_early(kern, (unsigned)((int64_t)B * H * n_rt), SimtCfg<D, R>::kThreads, smem, s, static_cast<const float *>(Q),
+                   static_cast<const float *>(K), static_cast<const float *>(V), t.row_ptr, t.col_idx, t.flags, t.bitmap,
+                   static_cast<float *>(O), H, Lq, Lk, t.n_qt, n_rt, scale);
   count_launches(1);
-  return cudaGetLastError();
+  return e;
 }
 
 // Query rows per CTA: the most (they share the K and V copies and the register tile grows) that still

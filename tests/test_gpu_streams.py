@@ -150,33 +150,31 @@ def test_calls_in_a_row_see_each_others_results(dtype, d):
     B, H, L = 5, 7, 300
     gen = torch.Generator().manual_seed(4500 + d)
     q, k, v = (torch.randn((B, H, L, d), generator=gen).to(dtype).cuda() for _ in range(3))
+    grads = [torch.empty_like(q) for _ in range(3)]
     acc = torch.zeros((H, L, L), device="cuda")
     tiles = ap.Tiles(H, L, L)
     mask = torch.zeros((H, L, L), dtype=torch.uint8, device="cuda")
 
     def chain(wait):
         done = torch.cuda.synchronize if wait else lambda: None
-        x, y, a = q.clone(), torch.empty_like(q), acc.clone()
+        x, y, z, a = q.clone(), torch.empty_like(q), torch.empty_like(q), acc.clone()
         out = []
-        for step in range(12):
+        for step in range(12):  # (an output is never one of the same call's inputs)
             ap.ap_accumulate_attention(a, x, k, causal=True), done()
             ap.ap_build_mask(a, 0.2 + 0.05 * (step % 4), True, True, mask, tiles), done()
             ap.ap_sparse_attention_fwd(x, k, v, tiles, y), done()
-            if dtype == torch.float32:
-                ap.ap_sparse_attention_entmax15_fwd(y, k, v, tiles, x), done()
-            else:
-                ap.ap_sparse_attention_entmax15_fwd(y, x, v, tiles, x.clone() if step % 2 else x.new_empty(x.shape)), done()
-                g = ap.ap_sparse_attention_bwd(x, k, v, y, q, tiles)
-                done()
-                out += [t.clone() for t in g]
-                ap.ap_sparse_attention_fwd(y, x, g[0], tiles, x), done()
-            ap.ap_sparse_attention_fwd(x, k, y, tiles, y), done()
-            x, y = y, x
-            out += [x.clone(), y.clone(), mask.clone()]
+            ap.ap_sparse_attention_entmax15_fwd(x, y, v, tiles, z), done()
+            ap.ap_accumulate_attention_entmax15(a, z, y, causal=True), done()
+            if dtype != torch.float32:
+                ap.ap_sparse_attention_bwd(x, k, v, y, z, tiles, *grads), done()
+                out += [t.clone() for t in grads]
+                ap.ap_sparse_attention_fwd(grads[0], y, grads[2], tiles, x), done()
+            ap.ap_sparse_attention_fwd(z, y, v, tiles, x), done()
+            out += [x.clone(), y.clone(), z.clone(), mask.clone()]
         return out + [a]
 
     want = chain(True)
     for _ in range(3):
         got = chain(False)
-        assert all(torch.equal(w.nan_to_num(7.0), g.nan_to_num(7.0)) for w, g in zip(want, got))
+        assert all(torch.equal(w, g) for w, g in zip(want, got))
     assert ap.ap_device_status() == ap.AP_OK
