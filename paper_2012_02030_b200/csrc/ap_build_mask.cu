@@ -961,7 +961,8 @@ struct Held {
 //
 // What bounds it: latency, three times a histogram, its merging into global memory, a barrier of the selection's CTAs and the pick of
 // a digit.  The accumulator is read once; with a scan of it per digit and an emit pass of its own one layer of 16 heads x 512
-// took 60 us, 39 with this kernel, some 20 of them its own (59 with whole tiles instead of quarters, of which a few CTAs then have two).  The first histogram's
+// took 60 us, 39 with this kernel, some 20 of them its own (59 with whole tiles instead of quarters, of which a few CTAs then have two; 32 with
+// the list's and the launches' part shortened as well).  The first histogram's
 // counts fall into few bins (a digit is little more than the exponent), so a warp takes entries of different rows and columns:
 // neighbours, which are alike, would queue for the same bin.
 __global__ void __launch_bounds__(kHeldThreads, 1)
