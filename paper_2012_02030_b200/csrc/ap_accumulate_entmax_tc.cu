@@ -121,25 +121,19 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     for (int s = 0; s < kMaxNewton + 2; ++s) bars->more[s] = 0;
     fence_mbar_init();
   }
-  if (warp == 9) {
-    tmem_alloc(&bars->tmem_base, kTmemCols);
-    tmem_relinquish();
+  if (threadIdx.x == 32 * 8) {
+    prefetch_tensormap(&map_q);
+    prefetch_tensormap(&map_k);
+    if (bias_by_tma) prefetch_tensormap(&map_bias);
   }
-  after_previous();
+  const uint32_t tmem = begin_with_tmem(&bars->tmem_base, kTmemCols, warp == 9);
   bias = from_here(bias);
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = bars->tmem_base;
   volatile int *abort_flag = &bars->abort_flag;
   const Waiter wait{abort_flag, err, kMaxPolls};
 
   if (warp == 8) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      prefetch_tensormap(&map_q);
-      prefetch_tensormap(&map_k);
-      if (bias_by_tma) prefetch_tensormap(&map_bias);
       int v = 0, tl = 0;  // visits issued, bias tiles issued
       bool last = false, ok = true;
       for (int sw = 0; ok; ++sw) {

@@ -210,16 +210,13 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     bars->abort_flag = 0;
     fence_mbar_init();
   }
-  if (warp == kIssuer) {
-    tmem_alloc(&bars->tmem_base, kTmemCols);
-    tmem_relinquish();
+  if (threadIdx.x == 32 * kProducer) {
+    prefetch_tensormap(&map_q);
+    prefetch_tensormap(&map_k);
+    if (bias_by_tma) prefetch_tensormap(&map_bias);
   }
-  after_previous();
+  const uint32_t tmem = begin_with_tmem(&bars->tmem_base, kTmemCols, warp == kIssuer);
   bias = from_here(bias);
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = bars->tmem_base;
   volatile int *abort_flag = &bars->abort_flag;
   const Waiter wait{abort_flag, err, max_polls};
 
@@ -227,9 +224,6 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // ------------------------------------------------------------ TMA producer
     {
       if (lane == 0) {
-        prefetch_tensormap(&map_q);
-        prefetch_tensormap(&map_k);
-        if (bias_by_tma) prefetch_tensormap(&map_bias);
       }
       int v = 0, bias_loads = 0;
       for (; v < n_visits; ++v) {

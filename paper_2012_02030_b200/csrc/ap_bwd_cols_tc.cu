@@ -146,11 +146,16 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
     sh->abort_flag = 0;
     fence_mbar_init();
   }
-  if (warp == kIssuer) {
-    tmem_alloc(&sh->tmem_base, kTmemCols);
-    tmem_relinquish();
+  if (warp == kProducer) {
+    if (lane < 4) {
+      prefetch_tensormap(&maps.k[lane]);
+      prefetch_tensormap(&maps.v[lane]);
+    } else if (lane == 4) {
+      prefetch_tensormap(&maps.q);
+      prefetch_tensormap(&maps.d_o);
+    }
   }
-  after_previous();
+  const uint32_t tmem = begin_with_tmem(&sh->tmem_base, kTmemCols, warp == kIssuer);
   table = from_here(table);
   const bool ordered = n_qt >= kMinOrderedTiles && H * n_kt <= kMaxHeavy && (int64_t)H * n_qt * n_kt <= kMaxTable;
   if (ordered) {
@@ -191,24 +196,14 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
         below += __shfl_sync(0xffffffffu, incl, 31);
       }
     }
+    __syncthreads();
   }
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = sh->tmem_base;
   const Waiter wait{&sh->abort_flag, err, max_polls};
   // accumulators of item n: dV at acc, dK at acc + D
   auto acc_of = [&](uint32_t n) { return tmem + kTmemAcc + (C::kAccBufs == 2u ? 128u * (n & 1u) : 0u); };
 
   if (warp == kProducer) {
     // ------------------------------------------------------------ producer
-    if (lane < 4) {
-      prefetch_tensormap(&maps.k[lane]);
-      prefetch_tensormap(&maps.v[lane]);
-    } else if (lane == 4) {
-      prefetch_tensormap(&maps.q);
-      prefetch_tensormap(&maps.d_o);
-    }
     bool ok = dbg_skip == 0;  // (test hook: nothing is copied, the other roles' waits run out)
     uint32_t g = 0, n = 0;    // visits / items with visits so far
     int k_armed = -1, v_armed = -1;

@@ -152,19 +152,7 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
     sh->abort_flag = 0;
     fence_mbar_init();
   }
-  if (warp == kIssuer) {
-    tmem_alloc(&sh->tmem_base, kTmemCols);
-    tmem_relinquish();
-  }
-  after_previous();
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = sh->tmem_base;
-  const Waiter wait{&sh->abort_flag, err, max_polls};
-
   if (warp == kProducer) {
-    // ------------------------------------------------------------ producer
     if (lane < 4) {
       prefetch_tensormap(&maps.k[lane]);
       prefetch_tensormap(&maps.v[lane]);
@@ -172,6 +160,12 @@ rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ 
       prefetch_tensormap(&maps.q);
       prefetch_tensormap(&maps.d_o);
     }
+  }
+  const uint32_t tmem = begin_with_tmem(&sh->tmem_base, kTmemCols, warp == kIssuer);
+  const Waiter wait{&sh->abort_flag, err, max_polls};
+
+  if (warp == kProducer) {
+    // ------------------------------------------------------------ producer
     bool ok = dbg_skip == 0;  // (test hook: nothing is copied, the other roles' waits run out)
     uint32_t g = 0, n = 0;    // rounds / non-empty items so far
     // The next item is asked for when the current one begins (every CTA begins with the item of its own number) and looked up

@@ -117,10 +117,11 @@ __device__ __forceinline__ T *from_here(T *p) {
 cudaError_t launch_clear(void *p, size_t bytes, cudaStream_t s);
 
 // By every thread, before it touches global memory: waits until the kernel before in the stream is over and its writes are
-// visible.  After it, the same is allowed to the kernel behind.
+// visible.  After it, the same is allowed to the kernel behind.  (Kernels that hold tensor memory: begin_with_tmem.)
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void after_previous() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  wait_previous();
   allow_next();
 }
 

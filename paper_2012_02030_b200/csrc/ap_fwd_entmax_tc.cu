@@ -203,18 +203,17 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     for (int s = 0; s < kMaxNewton + 2; ++s) bars->more[s] = 0;
     fence_mbar_init();
   }
-  if (warp == 9) {
-    tmem_alloc(&bars->tmem_base, kTmemCols);
-    tmem_relinquish();
+  if (threadIdx.x == 32 * 8) {
+    prefetch_tensormap(&maps.q);
+    prefetch_tensormap(&maps.k16);
+    prefetch_tensormap(&maps.k128);
+    prefetch_tensormap(&maps.v16);
+    prefetch_tensormap(&maps.v128);
   }
-  after_previous();
-  round_ptr = from_here(round_ptr);  // (the other loads depend on it)
-  const int t0 = round_ptr[h * n_qt + qt];
-  const int T = round_ptr[h * n_qt + qt + 1] - t0;  // rounds of this query tile: visits per sweep
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = bars->tmem_base;
+  wait_previous();  // (the loads are under way while the columns are taken)
+  const int t0 = (int)ldg_now_u32(round_ptr + h * n_qt + qt), t1 = (int)ldg_now_u32(round_ptr + h * n_qt + qt + 1);
+  const uint32_t tmem = begin_with_tmem(&bars->tmem_base, kTmemCols, warp == 9);
+  const int T = t1 - t0;  // rounds of this query tile: visits per sweep
   volatile int *abort_flag = &bars->abort_flag;
   const Waiter wait{abort_flag, err, kMaxPolls};
 
@@ -236,11 +235,6 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     // rows of the first visits of the next sweep are copied before the rows have decided whether that
     // sweep is the last one: the decision costs no copy latency.
     if (lane == 0) {
-      prefetch_tensormap(&maps.q);
-      prefetch_tensormap(&maps.k16);
-      prefetch_tensormap(&maps.k128);
-      prefetch_tensormap(&maps.v16);
-      prefetch_tensormap(&maps.v128);
       mbar_arrive_expect_tx(&bars->q_full, C::kTileBytes);
 #pragma unroll
       for (int s = 0; s < C::kSub; ++s) tma_load_3d(smem + s * kSubBytes, &maps.q, &bars->q_full, 64 * s, qt * kTile, bh);

@@ -176,15 +176,14 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
     sh->n_items = 0xffffffffu;
     fence_mbar_init();
   }
-  if (warp == 9) {
-    tmem_alloc(&sh->tmem_base, kTmemCols);
-    tmem_relinquish();
+  if (warp == 8) {
+    if (lane < 4) {
+      prefetch_tensormap(&maps.k[lane]);
+      prefetch_tensormap(&maps.v[lane]);
+    }
+    if (lane == 4) prefetch_tensormap(&maps.q);
   }
-  after_previous();
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = sh->tmem_base;
+  const uint32_t tmem = begin_with_tmem(&sh->tmem_base, kTmemCols, warp == 9);
   // The two groups' accumulators of an item.  At d = 64 they take 128 columns together and TMEM has
   // room for two items' worth: items alternate between them, so that the next item's first
   // O += P V need not wait until the epilogue has read this item's result.
@@ -198,11 +197,6 @@ fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
 
   if (warp == 8) {
     // ------------------------------------------------------------ producer
-    if (lane < 4) {
-      prefetch_tensormap(&maps.k[lane]);
-      prefetch_tensormap(&maps.v[lane]);
-    }
-    if (lane == 4) prefetch_tensormap(&maps.q);
     bool ok = true;
     uint32_t g = 0, n = 0;   // rounds / non-empty items so far
     int armed_q = -1;        // non-empty item whose Q copy was armed last

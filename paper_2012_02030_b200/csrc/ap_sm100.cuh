@@ -311,6 +311,25 @@ __device__ __forceinline__ void tc_fence_after_sync() {
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// What a kernel that holds tensor memory has in the place of after_previous(), by all threads of the block behind their
+// set-up (barriers, prefetched tensor maps; `mine` in one warp): returns the address of the block's columns.
+// The order keeps kernels that are launched early from waiting for one another in a ring, whatever shares an SM: an allocation
+// blocks until columns are free, so no block may hold some while it waits for the kernel before (a block of that kernel could be
+// the one that still needs them), and the kernel behind may be set up only when this block has its own.  One thread's
+// launch_dependents counts for the whole block, hence the barrier before it.
+__device__ __forceinline__ uint32_t begin_with_tmem(uint32_t *base, uint32_t ncols, bool mine) {
+  wait_previous();
+  if (mine) {
+    tmem_alloc(base, ncols);
+    tmem_relinquish();
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  allow_next();
+  return *base;
+}
+
 // 32 lanes x 32 bit, 32 consecutive columns: thread i of the warp gets columns
 // [col, col+32) of TMEM lane (lane_base + i).  taddr = (lane_base << 16) | col.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t r[32]) {
