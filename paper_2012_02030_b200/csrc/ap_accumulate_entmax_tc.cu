@@ -85,7 +85,7 @@ template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                          const __grid_constant__ CUtensorMap map_bias, int bias_by_tma, float *__restrict__ acc,
-                         const float *__restrict__ bias, int b0, int Bc, int H, int Lq, int Lk, int n_qt, int n_kt,
+                         const float *bias, int b0, int Bc, int H, int Lq, int Lk, int n_qt, int n_kt,
                          int causal, int f16, float half_scale, unsigned *err) {
   using C = Cfg<D>;
   extern __shared__ unsigned char smem_raw[];
@@ -127,7 +127,6 @@ accumulate_entmax_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     if (bias_by_tma) prefetch_tensormap(&map_bias);
   }
   const uint32_t tmem = begin_with_tmem(&bars->tmem_base, kTmemCols, warp == 9);
-  bias = from_here(bias);
   volatile int *abort_flag = &bars->abort_flag;
   const Waiter wait{abort_flag, err, kMaxPolls};
 

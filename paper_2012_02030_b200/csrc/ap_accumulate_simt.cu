@@ -38,23 +38,23 @@ __device__ __forceinline__ void load_piece(const float *p, float v[kPiece], bool
   if (wide) {
 #pragma unroll
     for (int t = 0; t < kPiece; t += 8)
-      asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                    : "=f"(v[t]), "=f"(v[t + 1]), "=f"(v[t + 2]), "=f"(v[t + 3]), "=f"(v[t + 4]), "=f"(v[t + 5]),
                      "=f"(v[t + 6]), "=f"(v[t + 7])
                    : "l"(p + t));
   } else {
 #pragma unroll
     for (int t = 0; t < kPiece; t += 4)
-      asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+      asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
                    : "=f"(v[t]), "=f"(v[t + 1]), "=f"(v[t + 2]), "=f"(v[t + 3])
                    : "l"(p + t));
   }
 }
 
 template <int D, bool kEntmax>
-__global__ void __launch_bounds__(kThreads) accumulate_simt_kernel(float *__restrict__ acc, const float *__restrict__ Q,
-                                                                   const float *__restrict__ K,
-                                                                   const float *__restrict__ bias, int B, int H,
+__global__ void __launch_bounds__(kThreads) accumulate_simt_kernel(float *__restrict__ acc, const float *Q,
+                                                                   const float *K,
+                                                                   const float *bias, int B, int H,
                                                                    int Lq, int Lk, int rows, int causal,
                                                                    float scale) {
   extern __shared__ __align__(16) float smem[];
@@ -69,7 +69,6 @@ __global__ void __launch_bounds__(kThreads) accumulate_simt_kernel(float *__rest
   const int jmax = causal ? min(Lk, i0 + n_rows + off) : Lk;
 
   after_previous();
-  Q = from_here(Q), K = from_here(K), bias = from_here(bias), acc = from_here(acc);
   const bool wide = (reinterpret_cast<uintptr_t>(K) & 31) == 0;
   for (int b = 0; b < B; ++b) {
     const float *Qb = Q + (((size_t)b * H + h) * Lq + i0) * D;

@@ -154,7 +154,7 @@ template <int D, bool kChunked, int kGroups>
 __global__ void __launch_bounds__(Roles<kGroups>::kRegThreads, 1)
 accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_bias, const __grid_constant__ CUtensorMap map_acc,
-                     int bias_by_tma, int acc_by_tma, float *__restrict__ acc, const float *__restrict__ bias, int b0,
+                     int bias_by_tma, int acc_by_tma, float *__restrict__ acc, const float *bias, int b0,
                      int Bc_all, int chunk_visits, unsigned *__restrict__ turn, int H, int Lq, int Lk, int n_qt,
                      int n_kt, int causal, int f16, float scale_log2, unsigned *err, uint32_t max_polls, int dbg_skip) {
   using C = Cfg<D>;
@@ -216,7 +216,6 @@ accumulate_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     if (bias_by_tma) prefetch_tensormap(&map_bias);
   }
   const uint32_t tmem = begin_with_tmem(&bars->tmem_base, kTmemCols, warp == kIssuer);
-  bias = from_here(bias);
   volatile int *abort_flag = &bars->abort_flag;
   const Waiter wait{abort_flag, err, max_polls};
 

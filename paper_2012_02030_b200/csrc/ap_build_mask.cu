@@ -197,7 +197,7 @@ __device__ uint32_t block_select22(const uint32_t *keys, uint32_t n, uint32_t ra
 // way, and then the histograms (most keys fall into a few bins).  A pair of CTAs that made all draws, in no order: 28 us for 16
 // heads x 2048, 14 of them the draws; 16 x 4096 as a whole 265 us, 259 with a cluster.  32768 draws: 263.
 __global__ void __cluster_dims__(kSampleCtas, 1, 1) __launch_bounds__(1024)
-sample_pivots_kernel(const float *__restrict__ acc, int rows, int Lk, int period, int causal, int diag,
+sample_pivots_kernel(const float *acc, int rows, int Lk, int period, int causal, int diag,
                      unsigned long long k_rest, unsigned long long n_rest, SelectState *state) {
   extern __shared__ uint32_t sm_dyn[];
   uint32_t *keys = sm_dyn;               // kSamples; 0 where a draw was dropped
@@ -206,7 +206,6 @@ sample_pivots_kernel(const float *__restrict__ acc, int rows, int Lk, int period
   __shared__ uint32_t n_valid_s;
   cg::cluster_group cluster = cg::this_cluster();
   after_previous();
-  acc = from_here(acc);
   const int h = blockIdx.x / kSampleCtas, part = blockIdx.x % kSampleCtas, t = threadIdx.x, lane = t & 31;
   if (t == 0) n_valid_s = 0u;
   const int off = (causal || diag) ? Lk - period : 0;
@@ -475,9 +474,9 @@ __device__ __forceinline__ void patch(const uint2 *__restrict__ cand, uint32_t n
 // What bounds it: three times (load latency + a few microseconds of shared-memory histogram + a barrier of about
 // 1.5 us); the passes read from L2.  Two CTAs of 512 threads per SM, so that one's loads run under the other's counting.
 __global__ void __launch_bounds__(kSelThreads, kSelCtasPerSm)
-select_kernel(const float *__restrict__ acc, int rows, int Lk, int period, int causal, int diag,
+select_kernel(const float *acc, int rows, int Lk, int period, int causal, int diag,
               unsigned long long k_rest, int n_sel, int per_sel, SelectState *state, uint32_t *hist,
-              const uint2 *__restrict__ cand, uint32_t cand_cap, int keep_ties, int H, long long nnz_init,
+              const uint2 *cand, uint32_t cand_cap, int keep_ties, int H, long long nnz_init,
               int64_t *__restrict__ nnz, int classified, int Lq, int n_qt, int n_kt, uint8_t *__restrict__ mask,
               uint32_t *__restrict__ stage_bitmap, int32_t *__restrict__ stage_count,
               uint32_t *__restrict__ stage_groups, unsigned *err) {
@@ -487,8 +486,6 @@ select_kernel(const float *__restrict__ acc, int rows, int Lk, int period, int c
   __shared__ unsigned long long pick_rest;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   after_previous();
-  acc = from_here(acc);
-  cand = from_here(cand);
   if (nnz)
     for (int x = blockIdx.x * kSelThreads + threadIdx.x; x < H; x += gridDim.x * kSelThreads) nnz[x] = nnz_init;
   const int rank = (int)blockIdx.x % per_sel;
@@ -822,7 +819,7 @@ __device__ __forceinline__ void emit_rows_by_column(const float *__restrict__ ac
 // left out, and the select adds the collected entries that turn out to be kept.  Only for exact
 // per-head selections (the kept count is known beforehand, nothing is counted here).
 template <bool kClassify, int kCtaWarps>
-__global__ void __launch_bounds__(32 * kCtaWarps, kCtaWarps == 4 ? 8 : 2) emit_kernel(const float *__restrict__ acc, int Lq, int Lk, int n_qt,
+__global__ void __launch_bounds__(32 * kCtaWarps, kCtaWarps == 4 ? 8 : 2) emit_kernel(const float *acc, int Lq, int Lk, int n_qt,
                                                               int n_kt, int n_tiles, int causal, int diag, int per_layer,
                                                               int keep_ties, SelectState *state,
                                                               uint8_t *__restrict__ mask,
@@ -836,7 +833,6 @@ __global__ void __launch_bounds__(32 * kCtaWarps, kCtaWarps == 4 ? 8 : 2) emit_k
   __shared__ uint2 stage_all[kClassify ? kCtaWarps : 1][kClassify ? kWarpStage : 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   after_previous();
-  acc = from_here(acc);
   // rows of the scores start on 32-byte boundaries and rows of the mask on 16-byte ones
   const bool aligned4 = (Lk & 3) == 0 && ((reinterpret_cast<uintptr_t>(acc) & 15) | (reinterpret_cast<uintptr_t>(mask) & 3)) == 0;
   const bool aligned = (Lk & 15) == 0 && ((reinterpret_cast<uintptr_t>(acc) & 31) | (reinterpret_cast<uintptr_t>(mask) & 15)) == 0;
@@ -966,7 +962,7 @@ struct Held {
 // counts fall into few bins (a digit is little more than the exponent), so a warp takes entries of different rows and columns:
 // neighbours, which are alike, would queue for the same bin.
 __global__ void __launch_bounds__(kHeldThreads, 1)
-held_kernel(const float *__restrict__ acc, const Held p, int diag, unsigned long long k_rest, SelectState *state,
+held_kernel(const float *acc, const Held p, int diag, unsigned long long k_rest, SelectState *state,
             uint32_t *hist, int keep_ties, long long nnz_init, int64_t *__restrict__ nnz, uint8_t *__restrict__ mask,
             uint32_t *__restrict__ stage_bitmap, int32_t *__restrict__ stage_count, uint32_t *__restrict__ stage_groups,
             unsigned *err) {
@@ -990,7 +986,6 @@ held_kernel(const float *__restrict__ acc, const Held p, int diag, unsigned long
   const int u0 = p.first_of(cta, ctas), n_units = p.first_of(cta + 1, ctas) - u0;
   const int sel0 = p.sel_of(u0), n_sel = p.sel_of(u0 + n_units - 1) - sel0 + 1;
   after_previous();
-  acc = from_here(acc);
   if (t < n_units) {
     const int h = (u0 + t) / p.per_head, in_head = (u0 + t) - h * p.per_head;
     int qt = 0;

@@ -107,8 +107,8 @@ __device__ __forceinline__ void cp_async4(void *smem_dst, const void *gmem_src) 
 template <int D, bool kF16>
 __global__ void __launch_bounds__(kThreads, 1)
 cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, uint16_t *__restrict__ dV,
-            const float *__restrict__ neg_l, const float *__restrict__ stat_d,
-            const uint32_t *__restrict__ table, const uint32_t *__restrict__ bitmap, int last_tile, int BH, int H, int Lq, int Lk,
+            const float *neg_l, const float *stat_d,
+            const uint32_t *table, const uint32_t *bitmap, int last_tile, int BH, int H, int Lq, int Lk,
             int n_qt, int n_kt, float scale, unsigned *err, uint32_t max_polls, int dbg_skip) {
   using C = Cfg<D>;
   using L = TileLayout<D, false>;
@@ -156,7 +156,6 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
     }
   }
   const uint32_t tmem = begin_with_tmem(&sh->tmem_base, kTmemCols, warp == kIssuer);
-  table = from_here(table);
   const bool ordered = n_qt >= kMinOrderedTiles && H * n_kt <= kMaxHeavy && (int64_t)H * n_qt * n_kt <= kMaxTable;
   if (ordered) {
     for (int x = threadIdx.x; x < H * n_kt; x += kThreads) {
@@ -164,7 +163,7 @@ cols_kernel(const __grid_constant__ ColsMaps maps, uint16_t *__restrict__ dK, ui
       uint32_t c[4] = {0u, 0u, 0u, 0u};  // query tiles per group, two 16-bit counts each
 #pragma unroll 8
       for (int qt = 0; qt < n_qt; ++qt) {
-        const uint32_t gm = __ldg(col + (size_t)qt * n_kt) >> 24;
+        const uint32_t gm = col[(size_t)qt * n_kt] >> 24;
 #pragma unroll
         for (int p = 0; p < 4; ++p) c[p] += ((gm >> (2 * p)) & 1u) | (((gm >> (2 * p + 1)) & 1u) << 16);
       }

@@ -106,10 +106,10 @@ __device__ __forceinline__ void write_table(const ListRows &l, int lr, int lane)
 
 template <int D, bool kSplit, bool kF16>
 __global__ void __launch_bounds__(kThreads, 1)
-rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *__restrict__ O, const uint16_t *__restrict__ dO,
+rows_kernel(const __grid_constant__ RowsMaps maps, const uint16_t *O, const uint16_t *dO,
             uint16_t *__restrict__ dQ, float *__restrict__ neg_l, float *__restrict__ stat_d,
-            const int32_t *__restrict__ round_ptr, const int32_t *__restrict__ round_rows,
-            const uint8_t *__restrict__ round_info, const uint32_t *__restrict__ round_bitmap, const ListRows list, int n_items,
+            const int32_t *round_ptr, const int32_t *round_rows,
+            const uint8_t *round_info, const uint32_t *round_bitmap, const ListRows list, int n_items,
             int H, int Lq, int n_qt, float scale, unsigned *err, uint32_t max_polls, int dbg_skip) {
   using C = Cfg<D, kSplit>;
   using L = TileLayout<D, kSplit>;

@@ -78,7 +78,9 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
 int sm_count();
 
 // Launches a kernel that begins with after_previous(): its blocks may take the SMs that the kernel before it in the stream has
-// left, set themselves up there and wait.
+// left, set themselves up there and wait.  What such a kernel reads may still be written while it is resident, so it is not
+// read-only data in the sense of ld.global.nc: no such loads or __ldg, and no const __restrict__ parameters, which the compiler
+// reads that way, and ahead of the wait if it likes.
 struct EarlyLaunch {
   cudaLaunchAttribute attrs[2];
   cudaLaunchConfig_t cfg = {};
@@ -105,13 +107,6 @@ inline cudaError_t launch_early_cooperative(const void *kern, unsigned grid, uns
                                             cudaStream_t s) {
   const EarlyLaunch l(grid, block, smem, s, true);
   return cudaLaunchKernelExC(&l.cfg, kern, args);
-}
-// The same pointer, as the compiler sees it only known from here on: loads through a const __restrict__ parameter, which it may
-// take for loads of constant memory, stay behind after_previous().
-template <class T>
-__device__ __forceinline__ T *from_here(T *p) {
-  asm volatile("" : "+l"(p));
-  return p;
 }
 // Zeroes a multiple of four bytes: a kernel, since a memset between two kernels would end what launch_early gains.
 cudaError_t launch_clear(void *p, size_t bytes, cudaStream_t s);

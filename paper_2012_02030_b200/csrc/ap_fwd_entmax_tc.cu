@@ -103,13 +103,13 @@ struct Maps {
 // round's descriptor stay in flight while the current round is worked on) ...
 struct RawRound {
   uint32_t info;
-  int4 a, b;
+  uint4 a, b;
 };
 __device__ __forceinline__ RawRound load_round(const int32_t *round_rows, const uint8_t *round_info, int t) {
   RawRound r;
-  r.info = __ldg(round_info + t);
-  r.a = __ldg(reinterpret_cast<const int4 *>(round_rows + (size_t)t * 8));
-  r.b = __ldg(reinterpret_cast<const int4 *>(round_rows + (size_t)t * 8) + 1);
+  r.info = ldg_now_u8(round_info + t);
+  r.a = ldg_now_v4(round_rows + (size_t)t * 8);
+  r.b = ldg_now_v4(round_rows + (size_t)t * 8 + 4);
   return r;
 }
 // ... and decoded: its groups and whether they are eight adjacent ones (one box of 128 rows brings them).
@@ -163,9 +163,9 @@ __device__ __forceinline__ void add_pair(float &s0, float &s1, uint32_t v) {
 
 template <int D, int kCtas, bool kF16>
 __global__ void __launch_bounds__(kThreads, kCtas)
-fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, const int32_t *__restrict__ round_ptr,
-                  const int32_t *__restrict__ round_rows, const uint8_t *__restrict__ round_info,
-                  const uint32_t *__restrict__ round_bitmap, int BH, int H, int Lq, int n_qt, float half_scale,
+fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, const int32_t *round_ptr,
+                  const int32_t *round_rows, const uint8_t *round_info,
+                  const uint32_t *round_bitmap, int BH, int H, int Lq, int n_qt, float half_scale,
                   unsigned *err) {
   using C = Cfg<D, kCtas>;
   constexpr int kSBufs = C::kSBufs;
@@ -315,14 +315,14 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
       const uint32_t v_lo = smem_desc_lo(smem_u32(smem + C::kVOffset), kSubBytes);
       bool ok = wait(&bars->q_full, 0u);
       int v = 0;  // visits whose S has been issued
-      auto ng_of = [&](int vv) { return (int)(__ldg(round_info + t0 + vv) & 15u); };
-      uint32_t info_next = __ldg(round_info + t0);  // used one visit later: the load stays in flight
+      auto ng_of = [&](int vv) { return (int)(ldg_now_u8(round_info + t0 + vv) & 15u); };
+      uint32_t info_next = ldg_now_u8(round_info + t0);  // used one visit later: the load stays in flight
       int vv_next = 0;
       auto issue_qk = [&]() -> bool {
         const int st = v % C::kStages, buf = v % kSBufs;
         const uint32_t idesc_qk = idesc_bf16_f32(128, 16 * (int)(info_next & 15u), false, false, kF16);
         vv_next = vv_next + 1 == T ? 0 : vv_next + 1;
-        info_next = __ldg(round_info + t0 + vv_next);
+        info_next = ldg_now_u8(round_info + t0 + vv_next);
         if (!wait(&bars->in_full[st], (uint32_t)(v / C::kStages) & 1u)) return false;
         // S[buf] was read (and, in the last sweep, its P consumed by a product issued earlier by
         // this thread: products execute in issue order) kSBufs visits ago
@@ -445,8 +445,8 @@ fwd_entmax_kernel(const __grid_constant__ Maps maps, uint16_t *__restrict__ O, c
     // (raw: nothing is computed from the loaded values before the visit that uses them)
     auto fetch = [&](int vv, uint32_t &info, uint2 &bits) {
       const int t = t0 + vv;
-      info = __ldg(round_info + t);
-      bits = __ldg(reinterpret_cast<const uint2 *>(round_bitmap + ((size_t)t * kTile + r) * 4 + 2 * wg));
+      info = ldg_now_u8(round_info + t);
+      bits = ldg_now_v2(round_bitmap + ((size_t)t * kTile + r) * 4 + 2 * wg);
     };
     uint32_t info_next;
     uint2 bits_next;

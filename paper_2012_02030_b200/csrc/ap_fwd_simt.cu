@@ -114,9 +114,9 @@ struct SimtCfg {
 
 template <int D, int R>
 __global__ void __launch_bounds__((SimtCfg<D, R>::kThreads), (SimtCfg<D, R>::kCtas))
-fwd_simt_kernel(const float *__restrict__ Q, const float *__restrict__ K, const float *__restrict__ V,
-                const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col_idx,
-                const uint8_t *__restrict__ flags, const uint32_t *__restrict__ bitmap, float *__restrict__ O, int H,
+fwd_simt_kernel(const float *Q, const float *K, const float *V,
+                const int32_t *row_ptr, const int32_t *col_idx,
+                const uint8_t *flags, const uint32_t *bitmap, float *__restrict__ O, int H,
                 int Lq, int Lk, int n_qt, int n_rt, float scale) {
   using C = SimtCfg<D, R>;
   constexpr int kThreads = C::kThreads;
@@ -132,8 +132,6 @@ fwd_simt_kernel(const float *__restrict__ Q, const float *__restrict__ K, const 
   const int i0 = rt * R, qt = i0 / kTile, h = (int)(bh % H);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   after_previous();
-  Q = from_here(Q), K = from_here(K), V = from_here(V);
-  row_ptr = from_here(row_ptr);  // (the list's other arrays are read behind it)
   const int t_begin = row_ptr[h * n_qt + qt], t_end = row_ptr[h * n_qt + qt + 1];
 
   for (int e = threadIdx.x; e < R * CH; e += kThreads) {
@@ -384,12 +382,12 @@ fwd_simt_kernel(const float *__restrict__ Q, const float *__restrict__ K, const 
 // 5e-7 max(1, |tau|) (at most 30 sweeps), then the sweep that forms the weights and adds p V.
 // Both threads of a row see the same scores and keep the same statistics.
 template <typename T, int D>
-__global__ void __launch_bounds__(kEntmaxThreads) fwd_entmax_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K,
-                                                                   const T *__restrict__ V,
-                                                                   const int32_t *__restrict__ row_ptr,
-                                                                   const int32_t *__restrict__ col_idx,
-                                                                   const uint8_t *__restrict__ flags,
-                                                                   const uint32_t *__restrict__ bitmap,
+__global__ void __launch_bounds__(kEntmaxThreads) fwd_entmax_simt_kernel(const T *Q, const T *K,
+                                                                   const T *V,
+                                                                   const int32_t *row_ptr,
+                                                                   const int32_t *col_idx,
+                                                                   const uint8_t *flags,
+                                                                   const uint32_t *bitmap,
                                                                    T *__restrict__ O, int H, int Lq, int Lk, int n_qt,
                                                                    float half_scale) {
   constexpr int G = D / 8;
@@ -404,8 +402,6 @@ __global__ void __launch_bounds__(kEntmaxThreads) fwd_entmax_simt_kernel(const T
   const size_t bh = (size_t)b * H + h;
 
   after_previous();
-  Q = from_here(Q), K = from_here(K), V = from_here(V);
-  row_ptr = from_here(row_ptr);  // (the list's other arrays are read behind it)
   float4 q[G], o[G];
 #pragma unroll
   for (int g = 0; g < G; ++g) {

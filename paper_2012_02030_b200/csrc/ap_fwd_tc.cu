@@ -139,8 +139,8 @@ struct Shared {
 template <int D, bool kSplit, bool kF16, bool kGath, bool kPairs>
 __global__ void __launch_bounds__(kThreads, 1)
 fwd_tc_kernel(const __grid_constant__ FwdMaps maps, uint16_t *__restrict__ O,
-              const int32_t *__restrict__ round_ptr, const int32_t *__restrict__ round_rows,
-              const uint8_t *__restrict__ round_info, const uint32_t *__restrict__ round_bitmap,
+              const int32_t *round_ptr, const int32_t *round_rows,
+              const uint8_t *round_info, const uint32_t *round_bitmap,
               const Gathered gth, int B, int H, int Lq, int n_qt, float scale_log2, unsigned *err,
               uint32_t max_polls, int dbg_skip) {
   using C = Cfg<D, kSplit>;

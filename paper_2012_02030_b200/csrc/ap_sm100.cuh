@@ -263,27 +263,27 @@ __device__ __forceinline__ void store_sector(uint16_t *p, const uint32_t v[8], b
   }
 }
 
-// Read-only global loads that are issued where they are written: a plain load of read-only data may
-// be moved by the compiler down to its first use, which defeats a load meant as a prefetch into
-// registers (issued one loop iteration ahead of the use).
+// Global loads that are issued where they are written: a plain load may be moved by the compiler down
+// to its first use, which defeats a load meant as a prefetch into registers (issued one loop
+// iteration ahead of the use).
 __device__ __forceinline__ uint4 ldg_now_v4(const void *p) {
   uint4 v;
-  asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }
 __device__ __forceinline__ uint2 ldg_now_v2(const void *p) {
   uint2 v;
-  asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
   return v;
 }
 __device__ __forceinline__ uint32_t ldg_now_u32(const void *p) {
   uint32_t v;
-  asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
 }
 __device__ __forceinline__ uint32_t ldg_now_u8(const void *p) {
   uint32_t v;
-  asm volatile("ld.global.nc.u8 %0, [%1];" : "=r"(v) : "l"(p));
+  asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
 }
 

@@ -64,3 +64,15 @@ def test_tensor_memory_is_taken_between_the_kernel_before_and_the_kernel_behind(
     barrier = re.search(r"__syncthreads\(\)|bar\.sync", body[alloc:])
     allow = body.index("allow_next()")
     assert allow > alloc + barrier.end()
+
+
+@pytest.mark.parametrize("name", EARLY)
+def test_no_parameter_is_declared_read_only(name):
+    """The compiler may read through a const __restrict__ parameter as if nobody wrote there while the kernel is resident."""
+    parameters = KERNELS[name].split("{", 1)[0]
+    assert not re.search(r"const\s+[\w ]+\*\s*__restrict__", parameters)
+
+
+def test_no_load_takes_its_data_for_read_only():
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        assert not re.search(r"\.global\S*\.nc\b|\b__ldg\b", _source(path)), path
