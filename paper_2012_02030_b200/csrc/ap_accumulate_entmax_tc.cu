@@ -414,7 +414,6 @@ cudaError_t launch(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorM
     const int Bc = B - b0 < kMaxB ? B - b0 : kMaxB;
     e = launch_early(kern, (unsigned)(H * n_qt), kThreads, Cfg<D>::kSmemBytes, s, mq, mk, mb, bias_by_tma, acc, bias, b0, Bc, H, Lq,
                      Lk, n_qt, n_kt, causal, f16, 0.5f * scale, err);
-    count_launches(1);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

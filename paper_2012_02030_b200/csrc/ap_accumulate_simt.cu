@@ -181,7 +181,6 @@ cudaError_t launch(float *acc, const void *Q, const void *K, const float *bias, 
   dim3 grid(ceil_div(Lq, rows), H);
   e = launch_early(kern, grid, kThreads, smem, s, acc, static_cast<const float *>(Q), static_cast<const float *>(K), bias, B, H,
                    Lq, Lk, rows, causal, scale);
-  count_launches(1);
   return e;
 }
 

@@ -672,7 +672,6 @@ cudaError_t launch(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorM
     e = launch_early(
         t ? kern_chunked : kern, (unsigned)(knobs.skip_arrive ? 1 : l.grid), R::kThreads, Cfg<D>::kSmemBytes, s, mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, b0, l.samples, l.visits, t, p.H, Lq, Lk, p.n_qt, p.n_kt, causal,
         f16, scale * kLog2e, err, knobs.max_polls, knobs.skip_arrive);
-    count_launches(1);
     if (e != cudaSuccess) return e;
     b0 += l.samples;
   }

@@ -1288,7 +1288,6 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
                     &stage_count, &stage_groups, &err};
     e = launch_early_cooperative(reinterpret_cast<const void *>(held_kernel), grid, kHeldThreads, args, smem, s);
     if (e != cudaSuccess) return e;
-    count_launches(1);
     if (!a.tiles) return cudaSuccess;
     return launch_compact_staged(a.stage_bitmap, a.stage_count, a.stage_groups, *a.tiles, reinterpret_cast<int2 *>(sc.hist),
                                  (size_t)kHistBuffers * kBins * sizeof(uint32_t) / sizeof(int2), &header->compact_barrier, s);
@@ -1329,9 +1328,9 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
       if (collect_blocks > 148 * 5 / n_sel) collect_blocks = max(148 * 5 / n_sel, 1);
       collect_kernel<<<dim3(collect_blocks, n_sel), kThreads, 0, s>>>(a.acc, rows, a.Lk, period, a.causal, diag, sc.state,
                                                                      sc.cand, (uint32_t)cap);
+      e = launched(cudaGetLastError());
     }
-    count_launches(2);
-    if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
   }
   {
     const int grid = per_sel > 1 ? n_sel * per_sel : n_sel < max_ctas ? n_sel : max_ctas;
@@ -1352,7 +1351,6 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
                     &mask, &stage_bitmap, &stage_count, &stage_groups, &err};
     e = launch_early_cooperative(reinterpret_cast<const void *>(select_kernel), grid, kSelThreads, args, 0, s);
     if (e != cudaSuccess) return e;
-    count_launches(1);
   }
   // Few tiles: sixteen warps each, so that a tile's rows are all in flight at once.  With the mask written by then (the
   // usual end of a classified selection) the launch only has to look.
@@ -1365,7 +1363,6 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
                      n_tiles, a.causal, diag, a.per_layer, a.keep_ties, sc.state, a.mask, a.stage_bitmap, a.stage_count,
                      a.stage_groups, a.nnz, nullptr, 0u);
   }
-  count_launches(1);
   if (e != cudaSuccess || !a.tiles) return e;
   // the histograms are free by now: the compaction keeps its CTAs' totals there
   return launch_compact_staged(a.stage_bitmap, a.stage_count, a.stage_groups, *a.tiles, reinterpret_cast<int2 *>(sc.hist),

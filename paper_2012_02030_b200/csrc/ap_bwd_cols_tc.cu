@@ -727,7 +727,6 @@ cudaError_t launch(const ColsMaps &maps, const Args &a) {
       kern, (unsigned)grid, kThreads, C::kSmemBytes, a.s, maps, static_cast<uint16_t *>(a.dK), static_cast<uint16_t *>(a.dV), a.plan.neg_l, a.plan.dsum, a.plan.table,
       a.t->bitmap, a.t->cap > 0 ? a.t->cap - 1 : 0, a.B * a.H, a.H, a.Lq, a.Lk, a.t->n_qt, a.t->n_kt, a.scale, a.err, knobs.max_polls,
       knobs.skip_arrive);
-  count_launches(1);
   return e;
 }
 

@@ -722,7 +722,6 @@ cudaError_t launch(const RowsMaps &maps, const Args &a) {
       kern, (unsigned)grid, kThreads, C::kSmemBytes, a.s, maps, static_cast<const uint16_t *>(a.O), static_cast<const uint16_t *>(a.dO), static_cast<uint16_t *>(a.dQ),
       a.plan.neg_l, a.plan.dsum, a.t->round_ptr, a.t->round_rows, a.t->round_info, a.t->round_bitmap,
       ListRows{a.t->row_ptr, a.t->col_idx, a.t->flags, a.t->groups, a.plan.table, a.t->n_kt}, n_items, a.H, a.Lq, a.t->n_qt, a.scale, a.err, knobs.max_polls, knobs.skip_arrive);
-  count_launches(1);
   return e;
 }
 

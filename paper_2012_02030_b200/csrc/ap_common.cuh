@@ -77,6 +77,18 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
 // SMs of the current device (0 if it cannot be queried).
 int sm_count();
 
+// Kernels launched by this library in this process (see ap_launch_count in ap.h).
+void count_launches(int n);
+// What a launch has returned: counted, or the error, which the runtime also keeps for whoever asks for the last one; a later
+// launch of this thread that is checked that way would take it for its own.
+inline cudaError_t launched(cudaError_t e) {
+  if (e == cudaSuccess)
+    count_launches(1);
+  else
+    cudaGetLastError();
+  return e;
+}
+
 // Launches a kernel that begins with after_previous(): its blocks may take the SMs that the kernel before it in the stream has
 // left, set themselves up there and wait.  What such a kernel reads may still be written while it is resident, so it is not
 // read-only data in the sense of ld.global.nc: no such loads or __ldg, and no const __restrict__ parameters, which the compiler
@@ -100,13 +112,13 @@ struct EarlyLaunch {
 template <class... Params, class... Args>
 cudaError_t launch_early(void (*kern)(Params...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, Args &&...args) {
   const EarlyLaunch l(grid, block, smem, s, false);
-  return cudaLaunchKernelEx(&l.cfg, kern, static_cast<Args &&>(args)...);
+  return launched(cudaLaunchKernelEx(&l.cfg, kern, static_cast<Args &&>(args)...));
 }
 // The same for a cooperative kernel, arguments by address.
 inline cudaError_t launch_early_cooperative(const void *kern, unsigned grid, unsigned block, void **args, size_t smem,
                                             cudaStream_t s) {
   const EarlyLaunch l(grid, block, smem, s, true);
-  return cudaLaunchKernelExC(&l.cfg, kern, args);
+  return launched(cudaLaunchKernelExC(&l.cfg, kern, args));
 }
 // Zeroes a multiple of four bytes: a kernel, since a memset between two kernels would end what launch_early gains.
 cudaError_t launch_clear(void *p, size_t bytes, cudaStream_t s);
@@ -119,9 +131,6 @@ __device__ __forceinline__ void after_previous() {
   wait_previous();
   allow_next();
 }
-
-// Kernels launched by this library in this process (see ap_launch_count in ap.h).
-void count_launches(int n);
 
 // Host: entries kept per head (see ap_build_mask in ap.h).
 int64_t keep_count(int64_t n_valid, int64_t n_forced, double keep_frac);

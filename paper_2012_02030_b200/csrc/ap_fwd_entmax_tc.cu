@@ -674,7 +674,6 @@ cudaError_t launch(const Maps &maps, const ap_tiles &t, void *O, int B, int H, i
   if (e != cudaSuccess) return e;
   e = launch_early(kern, (unsigned)(B * H * t.n_qt), kThreads, Cfg<D, kCtas>::kSmemBytes, s, maps, static_cast<uint16_t *>(O),
                    t.round_ptr, t.round_rows, t.round_info, t.round_bitmap, B * H, H, Lq, t.n_qt, 0.5f * scale, err);
-  count_launches(1);
   return e;
 }
 

@@ -874,7 +874,6 @@ cudaError_t launch_kernel(const FwdMaps &maps, const void *K, const void *V, voi
   e = launch_early(kern, dbg.skip_arrive ? 1 : (n_units < sms ? n_units : ctas), kThreads, C::kSmemBytes, s, maps,
                    static_cast<uint16_t *>(O), t.round_ptr, t.round_rows, t.round_info, t.round_bitmap, gth, B, H, Lq, t.n_qt,
                    scale_log2, err, dbg.max_polls, dbg.skip_arrive);
-  count_launches(1);
   return e;
 }
 

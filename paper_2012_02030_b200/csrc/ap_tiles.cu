@@ -1041,16 +1041,15 @@ cudaError_t launch_compact_staged(const uint32_t *stage_bitmap, const int32_t *s
     if (e != cudaSuccess) return e;
     e = launch_early(row_sums_kernel, 1, 1024, n_rows * sizeof(int2), s, l);
     if (e == cudaSuccess) e = launch_early(rows_kernel, (unsigned)(n_rows * parts), 128, 0, s, l, parts);
-    count_launches(1);
   } else {
     if (grid > (long long)n_totals) grid = (long long)n_totals;
     int parts = (int)(grid / n_rows);
     parts = parts < 1 ? 1 : parts > 8 ? 8 : parts;
     void *args[] = {&l, &parts, &totals, &barrier, &err};
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(compact_kernel), dim3((unsigned)grid), dim3(128), args, 0, s);
+    e = launched(
+        cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(compact_kernel), dim3((unsigned)grid), dim3(128), args, 0, s));
   }
   if (e != cudaSuccess) return e;
-  count_launches(1);
   return launch_options(t, s, true);
 }
 

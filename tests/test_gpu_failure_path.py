@@ -94,3 +94,24 @@ def test_backward_expired_wait_returns_timeout_once_and_the_next_call_is_correct
     for got, want, name in zip((dq, dk, dv), ref, ("dQ", "dK", "dV")):
         err = np.linalg.norm(got.float().cpu().numpy() - want) / np.linalg.norm(want)
         assert err < 1e-2, (name, err)
+
+
+@pytest.mark.gpu
+def test_a_refused_launch_is_that_calls_error_only():
+    """65 536 heads are one more than a grid has rows: the runtime refuses the launch (nothing runs).  The call says so, it is not
+    counted, and the next call of the thread does not report it again."""
+    from paper_2012_02030_b200 import binding as ap
+
+    H = 65536
+    q = torch.zeros((1, H, 1, 64), device="cuda")
+    acc = torch.zeros((H, 1, 1), device="cuda")
+    mask = torch.ones((1, 128, 128), dtype=torch.uint8, device="cuda")
+    tiles = ap.Tiles(1, 128, 128)
+    before = ap.ap_launch_count()
+    status = ap.lib.ap_accumulate_attention(acc.data_ptr(), q.data_ptr(), q.data_ptr(), None, 1, H, 1, 1, 64, ap.AP_F32, 0, 0.0, None)
+    assert status == ap.AP_ERR_CUDA
+    assert ap.ap_launch_count() == before
+    ap.ap_mask_to_tiles(mask, tiles)
+    assert ap.ap_device_status() == ap.AP_OK
+    assert int(tiles.row_ptr[1]) == 1
+    assert float(acc.abs().sum()) == 0.0
