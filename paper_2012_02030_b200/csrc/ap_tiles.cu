@@ -645,7 +645,10 @@ compact_kernel(const List l, int parts, int2 *totals, uint32_t *barrier, unsigne
 
 // The same for lists of at most kSmallList grid tiles that cannot outgrow their capacity, without barriers: every CTA adds up
 // what lies before its list row for itself.  One layer of 16 heads x 512 (256 grid tiles): the mask of such a layer as a whole 39 -> 33 us.
-constexpr int kSmallList = 4096;
+// The limit: each CTA reads all counts, so the work grows with tiles times rows.  Whole masks, in us, here / by the two kernels below /
+// by the cooperative kernel: 4 heads x 1024 (256 tiles) 34.9 / 36.8 / 41.1, 64 heads x 256 (256) 41.0 / 42.1 / 51.9, 512 heads x
+// 64 (512) 65.6 / 65.6 / 78.3, 16 heads x 1 x 4096 (512) 37.9 / 34.9 / 39.0, 64 heads x 1024 (4096) 170 / 161 / 173.
+constexpr int kSmallList = 512;
 __global__ void __launch_bounds__(128) small_list_kernel(const List l, int parts) {
   extern __shared__ int slots_s[];  // [n_rows]: slots of the list rows
   __shared__ RowShared sh;
@@ -693,7 +696,12 @@ __global__ void __launch_bounds__(128) small_list_kernel(const List l, int parts
 // Larger lists that cannot outgrow their capacity: one CTA adds up the tiles and rounds of all list rows, then the rows are
 // written by as many CTAs as there is work for.  Barriers of a thousand CTAs, each an addition to the same word, cost more than
 // the second launch (16 heads x 4096: 23 us in one cooperative kernel, 8 + 10 in two).
-constexpr int kMediumList = 1 << 17, kMediumRows = 8192;
+// The limit: the one CTA's time grows with the tiles, more with those that are stored.  Whole masks, in us, this way / by the
+// cooperative kernel, causal with 5 % kept: 16 heads x 4096 (2^14 tiles) 286 / 296, 32 x 4096 (2^15) 519 / 523, 128 x 2048 (2^15)
+// 580 / 593, 64 x 4096 (2^16) 995 / 1010, 16 x 8192 (2^16) 996 / 992, 32 x 8192 (2^17) 1873 / 1852; every tile stored: 1024 x 256
+// (2^12) 437 / 449, 32 x 4096 (2^15) 796 / 793, 256 x 1 x 16384 (2^15) 193 / 189, 64 x 4096 (2^16) 1632 / 1613, 1024 x 1 x 16384
+// (2^17) 735 / 680.
+constexpr int kMediumList = 1 << 15, kMediumRows = 8192;
 __global__ void __launch_bounds__(1024) row_sums_kernel(const List l) {
   extern __shared__ int2 rows_s[];  // [n_rows]: tiles and slots
   __shared__ int2 warp_sums[32];

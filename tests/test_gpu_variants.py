@@ -334,3 +334,21 @@ def test_build_mask_held_in_shared_memory(ap, H, Lq, Lk, causal, rule, distinct)
     assert np.array_equal(mask.cpu().numpy(), want)
     assert np.array_equal(nnz.cpu().numpy(), want_nnz)
     pu.assert_tiles_equal(tiles.to_host(), orc.mask_to_tiles(want))
+
+
+@pytest.mark.parametrize("H,Lq,Lk", [(128, 129, 200), (57, 300, 300),       # 512 and 513 tiles
+                                     (300, 513, 600),                       # 1500 list rows: sums are carried from 1024 to the next
+                                     (8192, 1, 512), (2731, 8, 1500),    # 32768 and 32772 tiles; the most list rows
+                                     (8193, 1, 130), (8, 1, 262400)])    # more list rows; 2050 tiles to a row
+def test_list_of_every_size(ap, H, Lq, Lk):
+    """The list of a mask, at the limits between the ways of writing it; some rows and tiles are empty."""
+    g = torch.Generator().manual_seed(631 + H)
+    acc = torch.rand((H, Lq, Lk), generator=g)
+    acc[:, :, (Lk // 256) * 128:] *= 0.4  # below the threshold
+    mask = torch.empty(acc.shape, dtype=torch.uint8, device="cuda")
+    tiles = ap.Tiles(H, Lq, Lk)
+    ap.ap_build_mask(acc.cuda(), 0.03, False, False, mask, tiles)
+    assert ap.ap_device_status() == ap.AP_OK
+    want, _ = orc.build_mask(acc.numpy(), 0.03, False, False)
+    assert np.array_equal(mask.cpu().numpy(), want)
+    pu.assert_tiles_equal(tiles.to_host(), orc.mask_to_tiles(want))
