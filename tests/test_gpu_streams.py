@@ -178,3 +178,77 @@ def test_calls_in_a_row_see_each_others_results(dtype, d):
         got = chain(False)
         assert all(torch.equal(w, g) for w, g in zip(want, got))
     assert ap.ap_device_status() == ap.AP_OK
+
+
+def _mask_chain(ap, shape, seed, dtype=torch.bfloat16):
+    """The whole procedure a few times over, each call reading what the one before has written: averages, masks under both rules from
+    the one workspace, both forwards and the backward.  Returns the function (which takes what to do between two calls) and its
+    outputs' buffers."""
+    H, Lq, Lk, causal = shape
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    q, d_o = (torch.randn((1, H, Lq, 64), generator=gen, device="cuda").to(dtype) for _ in range(2))
+    k, v = (torch.randn((1, H, Lk, 64), generator=gen, device="cuda").to(dtype) for _ in range(2))
+    acc = torch.zeros((H, Lq, Lk), device="cuda")
+    ws = torch.empty(ap.ap_build_mask_workspace_bytes(H, Lq, Lk), dtype=torch.uint8, device="cuda")
+    bwd_ws = torch.empty(ap.ap_sparse_attention_bwd_workspace_bytes(1, H, Lq, Lk), dtype=torch.uint8, device="cuda")
+    tiles = ap.Tiles(H, Lq, Lk)
+    rules = [(ap.ap_build_mask, 0.1), (ap.ap_build_mask_layer, 0.02), (ap.ap_build_mask, 0.4)]
+    steps = []
+    for _ in rules:
+        steps.append(dict(x=torch.empty_like(q), y=torch.empty_like(q), grads=[torch.empty_like(t) for t in (q, k, v)],
+                          mask=torch.empty((H, Lq, Lk), dtype=torch.uint8, device="cuda"),
+                          nnz=torch.empty(H, dtype=torch.int64, device="cuda")))
+
+    def run(between):
+        acc.zero_()
+        x = q
+        for (build, keep), s in zip(rules, steps):
+            ap.ap_accumulate_attention(acc, x, k, causal=causal), between()
+            build(acc, keep, causal, causal, s["mask"], tiles, s["nnz"], workspace=ws), between()
+            ap.ap_sparse_attention_fwd(x, k, v, tiles, s["x"]), between()
+            ap.ap_sparse_attention_entmax15_fwd(s["x"], k, v, tiles, s["y"]), between()
+            ap.ap_accumulate_attention_entmax15(acc, s["y"], k, causal=causal), between()
+            ap.ap_sparse_attention_bwd(x, k, v, s["x"], d_o, tiles, *s["grads"], workspace=bwd_ws), between()
+            x = s["y"]
+
+    return run, [acc] + [t for s in steps for t in (s["x"], s["y"], s["mask"], s["nnz"], *s["grads"])]
+
+
+# Entries held in shared memory; selected straight over the accumulator; pivots
+CHAINS = [(3, 300, 300, True), (9, 1024, 1000, False), (4, 1792, 1800, False), (1, 5120, 5120, True), (16, 896, 896 + 448, True)]
+
+
+@pytest.mark.parametrize("shape", CHAINS)
+def test_masks_in_a_row_see_each_others_results(ap, shape):
+    run, out = _mask_chain(ap, shape, 61)
+    run(torch.cuda.synchronize)
+    want = [t.clone() for t in out]
+    for _ in range(3):
+        for t in out[1:]:
+            t.fill_(99)
+        run(lambda: None)
+        assert all(torch.equal(w, g) for w, g in zip(want, out))
+    assert ap.ap_device_status() == ap.AP_OK
+
+
+@pytest.mark.parametrize("shape", CHAINS)
+def test_captured_procedure(ap, shape):
+    """The same calls captured once and replayed, also beside other work on the device."""
+    run, out = _mask_chain(ap, shape, 62)
+    run(torch.cuda.synchronize)
+    want = [t.clone() for t in out]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run(lambda: None)
+    side = torch.cuda.Stream()
+    for beside in (False, True):
+        for t in out[1:]:
+            t.fill_(99)
+        torch.cuda.synchronize()
+        if beside:
+            _busy(side, 0.01)
+        graph.replay()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(w, g) for w, g in zip(want, out))
+    assert ap.ap_device_status() == ap.AP_OK
