@@ -252,3 +252,29 @@ def test_captured_procedure(ap, shape):
         torch.cuda.synchronize()
         assert all(torch.equal(w, g) for w, g in zip(want, out))
     assert ap.ap_device_status() == ap.AP_OK
+
+
+# Entries held in the shared memory of every SM; of eight SMs; pivots
+@pytest.mark.parametrize("shape", [(8, 1280, 1280, True), (2, 256, 256, False), (4, 1792, 1800, False)])
+def test_masks_on_several_streams(ap, shape):
+    """Selections wait for all of their thread blocks.  On several streams at once each finds room for all of them, behind averages
+    that leave the SMs one by one, and gives the bits that it gives alone."""
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    chains = [_mask_chain(ap, shape, 71 + x) for x in range(3)]
+    want = []
+    for run, out in chains:
+        run(torch.cuda.synchronize)
+        want.append([t.clone() for t in out])
+    for _ in range(8):
+        for _, out in chains:
+            for t in out[1:]:
+                t.fill_(99)
+        torch.cuda.synchronize()
+        for _ in range(5):
+            for (run, _), stream in zip(chains, streams):
+                with torch.cuda.stream(stream):
+                    run(lambda: None)
+        torch.cuda.synchronize()
+        assert ap.ap_device_status() == ap.AP_OK
+        for (_, out), ref in zip(chains, want):
+            assert all(torch.equal(w, g) for w, g in zip(ref, out))
