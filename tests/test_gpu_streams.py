@@ -278,3 +278,81 @@ def test_masks_on_several_streams(ap, shape):
         assert ap.ap_device_status() == ap.AP_OK
         for (_, out), ref in zip(chains, want):
             assert all(torch.equal(w, g) for w, g in zip(ref, out))
+
+
+def _blocking_stream():
+    """A stream that the default stream waits for and that waits for the default stream (torch's own do neither)."""
+    from cuda.bindings import runtime
+
+    err, handle = runtime.cudaStreamCreate()
+    assert int(err) == 0
+    return torch.cuda.ExternalStream(int(handle))
+
+
+@pytest.mark.parametrize("how", ["event", "default stream"])
+def test_calls_wait_for_what_other_streams_write(ap, how):
+    """A kernel that may be set up early waits for all that its stream waits for, not only for the kernel before it."""
+    args, grads, ws = _attention(ap, 2, 4, 384, 64, 8)
+    q, k, v, _, d_o, tiles = args
+    other = [torch.randn(q.shape, generator=torch.Generator(device="cuda").manual_seed(90 + x), device="cuda").to(q.dtype)
+             for x in range(4)]
+    out = torch.empty_like(q)
+    x = q.clone()
+    want = [ap.ap_sparse_attention_fwd(t, k, v, tiles) for t in other]
+    side = torch.cuda.Stream() if how == "event" else _blocking_stream()
+    torch.cuda.synchronize()
+    here = torch.cuda.default_stream()
+    for _ in range(3):
+        got = []
+        for t in other:
+            ap.ap_sparse_attention_fwd(x, k, v, tiles, out)
+            if how == "event":
+                side.wait_stream(here)
+            _busy(side, 0.005)
+            with torch.cuda.stream(side):
+                x.copy_(t)
+            if how == "event":
+                here.wait_stream(side)
+            ap.ap_sparse_attention_fwd(x, k, v, tiles, out)
+            got.append(out.clone())
+        torch.cuda.synchronize()
+        assert all(torch.equal(w, g) for w, g in zip(want, got))
+
+
+def test_captured_fork_and_join(ap):
+    """In a captured graph, too: the second call depends on the first one and on another stream's calls."""
+    args, grads, ws = _attention(ap, 2, 4, 384, 64, 9)
+    q, k, v, _, _, tiles = args
+    x, y, z = (torch.empty_like(q) for _ in range(3))
+    acc = torch.zeros((4, 384, 384), device="cuda")
+    mask = torch.empty((4, 384, 384), dtype=torch.uint8, device="cuda")
+    tiles2 = ap.Tiles(4, 384, 384)
+    mask_ws = torch.empty(ap.ap_build_mask_workspace_bytes(4, 384, 384), dtype=torch.uint8, device="cuda")
+    side = torch.cuda.Stream()
+
+    def calls(main):
+        acc.zero_()
+        ap.ap_sparse_attention_fwd(q, k, v, tiles, x)
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            ap.ap_accumulate_attention(acc, x, k, causal=True)
+            ap.ap_build_mask(acc, 0.2, True, True, mask, tiles2, workspace=mask_ws)
+            ap.ap_sparse_attention_fwd(x, k, v, tiles2, z)
+        ap.ap_sparse_attention_fwd(x, k, v, tiles, y)
+        main.wait_stream(side)
+        ap.ap_sparse_attention_fwd(y, z, v, tiles2, x)
+
+    out = [acc, mask, x, y, z]
+    calls(torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    want = [t.clone() for t in out]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        calls(torch.cuda.current_stream())
+    for _ in range(3):
+        for t in out[1:]:
+            t.fill_(99)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(w, g) for w, g in zip(want, out))
+    assert ap.ap_device_status() == ap.AP_OK
