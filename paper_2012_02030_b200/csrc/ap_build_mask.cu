@@ -473,6 +473,9 @@ __device__ __forceinline__ void patch(const uint2 *__restrict__ cand, uint32_t n
 //
 // What bounds it: three times (load latency + a few microseconds of shared-memory histogram + a barrier of about
 // 1.5 us); the passes read from L2.  Two CTAs of 512 threads per SM, so that one's loads run under the other's counting.
+// kCand: the launch has collected entries.  Without any, the scan alone: beside the rest it compiles to slower code (32 heads x
+// 1407, causal: 337 us with it, 291 without).
+template <bool kCand>
 __global__ void __launch_bounds__(kSelThreads, kSelCtasPerSm)
 select_kernel(const float *acc, int rows, int Lk, int period, int causal, int diag,
               unsigned long long k_rest, int n_sel, int per_sel, SelectState *state, uint32_t *hist,
@@ -496,7 +499,7 @@ select_kernel(const float *acc, int rows, int Lk, int period, int causal, int di
       continue;
     }
     // the bracket holds the threshold and every key of the bracket was collected
-    const bool from_cand = st.use_shortcut && st.n_cand <= cand_cap && st.above_hi < k_rest &&
+    const bool from_cand = kCand && st.use_shortcut && st.n_cand <= cand_cap && st.above_hi < k_rest &&
                            k_rest - st.above_hi <= st.n_cand;
     // offsets from the lower pivot, moved up so that the bracket's span begins with the leading digit: the last digits are
     // zero for all, and skipped, where the span is short (as a rule the last one: two digits instead of three)
@@ -1349,7 +1352,8 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
     void *args[] = {&acc, &rows_arg, &Lk, &period_arg, &causal, &diag_arg, &k_rest, &n_sel_arg, &per_sel_arg, &sc.state,
                     &sc.hist, &cand, &cap_arg, &keep_ties, &H, &nnz_init, &nnz, &classified, &Lq, &n_qt_arg, &n_kt_arg,
                     &mask, &stage_bitmap, &stage_count, &stage_groups, &err};
-    e = launch_early_cooperative(reinterpret_cast<const void *>(select_kernel), grid, kSelThreads, args, 0, s);
+    e = launch_early_cooperative(reinterpret_cast<const void *>(shortcut ? select_kernel<true> : select_kernel<false>), grid,
+                                 kSelThreads, args, 0, s);
     if (e != cudaSuccess) return e;
   }
   // Few tiles: sixteen warps each, so that a tile's rows are all in flight at once.  With the mask written by then (the
