@@ -669,9 +669,9 @@ cudaError_t launch(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorM
     const Launch l = plan_launch(p, p.B - b0, R::kMaxB, turn != nullptr);
     unsigned *t = l.visits ? turn : nullptr;
     if (t && (e = launch_clear(t, (size_t)p.H * p.n_qt * p.n_kt * sizeof(unsigned), s)) != cudaSuccess) return e;
-    e = launch_early(
-        t ? kern_chunked : kern, (unsigned)(knobs.skip_arrive ? 1 : l.grid), R::kThreads, Cfg<D>::kSmemBytes, s, mq, mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, b0, l.samples, l.visits, t, p.H, Lq, Lk, p.n_qt, p.n_kt, causal,
-        f16, scale * kLog2e, err, knobs.max_polls, knobs.skip_arrive);
+    e = launch_early(t ? kern_chunked : kern, (unsigned)(knobs.skip_arrive ? 1 : l.grid), R::kThreads, Cfg<D>::kSmemBytes, s, mq,
+                     mk, mb, ma, bias_by_tma, acc_by_tma, acc, bias, b0, l.samples, l.visits, t, p.H, Lq, Lk, p.n_qt, p.n_kt,
+                     causal, f16, scale * kLog2e, err, knobs.max_polls, knobs.skip_arrive);
     if (e != cudaSuccess) return e;
     b0 += l.samples;
   }

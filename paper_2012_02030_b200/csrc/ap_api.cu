@@ -71,7 +71,9 @@ __global__ void __launch_bounds__(256) clear_kernel(uint32_t *p, size_t n) {
 cudaError_t launch_clear(void *p, size_t bytes, cudaStream_t s) {
   const size_t n = bytes / 4, blocks = (n + 1023) / 1024;
   if (n == 0) return cudaSuccess;
-  return launch_early(clear_kernel, (unsigned)(blocks < 148 ? blocks : 148), 256, 0, s, static_cast<uint32_t *>(p), n);
+  const size_t sms = (size_t)sm_count();
+  if (sms == 0) return cudaErrorUnknown;
+  return launch_early(clear_kernel, (unsigned)(blocks < sms ? blocks : sms), 256, 0, s, static_cast<uint32_t *>(p), n);
 }
 
 void count_launches(int n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }

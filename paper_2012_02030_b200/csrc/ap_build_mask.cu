@@ -651,11 +651,11 @@ struct TileSums {
   uint32_t groups, above;
 };
 
-// Tiles all of whose rows and columns exist, lie in the domain and are not forced.  kVec = 8: in arrays whose rows start on
-// 32-byte (scores) and 16-byte (mask) boundaries; 4: on 16-byte and 4-byte ones.  A lane takes 16 consecutive columns of one row, i.e. one group of the
-// tile: its bits are half a bitmap word, its mask bytes one 16-byte store, and where all 16 lie below the bracket (most of
-// them do: it sits near the top of the values) one comparison of their maximum says so.  A warp has four rows under way and
-// the next four loaded ahead.
+// Tiles all of whose rows and columns exist, lie in the domain and are not forced.  kVec = 8: in arrays whose rows
+// start on 32-byte (scores) and 16-byte (mask) boundaries; 4: on 16-byte and 4-byte ones.  A lane takes 16
+// consecutive columns of one row, i.e. one group of the tile: its bits are half a bitmap word, its mask bytes one
+// 16-byte store, and where all 16 lie below the bracket (most of them do: it sits near the top of the values) one
+// comparison of their maximum says so.  A warp has four rows under way and the next four loaded ahead.
 template <bool kClassify, int kCtaWarps, int kVec>
 __device__ __forceinline__ void emit_rows_by_group(const float *__restrict__ acc, int Lq, int Lk, int h, int qt, int kt,
                                                    int tile, const EmitSel &sel, uint8_t *__restrict__ mask,
@@ -811,8 +811,9 @@ __device__ __forceinline__ void emit_rows_by_column(const float *__restrict__ ac
   }
 }
 
-// A CTA per tile of the (h, qt, kt) grid (a CTA takes several in turn where the grid is smaller).  Writes the element mask, the tile's bitmap, popcount and group summary into the staging area.  Values are
-// compared with the threshold as floats (the same order as their keys).  per_layer:
+// A CTA per tile of the (h, qt, kt) grid (a CTA takes several in turn where the grid is smaller).
+// Writes the element mask, the tile's bitmap, popcount and group summary into the staging area.
+// Values are compared with the threshold as floats (the same order as their keys).  per_layer:
 // all heads share selection 0, ties are ordered by (h*Lq + i)*Lk + j, and the
 // tiles' popcounts are added up into nnz[h].  keep_ties: every entry equal to the threshold is
 // kept, and the popcounts are added up as well (the count is not known beforehand).
@@ -938,7 +939,7 @@ __global__ void __launch_bounds__(32 * kCtaWarps, kCtaWarps == 4 ? 8 : 2) emit_k
 constexpr int kHeldThreads = 1024;
 constexpr int kUnitRows = 32, kUnitWords = kUnitRows * kTile;  // a quarter of a 128 x 128 tile: a row per warp
 constexpr int kHeldUnits = 12;                                 // per CTA at most, one CTA per SM
-constexpr int kHeldSels = kHeldUnits / 4 + 1;                  // selections that these belong to (at least four units each), at most
+constexpr int kHeldSels = kHeldUnits / 4 + 1;                  // selections that these belong to at most (four units each or more)
 
 // The units of the domain's tiles, selection by selection, dealt out evenly to the CTAs of the grid.
 struct Held {
@@ -958,12 +959,13 @@ struct Held {
 // Cooperative.  The whole of a call but the compaction in one kernel: every CTA copies its units into shared memory as keys,
 // takes part in the select of the selections they belong to, and writes their mask and bitmaps.
 //
-// What bounds it: latency, three times a histogram, its merging into global memory, a barrier of the selection's CTAs and the pick of
-// a digit.  The accumulator is read once; with a scan of it per digit and an emit pass of its own one layer of 16 heads x 512
-// took 60 us, 39 with this kernel, some 20 of them its own (59 with whole tiles instead of quarters, of which a few CTAs then have two; 32 with
-// the list's and the launches' part shortened as well).  The first histogram's
-// counts fall into few bins (a digit is little more than the exponent), so a warp takes entries of different rows and columns:
-// neighbours, which are alike, would queue for the same bin.
+// What bounds it: latency, three times a histogram, its merging into global memory, a barrier of the selection's CTAs and the
+// pick of a digit.  The accumulator is read once; with a scan of it per digit and an emit pass of its own one layer of
+// 16 heads x 512 took 60 us, 39 with this kernel, some 20 of them its own (59 with whole tiles instead of quarters, of which a
+// few CTAs then have two; 31 with the list's and the launches' part shortened as well).  The first histogram's counts fall into
+// few bins (a digit is little more than the exponent), so a warp takes entries of different rows and columns: neighbours,
+// which are alike, would queue for the same bin.  The price of the shared memory: the CTAs have an SM each to themselves, all of
+// them at once, so beside another stream's kernel that fills the SMs the call begins when that one has left them.
 __global__ void __launch_bounds__(kHeldThreads, 1)
 held_kernel(const float *acc, const Held p, int diag, unsigned long long k_rest, SelectState *state,
             uint32_t *hist, int keep_ties, long long nnz_init, int64_t *__restrict__ nnz, uint8_t *__restrict__ mask,
@@ -1319,8 +1321,8 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
     const size_t smem = (kSamples + kBins) * sizeof(uint32_t);
     e = cudaFuncSetAttribute(sample_pivots_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = launch_early(sample_pivots_kernel, (unsigned)(n_sel * kSampleCtas), 1024, smem, s, a.acc, rows, a.Lk, period, a.causal, diag,
-                     (unsigned long long)a.k_rest, (unsigned long long)n_rest, sc.state);
+    e = launch_early(sample_pivots_kernel, (unsigned)(n_sel * kSampleCtas), 1024, smem, s, a.acc, rows, a.Lk, period, a.causal,
+                     diag, (unsigned long long)a.k_rest, (unsigned long long)n_rest, sc.state);
     if (e != cudaSuccess) return e;
     if (classify) {
       e = launch_early(emit_kernel<true, 4>, (unsigned)n_tiles, 128, 0, s, a.acc, a.Lq, a.Lk, n_qt, n_kt, n_tiles, a.causal, diag,
@@ -1328,7 +1330,7 @@ cudaError_t launch_build_mask(const BuildMaskArgs &a, cudaStream_t s) {
     } else {
       // one wave of CTAs (five fit an SM), so that no SM idles while a second, partial wave runs
       int collect_blocks = ceil_div(rows, kWarps);
-      if (collect_blocks > 148 * 5 / n_sel) collect_blocks = max(148 * 5 / n_sel, 1);
+      if (collect_blocks > sms * 5 / n_sel) collect_blocks = max(sms * 5 / n_sel, 1);
       collect_kernel<<<dim3(collect_blocks, n_sel), kThreads, 0, s>>>(a.acc, rows, a.Lk, period, a.causal, diag, sc.state,
                                                                      sc.cand, (uint32_t)cap);
       e = launched(cudaGetLastError());

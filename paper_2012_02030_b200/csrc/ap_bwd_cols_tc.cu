@@ -723,11 +723,10 @@ cudaError_t launch(const ColsMaps &maps, const Args &a) {
   const DebugKnobs knobs = debug_knobs();
   // (the test hook runs on the first wave only: none of its CTAs takes over another's item)
   const int n_items = a.B * a.H * a.t->n_kt, grid = knobs.skip_arrive && n_items > sms ? sms : n_items;
-  e = launch_early(
-      kern, (unsigned)grid, kThreads, C::kSmemBytes, a.s, maps, static_cast<uint16_t *>(a.dK), static_cast<uint16_t *>(a.dV), a.plan.neg_l, a.plan.dsum, a.plan.table,
-      a.t->bitmap, a.t->cap > 0 ? a.t->cap - 1 : 0, a.B * a.H, a.H, a.Lq, a.Lk, a.t->n_qt, a.t->n_kt, a.scale, a.err, knobs.max_polls,
-      knobs.skip_arrive);
-  return e;
+  return launch_early(kern, (unsigned)grid, kThreads, C::kSmemBytes, a.s, maps, static_cast<uint16_t *>(a.dK),
+                      static_cast<uint16_t *>(a.dV), a.plan.neg_l, a.plan.dsum, a.plan.table, a.t->bitmap,
+                      a.t->cap > 0 ? a.t->cap - 1 : 0, a.B * a.H, a.H, a.Lq, a.Lk, a.t->n_qt, a.t->n_kt, a.scale, a.err,
+                      knobs.max_polls, knobs.skip_arrive);
 }
 
 }  // namespace

@@ -14,12 +14,12 @@
 //
 // Warp roles (704 threads): warps 0-15 compute, 16 producer, 17 issues every MMA, 18-21 form D_i = dO_i . O_i of the
 // NEXT item straight from global memory and write the last item's dQ, -log2 sum and D, and the item's row of the table (as a
-// launch of its own in front the table took 4 of 117 us at 64 x 8 heads, 250 queries, 231 keys, forward and backward).  Sixteen compute warps, because
-// what a round costs a warp is mostly latency (barriers, tensor-memory loads), which four warps per scheduler hide
-// better than two.  TMEM (512 columns): S[2], dP, dQ.  The issuer runs one round ahead: S(g+1) and dP(g+1) are under way
-// while the threads work on round g.  Slots: V of a round is free after its dP, K only after its dQ, so the K that
-// comes kRing rounds later takes V's slot and that round's V takes K's, which gives both copies more than a
-// round's time to arrive.
+// launch of its own in front the table took 4 of 117 us at 64 x 8 heads, 250 queries, 231 keys, forward and backward).
+// Sixteen compute warps, because what a round costs a warp is mostly latency (barriers, tensor-memory loads), which
+// four warps per scheduler hide better than two.  TMEM (512 columns): S[2], dP, dQ.  The issuer runs one round ahead:
+// S(g+1) and dP(g+1) are under way while the threads work on round g.  Slots: V of a round is free after its dP, K
+// only after its dQ, so the K that comes kRing rounds later takes V's slot and that round's V takes K's, which gives
+// both copies more than a round's time to arrive.
 //
 // What bounds it: the threads' chain per round (S -> maximum, exchanged by the row's four warps -> exponentials ->
 // dP -> dS; 1 024 cycles of exponentials, 1 536 of products at d = 128).  The version it replaces had one CTA per query
@@ -718,11 +718,11 @@ cudaError_t launch(const RowsMaps &maps, const Args &a) {
   const DebugKnobs knobs = debug_knobs();
   // (the test hook runs on the first wave only: none of its CTAs takes over another's item)
   const int n_items = a.B * a.H * a.t->n_qt, grid = knobs.skip_arrive && n_items > sms ? sms : n_items;
-  e = launch_early(
-      kern, (unsigned)grid, kThreads, C::kSmemBytes, a.s, maps, static_cast<const uint16_t *>(a.O), static_cast<const uint16_t *>(a.dO), static_cast<uint16_t *>(a.dQ),
-      a.plan.neg_l, a.plan.dsum, a.t->round_ptr, a.t->round_rows, a.t->round_info, a.t->round_bitmap,
-      ListRows{a.t->row_ptr, a.t->col_idx, a.t->flags, a.t->groups, a.plan.table, a.t->n_kt}, n_items, a.H, a.Lq, a.t->n_qt, a.scale, a.err, knobs.max_polls, knobs.skip_arrive);
-  return e;
+  const ListRows list = {a.t->row_ptr, a.t->col_idx, a.t->flags, a.t->groups, a.plan.table, a.t->n_kt};
+  return launch_early(kern, (unsigned)grid, kThreads, C::kSmemBytes, a.s, maps, static_cast<const uint16_t *>(a.O),
+                      static_cast<const uint16_t *>(a.dO), static_cast<uint16_t *>(a.dQ), a.plan.neg_l, a.plan.dsum,
+                      a.t->round_ptr, a.t->round_rows, a.t->round_info, a.t->round_bitmap, list, n_items, a.H, a.Lq, a.t->n_qt,
+                      a.scale, a.err, knobs.max_polls, knobs.skip_arrive);
 }
 
 }  // namespace

@@ -644,10 +644,12 @@ compact_kernel(const List l, int parts, int2 *totals, uint32_t *barrier, unsigne
 }
 
 // The same for lists of at most kSmallList grid tiles that cannot outgrow their capacity, without barriers: every CTA adds up
-// what lies before its list row for itself.  One layer of 16 heads x 512 (256 grid tiles): the mask of such a layer as a whole 39 -> 33 us.
-// The limit: each CTA reads all counts, so the work grows with tiles times rows.  Whole masks, in us, here / by the two kernels below /
-// by the cooperative kernel: 4 heads x 1024 (256 tiles) 34.9 / 36.8 / 41.1, 64 heads x 256 (256) 41.0 / 42.1 / 51.9, 512 heads x
-// 64 (512) 65.6 / 65.6 / 78.3, 16 heads x 1 x 4096 (512) 37.9 / 34.9 / 39.0, 64 heads x 1024 (4096) 170 / 161 / 173.
+// what lies before its list row for itself.  One layer of 16 heads x 512 (256 grid tiles): the mask of such a layer as a whole
+// 39 -> 33 us.
+// The limit: each CTA reads all counts, so the work grows with tiles times rows.  Whole masks, in us, this way / by the two
+// kernels below / by the cooperative kernel: 4 heads x 1024 (256 tiles) 34.9 / 36.8 / 41.1, 64 heads x 256 (256) 41.0 / 42.1 /
+// 51.9, 512 heads x 64 (512) 65.6 / 65.6 / 78.3, 16 heads x 1 x 4096 (512) 37.9 / 34.9 / 39.0, 64 heads x 1024 (4096)
+// 170 / 161 / 173.
 constexpr int kSmallList = 512;
 __global__ void __launch_bounds__(128) small_list_kernel(const List l, int parts) {
   extern __shared__ int slots_s[];  // [n_rows]: slots of the list rows
