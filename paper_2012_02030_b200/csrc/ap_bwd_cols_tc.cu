@@ -32,7 +32,8 @@
 // The first frees dO's slot of visit g, which takes the Q that comes kRing visits later, the second Q's slot,
 // which takes that visit's dO: both copies have a whole visit's time to arrive.
 //
-// What bounds it: a visit takes some 5 600 cycles at 4 x 16 heads x 4096 x 128 (5 % kept; 190 us).  The threads' two phases
+// What bounds it: a visit takes some 6 000 cycles at 4 x 16 heads x 4096 x 128 (5 % kept; 66 visits per SM in 190 us in a stream
+// of calls, in 218 us alone with cold caches; the time between items counted in).  The threads' two phases
 // account for some 2 500 (1 024 of them exponentials), the chain dV(g) -> S^T(g+1) -> P(g+1) that one S^T buffer leaves and
 // the time between items of four to five visits for the rest; the products of a visit take the tensor cores 2 048 cycles at
 // d = 128.  (Sixteen compute warps, one chunk per thread, were slower: 246 against 209 us.)
